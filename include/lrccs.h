@@ -108,8 +108,8 @@ typedef struct lrccs_params {
 /* Launch plan of the transform kernels (tile and grouping choices that do not
  * change the result's definition, only its speed and summation grouping): a
  * zero field keeps the built-in default.
- *   fwd_tx      : image columns per block of the forward column transform
- *                 (even, divides nx, fwd_tx * r <= 256, and fits shared memory)
+ *   fwd_tx      : accepted and kept (plans saved by earlier builds carry it);
+ *                 the forward column transform's tile is fixed
  *   coil_groups : coil groups (thread-block cluster size, 1..8) of the column
  *                 adjoint and the line-mask row passes
  *   row_groups  : coil groups (1..8) of the general-mask row transforms
@@ -451,10 +451,9 @@ lrccs_status lrccs_get_plan(lrccs_ctx *ctx, lrccs_plan *plan);
 
 /* Autotuner of the launch plan (measurement-driven, per problem shape): after
  * lrccs_init, times n_iter iterations (directly launched, CUDA events on the
- * context's stream, best of 2) for every candidate plan -- fwd_tx in {2, 4,
- * 8, 16, 32}, coil_groups in {1, 2, 3, 4, 6, 8} and, for general masks,
- * row_groups in {1, 2, 4, 8}, each within the shape's limits, one field at a
- * time from the defaults -- applies the fastest, and restores the solver
+ * context's stream, best of 2) for every candidate plan -- coil_groups in {1,
+ * 2, 3, 4, 6, 8} and, for general masks, row_groups in {1, 2, 4, 8}, each within
+ * the shape's limits, one field at a time from the defaults -- applies the fastest, and restores the solver
  * state (U, U_{t-1}, B, step size and its schedule, right-hand sides), so the solve continues
  * exactly as if it had not been tuned.  cache_path (NULL: no cache) names a
  * text file of tuned plans, one line per shape (ny nx q C r mask-kind

@@ -93,7 +93,7 @@ static void free_all(lrccs_ctx *c) {
                     c->d_ufrow, c->d_upos, c->d_uidx, c->d_ufptr, c->d_uflist, c->d_fu, c->d_FU, c->d_Pu,
                     c->d_maskc, c->d_mec, c->d_mscal, c->d_mout, c->d_twq, c->d_Q, c->d_gdts, c->d_fpart,
                     c->d_tflag, c->d_tcA0, c->d_tcA1, c->d_tcscale, c->d_ZB, c->d_hpart,
-                    c->d_tcB0, c->d_tcB1};
+                    c->d_tcB0, c->d_tcB1, c->d_twsy, c->d_rowtab};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -174,7 +174,8 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     // against the free device memory before anything is allocated
     const size_t F2 = sizeof(float2), I4 = sizeof(int32_t), D8 = sizeof(double);
     const struct { void **p; size_t bytes; } plan[] = {
-        {(void **)&c->d_twy, ny * F2}, {(void **)&c->d_twx, c->nx * F2}, {(void **)&c->d_smaps, (size_t)nc * n * F2},
+        {(void **)&c->d_twy, ny * F2}, {(void **)&c->d_twx, c->nx * F2},
+        {(void **)&c->d_twsy, ny * F2}, {(void **)&c->d_rowtab, ((size_t)q + 17) * 32 * I4}, {(void **)&c->d_smaps, (size_t)nc * n * F2},
         {(void **)&c->d_rowcnt, (size_t)q * ny * I4}, {(void **)&c->d_rowidx, (size_t)q * ny * I4},
         {(void **)&c->d_framerows, (size_t)q * ny * I4}, {(void **)&c->d_lineptr, ((size_t)q + 1) * I4},
         {(void **)&c->d_rfptr, ((size_t)ny + 1) * I4}, {(void **)&c->d_rflist, (size_t)q * ny * I4},
@@ -254,6 +255,7 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     if (e == cudaSuccess) e = configure_kernels_solve(optin);
     if (e == cudaSuccess) {
         c->nsm = nsm;
+        cudaDeviceGetAttribute(&c->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         for (int rr = 1; rr <= 16; ++rr) c->bs_cap[rr] = rr <= rmax ? bstep_capacity(nc, c->nx, q, rr, optin, nsm) : 0;
     }
     if (e == cudaSuccess && !coop) e = cudaErrorNotSupported;
@@ -263,6 +265,7 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     if (e == cudaSuccess) e = launch_twiddles(c->d_twy, ny, c->stream);
     if (e == cudaSuccess) e = launch_twiddles(c->d_twx, c->nx, c->stream);
     if (e == cudaSuccess) e = launch_twiddles(c->d_twq, q, c->stream);
+    if (e == cudaSuccess) e = launch_col_twiddles(c);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_counters, 0, CNT_COUNT * sizeof(unsigned), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_scal, 0, SC_COUNT * sizeof(double), c->stream);
@@ -1512,14 +1515,7 @@ extern "C" lrccs_status lrccs_autotune(lrccs_ctx *c, int32_t n_iter, const char 
         return LRCCS_E_CUDA;
     }
     // one field at a time, starting from the defaults
-    const int txs[] = {2, 4, 8, 16, 32}, cgs[] = {1, 2, 3, 4, 6, 8}, rgs[] = {1, 2, 4, 8};
-    for (int v : txs) {
-        if (!fwd_tile_ok(v, c->r, c->nx, c->ny, c->dev_smem_optin)) continue;
-        lrccs_plan p = best;
-        p.fwd_tx = v;
-        const double ms = time_plan(c, p, n_iter, st);
-        if (ms >= 0.0 && ms < best_ms) best_ms = ms, best = p;
-    }
+    const int cgs[] = {1, 2, 3, 4, 6, 8}, rgs[] = {1, 2, 4, 8};
     for (int v : cgs) {
         if (v > c->nc) continue;
         lrccs_plan p = best;

@@ -12,8 +12,24 @@
 LRCCS_DEV float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 // conj(a) * b
 LRCCS_DEV float2 cmulc(float2 a, float2 b) { return make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }
-LRCCS_DEV float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-LRCCS_DEV float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// one packed instruction for both parts (the same two roundings): the transform
+// kernels are bound by instruction issue
+LRCCS_DEV float2 cadd(float2 a, float2 b) {
+    float2 d;
+    asm("{\n.reg .b64 a, b, d;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nadd.rn.f32x2 d, a, b;\n"
+        "mov.b64 {%0, %1}, d;\n}\n"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+LRCCS_DEV float2 csub(float2 a, float2 b) {
+    float2 d;
+    asm("{\n.reg .b64 a, b, d;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nsub.rn.f32x2 d, a, b;\n"
+        "mov.b64 {%0, %1}, d;\n}\n"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
 LRCCS_DEV float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 LRCCS_DEV float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 // acc += a * b
@@ -512,27 +528,14 @@ LRCCS_DEV void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "me
 // wait until at most one committed group is still pending (double buffering)
 LRCCS_DEV void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-// ---------------------------------------------------------------- tensor copies (TMA)
-// A 2D tile of a tensor map (cp.async.bulk.tensor) lands in shared memory and
-// completes a transaction count on an mbarrier: one thread arms the barrier
-// with the tile bytes and issues the copies, every thread waits on it.  The
-// wait is bounded: false when it gave up.
+// ---------------------------------------------------------------- bulk copies (TMA)
+// A bulk copy lands in shared memory and completes a transaction count on an
+// mbarrier: one thread arms the barrier with the bytes and issues the copies,
+// every thread waits on it.  The wait is bounded: false when it gave up.
 
 LRCCS_DEV void mbar_init(uint64_t *bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-LRCCS_DEV void mbar_expect_tx(uint64_t *bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-// tile at element coordinates (x, y) of the 2D map into dst (16-byte aligned)
-LRCCS_DEV void tma_load_2d(void *dst, const void *tmap, int x, int y, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-        "[%4];\n" ::"r"(smem_u32(dst)),
-        "l"(tmap), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
 }
 LRCCS_DEV bool mbar_wait(uint64_t *bar, unsigned parity, unsigned limit) {
     unsigned done = 0;

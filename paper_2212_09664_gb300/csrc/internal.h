@@ -102,6 +102,7 @@ struct lrccs_ctx {
     int nblk;          // blocks of the pixel-parallel init kernels
     int gd_grid;       // blocks of the cooperative GD/QR kernel (all resident)
     int nsm;           // multiprocessors of the device
+    int smem_sm;       // shared memory per multiprocessor (bytes)
     int bs_cap[17];    // resident k_bstep<r> blocks for this shape, r = 1..16 (0: rows do not fit)
     int n_used;        // host copy of MT_NUSED
     int n_lines;       // host copy of MT_NLINES
@@ -121,6 +122,8 @@ struct lrccs_ctx {
 
     // geometry / sampling
     float2 *d_twy, *d_twx;       // twiddles w_N^t, N = ny / nx
+    float2 *d_twsy;              // ny: twiddles of the column passes with their scale, [j2][k1]
+    uint32_t *d_rowtab;          // (q + 17) * 32 sampled-row tables of the column passes (k_row_tables)
     float2 *d_smaps;             // nc * n
     int32_t *d_rowcnt;           // q * ny  samples of frame k in row ky
     int32_t *d_rowidx;           // q * ny  line index of row ky in frame k, or -1
@@ -214,8 +217,12 @@ cudaError_t launch_iteration_general_back(lrccs_ctx *c);    // W per sample + in
 cudaError_t launch_fwd_rows(lrccs_ctx *c);
 cudaError_t launch_fwd_rows_r(lrccs_ctx *c, int r);
 cudaError_t launch_adj_rows_r(lrccs_ctx *c, int r);
-cudaError_t launch_fwd_cols_on(lrccs_ctx *c, const float2 *src, int r);   // T <- F_y(d_j o src) (n x r src)
-cudaError_t launch_adj_cols_to(lrccs_ctx *c, float2 *dst, int r);         // dst <- sum_j conj(d_j) F_y^H T_j
+// T <- F_y(d_j o src) (n x r src) on the rows of table entry e0 + l estep (column l), and
+// dst <- sum_j conj(d_j) F_y^H T_j from those rows
+cudaError_t launch_fwd_cols_on(lrccs_ctx *c, const float2 *src, int r, int e0, int estep);
+cudaError_t launch_adj_cols_to(lrccs_ctx *c, float2 *dst, int r, int e0, int estep);
+cudaError_t launch_row_tables(lrccs_ctx *c);
+cudaError_t launch_col_twiddles(lrccs_ctx *c);
 cudaError_t launch_sample_w(lrccs_ctx *c);
 cudaError_t launch_adj_rows(lrccs_ctx *c);
 cudaError_t launch_mean_resid_general(lrccs_ctx *c, const float2 *d_y, float2 *d_ytil);
@@ -255,7 +262,6 @@ cudaError_t launch_cg_init(lrccs_ctx *c, double *cg);
 cudaError_t launch_cg_step(lrccs_ctx *c, double *cg);
 cudaError_t launch_mean_resid(lrccs_ctx *c, const float2 *d_y, float2 *d_ytil, int nl_max);
 int npairs_of(int r);
-bool fwd_tile_ok(int tx, int r, int nx, int ny, int smem_optin);
 
 // Bits of the device status word ctx->d_status.
 enum {

@@ -154,7 +154,7 @@ cudaError_t launch_compact(lrccs_ctx *c, const uint8_t *d_mask, const int64_t *d
                                            c->d_usedrows, c->d_rowused, c->d_mks, c->d_fpk, c->d_rowoff, c->d_meta,
                                            c->d_status, c->d_scal);
     prof_end(c, KID_STRUCTURE);
-    return cudaGetLastError();
+    return launch_row_tables(c);
 }
 
 // Sample indices of masks that are unions of full lines (meta[MT_GENERAL] = 0).

@@ -24,12 +24,12 @@
 //   E k_adj_cols  : F_y^H, conj(d_j) coil sum                      -> Gk
 //   F k_gdqr      : grad = Gk - Z B^H, eta (t = 1), U - eta grad and its
 //                   Cholesky QR, partial sums of the next h = U^H Z, SD (kernels_gd.cu)
-// Tiles are staged into shared memory with cp.async so that each thread keeps
-// many loads in flight; the transforms run on the staged tiles (fft.cuh).
+// The column passes A and E load straight into registers; the row passes stage
+// their rows into shared memory with cp.async.
 #include <cooperative_groups.h>
-#include <cuda.h>   // CUtensorMap and its enums (the encoder is fetched through the runtime)
 #include <math.h>
-#include <string.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "fft.cuh"
@@ -55,76 +55,114 @@ namespace cg = cooperative_groups;
 int npairs_of(int r) { return r * (r + 1) / 2; }
 
 // ---------------------------------------------------------------- A: forward, along y
+//
+// The transforms along y act on the flat columns c = x r + l (rows of nx r
+// complex values) independently, so both column passes tile the flat columns
+// in groups of COLW = 16: a row of a tile is one 128-byte line whatever the
+// rank, and a half-warp holds one row (tiles of 8 columns measured 15.7 / 17.7 us
+// at 192 x 192 but 56 / 68 us at 256 x 256: half-lines).  A block of 16 max(R1, R2) threads
+// (N = R1 R2, fft.cuh) takes one tile through the coils of its group: thread
+// (lane, group g) runs the length-R1 DFT of rows g + R2 m, the groups exchange
+// through shared memory once per coil (one block barrier: two exchange tiles),
+// and thread (lane, g) finishes with the length-R2 DFT of rows g + R1 k2.  The
+// tiles sit in L2 and instruction issue bounds both passes, so every shared
+// address is a constant offset from a per-thread base, the scale rides in the
+// twiddles, and a half-warp stages the coil map's few x of its own rows by
+// cp.async one coil ahead, which needs no further block barrier.
+//
+// Which rows are sampled comes as bit tables (k_row_tables): entry e holds, per
+// group, the rows of pass 2 of the forward transform ([e][0..15]) and of pass 1
+// of the adjoint ([e][16..31]); column l uses entry e0 + l estep.
+#define COLW 16
 
-// The two tensor maps of a k_fwd_cols launch: U (rows of nx r complex, box
-// tx r complex x NY rows) and the coil maps (rows of nx complex over C ny
-// rows, box tx complex x NY rows).
-struct FwdMaps {
-    CUtensorMap u, s;
+// base + off bytes: a uniform base and a 32-bit per-thread offset address without 64-bit arithmetic
+template <class V>
+LRCCS_DEV V *at(V *base, unsigned off) {
+    return (V *)((uintptr_t)base + off);
+}
+
+template <int P>
+struct ColPlan {
+    static constexpr int NY = 32 * P, R1 = fft::Plan<NY>::R1, R2 = fft::Plan<NY>::R2;
+    static constexpr int NG = R1 > R2 ? R1 : R2, NT = COLW * NG;
 };
 
-// With TMA, one thread loads the tile of U and of d_j as two tensor copies
-// (the tile layouts are the boxes' dense row-major layouts); otherwise every
-// thread issues 16-byte cp.async copies.
-template <int P, bool TMA>
-__global__ void __launch_bounds__(256) k_fwd_cols(const float2 *__restrict__ U, const float2 *__restrict__ smaps,
-                                                   const uint8_t *__restrict__ rowused, float2 *__restrict__ T,
-                                                   int nx, int r, int tx, const float2 *__restrict__ g_tw,
-                                                   float scale, const __grid_constant__ FwdMaps maps,
-                                                   unsigned int *status) {
-    constexpr int NY = 32 * P;
-    extern __shared__ __align__(128) float2 smem_raw[];
-    // 128-byte aligned start (a TMA destination); the launch adds 128 bytes of slack
-    float2 *smem = (float2 *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    float2 *tile = smem;                // NY * C
-    float2 *sS = tile + NY * tx * r;    // NY * tx
-    float2 *s_tw = sS + NY * tx;        // NY
-    const int C = tx * r;
-    const int x0 = blockIdx.x * tx, j = blockIdx.y;
-    const size_t n = (size_t)NY * nx;
-    // one copy unit = (row y, 16-byte piece); rows of U are C complex, of d_j tx
-    // complex.  Every loop uses a fixed (column, row-step) thread mapping, so no
-    // per-element division by the runtime row lengths.
-    const int upr = C / 2;
-    const int uc = threadIdx.x % upr, uy = threadIdx.x / upr, ustep = blockDim.x / upr;
-    if constexpr (TMA) {
-        __shared__ __align__(8) uint64_t s_bar;
-        if (threadIdx.x == 0) mbar_init(&s_bar, 1);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            mbar_expect_tx(&s_bar, (unsigned)((NY * C + NY * tx) * sizeof(float2)));
-            tma_load_2d(tile, &maps.u, x0 * r * 2, 0, &s_bar);
-            tma_load_2d(sS, &maps.s, x0 * 2, j * NY, &s_bar);
-        }
-        load_twiddles(s_tw, g_tw, NY);
-        if (!mbar_wait(&s_bar, 0, 1u << 22) && threadIdx.x == 0) atomicOr(status, (unsigned)ST_TIMEOUT);
-        __syncthreads();
-    } else {
-        const int spr = tx / 2;
-        if (uy < ustep)
-            for (int y = uy; y < NY; y += ustep)
-                cp_async16(tile + y * C + 2 * uc, U + ((size_t)y * nx + x0) * r + 2 * uc);
-        {
-            const int sc = threadIdx.x % spr, sy = threadIdx.x / spr, sstep = blockDim.x / spr;
-            if (sy < sstep)
-                for (int y = sy; y < NY; y += sstep)
-                    cp_async16(sS + y * tx + 2 * sc, smaps + (size_t)j * n + (size_t)y * nx + x0 + 2 * sc);
-        }
-        cp_async_commit();
-        load_twiddles(s_tw, g_tw, NY);
-        cp_async_wait();
-        __syncthreads();
-    }
+// x values a tile of COLW flat columns can touch at rank r
+__host__ __device__ inline int col_nxt(int r) { return (COLW - 1 + r - 1) / r + 1; }
 
-    // F_y of d_j o U: the coil multiply happens as pass 1 reads the tile, and
-    // pass 2 stores the sampled rows straight to T
-    float2 *Tj = T + ((size_t)j * n + x0) * r;
-    const size_t rs = (size_t)nx * r;
-    fft::tile_dft_io<NY, false>(
-        tile, C, C, s_tw, [&](int y, int t) { return cmul(sS[y * tx + t / r], tile[y * C + t]); },
-        [&](int t, int ky, float2 v) {
-            if (rowused[ky]) Tj[(size_t)ky * rs + t] = cscale(v, scale);
-        });
+// The coil map at the rows of one group (CNT rows, rowstep apart, from src) and
+// the tile's nxt x values (the nxl of them inside the image), transposed to
+// dst[xi (CNT + 2) + m] (the pad keeps the 16-byte reads of different xi on
+// different banks); inv = ceil(2^16 / nxt).
+template <int CNT>
+LRCCS_DEV void stage_map(float2 *dst, const float2 *src, int rowstep, int nxt, int nxl, unsigned inv, int lane) {
+    for (unsigned e = lane; e < (unsigned)(CNT * nxt); e += COLW) {
+        const unsigned m = (e * inv) >> 16, xi = e - m * nxt;
+        if (xi < (unsigned)nxl) cp_async8(dst + xi * (CNT + 2) + m, src + m * rowstep + xi);
+    }
+}
+
+// Measured (kernel time, L2 warm), TMA-staged tiles of whole columns -> this form:
+// 192 x 192, C = 12, r = 10: 17.9 -> 15.3 us; 256 x 256, C = 20, r = 12: 58 -> 44 us;
+// 256 x 256, C = 32, r = 14: 136 -> 72 us
+template <int P>
+__global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_fwd_cols(
+    const float2 *__restrict__ U, const float2 *__restrict__ smaps, const uint32_t *__restrict__ rowtab, int e0,
+    int estep, float2 *__restrict__ T, int nx, int r, int nc, int nxt, unsigned inv, const float2 *__restrict__ g_tw) {
+    using PL = ColPlan<P>;
+    constexpr int NY = PL::NY, R1 = PL::R1, R2 = PL::R2, NG = PL::NG;
+    extern __shared__ __align__(16) float2 smem[];   // two exchange tiles, two map stages
+    const int lane = threadIdx.x & (COLW - 1), g = threadIdx.x / COLW, CG = gridDim.y;
+    const int rs = nx * r, c = blockIdx.x * COLW + lane, x0 = (int)((unsigned)(blockIdx.x * COLW) / (unsigned)r);
+    const int x = (int)((unsigned)c / (unsigned)r), l = c - x * r;
+    const bool first = R2 == NG || g < R2;
+    uint32_t rows = 0;
+    if (R1 == NG || g < R1) rows = __ldg(rowtab + (e0 + l * estep) * 32 + g);
+    const int mstage = nxt * (R1 + 2);
+    float2 *map = smem + 2 * NY * COLW + g * mstage;
+    const float2 *d = smaps + (size_t)g * nx + x0;
+    const int nxl = min(nxt, nx - x0);   // x values of this tile inside the image
+    float2 u[R1];
+    const unsigned off = (unsigned)(g * rs + c) * sizeof(float2);
+    int j = blockIdx.y;
+    if (first) {
+        stage_map<R1>(map, d + (size_t)j * NY * nx, R2 * nx, nxt, nxl, inv, lane);
+        cp_async_commit();
+#pragma unroll
+        for (int m = 0; m < R1; ++m) u[m] = __ldg(at(U + (size_t)(m * R2) * rs, off));
+    }
+    float2 *ex = smem;
+    for (int s = 0; j < nc; j += CG, s ^= 1) {
+        if (first) {
+            cp_async_wait();
+            __syncwarp();
+            const float4 *m4 = reinterpret_cast<const float4 *>(map + s * NG * mstage + (x - x0) * (R1 + 2));
+            float2 v[R1];
+#pragma unroll
+            for (int m = 0; m < R1; m += 2) {
+                const float4 w = m4[m / 2];
+                v[m] = cmul(make_float2(w.x, w.y), u[m]);
+                v[m + 1] = cmul(make_float2(w.z, w.w), u[m + 1]);
+            }
+            fft::dft_first<R1, R2, false>(v, g, g_tw, [&](int k1, float2 w) { ex[(k1 * R2 + g) * COLW + lane] = w; });
+        }
+        __syncthreads();
+        if (first && j + CG < nc) {
+            stage_map<R1>(map + (s ^ 1) * NG * mstage, d + (size_t)(j + CG) * NY * nx, R2 * nx, nxt, nxl, inv, lane);
+            cp_async_commit();
+        }
+        if (rows != 0) {
+            float2 v[R2];
+#pragma unroll
+            for (int j2 = 0; j2 < R2; ++j2) v[j2] = ex[(g * R2 + j2) * COLW + lane];
+            fft::Dft<R2, false>::run(v);
+            float2 *dst = T + (size_t)j * NY * rs;
+#pragma unroll
+            for (int k2 = 0; k2 < R2; ++k2)
+                if (rows >> k2 & 1) *at(dst + (size_t)(R1 * k2) * rs, off) = v[k2];
+        }
+        ex = ex == smem ? smem + NY * COLW : smem;
+    }
 }
 
 // ---------------------------------------------------------------- B: row Gram
@@ -270,124 +308,110 @@ __global__ void __launch_bounds__(256) k_row_w(float2 *__restrict__ T, const flo
 }
 
 // ---------------------------------------------------------------- E: adjoint, along y + coil sum
-// Gk = sum_j conj(d_j) o F_y^H (column x of coil j's row-transformed K_j);
+// Gk = sum_j conj(d_j) o F_y^H (flat column c of coil j's row-transformed K_j);
 // the - Z B^H term and the Grams are added by k_gdqr (kernels_gd.cu).
 //
-// Grid (nx, CG) in thread-block clusters of (1, CG): block (x, g) handles
-// coils g, g + CG, g + 2 CG, ... of column x and keeps its partial sum in
-// registers; the CG partial tiles are then added through distributed shared
-// memory in rank order (deterministic), each block writing 1/CG of the column.
-
-// (two chunks: registers capped for two blocks per SM; a third block per SM
-// made the one-chunk form slower)
-template <int P, int NCH>   // NCH: pass-2 chunks of the 2r transforms (1 or 2)
-__global__ void __launch_bounds__(256, NCH == 2 ? 2 : 1) k_adj_cols(const float2 *__restrict__ T, const float2 *__restrict__ smaps,
-                                                   const uint8_t *__restrict__ rowused, float2 *__restrict__ Gk,
-                                                   int nx, int r, int nc, const float2 *__restrict__ g_tw,
-                                                   float scale) {
-    constexpr int NY = 32 * P;
-    constexpr int R2 = fft::Plan<NY>::R2;
-    extern __shared__ __align__(16) float2 smem[];
-    // two coils per transform call: tile[y][c r + l], c = 0, 1 (two buffers)
-    float2 *tile0 = smem;                 // NY * 2r
-    float2 *tile1 = tile0 + NY * 2 * r;
-    float2 *sS0 = tile1 + NY * 2 * r;     // 2 NY (two buffers)
-    float2 *sS1 = sS0 + 2 * NY;
-    float2 *s_tw = sS1 + 2 * NY;          // NY
+// Grid (flat-column tiles, CG) in thread-block clusters of (1, CG): block
+// (tile, g) transforms coils g, g + CG, ... in turn and keeps its coil sum in
+// registers; the CG partial tiles are added through distributed shared memory
+// in rank order (deterministic), each block writing 1/CG of the tile.  Each
+// half-warp stages its own rows of T (and of the coil map) by cp.async while
+// the previous coil's second half runs, and transforms them in place: the
+// first half's output k1 replaces row g + R2 k1.  Rows that the tables leave
+// out are zero and not read.
+// Measured (kernel time, L2 warm), one image column per block staged by 8-byte
+// cp.async -> this form: 192 x 192, C = 12, r = 10: 28.9 -> 17.4 us; 256 x 256,
+// C = 20, r = 12: 121 -> 65 us; 256 x 256, C = 32, r = 14: 291 -> 114 us
+template <int P>
+__global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_adj_cols(
+    const float2 *__restrict__ T, const float2 *__restrict__ smaps, const uint32_t *__restrict__ rowtab, int e0,
+    int estep, float2 *__restrict__ Gk, int nx, int r, int nc, int nxt, unsigned inv, const float2 *__restrict__ g_tw) {
+    using PL = ColPlan<P>;
+    constexpr int NY = PL::NY, R1 = PL::R1, R2 = PL::R2, NG = PL::NG;
+    extern __shared__ __align__(16) float2 smem[];   // two tiles of NY x COLW, two map stages
     cg::cluster_group cluster = cg::this_cluster();
-    const int x = blockIdx.x, g = blockIdx.y, CG = gridDim.y;
-    const size_t n = (size_t)NY * nx;
-    const int cnt = NY * r, r2 = 2 * r;
-    // rows that no frame samples are zero-filled
-    __shared__ uint8_t s_used[32 * 8];
-    for (int y = threadIdx.x; y < NY; y += blockDim.x) s_used[y] = rowused[y];
-    // staging map: thread -> rank index l, rows y0, y0 + ystep, ...
-    const int sl = threadIdx.x % r, sy0 = threadIdx.x / r, systep = blockDim.x / r;
-    // pass-2 accumulators: conj(d_j) F_y^H of every coil of this block, per
-    // (chunk, k2) output of tile_dft_acc (a fixed (t, row) per thread)
-    float2 acc[NCH][R2];
+    const int lane = threadIdx.x & (COLW - 1), g = threadIdx.x / COLW, grp = blockIdx.y, CG = gridDim.y;
+    const int rs = nx * r, c0 = blockIdx.x * COLW, c = c0 + lane, x0 = (int)((unsigned)c0 / (unsigned)r);
+    const int x = (int)((unsigned)c / (unsigned)r), l = c - x * r;
+    const bool first = R2 == NG || g < R2, second = R1 == NG || g < R1;
+    const uint32_t rows = first ? __ldg(rowtab + (e0 + l * estep) * 32 + 16 + g) : 0u;
+    // rows either column of the lane pair needs: the pair's 16-byte pieces
+    const uint32_t prow = (rows | __shfl_xor_sync(0xffffffffu, rows, 1)) >> (lane & 1);
+    const size_t plane = (size_t)NY * rs;
+    const unsigned off = (unsigned)((g + R2 * (lane & 1)) * rs + c0 + (lane & ~1)) * sizeof(float2);
+    const int mstage = nxt * (R2 + 2);
+    float2 *map = smem + 2 * NY * COLW + g * mstage;
+    const float2 *d = smaps + (size_t)g * nx + x0;
+    const int nxl = min(nxt, nx - x0);   // x values of this tile inside the image
+    float2 acc[R2];
 #pragma unroll
-    for (int ch = 0; ch < NCH; ++ch)
+    for (int k2 = 0; k2 < R2; ++k2) acc[k2] = make_float2(0.f, 0.f);
+    auto stage = [&](int j, int s) {
+        if (first) {
+            float2 *dst = smem + s * NY * COLW + (g + R2 * (lane & 1)) * COLW + (lane & ~1);
+            const float2 *sj = T + j * plane;
 #pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) acc[ch][k2] = make_float2(0.f, 0.f);
-    __syncthreads();
-    // coils of this block: g, g + CG, g + 2 CG, ...; step s takes the pair (2s, 2s + 1) of them
-    const int mine = g < nc ? (nc - 1 - g) / CG + 1 : 0;
-    const int steps = (mine + 1) / 2;
-    auto stage = [&](float2 *tile, float2 *sS, int s) {
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int m = 2 * s + c;
-            const int j = g + m * CG;
-            const bool live = m < mine;
-            const float2 *Tj = T + (size_t)j * n * r + (size_t)x * r;
-            if (sy0 < systep)
-                for (int y = sy0; y < NY; y += systep) {
-                    float2 *dst = tile + y * r2 + c * r + sl;
-                    if (live && s_used[y]) cp_async8(dst, Tj + (size_t)y * nx * r + sl);
-                    else *dst = make_float2(0.f, 0.f);
-                }
-            for (int y = threadIdx.x; y < NY; y += blockDim.x) {
-                if (live) cp_async8(sS + c * NY + y, smaps + (size_t)j * n + (size_t)y * nx + x);
-                else sS[c * NY + y] = make_float2(0.f, 0.f);
-            }
+            for (int m = 0; m < R1; m += 2)
+                if (prow >> m & 1) cp_async16(dst + m * R2 * COLW, at(sj + (size_t)(m * R2) * rs, off));
         }
+        if (second) stage_map<R2>(map + s * NG * mstage, d + (size_t)j * NY * nx, R1 * nx, nxt, nxl, inv, lane);
         cp_async_commit();
     };
-    if (steps > 0) stage(tile0, sS0, 0);
-    load_twiddles(s_tw, g_tw, NY);
-    for (int s = 0; s < steps; ++s) {
-        float2 *tile = (s & 1) ? tile1 : tile0;
-        float2 *sS = (s & 1) ? sS1 : sS0;
-        if (s + 1 < steps) {
-            stage((s & 1) ? tile0 : tile1, (s & 1) ? sS0 : sS1, s + 1);
-            cp_async_wait_1();
-        } else {
-            cp_async_wait();
+    if (grp < nc) stage(grp, 0);
+    int s = 0;
+    for (int j = grp; j < nc; j += CG, s ^= 1) {
+        float2 *sm = smem + s * NY * COLW + lane;
+        cp_async_wait();
+        __syncwarp();
+        if (first) {
+            float2 v[R1];
+#pragma unroll
+            for (int m = 0; m < R1; ++m) v[m] = (rows >> m & 1) ? sm[(g + R2 * m) * COLW] : make_float2(0.f, 0.f);
+            fft::dft_first<R1, R2, true>(v, g, g_tw, [&](int k1, float2 w) { sm[(g + R2 * k1) * COLW] = w; });
         }
         __syncthreads();
-        fft::tile_dft_acc<NY, true, NCH>(tile, r2, r2, s_tw, [&](int ch, int k2, int t, int y, float2 v) {
-            cfmac(acc[ch][k2], sS[(t >= r ? NY : 0) + y], cscale(v, scale));
-        });
-        __syncthreads();
+        if (j + CG < nc) stage(j + CG, s ^ 1);
+        if (second) {
+            float2 v[R2];
+#pragma unroll
+            for (int j2 = 0; j2 < R2; ++j2) v[j2] = sm[(g * R2 + j2) * COLW];
+            fft::Dft<R2, true>::run(v);
+            const float4 *m4 = reinterpret_cast<const float4 *>(map + s * NG * mstage + (x - x0) * (R2 + 2));
+#pragma unroll
+            for (int k2 = 0; k2 < R2; k2 += 2) {
+                const float4 w = m4[k2 / 2];
+                cfmac(acc[k2], make_float2(w.x, w.y), v[k2]);
+                cfmac(acc[k2 + 1], make_float2(w.z, w.w), v[k2 + 1]);
+            }
+        }
     }
-    // this block's partial column: the two coil halves added, into tile0[y r + l]
-    fft::tile_dft_acc_slots<NY, NCH>(r2, [&](int ch, int k2, int t, int y) { tile1[y * r2 + t] = acc[ch][k2]; });
+    if (CG == 1) {
+        if (second) {
+#pragma unroll
+            for (int k2 = 0; k2 < R2; ++k2) Gk[(size_t)(R1 * k2 + g) * rs + c] = acc[k2];
+        }
+        return;
+    }
     __syncthreads();
-    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-        const int y = e / r, l = e - y * r;
-        tile0[e] = cadd(tile1[y * r2 + l], tile1[y * r2 + r + l]);
+    if (second) {
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) smem[(g + R1 * k2) * COLW + lane] = acc[k2];
     }
     cluster.sync();
-    const int per = (cnt + CG - 1) / CG;
-    const int e0 = g * per, e1 = min(cnt, e0 + per);
-    for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+    // rows y = grp, grp + CG, ... of the tile, by half-warps
+    for (int y = grp + CG * g; y < NY; y += CG * NG) {
         float2 sum = make_float2(0.f, 0.f);
-        for (int k = 0; k < CG; ++k) sum = cadd(sum, cluster.map_shared_rank(tile0, k)[e]);
-        const int y = e / r, l = e - y * r;
-        Gk[((size_t)y * nx + x) * r + l] = sum;
+        for (int k = 0; k < CG; ++k) sum = cadd(sum, cluster.map_shared_rank(smem, k)[y * COLW + lane]);
+        Gk[(size_t)y * rs + c] = sum;
     }
     cluster.sync();   // no block leaves while its tile may still be read
 }
 
 // ---------------------------------------------------------------- launchers
 
-// Columns per k_fwd_cols tile: even, and tx r <= 64 when possible; or the
-// context's tuned plan (lrccs_autotune / lrccs_set_plan) when it fits.
-bool fwd_tile_ok(int tx, int r, int nx, int ny, int smem_optin) {
-    const size_t smem = ((size_t)ny * tx * r + (size_t)ny * tx + ny) * sizeof(float2) + 128;
-    return tx >= 2 && (tx & 1) == 0 && nx % tx == 0 && tx * r <= 256 && smem + 256 <= (size_t)smem_optin;
-}
-static int fwd_tile_x(const lrccs_ctx *c, int r) {
-    if (c->plan.fwd_tx && fwd_tile_ok(c->plan.fwd_tx, r, c->nx, c->ny, c->dev_smem_optin)) return c->plan.fwd_tx;
-    int tx = 2;
-    while (tx * 2 * r <= 64 && tx * 2 <= c->nx) tx *= 2;
-    return tx;
-}
-
-// Coil groups (cluster size) of k_adj_cols, k_row_gram and k_row_w: groups of
-// about 4 coils, at most 8; or the tuned plan's.
-static int adj_cluster(const lrccs_ctx *c) {
+// Coil groups (cluster size) of k_row_gram and k_row_w: groups of about 4
+// coils, at most 8; or the tuned plan's.
+static int row_cluster(const lrccs_ctx *c) {
     if (c->plan.coil_groups >= 1 && c->plan.coil_groups <= 8 && c->plan.coil_groups <= c->nc)
         return c->plan.coil_groups;
     const int cg = (c->nc + 3) / 4;
@@ -403,82 +427,43 @@ static const row_w_t kRowW[RMAXC] = RANK_TABLE(k_row_w);
 
 // One launcher per iteration kernel, at the context's current rank c->r (the
 // _on / _to forms take the source or destination and the column count).
-// ---------------------------------------------------------------- tensor maps
-
-typedef CUresult (*encode_tiled_t)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// cuTensorMapEncodeTiled from the driver, through the runtime (no link-time
-// dependence on libcuda); NULL when unavailable, and the callers then stage
-// with cp.async.
-static encode_tiled_t tensor_map_encoder() {
-    static const encode_tiled_t fn = [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            p = nullptr;
-        }
-        return (encode_tiled_t)p;
-    }();
-    return fn;
+// Coil groups of a column pass whose blocks number tiles x groups, `res` of
+// them resident per multiprocessor: the fewest rounds of coils,
+// ceil(blocks / slots) (ceil(C / CG) + 1), the + 1 for a block's start and end.
+static int col_groups(const lrccs_ctx *c, int tiles, int res, int most) {
+    int best = 1;
+    double cost = 1e30;
+    for (int cg = 1; cg <= most && cg <= c->nc; ++cg) {
+        const int slots = res * c->nsm;
+        const double v = (double)((tiles * cg + slots - 1) / slots) * ((c->nc + cg - 1) / cg + 1.0);
+        if (v < cost) cost = v, best = cg;
+    }
+    return best;
 }
 
-// A 2D FP32 tensor map: `outer` rows of `inner` floats, `row_bytes` apart,
-// copied in boxes of box_inner x box_outer.  False (nothing encoded) unless
-// every TMA rule holds: base and row pitch 16-byte aligned, box edges <= 256
-// with an inner extent of a multiple of 16 bytes.
-bool encode_map_2d(CUtensorMap *m, const void *base, uint64_t inner, uint64_t outer, uint64_t row_bytes,
-                   uint32_t box_inner, uint32_t box_outer) {
-    const encode_tiled_t enc = tensor_map_encoder();
-    if (!enc || ((uintptr_t)base & 15) || (row_bytes & 15) || box_inner < 4 || box_inner > 256 || box_outer < 1 ||
-        box_outer > 256 || ((box_inner * 4) & 15) || box_inner > inner || box_outer > outer)
-        return false;
-    const cuuint64_t dims[2] = {inner, outer};
-    const cuuint64_t strides[1] = {row_bytes};
-    const cuuint32_t box[2] = {box_inner, box_outer};
-    const cuuint32_t es[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(base), dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+static size_t col_smem(int ny, int r, int ng, int cnt) {
+    return ((size_t)2 * ny * COLW + (size_t)2 * ng * col_nxt(r) * (cnt + 2)) * sizeof(float2);
 }
 
-cudaError_t launch_fwd_cols_on(lrccs_ctx *c, const float2 *src, int r) {
-    const int nx = c->nx, ny = c->ny;
-    const float sy = (float)(1.0 / sqrt((double)ny));
-    const int tx = fwd_tile_x(c, r);
-    // 128 bytes of slack: the TMA destination must start 128-byte aligned
-    const size_t smem = ((size_t)ny * tx * r + (size_t)ny * tx + ny) * sizeof(float2) + 128;
-    dim3 grid(nx / tx, c->nc);
-    // the tiles by TMA when both maps encode (x offsets x0 r and x0 are even
-    // complex counts: 16-byte aligned, since tx is even)
-    FwdMaps maps;
-    memset(&maps, 0, sizeof(maps));
-    const bool tma = (tx & 1) == 0 &&
-                     encode_map_2d(&maps.u, src, (uint64_t)nx * r * 2, (uint64_t)ny, (uint64_t)nx * r * 8,
-                                   (uint32_t)(tx * r * 2), (uint32_t)ny) &&
-                     encode_map_2d(&maps.s, c->d_smaps, (uint64_t)nx * 2, (uint64_t)c->nc * ny, (uint64_t)nx * 8,
-                                   (uint32_t)(tx * 2), (uint32_t)ny);
+cudaError_t launch_fwd_cols_on(lrccs_ctx *c, const float2 *src, int r, int e0, int estep) {
+    const int nx = c->nx, tiles = nx * r / COLW, nxt = col_nxt(r);
     DISPATCH_P(c->py, {
+        using PL = ColPlan<P_>;
+        const size_t smem = col_smem(PL::NY, r, PL::NG, PL::R1);
+        const int res = std::max(1, std::min(768 / PL::NT, (int)(c->smem_sm / (smem + 1024))));
+        const dim3 grid(tiles, col_groups(c, tiles, res, c->nc));
         prof_begin(c, KID_FWD_COLS);
-        if (tma)
-            k_fwd_cols<P_, true><<<grid, 256, smem, c->stream>>>(src, c->d_smaps, c->d_rowused, c->d_T, nx, r, tx,
-                                                                 c->d_twy, sy, maps, c->d_status);
-        else
-            k_fwd_cols<P_, false><<<grid, 256, smem, c->stream>>>(src, c->d_smaps, c->d_rowused, c->d_T, nx, r,
-                                                                  tx, c->d_twy, sy, maps, c->d_status);
+        k_fwd_cols<P_><<<grid, PL::NT, smem, c->stream>>>(src, c->d_smaps, c->d_rowtab, e0, estep, c->d_T, nx, r, c->nc,
+                                                          nxt, (65536u + nxt - 1) / nxt, c->d_twsy);
         prof_end(c, KID_FWD_COLS);
     });
-    return cudaSuccess;
+    return cudaGetLastError();
 }
 
 static cudaError_t launch_row_gram(lrccs_ctx *c) {
     const int r = c->r, nx = c->nx, ny = c->ny;
     const size_t smem = (size_t)2 * nx * r * sizeof(float2);
-    const int cgr = adj_cluster(c);
+    const int cgr = row_cluster(c);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c->n_used, cgr, 1);
     cfg.blockDim = dim3(256, 1, 1);
@@ -502,54 +487,91 @@ static void launch_row_w(lrccs_ctx *c) {
     const int r = c->r, nx = c->nx, ny = c->ny;
     const size_t smem = ((size_t)2 * nx * r + (size_t)c->q * r) * sizeof(float2);
     prof_begin(c, KID_ROW_W);
-    kRowW[r - 1]<<<dim3(c->n_used, adj_cluster(c)), 256, smem, c->stream>>>(
+    kRowW[r - 1]<<<dim3(c->n_used, row_cluster(c)), 256, smem, c->stream>>>(
         c->d_T, c->d_B, c->d_usedrows, c->d_rfptr, c->d_rflist, ny, nx, c->nc, c->q);
     prof_end(c, KID_ROW_W);
 }
 
-// coil-summed inverse transform into dst (n x r)
-cudaError_t launch_adj_cols_to(lrccs_ctx *c, float2 *dst, int r) {
-    const int nx = c->nx, ny = c->ny;
-    const float sy = (float)(1.0 / sqrt((double)ny));
-    const size_t smem = ((size_t)4 * ny * r + 5 * (size_t)ny) * sizeof(float2);
-    const int cg = adj_cluster(c);
+// coil-summed inverse transform into dst (n x r); cluster size: the plan's, or col_groups
+cudaError_t launch_adj_cols_to(lrccs_ctx *c, float2 *dst, int r, int e0, int estep) {
+    const int nx = c->nx, tiles = nx * r / COLW, nxt = col_nxt(r);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nx, cg, 1);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = smem;
     cfg.stream = c->stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 1;
-    at[0].val.clusterDim.y = cg;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    // pass-2 chunks of the 2r transforms: 256 / R1 transforms per chunk
-    static const int kR1[9] = {0, 4, 8, 12, 8, 10, 12, 14, 16};   // fft::Plan<32 P>::R1
-    const int nch = (2 * r + 256 / kR1[c->py] - 1) / (256 / kR1[c->py]);
-    if (nch > 2) return cudaErrorInvalidValue;
     cudaError_t el = cudaSuccess;
     DISPATCH_P(c->py, {
+        using PL = ColPlan<P_>;
+        const size_t smem = col_smem(PL::NY, r, PL::NG, PL::R2);
+        const int res = std::max(1, std::min(768 / PL::NT, (int)(c->smem_sm / (smem + 1024))));
+        int cgr = c->plan.coil_groups;
+        if (cgr < 1 || cgr > 8 || cgr > c->nc) cgr = col_groups(c, tiles, res, 8);
+        cfg.gridDim = dim3(tiles, cgr, 1);
+        at[0].val.clusterDim.y = cgr;
+        cfg.blockDim = dim3(PL::NT, 1, 1);
+        cfg.dynamicSmemBytes = smem;
         prof_begin(c, KID_ADJ_COLS);
-        if (nch == 1)
-            el = cudaLaunchKernelEx(&cfg, k_adj_cols<P_, 1>, (const float2 *)c->d_T, (const float2 *)c->d_smaps,
-                                    (const uint8_t *)c->d_rowused, dst, nx, r, c->nc, (const float2 *)c->d_twy, sy);
-        else
-            el = cudaLaunchKernelEx(&cfg, k_adj_cols<P_, 2>, (const float2 *)c->d_T, (const float2 *)c->d_smaps,
-                                    (const uint8_t *)c->d_rowused, dst, nx, r, c->nc, (const float2 *)c->d_twy, sy);
+        el = cudaLaunchKernelEx(&cfg, k_adj_cols<P_>, (const float2 *)c->d_T, (const float2 *)c->d_smaps,
+                                (const uint32_t *)c->d_rowtab, e0, estep, dst, nx, r, c->nc, nxt,
+                                (65536u + nxt - 1) / nxt, (const float2 *)c->d_twsy);
         prof_end(c, KID_ADJ_COLS);
     });
     return el;
 }
 
+// Sampled-row tables of the column passes: entry 0 the rows some frame samples,
+// entry 1 + k the rows of frame k, then 16 empty entries (frames past q).
+__global__ void k_row_tables(const int32_t *__restrict__ rowcnt, const uint8_t *__restrict__ rowused, int q, int ny,
+                             int R1, int R2, uint32_t *__restrict__ tab) {
+    const int e = blockIdx.x, t = threadIdx.x, g = t & 15;
+    uint32_t bits = 0;
+    const int step = t < 16 ? R1 : R2, cnt = t < 16 ? R2 : R1;
+    if (g < step)
+        for (int i = 0; i < cnt; ++i) {
+            const int y = g + step * i;
+            const bool used = e == 0 ? rowused[y] != 0 : (e <= q && rowcnt[(e - 1) * ny + y] > 0);
+            bits |= (uint32_t)used << i;
+        }
+    tab[e * 32 + t] = bits;
+}
+
+// Twiddles of the column passes, [j2][k1]: w_ny^(j2 k1) / sqrt(ny).
+__global__ void k_col_twiddles(float2 *tw, int N, int R1) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= N) return;
+    const int j2 = e / R1, k1 = e - j2 * R1;
+    double sn, cs;
+    sincospi(-2.0 * (double)(j2 * k1) / (double)N, &sn, &cs);
+    const double sc = 1.0 / sqrt((double)N);
+    tw[e] = make_float2((float)(cs * sc), (float)(sn * sc));
+}
+
+cudaError_t launch_col_twiddles(lrccs_ctx *c) {
+    DISPATCH_P(c->py, { k_col_twiddles<<<1, 256, 0, c->stream>>>(c->d_twsy, c->ny, ColPlan<P_>::R1); });
+    return cudaGetLastError();
+}
+
+cudaError_t launch_row_tables(lrccs_ctx *c) {
+    DISPATCH_P(c->py, {
+        prof_begin(c, KID_STRUCTURE);
+        k_row_tables<<<c->q + 17, 32, 0, c->stream>>>(c->d_rowcnt, c->d_rowused, c->q, c->ny, ColPlan<P_>::R1,
+                                                      ColPlan<P_>::R2, c->d_rowtab);
+        prof_end(c, KID_STRUCTURE);
+    });
+    return cudaGetLastError();
+}
+
 static cudaError_t launch_fwd_cols(lrccs_ctx *c) {
     // the precision forms run the sampled rows' DFT as a tensor-core GEMM
     if (c->dims.precision != LRCCS_PREC_FP32_FFT) return launch_fwd_gemm(c);
-    return launch_fwd_cols_on(c, c->d_U, c->r);
+    return launch_fwd_cols_on(c, c->d_U, c->r, 0, 0);
 }
 // the iteration's coil-summed inverse transform goes to the U+ buffer (free during iterations)
-static cudaError_t launch_adj_cols(lrccs_ctx *c) { return launch_adj_cols_to(c, c->d_Up, c->r); }
+static cudaError_t launch_adj_cols(lrccs_ctx *c) { return launch_adj_cols_to(c, c->d_Up, c->r, 0, 0); }
 
 // Z B^H on the context's side stream, forked from (and later joined back
 // into) its stream: a parallel branch when the iteration is captured.
@@ -679,19 +701,11 @@ cudaError_t launch_images(lrccs_ctx *c, float2 *d_X) {
     SET_SMEM(fn<1>); SET_SMEM(fn<2>); SET_SMEM(fn<3>); SET_SMEM(fn<4>); \
     SET_SMEM(fn<5>); SET_SMEM(fn<6>); SET_SMEM(fn<7>); SET_SMEM(fn<8>)
 cudaError_t configure_kernels_iter(int max_smem) {
-    SET_SMEM(k_fwd_cols<1, false>); SET_SMEM(k_fwd_cols<2, false>); SET_SMEM(k_fwd_cols<3, false>);
-    SET_SMEM(k_fwd_cols<4, false>); SET_SMEM(k_fwd_cols<5, false>); SET_SMEM(k_fwd_cols<6, false>);
-    SET_SMEM(k_fwd_cols<7, false>); SET_SMEM(k_fwd_cols<8, false>);
-    SET_SMEM(k_fwd_cols<1, true>); SET_SMEM(k_fwd_cols<2, true>); SET_SMEM(k_fwd_cols<3, true>);
-    SET_SMEM(k_fwd_cols<4, true>); SET_SMEM(k_fwd_cols<5, true>); SET_SMEM(k_fwd_cols<6, true>);
-    SET_SMEM(k_fwd_cols<7, true>); SET_SMEM(k_fwd_cols<8, true>);
     for (int i = 0; i < RMAXC; ++i) {
         SET_SMEM(kRowGram[i]);
         SET_SMEM(kRowW[i]);
     }
-    SET_SMEM(k_adj_cols<1, 1>); SET_SMEM(k_adj_cols<2, 1>); SET_SMEM(k_adj_cols<3, 1>); SET_SMEM(k_adj_cols<4, 1>);
-    SET_SMEM(k_adj_cols<5, 1>); SET_SMEM(k_adj_cols<6, 1>); SET_SMEM(k_adj_cols<7, 1>); SET_SMEM(k_adj_cols<8, 1>);
-    SET_SMEM(k_adj_cols<1, 2>); SET_SMEM(k_adj_cols<2, 2>); SET_SMEM(k_adj_cols<3, 2>); SET_SMEM(k_adj_cols<4, 2>);
-    SET_SMEM(k_adj_cols<5, 2>); SET_SMEM(k_adj_cols<6, 2>); SET_SMEM(k_adj_cols<7, 2>); SET_SMEM(k_adj_cols<8, 2>);
+    SET_SMEM_P(k_fwd_cols);
+    SET_SMEM_P(k_adj_cols);
     return cudaSuccess;
 }

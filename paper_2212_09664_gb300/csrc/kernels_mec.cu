@@ -14,7 +14,8 @@
 // transforms apply N to a whole chunk at once:
 //   N_k v = sum_j conj(d_j) o F^H [M_k o F(d_j o v)],
 // with the per-frame sampling M_k applied between the forward and inverse
-// transforms (k_mask_rows for line masks, k_mask_points for general ones).
+// transforms (in the column passes' row tables for line masks, by k_mask_points
+// for general ones).
 // Reductions per frame (dot products, norms) are FP64 in a fixed order.
 #include <math.h>
 
@@ -24,18 +25,6 @@
 #define MEC_G 152   // pixel blocks of the reduction kernels (one wave on 152 SMs)
 
 // ---------------------------------------------------------------- per-frame sampling between the transforms
-
-// Line masks: T_j[ky][x][l] of the used rows is kept only if frame k0 + l
-// samples row ky (frames >= q sample nothing).
-__global__ void k_mask_rows(float2 *__restrict__ T, const int32_t *__restrict__ usedrows,
-                            const int32_t *__restrict__ rowidx, int ny, int nx, int nc, int w, int k0, int q) {
-    const int ky = usedrows[blockIdx.x], j = blockIdx.y;
-    float2 *row = T + ((size_t)j * ny + ky) * nx * w;
-    for (int e = threadIdx.x; e < nx * w; e += blockDim.x) {
-        const int l = e % w, k = k0 + l;
-        if (k >= q || rowidx[k * ny + ky] < 0) row[e] = make_float2(0.f, 0.f);
-    }
-}
 
 // General masks: FU_j[u][l] is kept only if frame k0 + l samples union point u.
 __global__ void k_mask_points(float2 *__restrict__ FU, const uint8_t *__restrict__ maskc,
@@ -49,9 +38,12 @@ __global__ void k_mask_points(float2 *__restrict__ FU, const uint8_t *__restrict
     }
 }
 
-// dst (n x w) <- [N_{k0+l} src[:, l]]_l for one chunk of frames.
+// dst (n x w) <- [N_{k0+l} src[:, l]]_l for one chunk of frames.  With line
+// masks column l of the transforms only stores and reads the rows that frame
+// k0 + l samples (1/R of them; none for frames past q), which is the mask.
 cudaError_t launch_frame_normal_op(lrccs_ctx *c, const float2 *src, float2 *dst, int w, int k0) {
-    cudaError_t e = launch_fwd_cols_on(c, src, w);
+    const int e0 = c->general ? 0 : 1 + k0, es = c->general ? 0 : 1;
+    cudaError_t e = launch_fwd_cols_on(c, src, w, e0, es);
     if (e != cudaSuccess) return e;
     if (c->general) {
         e = launch_fwd_rows_r(c, w);
@@ -60,17 +52,12 @@ cudaError_t launch_frame_normal_op(lrccs_ctx *c, const float2 *src, float2 *dst,
         k_mask_points<<<4 * 152, 256, 0, c->stream>>>(c->d_FU, c->d_maskc, c->d_uidx, c->n, c->n_u, c->nc, w, k0,
                                                        c->q);
         prof_end(c, KID_MEC_MASK);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
         e = launch_adj_rows_r(c, w);
         if (e != cudaSuccess) return e;
-    } else {
-        prof_begin(c, KID_MEC_MASK);
-        k_mask_rows<<<dim3(c->n_used, c->nc), 256, 0, c->stream>>>(c->d_T, c->d_usedrows, c->d_rowidx, c->ny, c->nx,
-                                                                    c->nc, w, k0, c->q);
-        prof_end(c, KID_MEC_MASK);
     }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_adj_cols_to(c, dst, w);
+    return launch_adj_cols_to(c, dst, w, e0, es);
 }
 
 // ---------------------------------------------------------------- elementwise and reductions
