@@ -713,7 +713,7 @@ extern "C" lrccs_status lrccs_track_minibatch(lrccs_ctx *c, const void *d_y, con
 // CG on A^H A z = A^H y at rank 1 (the context's r is set to 1 by the caller).
 static lrccs_status mean_cg(lrccs_ctx *c, const void *d_y, double tol, int max_iter, void *d_zbar, void *d_ytil,
                            int32_t *out_iters) {
-    double *cg = (double *)c->d_tot;   // {gamma, alpha, stop}
+    double *cg = (double *)c->d_tot;   // {gamma, alpha, stop, beta}
     double h[3];
     CK(launch_cg_init(c, cg));
     CK(cudaMemcpyAsync(h, cg, sizeof(h), cudaMemcpyDeviceToHost, c->stream));

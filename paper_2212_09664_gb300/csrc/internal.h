@@ -37,7 +37,7 @@ enum {
 // Grid-reduction counters.
 // CNT_BAR and CNT_BAR + 1: the grid-barrier and exit counters of k_gdqr;
 // CNT_BS_BAR and CNT_BS_BAR + 1: those of k_bstep.
-enum { CNT_ENERGY = 0, CNT_GRAMX0, CNT_BAR, CNT_BAR_EXIT, CNT_BS_BAR, CNT_BS_EXIT, CNT_COUNT = 8 };
+enum { CNT_ENERGY = 0, CNT_GRAMX0, CNT_BAR, CNT_BAR_EXIT, CNT_BS_BAR, CNT_BS_EXIT, CNT_CG, CNT_COUNT = 8 };
 
 // Kernel ids (launch counting and optional CUDA-event timing).
 enum {

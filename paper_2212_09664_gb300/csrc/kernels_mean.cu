@@ -13,79 +13,101 @@
 // the gradient buffer.  The CG scalars are FP64, summed in a fixed order.
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "fft.cuh"
 #include "internal.h"
 
-#define CG_THREADS 1024
+#define CG_THREADS 256
+
+// The vectors (n complex values, L2 resident) are spread over every
+// multiprocessor and the FP64 scalars close each kernel: the last block to
+// arrive adds the blocks' partial sums in block order and forms the next
+// scalar, so a CG step is three short launches.  192 x 192, q = 48, kernel time,
+// one block of 1024 threads -> this form: right-hand side 868 -> 20 us,
+// one CG step 141 -> 15 us (the sum of its three kernels).
 
 // Sum over the block of one FP64 value per thread: warp shuffles, then the
-// warps in order (deterministic).  red holds 33 doubles.
-static __device__ double block_sum_fp64(double v, double *red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    __syncthreads();   // every thread has read red[32] of a previous call
+// warps in order (deterministic); valid in thread 0.
+static __device__ double block_sum_fp64(double v) {
+    __shared__ double red[CG_THREADS / 32];
+    v = warp_sum_d(v);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        red[32] = t;
-    }
-    __syncthreads();
-    return red[32];
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < CG_THREADS / 32; ++w) t += red[w];
+    return t;
+}
+
+// Grid-wide sum of one FP64 value per thread: true in the first warp of the
+// last block, where `total` is the sum of the blocks' partials (lane-strided,
+// then a fixed shuffle tree).
+static __device__ bool grid_sum_fp64(double v, double *part, unsigned int *counter, double &total) {
+    const double b = block_sum_fp64(v);
+    if (threadIdx.x == 0) part[blockIdx.x] = b;
+    if (!last_block_arrive(counter) || threadIdx.x >= 32) return false;
+    double t = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) t += __ldcg(part + i);
+    total = warp_sum_d(t);
+    return true;
 }
 
 // s = A^H y = sum_k Z[:, k] (Z = [A_k^H y_k], row-major i q + k), p = s, z = 0,
-// B = 1 (q x 1); cg = {||s||^2, 0, 0}.  One block.
+// B = 1 (q x 1); cg = {||s||^2, 0, 0, 0}.  One warp per pixel.
 __global__ void __launch_bounds__(CG_THREADS) k_cg_init(const float2 *__restrict__ Z, int n, int q, float2 *s,
-                                                        float2 *p, float2 *z, float2 *B, double *cg) {
-    __shared__ double red[33];
+                                                        float2 *p, float2 *z, float2 *B, double *cg, double *part,
+                                                        unsigned int *counter) {
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (CG_THREADS / 32);
     double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = blockIdx.x * (CG_THREADS / 32) + (threadIdx.x >> 5); i < n; i += warps) {
         float2 v = make_float2(0.f, 0.f);
-        for (int k = 0; k < q; ++k) {
-            const float2 a = Z[(size_t)i * q + k];
-            v.x += a.x;
-            v.y += a.y;
+        for (int k = lane; k < q; k += 32) v = cadd(v, __ldg(Z + (size_t)i * q + k));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = cadd(v, shfl_xor2(v, o));
+        if (lane == 0) {
+            s[i] = v;
+            p[i] = v;
+            z[i] = make_float2(0.f, 0.f);
+            acc += (double)v.x * v.x + (double)v.y * v.y;
         }
-        s[i] = v;
-        p[i] = v;
-        z[i] = make_float2(0.f, 0.f);
-        acc += (double)v.x * v.x + (double)v.y * v.y;
     }
-    for (int k = threadIdx.x; k < q; k += blockDim.x) B[k] = make_float2(1.f, 0.f);
-    const double g = block_sum_fp64(acc, red);
-    if (threadIdx.x == 0) {
+    if (blockIdx.x == 0)
+        for (int k = threadIdx.x; k < q; k += blockDim.x) B[k] = make_float2(1.f, 0.f);
+    double g;
+    if (grid_sum_fp64(acc, part, counter, g) && lane == 0) {
         cg[0] = g;
-        cg[1] = 0.0;
-        cg[2] = 0.0;
+        cg[1] = cg[2] = cg[3] = 0.0;
     }
 }
 
-// One CG step on A^H A z = A^H y, given w = A^H A p:
-//   alpha = gamma / <p, w>;  z += alpha p;  s -= alpha w;
-//   gamma' = ||s||^2;  p = s + (gamma' / gamma) p.
-// cg = {gamma, alpha, stop}: stop = 1 (and nothing updated) when <p, w> <= 0.
-// One block; each thread updates the same entries in every pass.
-__global__ void __launch_bounds__(CG_THREADS) k_cg_step(float2 *p, const float2 *__restrict__ w, float2 *z,
-                                                        float2 *s, int n, double *cg) {
-    __shared__ double red[33];
+// One CG step on A^H A z = A^H y, given w = A^H A p, in three kernels:
+//   k_cg_dot    alpha = gamma / <p, w>
+//   k_cg_update z += alpha p;  s -= alpha w;  gamma' = ||s||^2;  beta = gamma' / gamma
+//   k_cg_dir    p = s + beta p
+// cg = {gamma, alpha, stop, beta}: stop = 1 (and nothing updated) when <p, w> <= 0.
+__global__ void __launch_bounds__(CG_THREADS) k_cg_dot(const float2 *__restrict__ p, const float2 *__restrict__ w, int n,
+                                                       double *cg, double *part, unsigned int *counter) {
     double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = blockIdx.x * CG_THREADS + threadIdx.x; i < n; i += gridDim.x * CG_THREADS) {
         const float2 a = p[i], b = w[i];
         acc += (double)a.x * b.x + (double)a.y * b.y;   // Re(conj(p_i) w_i)
     }
-    const double dot = block_sum_fp64(acc, red);
-    const double gamma = cg[0];
-    if (!(dot > 0.0) || !(gamma > 0.0)) {
-        if (threadIdx.x == 0) cg[2] = 1.0;
-        return;
+    double dot;
+    if (grid_sum_fp64(acc, part, counter, dot) && threadIdx.x == 0) {
+        if (dot > 0.0 && cg[0] > 0.0) cg[1] = cg[0] / dot;
+        else cg[2] = 1.0;
     }
-    const double alpha_d = gamma / dot;
-    const float alpha = (float)alpha_d;
-    acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+}
+__global__ void __launch_bounds__(CG_THREADS) k_cg_update(const float2 *__restrict__ p, const float2 *__restrict__ w,
+                                                          float2 *z, float2 *s, int n, double *cg, double *part,
+                                                          unsigned int *counter) {
+    if (cg[2] != 0.0) return;   // the same for every thread of the grid
+    const float alpha = (float)cg[1];
+    const double gamma = cg[0];
+    double acc = 0.0;
+    for (int i = blockIdx.x * CG_THREADS + threadIdx.x; i < n; i += gridDim.x * CG_THREADS) {
         const float2 a = p[i], b = w[i];
         float2 zz = z[i], ss = s[i];
         zz.x = fmaf(alpha, a.x, zz.x);
@@ -96,15 +118,19 @@ __global__ void __launch_bounds__(CG_THREADS) k_cg_step(float2 *p, const float2 
         s[i] = ss;
         acc += (double)ss.x * ss.x + (double)ss.y * ss.y;
     }
-    const double g2 = block_sum_fp64(acc, red);
-    const float beta = (float)(g2 / gamma);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    double g2;
+    if (grid_sum_fp64(acc, part, counter, g2) && threadIdx.x == 0) {   // every block has read cg[0]
+        cg[0] = g2;
+        cg[3] = g2 / gamma;
+    }
+}
+__global__ void __launch_bounds__(CG_THREADS) k_cg_dir(float2 *p, const float2 *__restrict__ s, int n,
+                                                       const double *__restrict__ cg) {
+    if (cg[2] != 0.0) return;
+    const float beta = (float)cg[3];
+    for (int i = blockIdx.x * CG_THREADS + threadIdx.x; i < n; i += gridDim.x * CG_THREADS) {
         const float2 ss = s[i], a = p[i];
         p[i] = make_float2(fmaf(beta, a.x, ss.x), fmaf(beta, a.y, ss.y));
-    }
-    if (threadIdx.x == 0) {
-        cg[0] = g2;
-        cg[1] = alpha_d;
     }
 }
 
@@ -164,16 +190,26 @@ __global__ void __launch_bounds__(256) k_mean_resid(const float2 *__restrict__ y
         default: return cudaErrorInvalidValue;                         \
     }
 
+// blocks of the CG kernels (their partial sums go to d_gpart)
+static int cg_blocks(const lrccs_ctx *c) { return std::min(c->nsm, (c->n + CG_THREADS - 1) / CG_THREADS); }
+
 cudaError_t launch_cg_init(lrccs_ctx *c, double *cg) {
     prof_begin(c, KID_CG_INIT);
-    k_cg_init<<<1, CG_THREADS, 0, c->stream>>>(c->d_Z, c->n, c->q, c->d_G, c->d_U, c->d_Uprev, c->d_B, cg);
+    // 8 warps a block, one pixel each: four blocks per multiprocessor
+    k_cg_init<<<4 * c->nsm < 1024 ? 4 * c->nsm : 1024, CG_THREADS, 0, c->stream>>>(
+        c->d_Z, c->n, c->q, c->d_G, c->d_U, c->d_Uprev, c->d_B, cg, (double *)c->d_gpart, c->d_counters + CNT_CG);
     prof_end(c, KID_CG_INIT);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cg_step(lrccs_ctx *c, double *cg) {
+    const int nb = cg_blocks(c);
+    double *part = (double *)c->d_gpart;
+    unsigned int *cnt = c->d_counters + CNT_CG;
     prof_begin(c, KID_CG_STEP);
-    k_cg_step<<<1, CG_THREADS, 0, c->stream>>>(c->d_U, c->d_Up, c->d_Uprev, c->d_G, c->n, cg);
+    k_cg_dot<<<nb, CG_THREADS, 0, c->stream>>>(c->d_U, c->d_Up, c->n, cg, part, cnt);
+    k_cg_update<<<nb, CG_THREADS, 0, c->stream>>>(c->d_U, c->d_Up, c->d_Uprev, c->d_G, c->n, cg, part, cnt);
+    k_cg_dir<<<nb, CG_THREADS, 0, c->stream>>>(c->d_U, c->d_G, c->n, cg);
     prof_end(c, KID_CG_STEP);
     return cudaGetLastError();
 }
