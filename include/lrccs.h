@@ -256,10 +256,11 @@ lrccs_status lrccs_mean_step(lrccs_ctx *ctx, const void *d_y, const int64_t *d_f
  *   d_E    : NULL, or device complex64 q x n (row k = e_k), receives E
  *   d_X    : NULL, or device complex64 q x n, receives x_k = zbar + U_{t-1} b_k + e_k
  *   out_iters (MEC-2): NULL, or the number of ISTA updates made
- * The frames are processed rank_max at a time through the per-frame normal
+ * The frames are processed up to 16 at a time through the per-frame normal
  * operators A_k^H A_k (the iteration's transforms with each frame's own
  * sampling between them).  The first call allocates 5 q n complex64 of work
- * space in the context.  Both calls synchronise (MEC-2 reads its stopping test
+ * space in the context and, where the memory allows, widens its transform
+ * buffers to the frames processed at a time.  Both calls synchronise (MEC-2 reads its stopping test
  * after every step).  Errors: LRCCS_E_STATE (no iterate yet), LRCCS_E_INVALID,
  * LRCCS_E_NOMEM, LRCCS_E_CUDA. */
 lrccs_status lrccs_mec1(lrccs_ctx *ctx, int32_t iters, const void *d_zbar, void *d_E, void *d_X);

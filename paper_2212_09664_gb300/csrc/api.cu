@@ -364,6 +364,7 @@ static lrccs_status ensure_general_buffers(lrccs_ctx *c) {
                     dalloc(c, &c->d_fpart, frame_gram_part_count(c->q, c->rmax));
     if (!ok) return LRCCS_E_NOMEM;
     c->gen_cap_q = q;
+    c->FU_cap = (size_t)c->nc * n * c->rmax;
     return LRCCS_OK;
 }
 
@@ -772,11 +773,41 @@ extern "C" lrccs_status lrccs_mean_step(lrccs_ctx *c, const void *d_y, const int
 
 // ---------------------------------------------------------------- model-error correction (Alg. 3)
 
+// Grow a transform work buffer to `need` complex values, keeping the old one
+// when the larger does not fit the device memory.
+static bool grow_work(lrccs_ctx *c, float2 **buf, size_t *cap, size_t need) {
+    if (need <= *cap) return true;
+    float2 *p = nullptr;
+    if (cudaMalloc((void **)&p, need * sizeof(float2)) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    drop_iter_graph(c);   // captured iterations hold the old buffer's address
+    cudaFree(*buf);       // waits for the work that may still use it
+    *buf = p;
+    *cap = need;
+    return true;
+}
+
+// Work space and chunk width of the frames' normal operators.  A transform
+// costs little more for 16 columns than for 4, so the frames go in the fewest
+// chunks of at most 16 with the least padding: w = ceil(q / ceil(q / 16)), which
+// is also one column instead of rank_max for a single online frame.  Wider than
+// rank_max, the transform buffers grow once; when they cannot, w = rank_max.
 static lrccs_status mec_ensure(lrccs_ctx *c) {
-    if (c->d_mec) return LRCCS_OK;
-    const int w = c->rmax, nch = (c->q + w - 1) / w;
+    int nch = (c->q + 15) / 16, w = (c->q + nch - 1) / nch;
+    const size_t need = (size_t)c->nc * c->n * w;
+    if (!grow_work(c, &c->d_T, &c->T_cap, need) || (c->general && !grow_work(c, &c->d_FU, &c->FU_cap, need))) {
+        w = w < c->rmax ? w : c->rmax;
+        nch = (c->q + w - 1) / w;
+    }
+    if (c->d_mec && c->mec_w == w) return LRCCS_OK;
+    if (c->d_mec) cudaFree(c->d_mec);
+    if (c->d_mscal) cudaFree(c->d_mscal);
+    c->d_mec = nullptr;
+    c->d_mscal = nullptr;
     if (!dalloc(c, &c->d_mec, (size_t)5 * nch * c->n * w) || !dalloc(c, &c->d_mscal, mec_scal_count(c->n, c->q, w)) ||
-        !dalloc(c, &c->d_mout, 8)) {
+        (!c->d_mout && !dalloc(c, &c->d_mout, 8))) {
         if (c->d_mec) cudaFree(c->d_mec);
         if (c->d_mscal) cudaFree(c->d_mscal);
         c->d_mec = nullptr;

@@ -37,7 +37,7 @@ enum {
 // Grid-reduction counters.
 // CNT_BAR and CNT_BAR + 1: the grid-barrier and exit counters of k_gdqr;
 // CNT_BS_BAR and CNT_BS_BAR + 1: those of k_bstep.
-enum { CNT_ENERGY = 0, CNT_GRAMX0, CNT_BAR, CNT_BAR_EXIT, CNT_BS_BAR, CNT_BS_EXIT, CNT_CG, CNT_COUNT = 8 };
+enum { CNT_ENERGY = 0, CNT_GRAMX0, CNT_BAR, CNT_BAR_EXIT, CNT_BS_BAR, CNT_BS_EXIT, CNT_CG, CNT_MEC, CNT_COUNT = 8 };
 
 // Kernel ids (launch counting and optional CUDA-event timing).
 enum {
@@ -111,6 +111,7 @@ struct lrccs_ctx {
     int general;       // the loaded masks have partly sampled rows: 2D transforms per iteration
     int n_u;           // host copy of MT_NU (general masks)
     size_t gen_cap_q;  // frames the general-mask buffers were allocated for (0: none yet)
+    size_t FU_cap;     // capacity of d_FU in float2
     int dev_smem_optin;
     int test_timeout;  // lrccs_test_wait_timeout: the next direct k_gdqr launch waits for an unreachable barrier
     int device;        // CUDA device current at lrccs_create
@@ -185,8 +186,8 @@ struct lrccs_ctx {
     uint8_t *d_tflag;            // C sum_k m_k  truncation flags of the init (capacity tflag_cap)
     size_t tflag_cap;
 
-    // model-error correction (Alg. 3): frames in chunks of mec_w = rank_max
-    // columns, vectors V[c][i][l] (frame c mec_w + l)
+    // model-error correction (Alg. 3): frames in chunks of mec_w <= 16 columns,
+    // vectors V[c][i][l] (frame c mec_w + l)
     uint8_t *d_maskc;            // q * n   copy of the loaded masks (per-frame sampling inside N_k)
     float2 *d_mec;               // 5 vectors of mec_nch * n * mec_w: E, S, P, W, and M_prev (MEC-2)
     double *d_mscal;             // gamma, alpha, beta (q each), then reduction partials

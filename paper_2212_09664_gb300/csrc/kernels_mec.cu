@@ -9,15 +9,17 @@
 // Both only need the frames' normal operators N_k = A_k^H A_k and
 // s_k = A_k^H ytt_k = Z[:, k] - N_k x_k (Z = [A_k^H y~_k] from the init).
 //
-// Frames are processed in chunks of w = rank_max columns, vectors laid out as
-// V[c][i][l] (frame k = c w + l, pixel i), so that the iteration's column
-// transforms apply N to a whole chunk at once:
+// Frames are processed in chunks of w <= 16 columns (lrccs_mec1 chooses w),
+// vectors laid out as V[c][i][l] (frame k = c w + l, pixel i), so that the
+// iteration's column transforms apply N to a whole chunk at once:
 //   N_k v = sum_j conj(d_j) o F^H [M_k o F(d_j o v)],
 // with the per-frame sampling M_k applied between the forward and inverse
 // transforms (in the column passes' row tables for line masks, by k_mask_points
 // for general ones).
 // Reductions per frame (dot products, norms) are FP64 in a fixed order.
 #include <math.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "internal.h"
@@ -62,130 +64,161 @@ cudaError_t launch_frame_normal_op(lrccs_ctx *c, const float2 *src, float2 *dst,
 
 // ---------------------------------------------------------------- elementwise and reductions
 
+// Element (pixel i, column l) of chunk cc is at (cc n + i) w + l; the grids are
+// (pixel blocks, chunks), so an index needs one 32-bit division at most.
+
 // X[c][i][l] = U_{t-1}[i, :] b_k (k = c w + l < q, else 0); with zbar != NULL
 // (and Uprev == NULL) X[c][i][l] = zbar[i] for every frame instead.
-__global__ void k_mec_x(const float2 *__restrict__ Uprev, const float2 *__restrict__ B, const float2 *__restrict__ zbar,
-                        int n, int q, int r, int w, int nch, float2 *__restrict__ X) {
-    const size_t total = (size_t)nch * n * w;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int l = (int)(e % w);
-        const size_t ci = e / w;
-        const int i = (int)(ci % n), cc = (int)(ci / n);
-        const int k = cc * w + l;
+__global__ void __launch_bounds__(256) k_mec_x(const float2 *__restrict__ Uprev, const float2 *__restrict__ B,
+                                               const float2 *__restrict__ zbar, int n, int q, int r, int w,
+                                               float2 *__restrict__ X) {
+    const unsigned total = (unsigned)n * w;
+    const int cc = blockIdx.y;
+    float2 *Xc = X + (size_t)cc * total;
+    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const unsigned i = e / (unsigned)w;
+        const int k = cc * w + (int)(e - i * w);
         float2 v = make_float2(0.f, 0.f);
         if (k < q) {
             if (Uprev) {
-                for (int a = 0; a < r; ++a) cfma(v, Uprev[(size_t)i * r + a], B[(size_t)k * r + a]);
+                for (int a = 0; a < r; ++a) cfma(v, __ldg(Uprev + (size_t)i * r + a), __ldg(B + (size_t)k * r + a));
             } else {
-                v = zbar[i];
+                v = __ldg(zbar + i);
             }
         }
-        X[e] = v;
+        Xc[e] = v;
     }
 }
 
 // Z[i][k] -= V[c][i][l] (the mean's normal-operator image, online tracking).
-__global__ void k_mec_subz(float2 *__restrict__ Z, const float2 *__restrict__ V, int n, int q, int w) {
-    const size_t total = (size_t)n * q;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / q), k = (int)(e % q);
-        const float2 v = V[((size_t)(k / w) * n + i) * w + (k % w)];
-        Z[e] = csub(Z[e], v);
+__global__ void __launch_bounds__(256) k_mec_subz(float2 *__restrict__ Z, const float2 *__restrict__ V, int n, int q,
+                                                  int w) {
+    const unsigned total = (unsigned)n * w;
+    const int cc = blockIdx.y;
+    const float2 *Vc = V + (size_t)cc * total;
+    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const unsigned i = e / (unsigned)w;
+        const int k = cc * w + (int)(e - i * w);
+        if (k < q) {
+            float2 *z = Z + (size_t)i * q + k;
+            *z = csub(*z, __ldg(Vc + e));
+        }
     }
 }
 
-// Block (pixel range b, chunk cc); thread (column l, slice): per-frame FP64
-// partial sums of the value returned by f(index), written to part[b][cc w + l].
-template <class F>
-__device__ void mec_block_partial(int n, int w, double *part, F f) {
+// Per-frame FP64 sums over the pixels: thread (column l, slice) of block
+// (b, cc) adds f(i, l) over its slice of the block's pixels, the slices add in a
+// fixed tree, and the last block to arrive adds the blocks' partials (a warp per
+// frame: lane-strided, then a fixed shuffle tree) and hands each frame's total
+// to done(k, total).  The separate one-block finish kernel this replaces took
+// 10-12 us a launch, and the indices of the pixel loop another 20 (160 x 128,
+// 27 frames: dot product 27 + 11 -> 20 us; one 128 x 128 frame: 6 + 10 -> 7 us).
+template <class F, class DONE>
+__device__ void mec_frame_sums(int n, int w, int q, double *part, unsigned int *counter, F f, DONE done) {
     __shared__ double s_red[256];
     const int b = blockIdx.x, cc = blockIdx.y, G = gridDim.x, NW = gridDim.y * w;
     const int per = (n + G - 1) / G;
     const int i0 = min(n, b * per), i1 = min(n, i0 + per);
-    const int S = blockDim.x / w, l = threadIdx.x % w, sl = threadIdx.x / w;
+    const int S = blockDim.x / w, sl = threadIdx.x / w, l = threadIdx.x - sl * w;
     double acc = 0.0;
-    if (sl < S)
-        for (int i = i0 + sl; i < i1; i += S) acc += f(((size_t)cc * n + i) * w + l);
+    if (sl < S) {
+#pragma unroll 4
+        for (int i = i0 + sl; i < i1; i += S) acc += f(i, l);
+    }
     s_red[threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.x < w) {
-        double s = 0.0;
-        for (int v = 0; v < S; ++v) s += s_red[v * w + threadIdx.x];
-        part[(size_t)b * NW + cc * w + threadIdx.x] = s;
+    int h = 1;
+    while (2 * h < S) h <<= 1;
+    for (; h > 0; h >>= 1) {   // slices sl and sl + h, a fixed tree
+        __syncthreads();
+        if (sl < h && sl + h < S) s_red[threadIdx.x] += s_red[threadIdx.x + h * w];
+    }
+    if (threadIdx.x < w) part[(size_t)b * NW + cc * w + threadIdx.x] = s_red[threadIdx.x];
+    if (!last_block_arrive(counter)) return;
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < q; k += blockDim.x >> 5) {
+        double t = 0.0;
+        for (int g = lane; g < G; g += 32) t += __ldcg(part + (size_t)g * NW + k);
+        t = warp_sum_d(t);
+        if (lane == 0) done(k, t);
     }
 }
 
-// S = Z - V, P = S, E = 0 and the partials of gamma_k = ||S_k||^2.
+// S = Z - V, P = S, E = 0 and gamma_k = ||S_k||^2.
 __global__ void __launch_bounds__(256) k_mec_start(const float2 *__restrict__ Z, const float2 *__restrict__ V, int n,
                                                    int q, int w, float2 *__restrict__ S, float2 *__restrict__ P,
-                                                   float2 *__restrict__ E, double *part) {
-    mec_block_partial(n, w, part, [&](size_t e) {
-        const int l = (int)(e % w), i = (int)((e / w) % n), k = (int)(e / ((size_t)n * w)) * w + l;
-        float2 s = make_float2(0.f, 0.f);
-        if (k < q) s = csub(Z[(size_t)i * q + k], V[e]);
-        S[e] = s;
-        P[e] = s;
-        E[e] = make_float2(0.f, 0.f);
-        return (double)s.x * s.x + (double)s.y * s.y;
-    });
+                                                   float2 *__restrict__ E, double *part, unsigned int *counter,
+                                                   double *gamma) {
+    const int cc = blockIdx.y;
+    const size_t base = (size_t)cc * n * w;
+    mec_frame_sums(
+        n, w, q, part, counter,
+        [&](int i, int l) {
+            const size_t e = base + (size_t)i * w + l;
+            const int k = cc * w + l;
+            float2 s = make_float2(0.f, 0.f);
+            if (k < q) s = csub(__ldg(Z + (size_t)i * q + k), __ldg(V + e));
+            S[e] = s;
+            P[e] = s;
+            E[e] = make_float2(0.f, 0.f);
+            return (double)s.x * s.x + (double)s.y * s.y;
+        },
+        [&](int k, double t) { gamma[k] = t; });
 }
 
-// partials of Re<p_k, w_k> (= ||A_k p_k||^2)
+// alpha_k = gamma_k / Re<p_k, w_k> (= ||A_k p_k||^2; 0 if the frame's direction has no energy)
 __global__ void __launch_bounds__(256) k_mec_dot(const float2 *__restrict__ P, const float2 *__restrict__ W, int n,
-                                                 int w, double *part) {
-    mec_block_partial(n, w, part, [&](size_t e) {
-        const float2 a = P[e], b = W[e];
-        return (double)a.x * b.x + (double)a.y * b.y;
-    });
+                                                 int q, int w, double *part, unsigned int *counter,
+                                                 const double *__restrict__ gamma, double *alpha) {
+    const size_t base = (size_t)blockIdx.y * n * w;
+    mec_frame_sums(
+        n, w, q, part, counter,
+        [&](int i, int l) {
+            const size_t e = base + (size_t)i * w + l;
+            const float2 a = __ldg(P + e), b = __ldg(W + e);
+            return (double)a.x * b.x + (double)a.y * b.y;
+        },
+        [&](int k, double t) { alpha[k] = (t > 0.0 && gamma[k] > 0.0) ? gamma[k] / t : 0.0; });
 }
 
-// e += alpha p, s -= alpha w, and the partials of the new ||s_k||^2
+// e += alpha p, s -= alpha w; beta_k = (new ||s_k||^2) / gamma_k, gamma_k = the new norm
 __global__ void __launch_bounds__(256) k_mec_update(const float2 *__restrict__ P, const float2 *__restrict__ W,
                                                     float2 *__restrict__ E, float2 *__restrict__ S,
-                                                    const double *__restrict__ alpha, int n, int w, double *part) {
-    mec_block_partial(n, w, part, [&](size_t e) {
-        const int k = (int)(e / ((size_t)n * w)) * w + (int)(e % w);
-        const float a = (float)alpha[k];
-        const float2 p = P[e], ww = W[e];
-        float2 ee = E[e], ss = S[e];
-        ee.x = fmaf(a, p.x, ee.x);
-        ee.y = fmaf(a, p.y, ee.y);
-        ss.x = fmaf(-a, ww.x, ss.x);
-        ss.y = fmaf(-a, ww.y, ss.y);
-        E[e] = ee;
-        S[e] = ss;
-        return (double)ss.x * ss.x + (double)ss.y * ss.y;
-    });
+                                                    const double *__restrict__ alpha, int n, int q, int w, double *part,
+                                                    unsigned int *counter, double *gamma, double *beta) {
+    const int cc = blockIdx.y, l0 = threadIdx.x % w;
+    const size_t base = (size_t)cc * n * w;
+    const float a = cc * w + l0 < q ? (float)alpha[cc * w + l0] : 0.f;
+    mec_frame_sums(
+        n, w, q, part, counter,
+        [&](int i, int l) {
+            const size_t e = base + (size_t)i * w + l;
+            const float2 p = __ldg(P + e), ww = __ldg(W + e);
+            float2 ee = E[e], ss = S[e];
+            ee.x = fmaf(a, p.x, ee.x);
+            ee.y = fmaf(a, p.y, ee.y);
+            ss.x = fmaf(-a, ww.x, ss.x);
+            ss.y = fmaf(-a, ww.y, ss.y);
+            E[e] = ee;
+            S[e] = ss;
+            return (double)ss.x * ss.x + (double)ss.y * ss.y;
+        },
+        [&](int k, double t) {
+            beta[k] = gamma[k] > 0.0 ? t / gamma[k] : 0.0;
+            gamma[k] = t;
+        });
 }
 
 // p = s + beta p
-__global__ void k_mec_dir(const float2 *__restrict__ S, float2 *__restrict__ P, const double *__restrict__ beta, int n,
-                          int w, int nch) {
-    const size_t total = (size_t)nch * n * w;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(e / ((size_t)n * w)) * w + (int)(e % w);
-        const float bb = (float)beta[k];
-        const float2 s = S[e], p = P[e];
-        P[e] = make_float2(fmaf(bb, p.x, s.x), fmaf(bb, p.y, s.y));
-    }
-}
-
-// Per frame k < q: total = sum over the G pixel blocks of part[b][k] (in b
-// order), then   mode 0: gamma = total;   mode 1: alpha = gamma / total (0 if
-// the frame's direction has no energy);   mode 2: beta = total / gamma, gamma = total.
-__global__ void k_mec_finish(const double *__restrict__ part, int G, int NW, int q, int mode, double *gamma,
-                             double *alpha, double *beta) {
-    for (int k = threadIdx.x; k < q; k += blockDim.x) {
-        double t = 0.0;
-        for (int b = 0; b < G; ++b) t += part[(size_t)b * NW + k];
-        if (mode == 0) {
-            gamma[k] = t;
-        } else if (mode == 1) {
-            alpha[k] = (t > 0.0 && gamma[k] > 0.0) ? gamma[k] / t : 0.0;
-        } else {
-            beta[k] = gamma[k] > 0.0 ? t / gamma[k] : 0.0;
-            gamma[k] = t;
-        }
+__global__ void __launch_bounds__(256) k_mec_dir(const float2 *__restrict__ S, float2 *__restrict__ P,
+                                                 const double *__restrict__ beta, int n, int q, int w) {
+    const unsigned total = (unsigned)n * w;
+    const int cc = blockIdx.y;
+    const size_t base = (size_t)cc * total;
+    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int k = cc * w + (int)(e % (unsigned)w);
+        const float bb = k < q ? (float)beta[k] : 0.f;
+        const float2 s = __ldg(S + base + e), p = P[base + e];
+        P[base + e] = make_float2(fmaf(bb, p.x, s.x), fmaf(bb, p.y, s.y));
     }
 }
 
@@ -337,16 +370,22 @@ __global__ void __launch_bounds__(256) k_tdft_inv(const float2 *__restrict__ M, 
 
 static int mec_blocks(int n) { return n < MEC_G * 64 ? (n + 63) / 64 : MEC_G; }
 
+// blocks along the pixels of the elementwise kernels: four per multiprocessor over all chunks
+static dim3 mec_grid(const lrccs_ctx *c) {
+    const int need = (int)(((size_t)c->n * c->mec_w + 255) / 256);
+    return dim3(std::min(need, std::max(1, 4 * c->nsm / c->mec_nch)), c->mec_nch);
+}
+
 cudaError_t launch_mec_x(lrccs_ctx *c, const float2 *Uprev, const float2 *zbar, float2 *X) {
     prof_begin(c, KID_MEC_ELEM);
-    k_mec_x<<<4 * 152, 256, 0, c->stream>>>(Uprev, c->d_B, zbar, c->n, c->q, c->r, c->mec_w, c->mec_nch, X);
+    k_mec_x<<<mec_grid(c), 256, 0, c->stream>>>(Uprev, c->d_B, zbar, c->n, c->q, c->r, c->mec_w, X);
     prof_end(c, KID_MEC_ELEM);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mec_subz(lrccs_ctx *c, const float2 *V) {
     prof_begin(c, KID_MEC_ELEM);
-    k_mec_subz<<<4 * 152, 256, 0, c->stream>>>(c->d_Z, V, c->n, c->q, c->mec_w);
+    k_mec_subz<<<mec_grid(c), 256, 0, c->stream>>>(c->d_Z, V, c->n, c->q, c->mec_w);
     prof_end(c, KID_MEC_ELEM);
     return cudaGetLastError();
 }
@@ -354,23 +393,16 @@ cudaError_t launch_mec_subz(lrccs_ctx *c, const float2 *V) {
 // kind: 0 start (S = Z - V, P = S, E = 0, gamma), 1 alpha (from P, W), 2
 // update (E, S, then beta and gamma), 3 direction (P = S + beta P).
 cudaError_t launch_mec_cg(lrccs_ctx *c, int kind, const float2 *V) {
-    const int n = c->n, w = c->mec_w, nch = c->mec_nch, G = mec_blocks(n), NW = nch * w;
-    double *gamma = c->d_mscal, *alpha = gamma + c->q, *beta = alpha + c->q, *part = beta + c->q;
+    const int n = c->n, q = c->q, w = c->mec_w, nch = c->mec_nch;
+    double *gamma = c->d_mscal, *alpha = gamma + q, *beta = alpha + q, *part = beta + q;
     float2 *E = c->d_mec, *S = E + (size_t)nch * n * w, *P = S + (size_t)nch * n * w, *W = P + (size_t)nch * n * w;
-    dim3 grid(G, nch);
+    unsigned int *cnt = c->d_counters + CNT_MEC;
+    const dim3 grid(mec_blocks(n), nch);
     prof_begin(c, KID_MEC_ELEM);
-    if (kind == 0) {
-        k_mec_start<<<grid, 256, 0, c->stream>>>(c->d_Z, V, n, c->q, w, S, P, E, part);
-        k_mec_finish<<<1, 128, 0, c->stream>>>(part, G, NW, c->q, 0, gamma, alpha, beta);
-    } else if (kind == 1) {
-        k_mec_dot<<<grid, 256, 0, c->stream>>>(P, W, n, w, part);
-        k_mec_finish<<<1, 128, 0, c->stream>>>(part, G, NW, c->q, 1, gamma, alpha, beta);
-    } else if (kind == 2) {
-        k_mec_update<<<grid, 256, 0, c->stream>>>(P, W, E, S, alpha, n, w, part);
-        k_mec_finish<<<1, 128, 0, c->stream>>>(part, G, NW, c->q, 2, gamma, alpha, beta);
-    } else {
-        k_mec_dir<<<4 * 152, 256, 0, c->stream>>>(S, P, beta, n, w, nch);
-    }
+    if (kind == 0) k_mec_start<<<grid, 256, 0, c->stream>>>(c->d_Z, V, n, q, w, S, P, E, part, cnt, gamma);
+    else if (kind == 1) k_mec_dot<<<grid, 256, 0, c->stream>>>(P, W, n, q, w, part, cnt, gamma, alpha);
+    else if (kind == 2) k_mec_update<<<grid, 256, 0, c->stream>>>(P, W, E, S, alpha, n, q, w, part, cnt, gamma, beta);
+    else k_mec_dir<<<mec_grid(c), 256, 0, c->stream>>>(S, P, beta, n, q, w);
     prof_end(c, KID_MEC_ELEM);
     return cudaGetLastError();
 }

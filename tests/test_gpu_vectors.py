@@ -1,4 +1,4 @@
-"""GPU tests of the vector kernels around the transforms (the mean step's CG)
+"""GPU tests of the vector kernels around the transforms (the mean step's CG, MEC)
 against FP64 torch: one block and many, single frames and coils, frame counts
 that leave a warp partly idle."""
 import numpy as np
@@ -74,4 +74,33 @@ def test_mean_step_matches_torch(ny, nx, q, nc, kind):
     res = torch.cat([(c.y[k] - c.apply(k, z))[:, c.m[k] > 0].reshape(-1) for k in range(q)])
     scale = torch.linalg.norm(c.inp[0].to(torch.complex128))
     assert float(torch.linalg.norm(ytil - res)) < 5e-6 * float(scale)
+    s.close()
+
+
+# chunks of the frames' normal operators: one column, padded chunks, wider and narrower than the rank
+@pytest.mark.parametrize("ny,nx,q,nc,rank,kind", [(64, 64, 1, 3, 1, "lines"), (32, 96, 16, 2, 2, "lines"),
+                                                  (64, 64, 17, 3, 5, "radial"), (96, 64, 33, 2, 3, "lines"),
+                                                  (64, 32, 5, 4, 4, "radial")])
+def test_mec1_matches_torch(ny, nx, q, nc, rank, kind):
+    c = Case(ny, nx, q, nc, rank, kind, nx + q)
+    s = lrccs.Solver(ny, nx, q, nc, rank)
+    s.init(*c.inp)
+    s.iterate(3)
+    E, X = s.mec1(2)
+    U, B = s.factors()
+    s.sync()
+    low = (U.to(torch.complex128) @ B.to(torch.complex128).T).T
+    scale = torch.linalg.norm(low) / q ** 0.5
+    for k in range(q):
+        r = c.adjoint(k, c.y[k]) - c.adjoint(k, c.apply(k, low[k]))
+        e, p, g = torch.zeros_like(r), r.clone(), (r.abs() ** 2).sum()
+        for _ in range(2):
+            w = c.adjoint(k, c.apply(k, p))
+            a = g / (p.conj() * w).real.sum()
+            e, r = e + a * p, r - a * w
+            g2 = (r.abs() ** 2).sum()
+            p, g = r + (g2 / g) * p, g2
+        # the residual is a difference of FP32 terms of the image's size
+        assert float(torch.linalg.norm(E[k] - e)) < 3e-6 * float(scale)
+        assert float(torch.linalg.norm(X[k] - low[k] - e)) < 3e-6 * float(scale)
     s.close()
