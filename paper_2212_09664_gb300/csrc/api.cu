@@ -93,7 +93,7 @@ static void free_all(lrccs_ctx *c) {
                     c->d_ufrow, c->d_upos, c->d_uidx, c->d_ufptr, c->d_uflist, c->d_fu, c->d_FU, c->d_Pu,
                     c->d_maskc, c->d_mec, c->d_mscal, c->d_mout, c->d_twq, c->d_Q, c->d_gdts, c->d_fpart,
                     c->d_tflag, c->d_tcA0, c->d_tcA1, c->d_tcscale, c->d_ZB, c->d_hpart,
-                    c->d_tcB0, c->d_tcB1, c->d_twsy, c->d_rowtab};
+                    c->d_tcB0, c->d_tcB1, c->d_twsy, c->d_twsx, c->d_rowtab, c->d_ptab};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -175,7 +175,7 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     const size_t F2 = sizeof(float2), I4 = sizeof(int32_t), D8 = sizeof(double);
     const struct { void **p; size_t bytes; } plan[] = {
         {(void **)&c->d_twy, ny * F2}, {(void **)&c->d_twx, c->nx * F2},
-        {(void **)&c->d_twsy, ny * F2}, {(void **)&c->d_rowtab, ((size_t)q + 17) * 32 * I4}, {(void **)&c->d_smaps, (size_t)nc * n * F2},
+        {(void **)&c->d_twsy, ny * F2}, {(void **)&c->d_twsx, c->nx * F2}, {(void **)&c->d_rowtab, ((size_t)q + 17) * 32 * I4}, {(void **)&c->d_smaps, (size_t)nc * n * F2},
         {(void **)&c->d_rowcnt, (size_t)q * ny * I4}, {(void **)&c->d_rowidx, (size_t)q * ny * I4},
         {(void **)&c->d_framerows, (size_t)q * ny * I4}, {(void **)&c->d_lineptr, ((size_t)q + 1) * I4},
         {(void **)&c->d_rfptr, ((size_t)ny + 1) * I4}, {(void **)&c->d_rflist, (size_t)q * ny * I4},
@@ -800,6 +800,10 @@ static lrccs_status mec_ensure(lrccs_ctx *c) {
     if (!grow_work(c, &c->d_T, &c->T_cap, need) || (c->general && !grow_work(c, &c->d_FU, &c->FU_cap, need))) {
         w = w < c->rmax ? w : c->rmax;
         nch = (c->q + w - 1) / w;
+    }
+    if (c->general) {   // the loaded masks' point tables
+        if (!c->d_ptab && !dalloc(c, &c->d_ptab, (size_t)c->q * c->ny * 32)) return LRCCS_E_NOMEM;
+        CK(launch_point_tables(c));
     }
     if (c->d_mec && c->mec_w == w) return LRCCS_OK;
     if (c->d_mec) cudaFree(c->d_mec);

@@ -123,7 +123,8 @@ struct lrccs_ctx {
 
     // geometry / sampling
     float2 *d_twy, *d_twx;       // twiddles w_N^t, N = ny / nx
-    float2 *d_twsy;              // ny: twiddles of the column passes with their scale, [j2][k1]
+    float2 *d_twsy, *d_twsx;     // ny, nx: twiddles of the column and row passes with their scale, [j2][k1]
+    uint16_t *d_ptab;            // q * ny * 32 sampled-point tables of the row passes (general masks, MEC)
     uint32_t *d_rowtab;          // (q + 17) * 32 sampled-row tables of the column passes (k_row_tables)
     float2 *d_smaps;             // nc * n
     int32_t *d_rowcnt;           // q * ny  samples of frame k in row ky
@@ -216,8 +217,11 @@ cudaError_t launch_init_general(lrccs_ctx *c, const float2 *d_y);   // Z and X0 
 cudaError_t launch_iteration_general_front(lrccs_ctx *c);   // forward rows + sample Grams + B-step
 cudaError_t launch_iteration_general_back(lrccs_ctx *c);    // W per sample + inverse rows
 cudaError_t launch_fwd_rows(lrccs_ctx *c);
-cudaError_t launch_fwd_rows_r(lrccs_ctx *c, int r);
-cudaError_t launch_adj_rows_r(lrccs_ctx *c, int r);
+// row passes on the union points (k0 < 0), or for column l on those frame k0 + l
+// samples (launch_point_tables first)
+cudaError_t launch_fwd_rows_r(lrccs_ctx *c, int r, int k0);
+cudaError_t launch_adj_rows_r(lrccs_ctx *c, int r, int k0);
+cudaError_t launch_point_tables(lrccs_ctx *c);
 // T <- F_y(d_j o src) (n x r src) on the rows of table entry e0 + l estep (column l), and
 // dst <- sum_j conj(d_j) F_y^H T_j from those rows
 cudaError_t launch_fwd_cols_on(lrccs_ctx *c, const float2 *src, int r, int e0, int estep);

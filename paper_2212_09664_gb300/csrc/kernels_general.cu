@@ -24,6 +24,8 @@
 // inverse DFT along kx of each frame row's few samples, then the column FFTs).
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "fft.cuh"
 #include "internal.h"
@@ -353,179 +355,300 @@ cudaError_t launch_init_general(lrccs_ctx *c, const float2 *d_y) {
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- A2: forward along x, gather
+// ---------------------------------------------------------------- A2, E: the row passes
+//
+// A row (nx x r complex values of T_j[ky], l innermost) is transformed along x
+// with the two register halves of fft.cuh, N = R1 R2.  Item i = g r + l of a
+// coil: its length-R1 DFT takes elements x = g + R2 m, at m R2 r + i of the row,
+// and its length-R2 DFT gives x = g + R1 k2, at k2 R1 r + i, so every access to
+// the row is contiguous over the items whatever the rank.  The exchange tile
+// holds element (k1, j2, l) at k1 S + j2 r + l; S = r modulo 16 keeps the second
+// half's reads on distinct banks.  Each thread stages its own elements by
+// cp.async while the previous coil's second half runs (two tiles, one block
+// barrier per step) and transforms them in place.  A block takes the coils of
+// its group, CB at a time (small ranks), of one row ky.
+//
+// Which points of the row exist: the union points (iterations), or with ftab
+// only those that frame k0 + l samples (the frames' normal operators): 16-bit
+// masks per (frame, row, g), over k2 for the forward pass ([..][0..15]) and over
+// m for the adjoint ([..][16..31]).
+struct RowArgs {
+    const int32_t *usedrows, *uptr, *upos;
+    const uint16_t *ftab;      // NULL: every union point
+    const float2 *tw;          // [j2][k1] twiddles with the scale 1 / sqrt(nx)
+    int ny, r, nc, nu, S, CB, k0, q;
+};
 
-// Block (row ky of Omega_u, coil group g) transforms the rows of coils g, g +
-// CG, ... in turn (double buffered with cp.async): T_j[ky][:][:] (nx x r) is
-// transformed along x and its union points written to FU[j][u][:].
-template <int PX>
-__global__ void __launch_bounds__(256) k_fwd_rows(const float2 *__restrict__ T, const int32_t *__restrict__ usedrows,
-                                                   const int32_t *__restrict__ uptr, const int32_t *__restrict__ uidx,
-                                                   float2 *__restrict__ FU, int ny, int r, int nc, int nu,
-                                                   const float2 *__restrict__ g_tw, float scale) {
-    constexpr int NX = 32 * PX;
-    extern __shared__ __align__(16) float2 smem[];
-    float2 *tile0 = smem, *tile1 = smem + NX * r, *s_tw = tile1 + NX * r;
-    __shared__ int s_kx[NX];
-    const int ky = usedrows[blockIdx.x], g = blockIdx.y, CG = gridDim.y;
-    const size_t plane = (size_t)ny * NX * r;
-    const float2 *row0 = T + (size_t)ky * NX * r;
-    const int u0 = uptr[ky], cnt = uptr[ky + 1] - u0;
-    if (g < nc) stage_row(tile0, row0 + (size_t)g * plane, NX * r, threadIdx.x, blockDim.x);
-    cp_async_commit();
-    load_twiddles(s_tw, g_tw, NX);
-    for (int s = threadIdx.x; s < cnt; s += blockDim.x) s_kx[s] = uidx[u0 + s] - ky * NX;
-    const int gl = threadIdx.x % r, gs = threadIdx.x / r, gstep = blockDim.x / r;
-    int b = 0;
-    for (int j = g; j < nc; j += CG, b ^= 1) {
-        float2 *tile = b ? tile1 : tile0;
-        if (j + CG < nc) {
-            stage_row(b ? tile0 : tile1, row0 + (size_t)(j + CG) * plane, NX * r, threadIdx.x, blockDim.x);
-            cp_async_commit();
-            cp_async_wait_1();
-        } else {
-            cp_async_wait();
-        }
-        __syncthreads();
-        fft::tile_dft<NX, false>(tile, r, r, s_tw, scale);   // ends with a barrier
-        if (gs < gstep) {
-            float2 *dst = FU + ((size_t)j * nu + u0) * r;
-            for (int s = gs; s < cnt; s += gstep) dst[(size_t)s * r + gl] = tile[s_kx[s] * r + gl];
-        }
-        __syncthreads();
+template <int P>
+struct RowPlan {
+    static constexpr int NX = 32 * P, R1 = fft::Plan<NX>::R1, R2 = fft::Plan<NX>::R2, NG = R1 > R2 ? R1 : R2;
+};
+
+// the row's union index of every x (-1: none) into s_up; ends with a barrier
+LRCCS_DEV void row_positions(int16_t *s_up, const RowArgs &a, int ky, int nx) {
+    const int u0 = a.uptr[ky];
+    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+        const int u = __ldg(a.upos + (size_t)ky * nx + x);
+        s_up[x] = (int16_t)(u < 0 ? -1 : u - u0);
     }
+    __syncthreads();
+}
+// the points x = g + step i, i < cnt, of column l as a bit mask
+LRCCS_DEV uint32_t row_bits(const int16_t *s_up, const RowArgs &a, int ky, int g, int l, int step, int cnt, int half) {
+    if (a.ftab) return a.k0 + l < a.q ? __ldg(a.ftab + ((size_t)(a.k0 + l) * a.ny + ky) * 32 + half + g) : 0u;
+    uint32_t bits = 0;
+    for (int i = 0; i < cnt; ++i) bits |= (uint32_t)(s_up[g + step * i] >= 0) << i;
+    return bits;
+}
+
+// Measured (kernel time, L2 warm), whole rows staged by cp.async and transformed
+// with shared-memory passes -> this form: 256 x 256, C = 20, r = 12, 28.9k
+// points: 56 -> 55 us (DRAM: 126 MB of T in, 126 MB of its dirty lines out);
+// 224 x 224, C = 18, r = 13, 8 frames: 44 -> 32 us
+template <int P>
+__global__ void __launch_bounds__(256, 3) k_fwd_rows(const float2 *__restrict__ T, float2 *__restrict__ FU,
+                                                     const RowArgs a) {
+    using PL = RowPlan<P>;
+    constexpr int NX = PL::NX, R1 = PL::R1, R2 = PL::R2, NG = PL::NG;
+    extern __shared__ __align__(16) float2 smem[];
+    __shared__ int16_t s_up[NX];
+    const int r = a.r, IT = NG * r, tile = R1 * a.S, ky = a.usedrows[blockIdx.x];
+    const int slot = threadIdx.x / IT, i = threadIdx.x - slot * IT, g = i / r, l = i - g * r;
+    const bool first = slot < a.CB && g < R2, second = slot < a.CB && g < R1;
+    const size_t rowlen = (size_t)NX * r;
+    const int u0 = a.uptr[ky], step = gridDim.y * a.CB;
+    float2 *mine = smem + slot * tile;
+    auto stage = [&](int j, int s) {
+        if (first && j < a.nc) {
+            float2 *dst = mine + s * a.CB * tile + i;
+            const float2 *src = T + ((size_t)j * a.ny + ky) * rowlen + i;
+#pragma unroll
+            for (int m = 0; m < R1; ++m) cp_async8(dst + m * a.S, src + m * R2 * r);
+        }
+        cp_async_commit();
+    };
+    stage(blockIdx.y * a.CB + slot, 0);
+    row_positions(s_up, a, ky, NX);
+    const uint32_t bits = second ? row_bits(s_up, a, ky, g, l, R1, R2, 0) : 0u;
+    int s = 0;
+    for (int b = blockIdx.y * a.CB; b < a.nc; b += step, s ^= 1) {
+        const int j = b + slot;
+        float2 *ex = mine + s * a.CB * tile;
+        cp_async_wait();
+        if (first && j < a.nc) {
+            float2 v[R1];
+#pragma unroll
+            for (int m = 0; m < R1; ++m) v[m] = ex[m * a.S + i];
+            fft::dft_first<R1, R2, false>(v, g, a.tw, [&](int k1, float2 w) { ex[k1 * a.S + i] = w; });
+        }
+        __syncthreads();
+        if (b + step < a.nc) stage(j + step, s ^ 1);
+        if (bits != 0 && j < a.nc) {
+            float2 v[R2];
+            const float2 *e = ex + g * a.S + l;
+#pragma unroll
+            for (int j2 = 0; j2 < R2; ++j2) v[j2] = e[j2 * r];
+            fft::Dft<R2, false>::run(v);
+            float2 *dst = FU + ((size_t)j * a.nu + u0) * r + l;
+#pragma unroll
+            for (int k2 = 0; k2 < R2; ++k2)
+                if (bits >> k2 & 1) dst[s_up[g + R1 * k2] * r] = v[k2];
+        }
+    }
+}
+
+// The row's points scattered into a zero row, transformed back along x, the
+// full row written to T_j[ky] for the column pass.  Measured as above: 87 -> 53 us;
+// 65 -> 37 us.
+template <int P>
+__global__ void __launch_bounds__(256, 3) k_adj_rows(const float2 *__restrict__ FU, float2 *__restrict__ T,
+                                                     const RowArgs a) {
+    using PL = RowPlan<P>;
+    constexpr int NX = PL::NX, R1 = PL::R1, R2 = PL::R2, NG = PL::NG;
+    extern __shared__ __align__(16) float2 smem[];
+    __shared__ int16_t s_up[NX];
+    const int r = a.r, IT = NG * r, tile = R1 * a.S, ky = a.usedrows[blockIdx.x];
+    const int slot = threadIdx.x / IT, i = threadIdx.x - slot * IT, g = i / r, l = i - g * r;
+    const bool first = slot < a.CB && g < R2, second = slot < a.CB && g < R1;
+    const size_t rowlen = (size_t)NX * r;
+    const int u0 = a.uptr[ky], step = gridDim.y * a.CB;
+    float2 *mine = smem + slot * tile;
+    row_positions(s_up, a, ky, NX);
+    const uint32_t bits = first ? row_bits(s_up, a, ky, g, l, R2, R1, 16) : 0u;
+    auto stage = [&](int j, int s) {
+        if (j < a.nc) {
+            float2 *dst = mine + s * a.CB * tile + i;
+            const float2 *src = FU + ((size_t)j * a.nu + u0) * r + l;
+#pragma unroll
+            for (int m = 0; m < R1; ++m)
+                if (bits >> m & 1) cp_async8(dst + m * a.S, src + s_up[g + R2 * m] * r);
+        }
+        cp_async_commit();
+    };
+    stage(blockIdx.y * a.CB + slot, 0);
+    int s = 0;
+    for (int b = blockIdx.y * a.CB; b < a.nc; b += step, s ^= 1) {
+        const int j = b + slot;
+        float2 *ex = mine + s * a.CB * tile;
+        cp_async_wait();
+        if (first && j < a.nc) {
+            float2 v[R1];
+#pragma unroll
+            for (int m = 0; m < R1; ++m) v[m] = (bits >> m & 1) ? ex[m * a.S + i] : make_float2(0.f, 0.f);
+            fft::dft_first<R1, R2, true>(v, g, a.tw, [&](int k1, float2 w) { ex[k1 * a.S + i] = w; });
+        }
+        __syncthreads();
+        if (b + step < a.nc) stage(j + step, s ^ 1);
+        if (second && j < a.nc) {
+            float2 v[R2];
+            const float2 *e = ex + g * a.S + l;
+#pragma unroll
+            for (int j2 = 0; j2 < R2; ++j2) v[j2] = e[j2 * r];
+            fft::Dft<R2, true>::run(v);
+            float2 *dst = T + ((size_t)j * a.ny + ky) * rowlen + i;
+#pragma unroll
+            for (int k2 = 0; k2 < R2; ++k2) dst[k2 * R1 * r] = v[k2];
+        }
+    }
+}
+
+// The frames' point masks of the row passes (see RowArgs): block (row ky,
+// frame k), thread t < 32.
+__global__ void k_point_tables(const uint8_t *__restrict__ mask, int ny, int nx, int R1, int R2,
+                               uint16_t *__restrict__ tab) {
+    const int ky = blockIdx.x, k = blockIdx.y, t = threadIdx.x, g = t & 15;
+    const uint8_t *m = mask + ((size_t)k * ny + ky) * nx;
+    const int step = t < 16 ? R1 : R2, cnt = t < 16 ? R2 : R1;
+    uint32_t bits = 0;
+    if (g < step)
+        for (int i = 0; i < cnt; ++i) bits |= (uint32_t)(m[g + step * i] != 0) << i;
+    tab[((size_t)k * ny + ky) * 32 + t] = (uint16_t)bits;
 }
 
 // ---------------------------------------------------------------- B: per-point Gram
 
-// Block of SU = 32 union points: per coil (double buffered) the points' rows
-// FU_j[u][:] are staged and every thread adds conj(FU[a]) FU[b] for its
-// (point, pair) items; P_u holds the coil sum of the upper triangle.
+// Block of SU union points, thread (point, 2 x 2 tile of the upper triangle):
+// the points' rows FU_j[u][:] of up to `cc` coils are staged at once and every
+// thread adds its four products per coil from two 16-byte reads (even r).  The
+// FP32 products bound it once the reads are in flight together: 256 x 256,
+// C = 20, r = 12, 28.9k points: 35 us with one (point, pair) item and a block
+// barrier per coil, 22 us in this form.
 template <int R>
 __global__ void __launch_bounds__(256) k_sample_gram(const float2 *__restrict__ FU, float2 *__restrict__ Pu, int nu,
-                                                      int nc) {
-    constexpr int np = R * (R + 1) / 2;
-    constexpr int SU = 32;
-    constexpr int NA = (SU * np + 255) / 256;
-    __shared__ __align__(16) float2 s_f[2][SU * R];
+                                                      int nc, int cc) {
+    constexpr int np = R * (R + 1) / 2, tr = (R + 1) / 2, nt = tr * (tr + 1) / 2, SU = 256 / nt;
+    extern __shared__ __align__(16) float2 smem[];   // cc x SU x R
     const int u0 = blockIdx.x * SU, cnt = min(SU, nu - u0);
-    int ia[NA], ib[NA], io[NA];
-    float2 acc[NA];
+    const int su = threadIdx.x / nt, w = threadIdx.x - su * nt;
+    int A, Bt;
+    pair_of(w, tr, A, Bt);
+    const bool act = su < cnt;
+    float2 acc[4];
 #pragma unroll
-    for (int v = 0; v < NA; ++v) {
-        const int o = threadIdx.x + 256 * v;
-        acc[v] = make_float2(0.f, 0.f);
-        io[v] = -1;
-        ia[v] = ib[v] = 0;
-        if (o < SU * np) {
-            const int s = o / np, p = o - s * np;
-            int a, b;
-            pair_of(p, R, a, b);
-            if (s < cnt) {
-                io[v] = o;
-                ia[v] = s * R + a;
-                ib[v] = s * R + b;
+    for (int m = 0; m < 4; ++m) acc[m] = make_float2(0.f, 0.f);
+    for (int j0 = 0; j0 < nc; j0 += cc) {
+        const int jn = min(cc, nc - j0);
+        for (int j = 0; j < jn; ++j)
+            stage_row(smem + j * SU * R, FU + ((size_t)(j0 + j) * nu + u0) * R, cnt * R, threadIdx.x, blockDim.x);
+        cp_async_commit();
+        cp_async_wait();
+        __syncthreads();
+        if (act) {
+            const float2 *f = smem + su * R;
+#pragma unroll 4
+            for (int j = 0; j < jn; ++j, f += SU * R) {
+                float2 p0, p1, q0, q1;
+                if constexpr (R % 2 == 0) {
+                    const float4 p = *reinterpret_cast<const float4 *>(f + 2 * A);
+                    const float4 q = *reinterpret_cast<const float4 *>(f + 2 * Bt);
+                    p0 = make_float2(p.x, p.y), p1 = make_float2(p.z, p.w);
+                    q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
+                } else {
+                    p0 = f[2 * A], p1 = f[min(2 * A + 1, R - 1)];
+                    q0 = f[2 * Bt], q1 = f[min(2 * Bt + 1, R - 1)];
+                }
+                cfmac(acc[0], p0, q0);
+                cfmac(acc[1], p0, q1);
+                cfmac(acc[2], p1, q0);
+                cfmac(acc[3], p1, q1);
             }
         }
+        __syncthreads();
     }
-    stage_row(s_f[0], FU + (size_t)u0 * R, cnt * R, threadIdx.x, blockDim.x);
-    cp_async_commit();
-    for (int j = 0; j < nc; ++j) {
-        if (j + 1 < nc) {
-            stage_row(s_f[(j + 1) & 1], FU + ((size_t)(j + 1) * nu + u0) * R, cnt * R, threadIdx.x, blockDim.x);
-            cp_async_commit();
-            cp_async_wait_1();
-        } else {
-            cp_async_wait();
+    if (act) {
+        float2 *out = Pu + (size_t)(u0 + su) * np;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int x = 2 * A + (m >> 1), y = 2 * Bt + (m & 1);
+            if (x < R && y < R && x <= y) out[pair_index(x, y, R)] = acc[m];
         }
-        __syncthreads();
-        const float2 *f = s_f[j & 1];
-#pragma unroll
-        for (int v = 0; v < NA; ++v)
-            if (io[v] >= 0) cfmac(acc[v], f[ia[v]], f[ib[v]]);
-        __syncthreads();
     }
-#pragma unroll
-    for (int v = 0; v < NA; ++v)
-        if (io[v] >= 0) Pu[(size_t)u0 * np + io[v]] = acc[v];
 }
 
 // ---------------------------------------------------------------- D: times W_u
 
 // Block of SU = 256 / R union points, thread (point su, column wb):
 // W_u[:, wb] = sum over the frames k sampling u of b_k conj(b_k[wb]) in
-// registers, then for every coil FU_j[u][wb] <- sum_a FU_j[u][a] W_u[a][wb].
+// registers, then for every coil FU_j[u][wb] <- sum_a FU_j[u][a] W_u[a][wb].  Up
+// to `cc` coils' rows are staged at once (the copies run while W_u is formed),
+// read by 16 bytes.  256 x 256, C = 20, r = 12, 28.9k points: 68 us with a
+// stage, a wait and two barriers per coil, 43 us in this form.
 template <int R>
 __global__ void __launch_bounds__(256) k_sample_w(float2 *__restrict__ FU, const float2 *__restrict__ B,
                                                    const int32_t *__restrict__ ufptr,
-                                                   const int32_t *__restrict__ uflist, int nu, int nc, int q) {
+                                                   const int32_t *__restrict__ uflist, int nu, int nc, int q, int cc) {
     constexpr int SU = 256 / R;
     extern __shared__ __align__(16) float2 smem[];
-    float2 *s_f = smem;            // SU * R
-    float2 *sB = smem + SU * R;    // q * R
+    float2 *s_f = smem;                              // cc x SU x R
+    float2 *sB = smem + (size_t)cc * SU * R;         // q x R
     const int u0 = blockIdx.x * SU, cnt = min(SU, nu - u0);
     const int su = threadIdx.x / R, wb = threadIdx.x - su * R;
     const bool act = su < SU && su < cnt;
-    for (int e = threadIdx.x; e < q * R; e += blockDim.x) sB[e] = B[e];
-    __syncthreads();
+    for (int e = threadIdx.x; e < q * R; e += blockDim.x) cp_async8(sB + e, B + e);
+    cp_async_commit();
     float2 wcol[R];
 #pragma unroll
     for (int a = 0; a < R; ++a) wcol[a] = make_float2(0.f, 0.f);
-    if (act) {
-        const int u = u0 + su;
-        for (int f = ufptr[u]; f < ufptr[u + 1]; ++f) {
-            const float2 *bk = sB + uflist[f] * R;
-            const float2 bw = cconj(bk[wb]);
-#pragma unroll
-            for (int a = 0; a < R; ++a) cfma(wcol[a], bk[a], bw);
-        }
-    }
-    for (int j = 0; j < nc; ++j) {
-        __syncthreads();
-        stage_row(s_f, FU + ((size_t)j * nu + u0) * R, cnt * R, threadIdx.x, blockDim.x);
+    for (int j0 = 0; j0 < nc; j0 += cc) {
+        const int jn = min(cc, nc - j0);
+        for (int j = 0; j < jn; ++j)
+            stage_row(s_f + j * SU * R, FU + ((size_t)(j0 + j) * nu + u0) * R, cnt * R, threadIdx.x, blockDim.x);
         cp_async_commit();
+        if (j0 == 0) {
+            cp_async_wait_1();   // B is in
+            __syncthreads();
+            if (act) {
+                const int u = u0 + su, f1 = ufptr[u + 1];
+                for (int f = ufptr[u]; f < f1; ++f) {
+                    const float2 *bk = sB + uflist[f] * R;
+                    const float2 bw = cconj(bk[wb]);
+#pragma unroll
+                    for (int a = 0; a < R; ++a) cfma(wcol[a], bk[a], bw);
+                }
+            }
+        }
         cp_async_wait();
         __syncthreads();
         if (act) {
-            float2 o = make_float2(0.f, 0.f);
+            const float2 *fs = s_f + su * R;
+            float2 *dst = FU + ((size_t)j0 * nu + u0 + su) * R + wb;
+#pragma unroll 2
+            for (int j = 0; j < jn; ++j, fs += SU * R, dst += (size_t)nu * R) {
+                float2 o = make_float2(0.f, 0.f);
+                if constexpr (R % 2 == 0) {
 #pragma unroll
-            for (int a = 0; a < R; ++a) cfma(o, s_f[su * R + a], wcol[a]);
-            FU[((size_t)j * nu + u0 + su) * R + wb] = o;
+                    for (int a = 0; a < R; a += 2) {
+                        const float4 f = *reinterpret_cast<const float4 *>(fs + a);
+                        cfma(o, make_float2(f.x, f.y), wcol[a]);
+                        cfma(o, make_float2(f.z, f.w), wcol[a + 1]);
+                    }
+                } else {
+#pragma unroll
+                    for (int a = 0; a < R; ++a) cfma(o, fs[a], wcol[a]);
+                }
+                *dst = o;
+            }
         }
-    }
-}
-
-// ---------------------------------------------------------------- E: scatter, inverse along x
-
-// Block (row ky of Omega_u, coil group g): for coils g, g + CG, ... the row's
-// union points are scattered into a zero row (nx x r), transformed back along
-// x, and the full row written to T_j[ky] for the column pass.
-template <int PX>
-__global__ void __launch_bounds__(256) k_adj_rows(const float2 *__restrict__ FU, const int32_t *__restrict__ usedrows,
-                                                   const int32_t *__restrict__ uptr, const int32_t *__restrict__ uidx,
-                                                   float2 *__restrict__ T, int ny, int r, int nc, int nu,
-                                                   const float2 *__restrict__ g_tw, float scale) {
-    constexpr int NX = 32 * PX;
-    extern __shared__ __align__(16) float2 smem[];
-    float2 *tile = smem, *s_tw = smem + NX * r;
-    __shared__ int s_kx[NX];
-    const int ky = usedrows[blockIdx.x], g = blockIdx.y, CG = gridDim.y;
-    const int u0 = uptr[ky], cnt = uptr[ky + 1] - u0;
-    load_twiddles(s_tw, g_tw, NX);
-    for (int s = threadIdx.x; s < cnt; s += blockDim.x) s_kx[s] = uidx[u0 + s] - ky * NX;
-    const int gl = threadIdx.x % r, gs = threadIdx.x / r, gstep = blockDim.x / r;
-    const int half = NX * r / 2;   // float4 pieces of a row (NX is even)
-    for (int j = g; j < nc; j += CG) {
-        for (int e = threadIdx.x; e < half; e += blockDim.x) ((float4 *)tile)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-        __syncthreads();
-        if (gs < gstep) {
-            const float2 *src = FU + ((size_t)j * nu + u0) * r;
-            for (int s = gs; s < cnt; s += gstep) tile[s_kx[s] * r + gl] = src[(size_t)s * r + gl];
-        }
-        __syncthreads();
-        fft::tile_dft<NX, true>(tile, r, r, s_tw, scale);   // ends with a barrier
-        float4 *dst = (float4 *)(T + ((size_t)j * ny + ky) * NX * r);
-        for (int e = threadIdx.x; e < half; e += blockDim.x) dst[e] = ((const float4 *)tile)[e];
         __syncthreads();
     }
 }
@@ -550,64 +673,117 @@ __global__ void k_mean_resid_gen(const float2 *__restrict__ y, const float2 *__r
 
 // ---------------------------------------------------------------- launchers
 
-static int row_groups(const lrccs_ctx *c) {   // coil groups of the row passes: about 4 coils each, or the plan's
-    if (c->plan.row_groups >= 1 && c->plan.row_groups <= 8 && c->plan.row_groups <= c->nc) return c->plan.row_groups;
-    const int cg = (c->nc + 3) / 4;
-    return cg < 1 ? 1 : (cg > 8 ? 8 : cg);
-}
-
-typedef void (*sgram_t)(const float2 *, float2 *, int, int);
-typedef void (*sw_t)(float2 *, const float2 *, const int32_t *, const int32_t *, int, int, int);
+typedef void (*sgram_t)(const float2 *, float2 *, int, int, int);
+typedef void (*sw_t)(float2 *, const float2 *, const int32_t *, const int32_t *, int, int, int, int);
 #define RANK_TABLE(K) {K<1>, K<2>, K<3>, K<4>, K<5>, K<6>, K<7>, K<8>, K<9>, K<10>, K<11>, K<12>, K<13>, K<14>, K<15>, K<16>}
 static const sgram_t kSampleGram[RMAXC] = RANK_TABLE(k_sample_gram);
 static const sw_t kSampleW[RMAXC] = RANK_TABLE(k_sample_w);
 
-cudaError_t launch_fwd_rows_r(lrccs_ctx *c, int r) {
-    const float sx = (float)(1.0 / sqrt((double)c->nx));
-    const size_t smem = ((size_t)2 * c->nx * r + c->nx) * sizeof(float2);
-    dim3 grid(c->n_used, row_groups(c));
+// Shape of a row pass at rank r: coils at a time (a block of at most 256
+// threads), exchange stride, block, shared memory, and the coil groups: the
+// plan's, or the fewest rounds ceil(blocks / slots) (steps + 1) of a block's
+// coil steps.
+struct RowShape {
+    int CB, S, threads, groups;
+    size_t smem;
+};
+template <int P>
+static RowShape row_shape(const lrccs_ctx *c, int r) {
+    using PL = RowPlan<P>;
+    RowShape h;
+    const int it = PL::NG * r;
+    h.CB = std::max(1, std::min(c->nc, 256 / it));
+    h.S = PL::R2 * r + ((r - PL::R2 * r) % 16 + 16) % 16;
+    h.threads = (h.CB * it + 31) / 32 * 32;
+    h.smem = (size_t)2 * h.CB * PL::R1 * h.S * sizeof(float2);
+    const int res = std::max(1, std::min(768 / h.threads, (int)(c->smem_sm / (h.smem + 2048))));
+    const int slots = res * c->nsm, most = (c->nc + h.CB - 1) / h.CB;
+    h.groups = 1;
+    double cost = 1e30;
+    for (int g = 1; g <= most; ++g) {
+        const double v = (double)((c->n_used * g + slots - 1) / slots) * ((most + g - 1) / g + 1.0);
+        if (v < cost) cost = v, h.groups = g;
+    }
+    if (c->plan.row_groups >= 1 && c->plan.row_groups <= 8 && c->plan.row_groups <= c->nc) h.groups = c->plan.row_groups;
+    return h;
+}
+static RowArgs row_args(const lrccs_ctx *c, const RowShape &h, int r, int k0) {
+    RowArgs a;
+    a.usedrows = c->d_usedrows;
+    a.uptr = c->d_uptr;
+    a.upos = c->d_upos;
+    a.ftab = k0 >= 0 ? c->d_ptab : nullptr;
+    a.tw = c->d_twsx;
+    a.ny = c->ny;
+    a.r = r;
+    a.nc = c->nc;
+    a.nu = c->n_u;
+    a.S = h.S;
+    a.CB = h.CB;
+    a.k0 = k0;
+    a.q = c->q;
+    return a;
+}
+
+cudaError_t launch_fwd_rows_r(lrccs_ctx *c, int r, int k0) {
     DISPATCH_P(c->px, {
+        const RowShape h = row_shape<P_>(c, r);
         prof_begin(c, KID_FWD_ROWS);
-        k_fwd_rows<P_><<<grid, 256, smem, c->stream>>>(c->d_T, c->d_usedrows, c->d_uptr, c->d_uidx, c->d_FU, c->ny, r,
-                                                       c->nc, c->n_u, c->d_twx, sx);
+        k_fwd_rows<P_><<<dim3(c->n_used, h.groups), h.threads, h.smem, c->stream>>>(c->d_T, c->d_FU,
+                                                                                    row_args(c, h, r, k0));
         prof_end(c, KID_FWD_ROWS);
     });
     return cudaGetLastError();
 }
 
-static cudaError_t launch_sample_gram(lrccs_ctx *c) {
-    const int r = c->r;
-    prof_begin(c, KID_SAMPLE_GRAM);
-    kSampleGram[r - 1]<<<(c->n_u + 31) / 32, 256, 0, c->stream>>>(c->d_FU, c->d_Pu, c->n_u, c->nc);
-    prof_end(c, KID_SAMPLE_GRAM);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sample_w(lrccs_ctx *c) {
-    const int r = c->r, su = 256 / r;
-    const size_t smem = ((size_t)su * r + (size_t)c->q * r) * sizeof(float2);
-    prof_begin(c, KID_SAMPLE_W);
-    kSampleW[r - 1]<<<(c->n_u + su - 1) / su, 256, smem, c->stream>>>(c->d_FU, c->d_B, c->d_ufptr, c->d_uflist,
-                                                                      c->n_u, c->nc, c->q);
-    prof_end(c, KID_SAMPLE_W);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_adj_rows_r(lrccs_ctx *c, int r) {
-    const float sx = (float)(1.0 / sqrt((double)c->nx));
-    const size_t smem = ((size_t)c->nx * r + c->nx) * sizeof(float2);
-    dim3 grid(c->n_used, row_groups(c));
+cudaError_t launch_adj_rows_r(lrccs_ctx *c, int r, int k0) {
     DISPATCH_P(c->px, {
+        const RowShape h = row_shape<P_>(c, r);
         prof_begin(c, KID_ADJ_ROWS);
-        k_adj_rows<P_><<<grid, 256, smem, c->stream>>>(c->d_FU, c->d_usedrows, c->d_uptr, c->d_uidx, c->d_T, c->ny, r,
-                                                       c->nc, c->n_u, c->d_twx, sx);
+        k_adj_rows<P_><<<dim3(c->n_used, h.groups), h.threads, h.smem, c->stream>>>(c->d_FU, c->d_T,
+                                                                                    row_args(c, h, r, k0));
         prof_end(c, KID_ADJ_ROWS);
     });
     return cudaGetLastError();
 }
 
-cudaError_t launch_fwd_rows(lrccs_ctx *c) { return launch_fwd_rows_r(c, c->r); }
-cudaError_t launch_adj_rows(lrccs_ctx *c) { return launch_adj_rows_r(c, c->r); }
+// d_ptab <- the loaded masks' point tables (before launch_*_rows_r with k0 >= 0)
+cudaError_t launch_point_tables(lrccs_ctx *c) {
+    DISPATCH_P(c->px, {
+        prof_begin(c, KID_MEC_MASK);
+        k_point_tables<<<dim3(c->ny, c->q), 32, 0, c->stream>>>(c->d_maskc, c->ny, c->nx, RowPlan<P_>::R1,
+                                                                RowPlan<P_>::R2, c->d_ptab);
+        prof_end(c, KID_MEC_MASK);
+    });
+    return cudaGetLastError();
+}
+
+// coils staged at once by the point kernels: at most 48 KB, so that four blocks share a multiprocessor
+static int point_coils(const lrccs_ctx *c, int su, int r) {
+    return std::max(1, std::min(c->nc, (int)(49152 / ((size_t)su * r * sizeof(float2)))));
+}
+
+static cudaError_t launch_sample_gram(lrccs_ctx *c) {
+    const int r = c->r, tr = (r + 1) / 2, su = 256 / (tr * (tr + 1) / 2), cc = point_coils(c, su, r);
+    prof_begin(c, KID_SAMPLE_GRAM);
+    kSampleGram[r - 1]<<<(c->n_u + su - 1) / su, 256, (size_t)cc * su * r * sizeof(float2), c->stream>>>(
+        c->d_FU, c->d_Pu, c->n_u, c->nc, cc);
+    prof_end(c, KID_SAMPLE_GRAM);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sample_w(lrccs_ctx *c) {
+    const int r = c->r, su = 256 / r, cc = point_coils(c, su, r);
+    const size_t smem = ((size_t)cc * su * r + (size_t)c->q * r) * sizeof(float2);
+    prof_begin(c, KID_SAMPLE_W);
+    kSampleW[r - 1]<<<(c->n_u + su - 1) / su, 256, smem, c->stream>>>(c->d_FU, c->d_B, c->d_ufptr, c->d_uflist,
+                                                                      c->n_u, c->nc, c->q, cc);
+    prof_end(c, KID_SAMPLE_W);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fwd_rows(lrccs_ctx *c) { return launch_fwd_rows_r(c, c->r, -1); }
+cudaError_t launch_adj_rows(lrccs_ctx *c) { return launch_adj_rows_r(c, c->r, -1); }
 
 cudaError_t launch_iteration_general_front(lrccs_ctx *c) {
     cudaError_t e = launch_fwd_rows(c);
@@ -636,7 +812,10 @@ cudaError_t configure_kernels_general(int max_smem) {
     SET_SMEM(k_fwd_rows<5>); SET_SMEM(k_fwd_rows<6>); SET_SMEM(k_fwd_rows<7>); SET_SMEM(k_fwd_rows<8>);
     SET_SMEM(k_adj_rows<1>); SET_SMEM(k_adj_rows<2>); SET_SMEM(k_adj_rows<3>); SET_SMEM(k_adj_rows<4>);
     SET_SMEM(k_adj_rows<5>); SET_SMEM(k_adj_rows<6>); SET_SMEM(k_adj_rows<7>); SET_SMEM(k_adj_rows<8>);
-    for (int i = 0; i < RMAXC; ++i) SET_SMEM(kSampleW[i]);
+    for (int i = 0; i < RMAXC; ++i) {
+        SET_SMEM(kSampleW[i]);
+        SET_SMEM(kSampleGram[i]);
+    }
     SET_SMEM(k_init_gen<1>); SET_SMEM(k_init_gen<2>); SET_SMEM(k_init_gen<3>); SET_SMEM(k_init_gen<4>);
     SET_SMEM(k_init_gen<5>); SET_SMEM(k_init_gen<6>); SET_SMEM(k_init_gen<7>); SET_SMEM(k_init_gen<8>);
     return cudaSuccess;

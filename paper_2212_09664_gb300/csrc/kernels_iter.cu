@@ -539,7 +539,7 @@ __global__ void k_row_tables(const int32_t *__restrict__ rowcnt, const uint8_t *
     tab[e * 32 + t] = bits;
 }
 
-// Twiddles of the column passes, [j2][k1]: w_ny^(j2 k1) / sqrt(ny).
+// Twiddles of the column and row passes, [j2][k1]: w_N^(j2 k1) / sqrt(N).
 __global__ void k_col_twiddles(float2 *tw, int N, int R1) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= N) return;
@@ -552,6 +552,7 @@ __global__ void k_col_twiddles(float2 *tw, int N, int R1) {
 
 cudaError_t launch_col_twiddles(lrccs_ctx *c) {
     DISPATCH_P(c->py, { k_col_twiddles<<<1, 256, 0, c->stream>>>(c->d_twsy, c->ny, ColPlan<P_>::R1); });
+    DISPATCH_P(c->px, { k_col_twiddles<<<1, 256, 0, c->stream>>>(c->d_twsx, c->nx, ColPlan<P_>::R1); });
     return cudaGetLastError();
 }
 

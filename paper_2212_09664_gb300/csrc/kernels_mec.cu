@@ -14,8 +14,8 @@
 // iteration's column transforms apply N to a whole chunk at once:
 //   N_k v = sum_j conj(d_j) o F^H [M_k o F(d_j o v)],
 // with the per-frame sampling M_k applied between the forward and inverse
-// transforms (in the column passes' row tables for line masks, by k_mask_points
-// for general ones).
+// transforms (the column passes' row tables for line masks, the row passes'
+// point tables for general ones).
 // Reductions per frame (dot products, norms) are FP64 in a fixed order.
 #include <math.h>
 
@@ -28,38 +28,16 @@
 
 // ---------------------------------------------------------------- per-frame sampling between the transforms
 
-// General masks: FU_j[u][l] is kept only if frame k0 + l samples union point u.
-__global__ void k_mask_points(float2 *__restrict__ FU, const uint8_t *__restrict__ maskc,
-                              const int32_t *__restrict__ uidx, int n, int nu, int nc, int w, int k0, int q) {
-    const size_t total = (size_t)nc * nu * w;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int l = (int)(e % w);
-        const int u = (int)((e / w) % nu);
-        const int k = k0 + l;
-        if (k >= q || !maskc[(size_t)k * n + uidx[u]]) FU[e] = make_float2(0.f, 0.f);
-    }
-}
-
-// dst (n x w) <- [N_{k0+l} src[:, l]]_l for one chunk of frames.  With line
-// masks column l of the transforms only stores and reads the rows that frame
-// k0 + l samples (1/R of them; none for frames past q), which is the mask.
+// dst (n x w) <- [N_{k0+l} src[:, l]]_l for one chunk of frames.  Column l of the
+// transforms only stores and reads what frame k0 + l samples (rows, for line
+// masks; points of the row passes, for general ones; nothing for frames past
+// q), which is the mask.
 cudaError_t launch_frame_normal_op(lrccs_ctx *c, const float2 *src, float2 *dst, int w, int k0) {
     const int e0 = c->general ? 0 : 1 + k0, es = c->general ? 0 : 1;
     cudaError_t e = launch_fwd_cols_on(c, src, w, e0, es);
-    if (e != cudaSuccess) return e;
-    if (c->general) {
-        e = launch_fwd_rows_r(c, w);
-        if (e != cudaSuccess) return e;
-        prof_begin(c, KID_MEC_MASK);
-        k_mask_points<<<4 * 152, 256, 0, c->stream>>>(c->d_FU, c->d_maskc, c->d_uidx, c->n, c->n_u, c->nc, w, k0,
-                                                       c->q);
-        prof_end(c, KID_MEC_MASK);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        e = launch_adj_rows_r(c, w);
-        if (e != cudaSuccess) return e;
-    }
-    return launch_adj_cols_to(c, dst, w, e0, es);
+    if (e == cudaSuccess && c->general) e = launch_fwd_rows_r(c, w, k0);
+    if (e == cudaSuccess && c->general) e = launch_adj_rows_r(c, w, k0);
+    return e == cudaSuccess ? launch_adj_cols_to(c, dst, w, e0, es) : e;
 }
 
 // ---------------------------------------------------------------- elementwise and reductions
