@@ -36,6 +36,7 @@ cudaError_t configure_kernels_general(int max_smem);
 cudaError_t configure_kernels_tc(int max_smem);
 cudaError_t configure_kernels_zh(int max_smem);
 cudaError_t configure_kernels_solve(int max_smem);
+cudaError_t configure_kernels_mec(int max_smem);
 
 #define CK(call)                                                                        \
     do {                                                                                \
@@ -253,6 +254,7 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     if (e == cudaSuccess) e = configure_kernels_tc(optin);
     if (e == cudaSuccess) e = configure_kernels_zh(optin);
     if (e == cudaSuccess) e = configure_kernels_solve(optin);
+    if (e == cudaSuccess) e = configure_kernels_mec(optin);
     if (e == cudaSuccess) {
         c->nsm = nsm;
         cudaDeviceGetAttribute(&c->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);

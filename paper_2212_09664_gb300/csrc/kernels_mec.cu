@@ -220,128 +220,215 @@ __global__ void k_mec_out(const float2 *__restrict__ E, const float2 *__restrict
 
 // ---------------------------------------------------------------- MEC-2: DFT along the frames
 
-#define TD_PIX 8   // pixels per block of the temporal transforms
+// Temporal transforms: every pixel's q values times the q x q DFT matrix.  A
+// thread forms output f (with q even also f + q/2, whose sum differs only in the
+// sign of the odd inputs, so half the products serve both) for TD_P pixels at
+// once: per input frame one twiddle and four broadcast 16-byte reads feed the
+// 8 complex products, which FP32 issue bounds.  H = q/2 or q output pairs by
+// 256 / H pixel groups fill the block.  192 x 192, q = 48, kernel time: 327 + 42
+// (the sums of its blocks) -> 63 us forward, 45 -> 29 us back.
+#define TD_P 8                  // pixels per thread
+#define TD_S (TD_P + 2)         // shared stride of a frame's pixels (16-byte aligned, spread over the banks)
 
-// M[:, i] = F_t (E + S0 - V)[i, :] (unitary DFT over the q frames, tw[t] =
-// exp(-2 pi i t / q)) for TD_PIX pixels per block, and the block's max |M|,
-// sum |M - Mprev|^2 and sum |Mprev|^2 (when have_prev) into part[blk][3].
-__global__ void __launch_bounds__(256) k_tdft_fwd(const float2 *__restrict__ E, const float2 *__restrict__ S0,
-                                                  const float2 *__restrict__ V, const float2 *__restrict__ Mprev,
-                                                  const float2 *__restrict__ tw, int n, int q, int w, int have_v,
-                                                  int have_prev, float2 *__restrict__ M, double *part) {
-    extern __shared__ float2 s_g[];           // TD_PIX * q, then tw (q)
-    float2 *s_tw = s_g + TD_PIX * q;
-    __shared__ double s_r[3][256];
-    const int i0 = blockIdx.x * TD_PIX;
-    const float sc = rsqrtf((float)q);
-    for (int t = threadIdx.x; t < q; t += blockDim.x) s_tw[t] = tw[t];
-    for (int e = threadIdx.x; e < TD_PIX * q; e += blockDim.x) {
-        const int p = e / q, k = e - p * q, i = i0 + p;
-        float2 g = make_float2(0.f, 0.f);
-        if (i < n) {
-            const size_t o = ((size_t)(k / w) * n + i) * w + (k % w);
-            g = cadd(E[o], S0[o]);
-            if (have_v) g = csub(g, V[o]);
+struct TdShape {
+    int H, groups, pix;         // output pairs, pixel groups per block, pixels per block
+    size_t smem;
+};
+__host__ __device__ inline TdShape td_shape(int q) {
+    TdShape t;
+    t.H = (q & 1) ? q : q / 2;
+    t.groups = 256 / t.H;
+    t.pix = t.groups * TD_P;
+    t.smem = ((size_t)t.groups * q * TD_S + q) * sizeof(float2);
+    return t;
+}
+
+// The block's sums over frames of s_g[(group q + k) TD_S + p] times tw^(f k):
+// thread (group pg, f) receives its outputs f in lo (and f + H in hi, q even).
+template <bool INV>
+LRCCS_DEV void td_dft(const float2 *s_g, const float2 *s_tw, int q, int H, int pg, int f, float2 (&lo)[TD_P],
+                      float2 (&hi)[TD_P]) {
+    float2 ev[TD_P], od[TD_P];
+#pragma unroll
+    for (int p = 0; p < TD_P; ++p) ev[p] = od[p] = make_float2(0.f, 0.f);
+    const float2 *g = s_g + (size_t)pg * q * TD_S;
+    auto step = [&](float2 (&acc)[TD_P], int k, int t) {
+        float2 w = s_tw[t];
+        if (INV) w.y = -w.y;
+        const float4 *g4 = reinterpret_cast<const float4 *>(g + k * TD_S);
+#pragma unroll
+        for (int p = 0; p < TD_P; p += 2) {
+            const float4 v = g4[p / 2];
+            cfma(acc[p], make_float2(v.x, v.y), w);
+            cfma(acc[p + 1], make_float2(v.z, v.w), w);
         }
-        s_g[e] = g;
-    }
-    __syncthreads();
-    double mx = 0.0, dd = 0.0, pp = 0.0;
-    for (int e = threadIdx.x; e < TD_PIX * q; e += blockDim.x) {
-        const int p = e / q, f = e - p * q, i = i0 + p;
-        if (i >= n) continue;
-        float2 acc = make_float2(0.f, 0.f);
-        int t = 0;
+    };
+    int t = 0;
+    if (q & 1) {
         for (int k = 0; k < q; ++k) {
-            cfma(acc, s_g[p * q + k], s_tw[t]);
+            step(ev, k, t);
             t += f;
             if (t >= q) t -= q;
         }
-        acc = cscale(acc, sc);
-        const size_t o = ((size_t)(f / w) * n + i) * w + (f % w);
-        M[o] = acc;
-        mx = fmax(mx, sqrt((double)acc.x * acc.x + (double)acc.y * acc.y));
-        if (have_prev) {
-            const float2 m0 = Mprev[o];
-            const double dx = (double)acc.x - m0.x, dy = (double)acc.y - m0.y;
-            dd += dx * dx + dy * dy;
-            pp += (double)m0.x * m0.x + (double)m0.y * m0.y;
-        }
+#pragma unroll
+        for (int p = 0; p < TD_P; ++p) lo[p] = ev[p];
+        return;
     }
-    s_r[0][threadIdx.x] = mx;
-    s_r[1][threadIdx.x] = dd;
-    s_r[2][threadIdx.x] = pp;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0, cc = 0.0;
-        for (int t = 0; t < (int)blockDim.x; ++t) {
-            a = fmax(a, s_r[0][t]);
-            b += s_r[1][t];
-            cc += s_r[2][t];
-        }
-        part[(size_t)blockIdx.x * 3 + 0] = a;
-        part[(size_t)blockIdx.x * 3 + 1] = b;
-        part[(size_t)blockIdx.x * 3 + 2] = cc;
+    for (int k = 0; k < q; k += 2) {
+        step(ev, k, t);
+        t += f;
+        if (t >= q) t -= q;
+        step(od, k + 1, t);
+        t += f;
+        if (t >= q) t -= q;
+    }
+#pragma unroll
+    for (int p = 0; p < TD_P; ++p) {
+        lo[p] = cadd(ev[p], od[p]);
+        hi[p] = csub(ev[p], od[p]);
     }
 }
 
-// out[0] = max, out[1], out[2] = sums of the nb block partials (fixed order).
-__global__ void k_tdft_finish(const double *__restrict__ part, int nb, double *out) {
-    __shared__ double s_r[3][256];
-    double a = 0.0, b = 0.0, c = 0.0;
-    for (int t = threadIdx.x; t < nb; t += blockDim.x) {
-        a = fmax(a, part[(size_t)t * 3]);
-        b += part[(size_t)t * 3 + 1];
-        c += part[(size_t)t * 3 + 2];
-    }
-    s_r[0][threadIdx.x] = a;
-    s_r[1][threadIdx.x] = b;
-    s_r[2][threadIdx.x] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {   // thread 0's own partials are in a, b, c already
-        for (int t = 1; t < (int)blockDim.x; ++t) {
-            a = fmax(a, s_r[0][t]);
-            b += s_r[1][t];
-            c += s_r[2][t];
+// Fill s_g from get(offset) at every (frame, pixel) of the block's pixels.
+template <class GET>
+LRCCS_DEV void td_fill(float2 *s_g, int q, int w, int n, int pix, GET get) {
+    const int i0 = blockIdx.x * pix, cnt = pix * w;
+    for (int cc = 0; cc * w < q; ++cc)
+        for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+            const int p = e / w, l = e - p * w, k = cc * w + l;
+            if (k < q)
+                s_g[((p / TD_P) * q + k) * TD_S + p % TD_P] =
+                    i0 + p < n ? get(((size_t)cc * n + i0 + p) * w + l) : make_float2(0.f, 0.f);
         }
-        out[0] = a;
-        out[1] = b;
-        out[2] = c;
+}
+
+// M[:, i] = F_t (E + S0 - V)[i, :] (unitary DFT over the q frames, tw[t] =
+// exp(-2 pi i t / q)), and over the whole grid max |M| (first step only, Mprev
+// NULL) or sum |M - Mprev|^2 and sum |Mprev|^2 into out[3]: FP32 pairs that keep
+// the rounding of every square and addition per thread, FP64 from there, in a
+// fixed order.
+LRCCS_DEV void fsum_sq(fsum2 &s, float x) {
+    const float p = __fmul_rn(x, x);
+    fsum_add(s, p);
+    s.lo += fmaf(x, x, -p);
+}
+__global__ void __launch_bounds__(256, 3) k_tdft_fwd(const float2 *__restrict__ E, const float2 *__restrict__ S0,
+                                                     const float2 *__restrict__ V, const float2 *__restrict__ Mprev,
+                                                     const float2 *__restrict__ tw, int n, int q, int w,
+                                                     float2 *__restrict__ M, double *part, unsigned int *counter,
+                                                     double *out) {
+    extern __shared__ __align__(16) float2 s_g[];
+    const TdShape t = td_shape(q);
+    float2 *s_tw = s_g + (size_t)t.groups * q * TD_S;
+    __shared__ double s_r[3][8];
+    const int i0 = blockIdx.x * t.pix, lane = threadIdx.x & 31;
+    const float sc = rsqrtf((float)q);
+    for (int i = threadIdx.x; i < q; i += blockDim.x) s_tw[i] = tw[i];
+    td_fill(s_g, q, w, n, t.pix, [&](size_t o) {
+        float2 g = cadd(E[o], S0[o]);
+        if (V) g = csub(g, V[o]);
+        return g;
+    });
+    __syncthreads();
+    double mx = 0.0;
+    fsum2 dd = {0.f, 0.f}, pp = {0.f, 0.f};
+    const int pg = threadIdx.x / t.H, f0 = threadIdx.x - pg * t.H;
+    if (pg < t.groups) {
+        float2 lo[TD_P], hi[TD_P];
+        td_dft<false>(s_g, s_tw, q, t.H, pg, f0, lo, hi);
+        auto put = [&](const float2 (&v)[TD_P], int f) {
+            const int cc = f / w, l = f - cc * w;
+#pragma unroll
+            for (int p = 0; p < TD_P; ++p) {
+                const int i = i0 + pg * TD_P + p;
+                if (i >= n) continue;
+                const size_t o = ((size_t)cc * n + i) * w + l;
+                const float2 m = cscale(v[p], sc);
+                M[o] = m;
+                if (Mprev) {
+                    const float2 m0 = Mprev[o];
+                    float d, e;   // the difference and its rounding, exactly
+                    two_sum(m.x, -m0.x, d, e);
+                    fsum_sq(dd, d);
+                    dd.lo += 2.f * d * e;
+                    two_sum(m.y, -m0.y, d, e);
+                    fsum_sq(dd, d);
+                    dd.lo += 2.f * d * e;
+                    fsum_sq(pp, m0.x);
+                    fsum_sq(pp, m0.y);
+                } else {
+                    mx = fmax(mx, (double)m.x * m.x + (double)m.y * m.y);
+                }
+            }
+        };
+        put(lo, f0);
+        if (!(q & 1)) put(hi, f0 + t.H);
     }
+    // block, then grid: [0] max |M|^2, [1] sum |M - Mprev|^2, [2] sum |Mprev|^2
+    double v[3] = {mx, (double)dd.hi + (double)dd.lo, (double)pp.hi + (double)pp.lo};
+    for (int o = 16; o > 0; o >>= 1) v[0] = fmax(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
+    v[1] = warp_sum_d(v[1]);
+    v[2] = warp_sum_d(v[2]);
+    if (lane == 0)
+        for (int c = 0; c < 3; ++c) s_r[c][threadIdx.x >> 5] = v[c];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double a = 0.0, b = 0.0, c = 0.0;
+        for (int x = 0; x < 8; ++x) {
+            a = fmax(a, s_r[0][x]);
+            b += s_r[1][x];
+            c += s_r[2][x];
+        }
+        part[(size_t)blockIdx.x * 3] = a;
+        part[(size_t)blockIdx.x * 3 + 1] = b;
+        part[(size_t)blockIdx.x * 3 + 2] = c;
+    }
+    if (!last_block_arrive(counter) || threadIdx.x >= 96) return;
+    const int c = threadIdx.x >> 5;   // a warp per result
+    double r = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) {
+        const double x = __ldcg(part + (size_t)b * 3 + c);
+        r = c == 0 ? fmax(r, x) : r + x;
+    }
+    if (c == 0) {
+        for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
+        r = sqrt(r);
+    } else {
+        r = warp_sum_d(r);
+    }
+    if (lane == 0) out[c] = r;
 }
 
 // E[i, :] = F_t^{-1} SThr_omega(M[:, i]): the complex soft threshold
 // m (|m| - omega) / |m| for |m| > omega, else 0, then the inverse unitary DFT.
-__global__ void __launch_bounds__(256) k_tdft_inv(const float2 *__restrict__ M, const float2 *__restrict__ tw, int n,
-                                                  int q, int w, float omega, float2 *__restrict__ E) {
-    extern __shared__ float2 s_g[];
-    float2 *s_tw = s_g + TD_PIX * q;
-    const int i0 = blockIdx.x * TD_PIX;
+__global__ void __launch_bounds__(256, 3) k_tdft_inv(const float2 *__restrict__ M, const float2 *__restrict__ tw, int n,
+                                                     int q, int w, float omega, float2 *__restrict__ E) {
+    extern __shared__ __align__(16) float2 s_g[];
+    const TdShape t = td_shape(q);
+    float2 *s_tw = s_g + (size_t)t.groups * q * TD_S;
+    const int i0 = blockIdx.x * t.pix;
     const float sc = rsqrtf((float)q);
-    for (int t = threadIdx.x; t < q; t += blockDim.x) s_tw[t] = tw[t];
-    for (int e = threadIdx.x; e < TD_PIX * q; e += blockDim.x) {
-        const int p = e / q, f = e - p * q, i = i0 + p;
-        float2 m = make_float2(0.f, 0.f);
-        if (i < n) {
-            m = M[((size_t)(f / w) * n + i) * w + (f % w)];
-            const float a = sqrtf(m.x * m.x + m.y * m.y);
-            m = a > omega ? cscale(m, (a - omega) / a) : make_float2(0.f, 0.f);
-        }
-        s_g[e] = m;
-    }
+    for (int i = threadIdx.x; i < q; i += blockDim.x) s_tw[i] = tw[i];
+    td_fill(s_g, q, w, n, t.pix, [&](size_t o) {
+        const float2 m = M[o];
+        const float a = sqrtf(m.x * m.x + m.y * m.y);
+        return a > omega ? cscale(m, (a - omega) / a) : make_float2(0.f, 0.f);
+    });
     __syncthreads();
-    for (int e = threadIdx.x; e < TD_PIX * q; e += blockDim.x) {
-        const int p = e / q, k = e - p * q, i = i0 + p;
-        if (i >= n) continue;
-        float2 acc = make_float2(0.f, 0.f);
-        int t = 0;
-        for (int f = 0; f < q; ++f) {
-            cfma(acc, s_g[p * q + f], cconj(s_tw[t]));
-            t += k;
-            if (t >= q) t -= q;
+    const int pg = threadIdx.x / t.H, f0 = threadIdx.x - pg * t.H;
+    if (pg >= t.groups) return;
+    float2 lo[TD_P], hi[TD_P];
+    td_dft<true>(s_g, s_tw, q, t.H, pg, f0, lo, hi);
+    auto put = [&](const float2 (&v)[TD_P], int k) {
+        const int cc = k / w, l = k - cc * w;
+#pragma unroll
+        for (int p = 0; p < TD_P; ++p) {
+            const int i = i0 + pg * TD_P + p;
+            if (i < n) E[((size_t)cc * n + i) * w + l] = cscale(v[p], sc);
         }
-        E[((size_t)(k / w) * n + i) * w + (k % w)] = cscale(acc, sc);
-    }
+    };
+    put(lo, f0);
+    if (!(q & 1)) put(hi, f0 + t.H);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -394,29 +481,32 @@ cudaError_t launch_mec_out(lrccs_ctx *c, const float2 *E, const float2 *zbar, fl
 
 cudaError_t launch_tdft_fwd(lrccs_ctx *c, const float2 *E, const float2 *S0, const float2 *V, const float2 *Mprev,
                             float2 *M, double *out) {
-    const int nb = (c->n + TD_PIX - 1) / TD_PIX;
-    const size_t smem = (size_t)(TD_PIX + 1) * c->q * sizeof(float2);
+    const TdShape t = td_shape(c->q);
     double *part = c->d_mscal + 3 * c->q;
     prof_begin(c, KID_MEC_TDFT);
-    k_tdft_fwd<<<nb, 256, smem, c->stream>>>(E, S0, V, Mprev, c->d_twq, c->n, c->q, c->mec_w, V != nullptr,
-                                             Mprev != nullptr, M, part);
-    k_tdft_finish<<<1, 256, 0, c->stream>>>(part, nb, out);
+    k_tdft_fwd<<<(c->n + t.pix - 1) / t.pix, 256, t.smem, c->stream>>>(E, S0, V, Mprev, c->d_twq, c->n, c->q, c->mec_w, M,
+                                                                      part, c->d_counters + CNT_MEC, out);
     prof_end(c, KID_MEC_TDFT);
     return cudaGetLastError();
 }
 
 cudaError_t launch_tdft_inv(lrccs_ctx *c, const float2 *M, float omega, float2 *E) {
-    const int nb = (c->n + TD_PIX - 1) / TD_PIX;
-    const size_t smem = (size_t)(TD_PIX + 1) * c->q * sizeof(float2);
+    const TdShape t = td_shape(c->q);
     prof_begin(c, KID_MEC_TDFT);
-    k_tdft_inv<<<nb, 256, smem, c->stream>>>(M, c->d_twq, c->n, c->q, c->mec_w, omega, E);
+    k_tdft_inv<<<(c->n + t.pix - 1) / t.pix, 256, t.smem, c->stream>>>(M, c->d_twq, c->n, c->q, c->mec_w, omega, E);
     prof_end(c, KID_MEC_TDFT);
     return cudaGetLastError();
 }
 
-// Scratch of the reductions: 3 q FP64 scalars, then max(G q', 3 ceil(n / TD_PIX)) partials.
+// Scratch of the reductions: 3 q FP64 scalars, then the partials of the frame
+// sums (G per column) or of the temporal transform (3 per block).
 size_t mec_scal_count(int n, int q, int w) {
-    const int nch = (q + w - 1) / w;
-    const size_t a = (size_t)MEC_G * nch * w, b = (size_t)3 * ((n + TD_PIX - 1) / TD_PIX);
+    const int nch = (q + w - 1) / w, pix = td_shape(q).pix;
+    const size_t a = (size_t)MEC_G * nch * w, b = (size_t)3 * ((n + pix - 1) / pix);
     return (size_t)3 * q + (a > b ? a : b) + 8;
+}
+
+cudaError_t configure_kernels_mec(int max_smem) {
+    cudaError_t e = allow_smem(k_tdft_fwd, max_smem);
+    return e == cudaSuccess ? allow_smem(k_tdft_inv, max_smem) : e;
 }

@@ -104,3 +104,32 @@ def test_mec1_matches_torch(ny, nx, q, nc, rank, kind):
         assert float(torch.linalg.norm(E[k] - e)) < 3e-6 * float(scale)
         assert float(torch.linalg.norm(X[k] - low[k] - e)) < 3e-6 * float(scale)
     s.close()
+
+
+# temporal transforms: one frame, odd, prime, even and the largest frame counts
+@pytest.mark.parametrize("ny,nx,q,nc,kind", [(32, 32, 1, 2, "lines"), (32, 64, 2, 3, "radial"), (32, 32, 13, 2, "lines"),
+                                             (64, 32, 30, 2, "lines"), (32, 32, 127, 1, "lines"), (32, 32, 128, 2, "lines")])
+def test_mec2_matches_torch(ny, nx, q, nc, kind):
+    c = Case(ny, nx, q, nc, 1, kind, ny + 3 * q)
+    s = lrccs.Solver(ny, nx, q, nc, 1)
+    s.init(*c.inp)
+    s.iterate(2)
+    E, X, it = s.mec2(3, 0.0, 0.02)
+    U, B = s.factors()
+    s.sync()
+    low = (U.to(torch.complex128) @ B.to(torch.complex128).T).T
+    s0 = torch.stack([c.adjoint(k, c.y[k]) - c.adjoint(k, c.apply(k, low[k])) for k in range(q)])
+    e = torch.zeros_like(s0)
+    for tau in range(3):
+        ne = torch.stack([c.adjoint(k, c.apply(k, e[k])) for k in range(q)])
+        m = torch.fft.fft(e + s0 - ne, dim=0, norm="ortho")
+        if tau == 0:
+            omega = 0.02 * float(m.abs().max())
+        a = m.abs()
+        e = torch.fft.ifft(torch.where(a > omega, m * (1 - omega / a.clamp_min(1e-300)), torch.zeros_like(m)), dim=0,
+                           norm="ortho")
+    assert it == 3
+    # FP32 sums of q terms, three steps, on the residual of FP32 images
+    scale = torch.linalg.norm(low) + torch.linalg.norm(e)
+    assert float(torch.linalg.norm(E - e)) < 3e-6 * float(scale)
+    s.close()
