@@ -261,6 +261,8 @@ cudaError_t launch_bstep_fused(lrccs_ctx *c);          // B + C + D in one coope
 int bstep_capacity(int nc, int nx, int q, int r, int smem_optin, int nsm);
 cudaError_t launch_iteration(lrccs_ctx *c);            // A .. H for one iteration
 cudaError_t launch_images(lrccs_ctx *c, float2 *d_X);
+cudaError_t launch_images_mec(lrccs_ctx *c, int kid, const float2 *zbar, const float2 *E, int w, float2 *Eout,
+                              float2 *X);
 cudaError_t launch_normal_op(lrccs_ctx *c);           // U+ <- A^H A U, rank 1, b_k = 1
 cudaError_t launch_fwd_only(lrccs_ctx *c);            // T <- F_y(d_j o U) on the sampled rows
 cudaError_t launch_cg_init(lrccs_ctx *c, double *cg);

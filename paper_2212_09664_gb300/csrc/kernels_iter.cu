@@ -679,22 +679,61 @@ cudaError_t launch_fwd_only(lrccs_ctx *c) {
     return cudaGetLastError();
 }
 
-__global__ void k_images(const float2 *__restrict__ Uprev, const float2 *__restrict__ B, float2 *__restrict__ X,
-                         int n, int q, int r) {
-    const size_t total = (size_t)n * q;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(e / n), i = (int)(e % n);
-        float2 acc = make_float2(0.f, 0.f);
-        for (int l = 0; l < r; ++l) cfma(acc, Uprev[(size_t)i * r + l], B[(size_t)k * r + l]);
-        X[e] = acc;
+// Caller layouts (frame k contiguous, X[k n + i]): X_k = zbar + U_{t-1} b_k + e_k
+// and, with Eout, E_k = e_k; zbar and E (chunks of w columns, kernels_mec.cu) may be
+// NULL.  Block = 256 pixels x IMG_F frames: a thread keeps its pixel's row of
+// U in registers and walks the frames (b_k broadcast from shared memory), so
+// every store is a full line.  One thread per (frame, pixel) re-read U's row
+// for each: n = 65536, q = 96, r = 14: 111 -> 25 us; n = 36864, q = 8, r = 10: 6.2 ->
+// 4.5 us.
+#define IMG_F 16
+template <int R>
+__global__ void __launch_bounds__(256) k_images(const float2 *__restrict__ Uprev, const float2 *__restrict__ B,
+                                                const float2 *__restrict__ zbar, const float2 *__restrict__ E, int w,
+                                                int n, int q, float2 *__restrict__ Eout, float2 *__restrict__ X) {
+    __shared__ float2 s_b[IMG_F * R];
+    const int i = blockIdx.x * 256 + threadIdx.x, k0 = blockIdx.y * IMG_F, kn = min(IMG_F, q - k0);
+    for (int e = threadIdx.x; e < kn * R; e += 256) s_b[e] = B[(size_t)k0 * R + e];
+    __syncthreads();
+    if (i >= n) return;
+    float2 u[R];
+    const float2 z = zbar ? zbar[i] : make_float2(0.f, 0.f);
+    if (X) {
+#pragma unroll
+        for (int a = 0; a < R; ++a) u[a] = __ldg(Uprev + (size_t)i * R + a);
+    }
+    int cc = w > 0 ? k0 / w : 0, l = w > 0 ? k0 - cc * w : 0;
+#pragma unroll 2
+    for (int f = 0; f < kn; ++f) {
+        float2 e = make_float2(0.f, 0.f);
+        const size_t o = (size_t)(k0 + f) * n + i;
+        if (E) {
+            e = __ldg(E + ((size_t)cc * n + i) * w + l);
+            if (++l == w) l = 0, ++cc;
+            if (Eout) Eout[o] = e;
+        }
+        if (X) {
+            float2 x = z;
+#pragma unroll
+            for (int a = 0; a < R; ++a) cfma(x, u[a], s_b[f * R + a]);
+            X[o] = E ? cadd(x, e) : x;
+        }
     }
 }
 
-cudaError_t launch_images(lrccs_ctx *c, float2 *d_X) {
-    prof_begin(c, KID_IMAGES);
-    k_images<<<608, 256, 0, c->stream>>>(c->d_Uprev, c->d_B, d_X, c->n, c->q, c->r);
-    prof_end(c, KID_IMAGES);
+typedef void (*images_t)(const float2 *, const float2 *, const float2 *, const float2 *, int, int, int, float2 *, float2 *);
+static const images_t kImages[RMAXC] = RANK_TABLE(k_images);
+
+cudaError_t launch_images_mec(lrccs_ctx *c, int kid, const float2 *zbar, const float2 *E, int w, float2 *Eout, float2 *X) {
+    prof_begin(c, kid);
+    kImages[c->r - 1]<<<dim3((c->n + 255) / 256, (c->q + IMG_F - 1) / IMG_F), 256, 0, c->stream>>>(
+        c->d_Uprev, c->d_B, zbar, E, w, c->n, c->q, Eout, X);
+    prof_end(c, kid);
     return cudaGetLastError();
+}
+
+cudaError_t launch_images(lrccs_ctx *c, float2 *d_X) {
+    return launch_images_mec(c, KID_IMAGES, nullptr, nullptr, 0, nullptr, d_X);
 }
 
 #define SET_SMEM(...) do { cudaError_t e_ = allow_smem(__VA_ARGS__, max_smem); if (e_ != cudaSuccess) return e_; } while (0)

@@ -200,24 +200,6 @@ __global__ void __launch_bounds__(256) k_mec_dir(const float2 *__restrict__ S, f
     }
 }
 
-// Caller layouts (frame k contiguous, X[k n + i]): E_out = e_k and
-// X_out = zbar + U_{t-1} b_k + e_k (zbar may be NULL).
-__global__ void k_mec_out(const float2 *__restrict__ E, const float2 *__restrict__ Uprev, const float2 *__restrict__ B,
-                          const float2 *__restrict__ zbar, int n, int q, int r, int w, float2 *__restrict__ Eout,
-                          float2 *__restrict__ Xout) {
-    const size_t total = (size_t)n * q;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(e / n), i = (int)(e % n);
-        const float2 ev = E[((size_t)(k / w) * n + i) * w + (k % w)];
-        if (Eout) Eout[e] = ev;
-        if (Xout) {
-            float2 x = zbar ? zbar[i] : make_float2(0.f, 0.f);
-            for (int a = 0; a < r; ++a) cfma(x, Uprev[(size_t)i * r + a], B[(size_t)k * r + a]);
-            Xout[e] = cadd(x, ev);
-        }
-    }
-}
-
 // ---------------------------------------------------------------- MEC-2: DFT along the frames
 
 // Temporal transforms: every pixel's q values times the q x q DFT matrix.  A
@@ -473,10 +455,7 @@ cudaError_t launch_mec_cg(lrccs_ctx *c, int kind, const float2 *V) {
 }
 
 cudaError_t launch_mec_out(lrccs_ctx *c, const float2 *E, const float2 *zbar, float2 *Eout, float2 *Xout) {
-    prof_begin(c, KID_MEC_ELEM);
-    k_mec_out<<<4 * 152, 256, 0, c->stream>>>(E, c->d_Uprev, c->d_B, zbar, c->n, c->q, c->r, c->mec_w, Eout, Xout);
-    prof_end(c, KID_MEC_ELEM);
-    return cudaGetLastError();
+    return launch_images_mec(c, KID_MEC_ELEM, zbar, E, c->mec_w, Eout, Xout);
 }
 
 cudaError_t launch_tdft_fwd(lrccs_ctx *c, const float2 *E, const float2 *S0, const float2 *V, const float2 *Mprev,
