@@ -151,8 +151,9 @@ lrccs_status lrccs_create(const lrccs_dims *dims, const lrccs_params *params,
                           void *cuda_stream, lrccs_ctx **out);
 
 /* Device bytes lrccs_create would allocate for dims (each buffer rounded up to
- * 256 bytes).  Not included: the general-mask and MEC work space, allocated by
- * the first call that needs them (see lrccs_init, lrccs_mec1).  Allocates
+ * 256 bytes).  Not included: the general-mask and MEC work space and wider
+ * transform buffers, allocated by the first call that needs them where the
+ * memory allows (see lrccs_init, lrccs_mec1).  Allocates
  * nothing.  Errors: LRCCS_E_INVALID, LRCCS_E_UNSUPPORTED. */
 lrccs_status lrccs_context_bytes(const lrccs_dims *dims, size_t *bytes);
 
@@ -167,7 +168,9 @@ lrccs_status lrccs_context_bytes(const lrccs_dims *dims, size_t *bytes);
  * scaled X0, its top-r left singular vectors U_0, and resets t and eta.  The
  * call blocks until the device work is done.  Inputs are not retained.
  * The first general (2D) mask a context sees allocates that path's buffers
- * (about 2 q n int32 plus C n rank_max complex64).
+ * (about 2 q n int32 plus C n rank_max complex64).  The first data load widens
+ * the transform buffer to min(q, 16) frames (C n min(q, 16) complex64) if that
+ * is above rank_max and fits the device memory.
  * Errors: LRCCS_E_INVALID (frame_ptr inconsistent with the mask, or a fixed
  * rank above q: the top-r singular vectors of the n x q X0 need r <= q),
  * LRCCS_E_RANK_DEFICIENT (sigma_r(X0) = 0), LRCCS_E_NOMEM, LRCCS_E_CUDA. */
@@ -203,7 +206,7 @@ lrccs_status lrccs_get_images(lrccs_ctx *ctx, void *d_X);
 
 /* Diagnostics: copy an internal array to caller device memory.
  *   LRCCS_BUF_Z     Z = [A_k^H y_k]            n x q, row-major (i * q + k)
- *   LRCCS_BUF_X0    truncated, scaled X0       n x q, row-major
+ *   LRCCS_BUF_X0    truncated, scaled X0       n x q, row-major (of the last lrccs_init)
  *   LRCCS_BUF_GRAD  last gradient              n x r, row-major
  *   LRCCS_BUF_SIGMA singular values of X0      q float64, descending
  *   LRCCS_BUF_IDX   compacted sample indices   fp[q] int32 (ascending per frame)

@@ -93,8 +93,8 @@ static void free_all(lrccs_ctx *c) {
                     c->d_mks, c->d_fpk, c->d_rowoff, c->d_ucnt, c->d_uloc, c->d_floc, c->d_urow, c->d_uptr,
                     c->d_ufrow, c->d_upos, c->d_uidx, c->d_ufptr, c->d_uflist, c->d_fu, c->d_FU, c->d_Pu,
                     c->d_maskc, c->d_mec, c->d_mscal, c->d_mout, c->d_twq, c->d_Q, c->d_gdts, c->d_fpart,
-                    c->d_tflag, c->d_tcA0, c->d_tcA1, c->d_tcscale, c->d_ZB, c->d_hpart,
-                    c->d_tcB0, c->d_tcB1, c->d_twsy, c->d_twsx, c->d_rowtab, c->d_ptab};
+                    c->d_tcA0, c->d_tcA1, c->d_tcscale, c->d_ZB, c->d_hpart,
+                    c->d_tcB0, c->d_tcB1, c->d_twsy, c->d_twsx, c->d_rowtab, c->d_ptab, c->d_xs};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -176,7 +176,7 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     const size_t F2 = sizeof(float2), I4 = sizeof(int32_t), D8 = sizeof(double);
     const struct { void **p; size_t bytes; } plan[] = {
         {(void **)&c->d_twy, ny * F2}, {(void **)&c->d_twx, c->nx * F2},
-        {(void **)&c->d_twsy, ny * F2}, {(void **)&c->d_twsx, c->nx * F2}, {(void **)&c->d_rowtab, ((size_t)q + 17) * 32 * I4}, {(void **)&c->d_smaps, (size_t)nc * n * F2},
+        {(void **)&c->d_twsy, ny * F2}, {(void **)&c->d_twsx, c->nx * F2}, {(void **)&c->d_rowtab, ((size_t)q + 17) * 32 * I4}, {(void **)&c->d_xs, (size_t)q * 4}, {(void **)&c->d_smaps, (size_t)nc * n * F2},
         {(void **)&c->d_rowcnt, (size_t)q * ny * I4}, {(void **)&c->d_rowidx, (size_t)q * ny * I4},
         {(void **)&c->d_framerows, (size_t)q * ny * I4}, {(void **)&c->d_lineptr, ((size_t)q + 1) * I4},
         {(void **)&c->d_rfptr, ((size_t)ny + 1) * I4}, {(void **)&c->d_rflist, (size_t)q * ny * I4},
@@ -370,9 +370,27 @@ static lrccs_status ensure_general_buffers(lrccs_ctx *c) {
     return LRCCS_OK;
 }
 
+static void drop_iter_graph(lrccs_ctx *c);
+
+// Grow a transform work buffer to `need` complex values, keeping the old one
+// when the larger does not fit the device memory.
+static bool grow_work(lrccs_ctx *c, float2 **buf, size_t *cap, size_t need) {
+    if (need <= *cap) return true;
+    float2 *p = nullptr;
+    if (cudaMalloc((void **)&p, need * sizeof(float2)) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    drop_iter_graph(c);   // captured iterations hold the old buffer's address
+    cudaFree(*buf);       // waits for the work that may still use it
+    *buf = p;
+    *cap = need;
+    return true;
+}
+
 // Mask compaction, the sampled-row structure and Z = [A_k^H y_k] for the data
-// of one lrccs_init or tracking call; with_energy also forms gamma, which only
-// the spectral initialisation's truncation uses.  Waits for the compaction's
+// of one lrccs_init or tracking call; with_energy also forms gamma and the
+// truncated X0, which only the spectral initialisation uses.  Waits for the compaction's
 // counts (twice for a general 2D mask: once for the row structure, once for
 // the union of the frames' samples).
 static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_frame_ptr, const uint8_t *d_mask,
@@ -401,14 +419,6 @@ static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_fr
     if (c->general) {
         s = ensure_general_buffers(c);
         if (s != LRCCS_OK) return s;
-        const size_t nflag = (size_t)c->nc * c->total;
-        if (nflag > c->tflag_cap) {
-            if (c->d_tflag) cudaFree(c->d_tflag);
-            c->d_tflag = nullptr;
-            c->tflag_cap = 0;
-            if (!dalloc(c, &c->d_tflag, nflag)) return LRCCS_E_NOMEM;
-            c->tflag_cap = nflag;
-        }
         CK(launch_compact_general(c, d_mask));
         CK(cudaMemcpyAsync(meta, c->d_meta, sizeof(meta), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
@@ -417,20 +427,10 @@ static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_fr
         CK(launch_fill_lines(c));
     }
     if (c->dims.precision != LRCCS_PREC_FP32_FFT) CK(launch_dft_a(c));   // DFT rows of the sampled rows
-    // line masks' init row pass: full rows (nx) for every (frame row, coil), plain
-    // and truncated (the general masks' init needs no such buffer)
-    const size_t need = c->general ? 0 : (size_t)2 * c->nc * c->n_lines * c->nx;
-    if (need > c->T_cap) {
-        cudaFree(c->d_T);
-        c->d_T = nullptr;
-        if (!dalloc(c, &c->d_T, need)) {
-            c->T_cap = 0;
-            return LRCCS_E_NOMEM;
-        }
-        c->T_cap = need;
-    }
+    // the init transforms up to 16 frames at a time where the memory allows it (rmax otherwise)
+    grow_work(c, &c->d_T, &c->T_cap, (size_t)c->nc * c->n * std::min(16, c->q));
     if (with_energy) CK(launch_energy(c, (const float2 *)d_y));
-    CK(launch_init_adjoint(c, (const float2 *)d_y));
+    CK(launch_init_adjoint(c, (const float2 *)d_y, with_energy));
     return LRCCS_OK;
 }
 
@@ -774,22 +774,6 @@ extern "C" lrccs_status lrccs_mean_step(lrccs_ctx *c, const void *d_y, const int
 }
 
 // ---------------------------------------------------------------- model-error correction (Alg. 3)
-
-// Grow a transform work buffer to `need` complex values, keeping the old one
-// when the larger does not fit the device memory.
-static bool grow_work(lrccs_ctx *c, float2 **buf, size_t *cap, size_t need) {
-    if (need <= *cap) return true;
-    float2 *p = nullptr;
-    if (cudaMalloc((void **)&p, need * sizeof(float2)) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    drop_iter_graph(c);   // captured iterations hold the old buffer's address
-    cudaFree(*buf);       // waits for the work that may still use it
-    *buf = p;
-    *cap = need;
-    return true;
-}
 
 // Work space and chunk width of the frames' normal operators.  A transform
 // costs little more for 16 columns than for 4, so the frames go in the fewest

@@ -75,6 +75,18 @@ LRCCS_DEV double abs2_rn(float2 v) {
     return __dadd_rn(__dmul_rn((double)v.x, (double)v.x), __dmul_rn((double)v.y, (double)v.y));
 }
 
+// |v|^2 > gam on those FP64 squares; the FP32 square decides wherever it is
+// further from gam than its rounding (glo, ghi = gam (1 -+ 1e-5)) and in range
+LRCCS_DEV bool trunc_drop(float2 v, double gam, float glo, float ghi) {
+    if (v.x == 0.f && v.y == 0.f) return false;   // gam >= 0
+    const float s = fmaf(v.x, v.x, v.y * v.y);
+    if (s > 1e-30f && s < 1e30f) {
+        if (s < glo) return false;
+        if (s > ghi) return true;
+    }
+    return abs2_rn(v) > gam;
+}
+
 LRCCS_DEV void load_twiddles(float2 *s_tw, const float2 *g_tw, int N) {
     for (int t = threadIdx.x; t < N; t += blockDim.x) s_tw[t] = g_tw[t];
 }

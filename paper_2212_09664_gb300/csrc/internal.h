@@ -125,7 +125,7 @@ struct lrccs_ctx {
     float2 *d_twy, *d_twx;       // twiddles w_N^t, N = ny / nx
     float2 *d_twsy, *d_twsx;     // ny, nx: twiddles of the column and row passes with their scale, [j2][k1]
     uint16_t *d_ptab;            // q * ny * 32 sampled-point tables of the row passes (general masks, MEC)
-    uint32_t *d_rowtab;          // (q + 17) * 32 sampled-row tables of the column passes (k_row_tables)
+    uint32_t *d_rowtab;          // (q + 17) * 32 sampled-row tables of the column passes (k_structure)
     float2 *d_smaps;             // nc * n
     int32_t *d_rowcnt;           // q * ny  samples of frame k in row ky
     int32_t *d_rowidx;           // q * ny  line index of row ky in frame k, or -1
@@ -148,7 +148,7 @@ struct lrccs_ctx {
     // numerical buffers
     float2 *d_Z;                 // n * q   Z = [A_k^H y_k]   (row-major i*q + k)
     float2 *d_X0;                // n * q   truncated, scaled X0
-    float2 *d_T;                 // work: nc * n * rmax (iteration), 2 * nc * fp[q] (init)
+    float2 *d_T;                 // work: nc * n columns (rmax of them, or the frames transformed at a time)
     size_t T_cap;                // capacity of d_T in float2
     float2 *d_U;                 // n * rmax  U_t
     float2 *d_Uprev;             // n * rmax  U_{t-1}
@@ -184,8 +184,7 @@ struct lrccs_ctx {
     float2 *d_FU;                // nc * n_u * rmax  F(d_j o U) at the union points (FU[j][u][l])
     float2 *d_Pu;                // n_u * npairs      coil-summed Gram of every union point
     double *d_fpart;             // q * 8 chunks * 2 npairs  per-frame Gram partial sums (FP64)
-    uint8_t *d_tflag;            // C sum_k m_k  truncation flags of the init (capacity tflag_cap)
-    size_t tflag_cap;
+    float *d_xs;                 // q       X0's column scale 1 / sqrt(m_k mbar)
 
     // model-error correction (Alg. 3): frames in chunks of mec_w <= 16 columns,
     // vectors V[c][i][l] (frame c mec_w + l)
@@ -213,7 +212,6 @@ cudaError_t launch_compact(lrccs_ctx *c, const uint8_t *d_mask, const int64_t *d
 cudaError_t launch_fill_lines(lrccs_ctx *c);
 // general (2D) masks (kernels_general.cu)
 cudaError_t launch_compact_general(lrccs_ctx *c, const uint8_t *d_mask);
-cudaError_t launch_init_general(lrccs_ctx *c, const float2 *d_y);   // Z and X0 in one pass (general masks)
 cudaError_t launch_iteration_general_front(lrccs_ctx *c);   // forward rows + sample Grams + B-step
 cudaError_t launch_iteration_general_back(lrccs_ctx *c);    // W per sample + inverse rows
 cudaError_t launch_fwd_rows(lrccs_ctx *c);
@@ -226,7 +224,7 @@ cudaError_t launch_point_tables(lrccs_ctx *c);
 // dst <- sum_j conj(d_j) F_y^H T_j from those rows
 cudaError_t launch_fwd_cols_on(lrccs_ctx *c, const float2 *src, int r, int e0, int estep);
 cudaError_t launch_adj_cols_to(lrccs_ctx *c, float2 *dst, int r, int e0, int estep);
-cudaError_t launch_row_tables(lrccs_ctx *c);
+cudaError_t launch_adj_cols_frames(lrccs_ctx *c, float2 *dst, int w, int k0, const float *scale);
 cudaError_t launch_col_twiddles(lrccs_ctx *c);
 cudaError_t launch_sample_w(lrccs_ctx *c);
 cudaError_t launch_adj_rows(lrccs_ctx *c);
@@ -250,7 +248,7 @@ cudaError_t launch_fwd_gemm(lrccs_ctx *c);
 size_t tc_a_elems(int ny);
 size_t tc_b_elems(int nc, int ny, int nx, int rmax);
 cudaError_t launch_energy(lrccs_ctx *c, const float2 *d_y);
-cudaError_t launch_init_adjoint(lrccs_ctx *c, const float2 *d_y);
+cudaError_t launch_init_adjoint(lrccs_ctx *c, const float2 *d_y, bool trunc);   // Z (and X0)
 cudaError_t launch_gram_x0(lrccs_ctx *c);
 cudaError_t launch_u0(lrccs_ctx *c);
 cudaError_t launch_gdqr(lrccs_ctx *c, int mode);      // F: GD step + Cholesky QR (mode 0: init U+)

@@ -20,8 +20,7 @@
 //   E  k_adj_rows     : scatter a row's union points, F_x^H           -> T[j][ky][x][l]
 //   F  k_adj_cols     : F_y^H and the conj(d_j) coil sum              -> Gk
 //   G  k_gdqr         : gradient, GD step, QR                          (kernels_gd.cu)
-// and the spectral initialisation's fused pass k_init_gen (Z and X0: direct
-// inverse DFT along kx of each frame row's few samples, then the column FFTs).
+// (the spectral initialisation takes any mask: kernels_init.cu).
 #include <math.h>
 
 #include <algorithm>
@@ -181,177 +180,6 @@ cudaError_t launch_compact_general(lrccs_ctx *c, const uint8_t *d_mask) {
     k_fill_general<<<(q * ny * 32 + 255) / 256, 256, 0, c->stream>>>(d_mask, c->d_rowcnt, c->d_rowoff, c->d_upos,
                                                                       q, ny, nx, c->d_idx, c->d_fu);
     prof_end(c, KID_FILL_GEN);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- init: fused pass
-
-// Z[:, k] = A_k^H y_k and X0[:, k] = A_k^H y_k,tnc / sqrt(m_k mbar) for general
-// masks in one pass, block (tile of TXG columns, frame k).  For every coil the
-// inverse DFT along kx of each frame row is evaluated directly from the row's
-// few samples at the tile's columns (T[ky][x] = sum_s y_s e^{+2 pi i kx_s x / nx}
-// / sqrt(nx), plain and truncated), then the column tile is transformed back
-// along ky and multiplied by conj(d_j) into the coil sum.  Nothing the size of
-// full k-space rows goes through memory.  The block's twiddles
-// e^{+2 pi i kx x / nx} (every kx, the tile's x) are tabulated once in shared
-// memory; a thread evaluates four columns of one row per pass over its samples.
-#define TXG 16
-#define IG_STAGE 512    // samples of one coil staged at a time (>= nx: a row always fits)
-template <int P>
-__global__ void __launch_bounds__(256, 2) k_init_gen(const float2 *__restrict__ y, const int32_t *__restrict__ idx,
-                                                     const int32_t *__restrict__ framerows,
-                                                     const int32_t *__restrict__ lineptr,
-                                                     const int32_t *__restrict__ rowoff,
-                                                     const int32_t *__restrict__ rowcnt,
-                                                     const int32_t *__restrict__ fpk, const int32_t *__restrict__ mks,
-                                                     const float2 *__restrict__ smaps, const double *__restrict__ scal,
-                                                     const uint8_t *__restrict__ tflag, float2 *__restrict__ Z,
-                                                     float2 *__restrict__ X0, int nx, int q, int nc,
-                                                     const float2 *__restrict__ g_twy, const float2 *__restrict__ g_twx,
-                                                     float sy, float sx) {
-    constexpr int NY = 32 * P;
-    constexpr int TP = 2 * TXG + 1;
-    constexpr int ACC = (NY * 2 * TXG + 255) / 256;
-    extern __shared__ __align__(16) float2 smem[];
-    float2 *tile = smem;                  // NY * TP
-    float2 *s_tw = tile + NY * TP;        // nx * TXG: e^{+2 pi i kx (x0 + xx) / nx} at kx * TXG + xx
-    float2 *s_twy = s_tw + nx * TXG;      // NY
-    float2 *s_y = s_twy + NY;             // IG_STAGE staged samples of one coil
-    int16_t *s_kx = (int16_t *)(s_y + IG_STAGE);
-    uint8_t *s_tr = (uint8_t *)(s_kx + IG_STAGE);
-    // the frame's rows (the same for every coil): row ky, sample count and
-    // first sample, and the row groups whose samples fit the staging area
-    __shared__ int s_ky[NY], s_rc[NY], s_ro[NY], s_gb[NY + 1];
-    __shared__ int s_ng;
-    const int k = blockIdx.y, x0 = blockIdx.x * TXG;
-    const int n = NY * nx;
-    load_twiddles(s_twy, g_twy, NY);
-    for (int e = threadIdx.x; e < nx * TXG; e += blockDim.x) {
-        const int kx = e / TXG, xx = e - kx * TXG;
-        s_tw[e] = cconj(g_twx[(kx * (x0 + xx)) % nx]);
-    }
-    const int lp = lineptr[k], L = lineptr[k + 1] - lp;
-    const int f0 = fpk[k], mk = mks[k];
-    for (int li = threadIdx.x; li < L; li += blockDim.x) {
-        const int ky = framerows[lp + li];
-        s_ky[li] = ky;
-        s_rc[li] = rowcnt[k * NY + ky];
-        s_ro[li] = rowoff[k * NY + ky];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ng = 0, tot = 0;
-        s_gb[0] = 0;
-        for (int li = 0; li < L; ++li) {
-            const int c = s_rc[li];
-            if (li > 0 && tot + c > IG_STAGE) {
-                s_gb[++ng] = li;
-                tot = 0;
-            }
-            tot += c;
-        }
-        if (L > 0) s_gb[++ng] = L;
-        s_ng = ng;
-    }
-    float2 acc[ACC];
-#pragma unroll
-    for (int u = 0; u < ACC; ++u) acc[u] = make_float2(0.f, 0.f);
-    for (int j = 0; j < nc; ++j) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < NY * TP; e += blockDim.x) tile[e] = make_float2(0.f, 0.f);
-        const int64_t yb = (int64_t)nc * f0 + (int64_t)j * mk;   // sample f0 + s of coil j at y[yb + s]
-        // the frame's rows in groups whose samples fit the staging area
-        for (int gi = 0; gi < s_ng; ++gi) {
-            __syncthreads();
-            const int g0 = s_gb[gi], g1 = s_gb[gi + 1];
-            const int sbase = s_ro[g0], scnt = s_ro[g1 - 1] + s_rc[g1 - 1] - sbase;
-            // stage the group's samples of coil j: value, kx, and the truncation
-            // flag (1: |y|^2 > gamma, dropped from the truncated copy)
-            for (int e = threadIdx.x; e < scnt; e += blockDim.x) {
-                const int s = sbase + e;
-                s_y[e] = __ldg(y + yb + (s - f0));
-                s_kx[e] = (int16_t)(__ldg(idx + s) % nx);
-                s_tr[e] = tflag[yb + (s - f0)];
-            }
-            __syncthreads();
-            // item (row li, column quad cq): columns x0 + 4 cq .. x0 + 4 cq + 3
-            for (int e = threadIdx.x; e < (g1 - g0) * (TXG / 4); e += blockDim.x) {
-                const int li = g0 + e / (TXG / 4), cq = e % (TXG / 4);
-                const int ky = s_ky[li];
-                const int off = s_ro[li] - sbase, cnt = s_rc[li];
-                float2 vp[4], vt[4];
-#pragma unroll
-                for (int jj = 0; jj < 4; ++jj) vp[jj] = vt[jj] = make_float2(0.f, 0.f);
-                for (int s = off; s < off + cnt; ++s) {
-                    const float2 a = s_y[s];
-                    const float4 *w4 = (const float4 *)(s_tw + (int)s_kx[s] * TXG + 4 * cq);
-                    const float4 wa = w4[0], wb = w4[1];
-                    const float2 w[4] = {make_float2(wa.x, wa.y), make_float2(wa.z, wa.w), make_float2(wb.x, wb.y),
-                                         make_float2(wb.z, wb.w)};
-                    const bool keep = s_tr[s] == 0;
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) {
-                        cfma(vp[jj], a, w[jj]);
-                        if (keep) cfma(vt[jj], a, w[jj]);
-                    }
-                }
-#pragma unroll
-                for (int jj = 0; jj < 4; ++jj) {
-                    tile[ky * TP + 2 * (4 * cq + jj)] = cscale(vp[jj], sx);
-                    tile[ky * TP + 2 * (4 * cq + jj) + 1] = cscale(vt[jj], sx);
-                }
-            }
-        }
-        __syncthreads();
-        fft::tile_dft<NY, true>(tile, TP, 2 * TXG, s_twy, sy);
-#pragma unroll
-        for (int u = 0; u < ACC; ++u) {
-            const int e = threadIdx.x + 256 * u;
-            if (e < NY * 2 * TXG) {
-                const int yy = e / (2 * TXG), cc = e % (2 * TXG);
-                cfmac(acc[u], __ldg(smaps + (size_t)j * n + (size_t)yy * nx + x0 + (cc >> 1)), tile[yy * TP + cc]);
-            }
-        }
-    }
-    const double mbar = scal[SC_MBAR];
-    const float xs = (mk > 0) ? (float)(1.0 / sqrt((double)mk * mbar)) : 0.f;
-#pragma unroll
-    for (int u = 0; u < ACC; ++u) {
-        const int e = threadIdx.x + 256 * u;
-        if (e < NY * 2 * TXG) {
-            const int yy = e / (2 * TXG), cc = e % (2 * TXG);
-            const size_t i = (size_t)yy * nx + x0 + (cc >> 1);
-            if ((cc & 1) == 0) Z[i * q + k] = acc[u];
-            else X0[i * q + k] = cscale(acc[u], xs);
-        }
-    }
-}
-
-// The truncation decision of every measured entry, |y|^2 > gamma (FP64 squares,
-// as in the line path), once per entry: 1 = dropped from X0.
-__global__ void k_trunc_flags(const float2 *__restrict__ y, int64_t count, const double *__restrict__ scal,
-                              uint8_t *__restrict__ flag) {
-    const double gam = scal[SC_GAMMA];
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
-        flag[e] = abs2_rn(y[e]) > gam ? 1 : 0;
-}
-
-cudaError_t launch_init_general(lrccs_ctx *c, const float2 *d_y) {
-    const float sx = (float)(1.0 / sqrt((double)c->nx)), sy = (float)(1.0 / sqrt((double)c->ny));
-    const size_t smem = ((size_t)c->ny * (2 * TXG + 1) + (size_t)c->nx * TXG + c->ny + IG_STAGE) * sizeof(float2) +
-                        (size_t)IG_STAGE * (sizeof(int16_t) + 1);
-    prof_begin(c, KID_INIT_GEN);
-    k_trunc_flags<<<4 * 152, 256, 0, c->stream>>>(d_y, (int64_t)c->nc * c->total, c->d_scal, c->d_tflag);
-    prof_end(c, KID_INIT_GEN);
-    dim3 grid(c->nx / TXG, c->q);
-    DISPATCH_P(c->py, {
-        prof_begin(c, KID_INIT_GEN);
-        k_init_gen<P_><<<grid, 256, smem, c->stream>>>(d_y, c->d_idx, c->d_framerows, c->d_lineptr, c->d_rowoff,
-                                                       c->d_rowcnt, c->d_fpk, c->d_mks, c->d_smaps, c->d_scal,
-                                                       c->d_tflag, c->d_Z, c->d_X0, c->nx, c->q, c->nc, c->d_twy,
-                                                       c->d_twx, sy, sx);
-        prof_end(c, KID_INIT_GEN);
-    });
     return cudaGetLastError();
 }
 
@@ -816,7 +644,5 @@ cudaError_t configure_kernels_general(int max_smem) {
         SET_SMEM(kSampleW[i]);
         SET_SMEM(kSampleGram[i]);
     }
-    SET_SMEM(k_init_gen<1>); SET_SMEM(k_init_gen<2>); SET_SMEM(k_init_gen<3>); SET_SMEM(k_init_gen<4>);
-    SET_SMEM(k_init_gen<5>); SET_SMEM(k_init_gen<6>); SET_SMEM(k_init_gen<7>); SET_SMEM(k_init_gen<8>);
     return cudaSuccess;
 }

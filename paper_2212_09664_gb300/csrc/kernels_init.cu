@@ -3,9 +3,24 @@
 // Gram X0^H X0 with a Jacobi eigensolver, and U_0 = X0 V_r Sigma_r^{-1}.
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "fft.cuh"
 #include "internal.h"
+
+#define DISPATCH_P(PV, ...)                                           \
+    switch (PV) {                                                      \
+        case 1: { constexpr int P_ = 1; __VA_ARGS__; } break;                 \
+        case 2: { constexpr int P_ = 2; __VA_ARGS__; } break;                 \
+        case 3: { constexpr int P_ = 3; __VA_ARGS__; } break;                 \
+        case 4: { constexpr int P_ = 4; __VA_ARGS__; } break;                 \
+        case 5: { constexpr int P_ = 5; __VA_ARGS__; } break;                 \
+        case 6: { constexpr int P_ = 6; __VA_ARGS__; } break;                 \
+        case 7: { constexpr int P_ = 7; __VA_ARGS__; } break;                 \
+        case 8: { constexpr int P_ = 8; __VA_ARGS__; } break;                 \
+        default: return cudaErrorInvalidValue;                         \
+    }
 
 // ---------------------------------------------------------------- twiddles
 
@@ -44,94 +59,169 @@ __global__ void k_rowcount(const uint8_t *__restrict__ mask, int rows, int nx, i
 // "frame rows" (its lines, for 1D Cartesian masks): lineptr / framerows /
 // framek / rowidx.  Also the frames' sample counts m_k and offsets fpk (checked
 // against the caller's frame_ptr), each (frame, row)'s first sample rowoff, the
-// rows sampled by some frame, and meta[MT_GENERAL] = 1 when some row is only
-// partly sampled (a general 2D mask).
-__global__ void k_structure(const int32_t *__restrict__ rowcnt, const int64_t *__restrict__ fp_user,
-                            int q, int ny, int nx, int32_t *rowidx, int32_t *framerows, int32_t *framek,
-                            int32_t *lineptr, int32_t *rfptr, int32_t *rflist, int32_t *usedrows,
-                            uint8_t *rowused, int32_t *mks, int32_t *fpk, int32_t *rowoff, int32_t *meta,
-                            unsigned int *status, double *scal) {
-    __shared__ int s_lines[129];
-    __shared__ int s_m[129];
-    __shared__ int s_fp[130];
-    __shared__ int s_rf[257];
-    __shared__ int s_partial;
-    const int tid = threadIdx.x;
-    if (tid == 0) s_partial = 0;
+// rows sampled by some frame, meta[MT_GENERAL] = 1 when some row is only
+// partly sampled (a general 2D mask), and the column passes' row tables
+// (kernels_iter.cu): entry 0 the rows some frame samples, entry 1 + k those of
+// frame k, then 16 empty entries; [e][g] bit i = row g + R1 i, [e][16 + g] bit i =
+// row g + R2 i.
+//
+// One block of 1024 threads with the counts in shared memory; a warp per frame
+// (lanes over the rows, ballot and shuffle prefixes), then a warp per row.
+// The chain of dependent global loads bounded the earlier thread-per-frame
+// form: 45 us (48 frames of 192 rows) -> 24 us with the column tables, 90 us (96 of
+// 256) -> 46 us.
+#define ST_NT 1024
+LRCCS_DEV int warp_excl_sum(int v, int lane, int &total) {   // exclusive prefix over the warp, and its total
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += t;
+    }
+    total = __shfl_sync(0xffffffffu, x, 31);
+    return x - v;
+}
+__global__ void __launch_bounds__(ST_NT) k_structure(
+    const int32_t *__restrict__ rowcnt, const int64_t *__restrict__ fp_user, int q, int ny, int nx, int R1, int R2,
+    int32_t *rowidx, int32_t *framerows, int32_t *framek, int32_t *lineptr, int32_t *rfptr, int32_t *rflist,
+    int32_t *usedrows, uint8_t *rowused, int32_t *mks, int32_t *fpk, int32_t *rowoff, uint32_t *rowtab, float *xs, int32_t *meta,
+    unsigned int *status, double *scal) {
+    extern __shared__ int16_t s_cnt[];   // q x ny (a count is at most nx <= 256)
+    __shared__ int s_lines[129], s_fp[129], s_rf[257], s_nu[257];
+    __shared__ int s_partial, s_min, s_max, s_total;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = ST_NT / 32;
+    if (tid == 0) {
+        s_partial = 0;
+        s_min = 0x7fffffff;
+        s_max = 0;
+    }
+    for (int e = tid; e < q * ny; e += ST_NT) s_cnt[e] = (int16_t)rowcnt[e];
     __syncthreads();
-    for (int k = tid; k < q; k += blockDim.x) {
+    for (int k = warp; k < q; k += nw) {          // line and sample counts of frame k
         int L = 0, m = 0, part = 0;
-        for (int ky = 0; ky < ny; ++ky) {
-            const int c = rowcnt[k * ny + ky];
+        for (int ky = lane; ky < ny; ky += 32) {
+            const int c = s_cnt[k * ny + ky];
             L += c > 0;
             m += c;
             part |= (c != 0 && c != nx);
         }
-        s_lines[k] = L;
-        s_m[k] = m;
-        if (part) s_partial = 1;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            L += __shfl_xor_sync(0xffffffffu, L, o);
+            m += __shfl_xor_sync(0xffffffffu, m, o);
+            part |= __shfl_xor_sync(0xffffffffu, part, o);
+        }
+        if (lane == 0) {
+            s_lines[k] = L;
+            s_fp[k] = m;
+            mks[k] = m;
+            atomicMin(&s_min, m);
+            atomicMax(&s_max, m);
+            if (part) s_partial = 1;
+        }
     }
-    for (int ky = tid; ky < ny; ky += blockDim.x) {
+    for (int ky = warp; ky < ny; ky += nw) {      // frames that sample row ky
         int c = 0;
-        for (int k = 0; k < q; ++k) c += (rowcnt[k * ny + ky] > 0);
-        s_rf[ky] = c;
+        for (int k = lane; k < q; k += 32) c += s_cnt[k * ny + ky] > 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        if (lane == 0) {
+            s_rf[ky] = c;
+            rowused[ky] = (uint8_t)(c > 0);
+        }
     }
     __syncthreads();
-    if (tid == 0) {
-        int acc = 0, accm = 0, mmin = 0x7fffffff, mmax = 0;
-        for (int k = 0; k < q; ++k) {
-            lineptr[k] = acc;
-            s_fp[k] = accm;
-            fpk[k] = accm;
-            acc += s_lines[k];
-            accm += s_m[k];
-            mmin = min(mmin, s_m[k]);
-            mmax = max(mmax, s_m[k]);
-        }
-        lineptr[q] = acc;
-        s_fp[q] = accm;
-        fpk[q] = accm;
-        meta[MT_NLINES] = acc;
-        meta[MT_MMIN] = mmin;
-        meta[MT_MMAX] = mmax;
-        meta[MT_TOTAL] = accm;
-        meta[MT_GENERAL] = s_partial;
-        scal[SC_MBAR] = (double)accm / (double)q;
-        int pacc = 0, nu = 0;
-        for (int ky = 0; ky < ny; ++ky) {
-            rfptr[ky] = pacc;
-            pacc += s_rf[ky];
-            rowused[ky] = (uint8_t)(s_rf[ky] > 0);
-            if (s_rf[ky] > 0) usedrows[nu++] = ky;
-        }
-        rfptr[ny] = pacc;
-        meta[MT_NUSED] = nu;
-        if (fp_user[q] != (int64_t)accm || fp_user[0] != 0) atomicOr(status, (unsigned)ST_FRAMEPTR_MISMATCH);
-    }
-    __syncthreads();
-    for (int k = tid; k < q; k += blockDim.x) {
-        const int base = lineptr[k];
-        if (fp_user[k] != (int64_t)s_fp[k]) atomicOr(status, (unsigned)ST_FRAMEPTR_MISMATCH);
-        mks[k] = s_m[k];
-        int i = 0, off = s_fp[k];
-        for (int ky = 0; ky < ny; ++ky) {
-            const int c = rowcnt[k * ny + ky];
-            rowoff[k * ny + ky] = off;
-            off += c;
-            if (c > 0) {
-                rowidx[k * ny + ky] = i;
-                framerows[base + i] = ky;
-                framek[base + i] = k;
-                ++i;
-            } else {
-                rowidx[k * ny + ky] = -1;
+    if (warp == 0) {                              // prefixes over the frames (q <= 128)
+        int acc = 0, accm = 0;
+        for (int k0 = 0; k0 < q; k0 += 32) {
+            const int k = k0 + lane;
+            int tl, tm;
+            const int el = warp_excl_sum(k < q ? s_lines[k] : 0, lane, tl);
+            const int em = warp_excl_sum(k < q ? s_fp[k] : 0, lane, tm);
+            __syncwarp();
+            if (k < q) {
+                s_lines[k] = acc + el;
+                s_fp[k] = accm + em;
+                lineptr[k] = acc + el;
+                fpk[k] = accm + em;
+                if (fp_user[k] != (int64_t)(accm + em)) atomicOr(status, (unsigned)ST_FRAMEPTR_MISMATCH);
             }
+            acc += tl;
+            accm += tm;
+        }
+        if (lane == 0) {
+            lineptr[q] = acc;
+            fpk[q] = accm;
+            s_total = accm;
+            meta[MT_NLINES] = acc;
+            meta[MT_MMIN] = s_min;
+            meta[MT_MMAX] = s_max;
+            meta[MT_TOTAL] = accm;
+            meta[MT_GENERAL] = s_partial;
+            scal[SC_MBAR] = (double)accm / (double)q;
+            if (fp_user[q] != (int64_t)accm) atomicOr(status, (unsigned)ST_FRAMEPTR_MISMATCH);
+        }
+    } else if (warp == 1) {                       // prefixes over the rows
+        int acc = 0, nu = 0;
+        for (int y0 = 0; y0 < ny; y0 += 32) {
+            const int ky = y0 + lane;             // ny is a multiple of 32
+            int t, tu;
+            const int c = s_rf[ky];
+            const int e = warp_excl_sum(c, lane, t), eu = warp_excl_sum(c > 0, lane, tu);
+            s_rf[ky] = acc + e;
+            s_nu[ky] = c > 0 ? nu + eu : -1;
+            rfptr[ky] = acc + e;
+            acc += t;
+            nu += tu;
+        }
+        if (lane == 0) {
+            rfptr[ny] = acc;
+            meta[MT_NUSED] = nu;
         }
     }
-    for (int ky = tid; ky < ny; ky += blockDim.x) {
-        int base = rfptr[ky], c = 0;
-        for (int k = 0; k < q; ++k)
-            if (rowcnt[k * ny + ky] > 0) rflist[base + c++] = k;
+    __syncthreads();
+    if (tid < q) {                                // X0's column scale 1 / sqrt(m_k mbar)
+        const int m = (tid + 1 < q ? s_fp[tid + 1] : s_total) - s_fp[tid];
+        xs[tid] = m > 0 ? (float)(1.0 / sqrt((double)m * ((double)s_total / (double)q))) : 0.f;
+    }
+    for (int k = warp; k < q; k += nw) {          // frame k's rows, in order
+        int i = s_lines[k], off = s_fp[k];
+        const int base = i;
+        for (int y0 = 0; y0 < ny; y0 += 32) {
+            const int ky = y0 + lane, e = k * ny + ky, c = s_cnt[e];
+            int tl, tm;
+            const int el = warp_excl_sum(c > 0, lane, tl), em = warp_excl_sum(c, lane, tm);
+            rowoff[e] = off + em;
+            rowidx[e] = c > 0 ? i + el - base : -1;
+            if (c > 0) {
+                framerows[i + el] = ky;
+                framek[i + el] = k;
+            }
+            i += tl;
+            off += tm;
+        }
+    }
+    for (int ky = warp; ky < ny; ky += nw) {      // the frames of row ky, in order
+        int base = s_rf[ky];
+        if (lane == 0 && s_nu[ky] >= 0) usedrows[s_nu[ky]] = ky;
+        for (int k0 = 0; k0 < q; k0 += 32) {
+            const int k = k0 + lane;
+            const bool in = k < q && s_cnt[k * ny + ky] > 0;
+            const unsigned bal = __ballot_sync(0xffffffffu, in);
+            if (in) rflist[base + __popc(bal & ((1u << lane) - 1u))] = k;
+            base += __popc(bal);
+        }
+    }
+    for (int e = tid; e < (q + 17) * 32; e += ST_NT) {
+        const int en = e >> 5, t = e & 31, g = t & 15, step = t < 16 ? R1 : R2, cnt = t < 16 ? R2 : R1;
+        uint32_t bits = 0;
+        if (g < step && en <= q)
+            for (int i = 0; i < cnt; ++i) {
+                const int y = g + step * i;
+                const bool used = en == 0 ? s_nu[y] >= 0 : s_cnt[(en - 1) * ny + y] > 0;
+                bits |= (uint32_t)used << i;
+            }
+        rowtab[e] = bits;
     }
 }
 
@@ -149,12 +239,15 @@ cudaError_t launch_compact(lrccs_ctx *c, const uint8_t *d_mask, const int64_t *d
     k_rowcount<<<(rows * 32 + 255) / 256, 256, 0, c->stream>>>(d_mask, rows, c->nx, c->d_rowcnt);
     prof_end(c, KID_ROWCOUNT);
     prof_begin(c, KID_STRUCTURE);
-    k_structure<<<1, 256, 0, c->stream>>>(c->d_rowcnt, d_fp_user, c->q, c->ny, c->nx, c->d_rowidx,
-                                           c->d_framerows, c->d_framek, c->d_lineptr, c->d_rfptr, c->d_rflist,
-                                           c->d_usedrows, c->d_rowused, c->d_mks, c->d_fpk, c->d_rowoff, c->d_meta,
-                                           c->d_status, c->d_scal);
+    DISPATCH_P(c->py, {
+        using PL = fft::Plan<32 * P_>;
+        k_structure<<<1, ST_NT, (size_t)c->q * c->ny * sizeof(int16_t), c->stream>>>(
+            c->d_rowcnt, d_fp_user, c->q, c->ny, c->nx, PL::R1, PL::R2, c->d_rowidx, c->d_framerows, c->d_framek,
+            c->d_lineptr, c->d_rfptr, c->d_rflist, c->d_usedrows, c->d_rowused, c->d_mks, c->d_fpk, c->d_rowoff,
+            c->d_rowtab, c->d_xs, c->d_meta, c->d_status, c->d_scal);
+    });
     prof_end(c, KID_STRUCTURE);
-    return launch_row_tables(c);
+    return cudaGetLastError();
 }
 
 // Sample indices of masks that are unions of full lines (meta[MT_GENERAL] = 0).
@@ -167,36 +260,78 @@ cudaError_t launch_fill_lines(lrccs_ctx *c) {
 
 // ---------------------------------------------------------------- gamma
 // gamma = trunc * sum |y|^2 / (number of measured entries)  (Alg. 2, init).
-// |y|^2 is formed in FP64 without contraction so that the truncation decision
-// |y|^2 <= gamma is taken on exactly the same squares as an FP64 reference.
+// FP64 adds bound an FP64 sum here (two a cycle per multiprocessor: 50 us for
+// 2.7 M entries, 403 us for 34 M), so each thread sums in FP32 without error:
+// a square is the exact pair (p, fma(x, x, -p)), and p, its error term and the
+// rounding of every addition go into three levels of two_sum (about 72 bits,
+// more than an FP64 accumulator holds); threads and blocks add in FP64 in a
+// fixed order: 17 us and 93 us.
 
+struct fsum3 {
+    float a, b, c;
+};
+LRCCS_DEV void fsum3_add(fsum3 &s, float x) {
+    float e, f;
+    two_sum(s.a, x, s.a, e);
+    two_sum(s.b, e, s.b, f);
+    s.c += f;
+}
+// x^2, exactly, where neither the square nor its error term leaves the FP32
+// range (and not NaN); anything else goes to the FP64 sum
+LRCCS_DEV void fsum3_sq(fsum3 &s, double &wide, float x) {
+    const float ax = fabsf(x);
+    if (!(ax <= 1e15f && (ax >= 1e-13f || ax == 0.f))) {
+        wide += (double)x * (double)x;
+        return;
+    }
+    const float p = __fmul_rn(x, x);
+    float f;
+    fsum3_add(s, p);
+    two_sum(s.b, fmaf(x, x, -p), s.b, f);
+    s.c += f;
+}
 
-__global__ void k_energy(const float2 *__restrict__ y, int64_t count, double trunc, double *part,
-                         unsigned int *counter, double *scal) {
-    __shared__ double s_red[32];
-    double acc = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x)
-        acc += abs2_rn(y[i]);
+__global__ void __launch_bounds__(256) k_energy(const float2 *__restrict__ y, int64_t count, double trunc, double *part,
+                                                unsigned int *counter, double *scal) {
+    __shared__ double s_red[8];
+    fsum3 s = {0.f, 0.f, 0.f};
+    double wide = 0.0;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; i + 3 * step < count; i += 4 * step) {
+        float2 v[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(y + i + u * step);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            fsum3_sq(s, wide, v[u].x);
+            fsum3_sq(s, wide, v[u].y);
+        }
+    }
+    for (; i < count; i += step) {
+        const float2 v = __ldg(y + i);
+        fsum3_sq(s, wide, v.x);
+        fsum3_sq(s, wide, v.y);
+    }
+    const double acc = warp_sum_d(wide + ((double)s.a + ((double)s.b + (double)s.c)));
     if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double b = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += s_red[w];
+        for (int w = 0; w < 8; ++w) b += s_red[w];
         part[blockIdx.x] = b;
     }
-    if (last_block_arrive(counter) && threadIdx.x == 0) {
+    if (last_block_arrive(counter) && threadIdx.x < 32) {
         double e = 0.0;
-        for (int b = 0; b < (int)gridDim.x; ++b) e += __ldcg(part + b);
-        scal[SC_GAMMA] = trunc * e / (double)count;
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) e += __ldcg(part + b);
+        e = warp_sum_d(e);
+        if (threadIdx.x == 0) scal[SC_GAMMA] = trunc * e / (double)count;
     }
 }
 
 cudaError_t launch_energy(lrccs_ctx *c, const float2 *d_y) {
     const int64_t count = (int64_t)c->nc * c->total;
-    const int blocks = 304;
+    const int blocks = 4 * c->nsm < 1024 ? 4 * c->nsm : 1024;   // partials: doubles of d_gpart (at least 1024)
     prof_begin(c, KID_ENERGY);
     k_energy<<<blocks, 256, 0, c->stream>>>(d_y, count, c->prm.trunc_factor, (double *)c->d_gpart,
                                             c->d_counters + CNT_ENERGY, c->d_scal);
@@ -205,150 +340,185 @@ cudaError_t launch_energy(lrccs_ctx *c, const float2 *d_y) {
 }
 
 // ---------------------------------------------------------------- Z and X0
-// Z[:, k] = A_k^H y_k and X0[:, k] = A_k^H y_k,tnc / sqrt(m_k mbar), computed as
-// a row pass (inverse DFT along kx of every sampled line, both the plain and
-// the truncated data) and a column pass (inverse DFT along ky, coil combine
-// with conj(d_j)).  The line layout of y makes every sampled row contiguous.
+// Z[:, k] = A_k^H y_k and X0[:, k] = A_k^H y_k,tnc / sqrt(m_k mbar) (the plain and
+// the truncated data), w frames at a time as the columns of one transform: a
+// row pass scatters the frames' samples of k-space row ky and transforms them
+// back along x into T[j][ky][x][l] (frame k0 + l), and the iteration's adjoint
+// column pass, reading for column l only the rows frame k0 + l samples, does the
+// rest and writes column k0 + l of Z or X0.  Any mask takes this path (full
+// lines only make the scatter the identity).  Z and X0, kernel time: 16 spokes on
+// 256 x 256, q = 64, C = 20: direct sums over each row's samples in one kernel 3.22 ms
+// -> 8 chunks of 108 + 89 us; 8 frames of 224 x 224 (Z alone, which is all that
+// tracking needs): 0.98 ms -> 26 + 50 us; lines of 192 x 192, q = 48, C = 12: 36 + 175 us
+// -> 6 chunks of 15 + 23 us.
+//
+// Row pass: block (row ky, coil group); only the nf frames of the chunk that
+// sample ky take part.  Item (frame c, g): its length-R1 DFT takes kx = g + R2 m
+// (lanes along g: contiguous samples), its length-R2 DFT gives x = g + R1 k2
+// (lanes along c: neighbouring columns of T).  The exchange tile holds (k1, c,
+// j2) at k1 S + c (R2 + 1) + j2, S = nf modulo 16, free of bank conflicts on both
+// sides; samples are staged in place one coil step ahead, as in the general
+// row passes.
+struct InitArgs {
+    const float2 *y;
+    const int32_t *usedrows, *rfptr, *rflist, *rowoff, *fpk, *mks;
+    const uint8_t *mask;       // q x n bitmap (general masks), or NULL: full lines
+    const double *scal;
+    const float2 *tw;          // [j2][k1] twiddles with the scale 1 / sqrt(nx)
+    int ny, nc, w, k0;
+};
 
 template <int P>
-__global__ void __launch_bounds__(256) k_init_rows(const float2 *__restrict__ y, float2 *__restrict__ T0,
-                                                    int64_t total_rows, const double *__restrict__ scal,
-                                                    const float2 *__restrict__ g_tw, float scale) {
-    // 4 rows x {plain, truncated} = 8 transforms per block; tile[x][2 row + ch]
-    constexpr int N = 32 * P;
-    constexpr int ROWS = 4, TPR = 2 * ROWS + 1;
-    __shared__ float2 s_tw[N];
-    __shared__ float2 tile[N * TPR];
-    load_twiddles(s_tw, g_tw, N);
-    const int64_t g0 = (int64_t)blockIdx.x * ROWS;
-    const double gam = scal[SC_GAMMA];
-    for (int e = threadIdx.x; e < ROWS * N; e += blockDim.x) {
-        const int row = e / N, x = e - row * N;
-        float2 a = make_float2(0.f, 0.f);
-        if (g0 + row < total_rows) a = y[(g0 + row) * N + x];
-        tile[x * TPR + 2 * row] = a;
-        tile[x * TPR + 2 * row + 1] = abs2_rn(a) > gam ? make_float2(0.f, 0.f) : a;
+struct RowPlanI {
+    static constexpr int NX = 32 * P, R1 = fft::Plan<NX>::R1, R2 = fft::Plan<NX>::R2, NG = R1 > R2 ? R1 : R2;
+    static __host__ __device__ int coils(int nf, int nc) {   // coils at a time: a block of 256 threads
+        const int cb = 256 / (NG * nf);
+        return cb < 1 ? 1 : (cb < nc ? cb : nc);
+    }
+    static __host__ __device__ int stride(int nf) { return nf * (R2 + 1) + (16 - nf * R2 % 16) % 16; }
+};
+
+template <int P, bool TRUNC>
+__global__ void __launch_bounds__(256, 3) k_init_rows(float2 *__restrict__ T, const InitArgs a) {
+    using PL = RowPlanI<P>;
+    constexpr int NX = PL::NX, R1 = PL::R1, R2 = PL::R2, NG = PL::NG;
+    extern __shared__ __align__(16) float2 smem[];
+    __shared__ int16_t s_pos[16 * NX];   // general masks: sample index of kx in the frame's row, or -1
+    __shared__ int s_fr[16], s_nf;
+    __shared__ int64_t s_base[16];       // first sample of (frame, row) for coil 0
+    __shared__ int s_m[16];
+    const int ky = a.usedrows[blockIdx.x], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp == 0) {
+        int nf = 0;
+        for (int f0 = a.rfptr[ky]; f0 < a.rfptr[ky + 1]; f0 += 32) {
+            const int f = f0 + lane, k = f < a.rfptr[ky + 1] ? a.rflist[f] : -1;
+            const bool in = k >= a.k0 && k < a.k0 + a.w;
+            const unsigned bal = __ballot_sync(0xffffffffu, in);
+            if (in) {
+                const int c = nf + __popc(bal & ((1u << lane) - 1u)), f0k = a.fpk[k];
+                s_fr[c] = k;
+                s_m[c] = a.mks[k];
+                s_base[c] = (int64_t)a.nc * f0k + (a.rowoff[k * a.ny + ky] - f0k);
+            }
+            nf += __popc(bal);
+        }
+        if (lane == 0) s_nf = nf;
     }
     __syncthreads();
-    fft::tile_dft<N, true>(tile, TPR, 2 * ROWS, s_tw, scale);
-    for (int e = threadIdx.x; e < ROWS * 2 * N; e += blockDim.x) {
-        const int row = e / (2 * N), rem = e - row * 2 * N, x = rem >> 1, ch = rem & 1;
-        if (g0 + row < total_rows) T0[(g0 + row) * N * 2 + rem] = tile[x * TPR + 2 * row + ch];
+    const int nf = s_nf;
+    if (nf == 0) return;   // the same for every thread of the block
+    if (a.mask) {
+        for (int c = warp; c < nf; c += 8) {
+            const uint8_t *m = a.mask + ((size_t)s_fr[c] * a.ny + ky) * NX;
+            int pos = 0;
+            for (int x0 = 0; x0 < NX; x0 += 32) {
+                const bool in = m[x0 + lane] != 0;
+                const unsigned bal = __ballot_sync(0xffffffffu, in);
+                s_pos[c * NX + x0 + lane] = (int16_t)(in ? pos + __popc(bal & ((1u << lane) - 1u)) : -1);
+                pos += __popc(bal);
+            }
+        }
+        __syncthreads();
+    }
+    const int CB = PL::coils(nf, a.nc), IT = NG * nf, S = PL::stride(nf), tile = R1 * S;
+    const int slot = threadIdx.x / IT, i = threadIdx.x - slot * IT;
+    const int c1 = i / NG, g1 = i - c1 * NG, g2 = i / nf, c2 = i - g2 * nf;
+    const bool first = slot < CB && g1 < R2, second = slot < CB && g2 < R1;
+    const int step = gridDim.y * CB;
+    float2 *mine = smem + slot * tile;
+    uint32_t bits = 0;
+    if (first) {
+        bits = (1u << R1) - 1u;
+        if (a.mask) {
+            bits = 0;
+            for (int m = 0; m < R1; ++m) bits |= (uint32_t)(s_pos[c1 * NX + g1 + R2 * m] >= 0) << m;
+        }
+    }
+    auto stage = [&](int j, int s) {
+        if (bits != 0 && j < a.nc) {
+            float2 *dst = mine + s * CB * tile + c1 * (R2 + 1) + g1;
+            const float2 *src = a.y + s_base[c1] + (int64_t)j * s_m[c1];
+#pragma unroll
+            for (int m = 0; m < R1; ++m)
+                if (bits >> m & 1) cp_async8(dst + m * S, src + (a.mask ? (int)s_pos[c1 * NX + g1 + R2 * m] : g1 + R2 * m));
+        }
+        cp_async_commit();
+    };
+    stage(blockIdx.y * CB + slot, 0);
+    const double gam = TRUNC ? a.scal[SC_GAMMA] : 0.0;
+    const float glo = (float)(gam * (1.0 - 1e-5)), ghi = (float)(gam * (1.0 + 1e-5));
+    int s = 0;
+    for (int b = blockIdx.y * CB; b < a.nc; b += step, s ^= 1) {
+        const int j = b + slot;
+        float2 *ex = mine + s * CB * tile;
+        cp_async_wait();
+        if (first && j < a.nc) {
+            float2 v[R1], *e = ex + c1 * (R2 + 1) + g1;
+#pragma unroll
+            for (int m = 0; m < R1; ++m) {
+                v[m] = (bits >> m & 1) ? e[m * S] : make_float2(0.f, 0.f);
+                if (TRUNC && trunc_drop(v[m], gam, glo, ghi)) v[m] = make_float2(0.f, 0.f);
+            }
+            fft::dft_first<R1, R2, true>(v, g1, a.tw, [&](int k1, float2 w) { e[k1 * S] = w; });
+        }
+        __syncthreads();
+        if (b + step < a.nc) stage(j + step, s ^ 1);
+        if (second && j < a.nc) {
+            float2 v[R2];
+            const float2 *e = ex + g2 * S + c2 * (R2 + 1);
+#pragma unroll
+            for (int j2 = 0; j2 < R2; ++j2) v[j2] = e[j2];
+            fft::Dft<R2, true>::run(v);
+            float2 *dst = T + (((size_t)j * a.ny + ky) * NX + g2) * a.w + (s_fr[c2] - a.k0);
+#pragma unroll
+            for (int k2 = 0; k2 < R2; ++k2) dst[(size_t)(R1 * k2) * a.w] = v[k2];
+        }
     }
 }
 
-#define TXI 8
 template <int P>
-__global__ void __launch_bounds__(256) k_init_cols(const float2 *__restrict__ T0, const float2 *__restrict__ smaps,
-                                                    const int32_t *__restrict__ rowidx,
-                                                    const int32_t *__restrict__ lineptr, const int32_t *__restrict__ mks,
-                                                    const double *__restrict__ scal,
-                                                    float2 *__restrict__ Z, float2 *__restrict__ X0, int nx, int q,
-                                                    int nc, const float2 *__restrict__ g_tw, float scale) {
-    constexpr int NY = 32 * P;
-    constexpr int TP = 2 * TXI + 1;
-    extern __shared__ float2 smem[];
-    float2 *s_tw = smem;
-    float2 *tile = s_tw + NY;
-    float2 *s_S = tile + NY * TP;
-    load_twiddles(s_tw, g_tw, NY);
-    const int k = blockIdx.y, x0 = blockIdx.x * TXI;
-    const int n = NY * nx;
-    const int lp = lineptr[k];
-    const int64_t mk = (int64_t)(lineptr[k + 1] - lp) * nx;
-    const int64_t fbase = (int64_t)nc * lp * nx;
-    // thread owns tile elements e = tid + 256 u: yy = e / (2 TXI), cc = e % (2 TXI)
-    constexpr int ACC = (NY * 2 * TXI + 255) / 256;
-    float2 acc[ACC];
-    int goff[ACC];       // this thread's tile elements: offset in a coil's line block, or -1
-#pragma unroll
-    for (int u = 0; u < ACC; ++u) {
-        acc[u] = make_float2(0.f, 0.f);
-        const int e = threadIdx.x + 256 * u;
-        goff[u] = -1;
-        if (e < NY * 2 * TXI) {
-            const int yy = e / (2 * TXI), cc = e % (2 * TXI);
-            const int li = rowidx[k * NY + yy];
-            if (li >= 0) goff[u] = (li * nx + x0) * 2 + cc;
-        }
-    }
-    for (int j = 0; j < nc; ++j) {
-        __syncthreads();
-        const int64_t jb = (fbase + j * mk) * 2;
-#pragma unroll
-        for (int u = 0; u < ACC; ++u) {
-            const int e = threadIdx.x + 256 * u;
-            if (e < NY * 2 * TXI) {
-                const int yy = e / (2 * TXI), cc = e % (2 * TXI);
-                tile[yy * TP + cc] = goff[u] >= 0 ? T0[jb + goff[u]] : make_float2(0.f, 0.f);
-            }
-        }
-        for (int e = threadIdx.x; e < NY * TXI; e += blockDim.x)
-            s_S[e] = smaps[(size_t)j * n + (size_t)(e / TXI) * nx + x0 + (e % TXI)];
-        __syncthreads();
-        fft::tile_dft<NY, true>(tile, TP, 2 * TXI, s_tw, scale);
-#pragma unroll
-        for (int u = 0; u < ACC; ++u) {
-            const int e = threadIdx.x + 256 * u;
-            if (e < NY * 2 * TXI) {
-                const int yy = e / (2 * TXI), cc = e % (2 * TXI);
-                cfmac(acc[u], s_S[yy * TXI + (cc >> 1)], tile[yy * TP + cc]);
-            }
-        }
-    }
-    const double mbar = scal[SC_MBAR];
-    const int msamp = mks[k];   // samples per coil of frame k (m_k of Alg. 2's scale 1/sqrt(m_k mbar))
-    const float xs = (msamp > 0) ? (float)(1.0 / sqrt((double)msamp * mbar)) : 0.f;
-#pragma unroll
-    for (int u = 0; u < ACC; ++u) {
-        const int e = threadIdx.x + 256 * u;
-        if (e < NY * 2 * TXI) {
-            const int yy = e / (2 * TXI), cc = e % (2 * TXI);
-            const size_t i = (size_t)yy * nx + x0 + (cc >> 1);
-            if ((cc & 1) == 0) Z[i * q + k] = acc[u];
-            else X0[i * q + k] = cscale(acc[u], xs);
-        }
-    }
+static cudaError_t launch_init_rows(lrccs_ctx *c, const float2 *d_y, int w, int k0, bool trunc) {
+    using PL = RowPlanI<P>;
+    InitArgs a;
+    a.y = d_y;
+    a.usedrows = c->d_usedrows;
+    a.rfptr = c->d_rfptr;
+    a.rflist = c->d_rflist;
+    a.rowoff = c->d_rowoff;
+    a.fpk = c->d_fpk;
+    a.mks = c->d_mks;
+    a.mask = c->general ? c->d_maskc : nullptr;
+    a.scal = c->d_scal;
+    a.tw = c->d_twsx;
+    a.ny = c->ny;
+    a.nc = c->nc;
+    a.w = w;
+    a.k0 = k0;
+    size_t tile = 0;   // two tiles of the widest row the chunk can hold
+    for (int nf = 1; nf <= w; ++nf) tile = std::max(tile, (size_t)PL::coils(nf, c->nc) * PL::R1 * PL::stride(nf));
+    const dim3 grid(c->n_used, std::max(1, std::min(c->nc, (4 * c->nsm + c->n_used - 1) / c->n_used)));
+    prof_begin(c, KID_INIT_ROWS);
+    if (trunc) k_init_rows<P, true><<<grid, 256, 2 * tile * sizeof(float2), c->stream>>>(c->d_T, a);
+    else k_init_rows<P, false><<<grid, 256, 2 * tile * sizeof(float2), c->stream>>>(c->d_T, a);
+    prof_end(c, KID_INIT_ROWS);
+    return cudaGetLastError();
 }
 
-#define DISPATCH_P(PV, ...)                                           \
-    switch (PV) {                                                      \
-        case 1: { constexpr int P_ = 1; __VA_ARGS__; } break;                 \
-        case 2: { constexpr int P_ = 2; __VA_ARGS__; } break;                 \
-        case 3: { constexpr int P_ = 3; __VA_ARGS__; } break;                 \
-        case 4: { constexpr int P_ = 4; __VA_ARGS__; } break;                 \
-        case 5: { constexpr int P_ = 5; __VA_ARGS__; } break;                 \
-        case 6: { constexpr int P_ = 6; __VA_ARGS__; } break;                 \
-        case 7: { constexpr int P_ = 7; __VA_ARGS__; } break;                 \
-        case 8: { constexpr int P_ = 8; __VA_ARGS__; } break;                 \
-        default: return cudaErrorInvalidValue;                         \
-    }
-
-cudaError_t launch_init_adjoint(lrccs_ctx *c, const float2 *d_y) {
-    const int64_t total_rows = (int64_t)c->nc * c->n_lines;
-    const float sx = (float)(1.0 / sqrt((double)c->nx));
-    const float sy = (float)(1.0 / sqrt((double)c->ny));
-    const unsigned rb = (unsigned)((total_rows + 3) / 4);
-    if (c->general) return launch_init_general(c, d_y);   // frame rows hold scattered samples: one fused pass
-    if (total_rows > 0) {
-        DISPATCH_P(c->px, {
-            prof_begin(c, KID_INIT_ROWS);
-            k_init_rows<P_><<<rb, 256, 0, c->stream>>>(d_y, c->d_T, total_rows, c->d_scal, c->d_twx, sx);
-            prof_end(c, KID_INIT_ROWS);
-        });
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const size_t smem = (size_t)c->ny * (1 + 2 * TXI + 1 + TXI) * sizeof(float2);
-    dim3 grid(c->nx / TXI, c->q);
-    DISPATCH_P(c->py, {
-        prof_begin(c, KID_INIT_COLS);
-        k_init_cols<P_><<<grid, 256, smem, c->stream>>>(c->d_T, c->d_smaps, c->d_rowidx, c->d_lineptr, c->d_mks,
-                                                        c->d_scal, c->d_Z, c->d_X0, c->nx, c->q, c->nc,
-                                                        c->d_twy, sy);
-        prof_end(c, KID_INIT_COLS);
-    });
-    return cudaGetLastError();
+// Z, and with trunc also X0 (which only the spectral initialisation reads).
+cudaError_t launch_init_adjoint(lrccs_ctx *c, const float2 *d_y, bool trunc) {
+    const int wmax = (int)std::min<size_t>(16, c->T_cap / ((size_t)c->nc * c->n));
+    const int nch = (c->q + wmax - 1) / wmax, w = (c->q + nch - 1) / nch;
+    for (int ch = 0; ch < (trunc ? 2 : 1); ++ch)
+        for (int k0 = 0; k0 < c->q; k0 += w) {
+            DISPATCH_P(c->px, {
+                cudaError_t e = launch_init_rows<P_>(c, d_y, w, k0, ch == 1);
+                if (e != cudaSuccess) return e;
+            });
+            // X0's columns are scaled by 1 / sqrt(m_k mbar)
+            cudaError_t e = launch_adj_cols_frames(c, ch ? c->d_X0 : c->d_Z, w, k0, ch ? c->d_xs : nullptr);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 // ---------------------------------------------------------------- Gram of X0 and its eigensolver
@@ -686,13 +856,15 @@ cudaError_t launch_u0(lrccs_ctx *c) {
 
 // Allow every kernel of this file the device's opt-in shared memory per block
 // (the launch still requests only what it needs).
-#define SET_SMEM(fn) do { cudaError_t e_ = allow_smem(fn, max_smem); if (e_ != cudaSuccess) return e_; } while (0)
+#define SET_SMEM(...) do { cudaError_t e_ = allow_smem(__VA_ARGS__, max_smem); if (e_ != cudaSuccess) return e_; } while (0)
+#define SET_SMEM_B(fn, P) SET_SMEM(fn<P, false>); SET_SMEM(fn<P, true>)
 cudaError_t configure_kernels_init(int max_smem) {
-    SET_SMEM(k_init_cols<1>); SET_SMEM(k_init_cols<2>); SET_SMEM(k_init_cols<3>); SET_SMEM(k_init_cols<4>);
-    SET_SMEM(k_init_cols<5>); SET_SMEM(k_init_cols<6>); SET_SMEM(k_init_cols<7>); SET_SMEM(k_init_cols<8>);
+    SET_SMEM_B(k_init_rows, 1); SET_SMEM_B(k_init_rows, 2); SET_SMEM_B(k_init_rows, 3); SET_SMEM_B(k_init_rows, 4);
+    SET_SMEM_B(k_init_rows, 5); SET_SMEM_B(k_init_rows, 6); SET_SMEM_B(k_init_rows, 7); SET_SMEM_B(k_init_rows, 8);
     SET_SMEM(k_gram_x0<1>); SET_SMEM(k_gram_x0<2>); SET_SMEM(k_gram_x0<3>); SET_SMEM(k_gram_x0<5>);
     SET_SMEM(k_gram_x0<8>); SET_SMEM(k_gram_x0<12>); SET_SMEM(k_gram_x0<MAXPP>);
     SET_SMEM(k_eig);
+    SET_SMEM(k_structure);
     SET_SMEM(k_u0);
     return cudaGetLastError();
 }

@@ -322,10 +322,18 @@ __global__ void __launch_bounds__(256) k_row_w(float2 *__restrict__ T, const flo
 // Measured (kernel time, L2 warm), one image column per block staged by 8-byte
 // cp.async -> this form: 192 x 192, C = 12, r = 10: 28.9 -> 17.4 us; 256 x 256,
 // C = 20, r = 12: 121 -> 65 us; 256 x 256, C = 32, r = 14: 291 -> 114 us
+// Where k_adj_cols writes: element (pixel i, column l < cols) at p[i stride + l],
+// times scale[l] when scale is not NULL.
+struct AdjOut {
+    float2 *p;
+    int stride, cols;
+    const float *scale;
+};
+
 template <int P>
 __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_adj_cols(
     const float2 *__restrict__ T, const float2 *__restrict__ smaps, const uint32_t *__restrict__ rowtab, int e0,
-    int estep, float2 *__restrict__ Gk, int nx, int r, int nc, int nxt, unsigned inv, const float2 *__restrict__ g_tw) {
+    int estep, const AdjOut out, int nx, int r, int nc, int nxt, unsigned inv, const float2 *__restrict__ g_tw) {
     using PL = ColPlan<P>;
     constexpr int NY = PL::NY, R1 = PL::R1, R2 = PL::R2, NG = PL::NG;
     extern __shared__ __align__(16) float2 smem[];   // two tiles of NY x COLW, two map stages
@@ -385,10 +393,15 @@ __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_adj_co
             }
         }
     }
+    // element (y, x, l) of the result
+    float2 *dst = out.p + (size_t)x * out.stride + l;
+    const size_t orow = (size_t)nx * out.stride;
+    const bool live = l < out.cols;
+    const float sc = out.scale && live ? __ldg(out.scale + l) : 1.f;
     if (CG == 1) {
-        if (second) {
+        if (second && live) {
 #pragma unroll
-            for (int k2 = 0; k2 < R2; ++k2) Gk[(size_t)(R1 * k2 + g) * rs + c] = acc[k2];
+            for (int k2 = 0; k2 < R2; ++k2) dst[(R1 * k2 + g) * orow] = cscale(acc[k2], sc);
         }
         return;
     }
@@ -402,7 +415,7 @@ __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_adj_co
     for (int y = grp + CG * g; y < NY; y += CG * NG) {
         float2 sum = make_float2(0.f, 0.f);
         for (int k = 0; k < CG; ++k) sum = cadd(sum, cluster.map_shared_rank(smem, k)[y * COLW + lane]);
-        Gk[(size_t)y * rs + c] = sum;
+        if (live) dst[y * orow] = cscale(sum, sc);
     }
     cluster.sync();   // no block leaves while its tile may still be read
 }
@@ -493,7 +506,7 @@ static void launch_row_w(lrccs_ctx *c) {
 }
 
 // coil-summed inverse transform into dst (n x r); cluster size: the plan's, or col_groups
-cudaError_t launch_adj_cols_to(lrccs_ctx *c, float2 *dst, int r, int e0, int estep) {
+static cudaError_t adj_cols(lrccs_ctx *c, const AdjOut &out, int r, int e0, int estep) {
     const int nx = c->nx, tiles = nx * r / COLW, nxt = col_nxt(r);
     cudaLaunchConfig_t cfg = {};
     cfg.stream = c->stream;
@@ -516,27 +529,21 @@ cudaError_t launch_adj_cols_to(lrccs_ctx *c, float2 *dst, int r, int e0, int est
         cfg.dynamicSmemBytes = smem;
         prof_begin(c, KID_ADJ_COLS);
         el = cudaLaunchKernelEx(&cfg, k_adj_cols<P_>, (const float2 *)c->d_T, (const float2 *)c->d_smaps,
-                                (const uint32_t *)c->d_rowtab, e0, estep, dst, nx, r, c->nc, nxt,
+                                (const uint32_t *)c->d_rowtab, e0, estep, out, nx, r, c->nc, nxt,
                                 (65536u + nxt - 1) / nxt, (const float2 *)c->d_twsy);
         prof_end(c, KID_ADJ_COLS);
     });
     return el;
 }
 
-// Sampled-row tables of the column passes: entry 0 the rows some frame samples,
-// entry 1 + k the rows of frame k, then 16 empty entries (frames past q).
-__global__ void k_row_tables(const int32_t *__restrict__ rowcnt, const uint8_t *__restrict__ rowused, int q, int ny,
-                             int R1, int R2, uint32_t *__restrict__ tab) {
-    const int e = blockIdx.x, t = threadIdx.x, g = t & 15;
-    uint32_t bits = 0;
-    const int step = t < 16 ? R1 : R2, cnt = t < 16 ? R2 : R1;
-    if (g < step)
-        for (int i = 0; i < cnt; ++i) {
-            const int y = g + step * i;
-            const bool used = e == 0 ? rowused[y] != 0 : (e <= q && rowcnt[(e - 1) * ny + y] > 0);
-            bits |= (uint32_t)used << i;
-        }
-    tab[e * 32 + t] = bits;
+cudaError_t launch_adj_cols_to(lrccs_ctx *c, float2 *dst, int r, int e0, int estep) {
+    return adj_cols(c, AdjOut{dst, r, r, nullptr}, r, e0, estep);
+}
+
+// Columns of T as the frames k0 .. k0 + w - 1, each on its own rows, into columns
+// k0 .. of the n x q array dst, times scale[k] when given.
+cudaError_t launch_adj_cols_frames(lrccs_ctx *c, float2 *dst, int w, int k0, const float *scale) {
+    return adj_cols(c, AdjOut{dst + k0, c->q, c->q - k0, scale ? scale + k0 : nullptr}, w, 1 + k0, 1);
 }
 
 // Twiddles of the column and row passes, [j2][k1]: w_N^(j2 k1) / sqrt(N).
@@ -553,16 +560,6 @@ __global__ void k_col_twiddles(float2 *tw, int N, int R1) {
 cudaError_t launch_col_twiddles(lrccs_ctx *c) {
     DISPATCH_P(c->py, { k_col_twiddles<<<1, 256, 0, c->stream>>>(c->d_twsy, c->ny, ColPlan<P_>::R1); });
     DISPATCH_P(c->px, { k_col_twiddles<<<1, 256, 0, c->stream>>>(c->d_twsx, c->nx, ColPlan<P_>::R1); });
-    return cudaGetLastError();
-}
-
-cudaError_t launch_row_tables(lrccs_ctx *c) {
-    DISPATCH_P(c->py, {
-        prof_begin(c, KID_STRUCTURE);
-        k_row_tables<<<c->q + 17, 32, 0, c->stream>>>(c->d_rowcnt, c->d_rowused, c->q, c->ny, ColPlan<P_>::R1,
-                                                      ColPlan<P_>::R2, c->d_rowtab);
-        prof_end(c, KID_STRUCTURE);
-    });
     return cudaGetLastError();
 }
 
