@@ -494,8 +494,8 @@ lrccs_status lrccs_forward_transform(lrccs_ctx *ctx, void *d_T, size_t bytes);
  * per-step timing markers, Sec. V).  enable != 0 allocates a stamp buffer and
  * makes every later GD/QR kernel of an iteration (launched directly or
  * replayed in the iteration graph, which is re-captured) record clock64() at
- * 9 points in each block: start, inputs staged, gradient and Gram partials
- * done, partials written, grid barrier 1 passed, totals reduced, barrier 2
+ * 9 points in each block: start, inputs staged and gradient formed, Gram
+ * partials written (two points), grid barrier 1 passed, totals reduced, barrier 2
  * passed, the r x r factors done, U_{t+1} written; and the global timer at
  * the block's entry and exit.  out (NULL, or 18 doubles) receives, for each of
  * the 8 intervals, the mean and the maximum over the blocks in SM cycles of

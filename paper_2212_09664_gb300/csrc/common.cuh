@@ -494,8 +494,9 @@ LRCCS_DEV void grid_sync(unsigned int *bar, unsigned int k, unsigned int *status
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned int target = k * gridDim.x + skew;
-        __threadfence();
-        atomicAdd(bar, 1u);
+        // the release covers the block's writes (ordered before it by the
+        // barrier above), the acquire orders the others' before the one below
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(bar) : "memory");
         unsigned int v = 0, spins = 0;
         while (true) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(bar) : "memory");
@@ -504,9 +505,7 @@ LRCCS_DEV void grid_sync(unsigned int *bar, unsigned int k, unsigned int *status
                 atomicOr(status, timeout_bit);
                 break;
             }
-            __nanosleep(32);
         }
-        __threadfence();
     }
     __syncthreads();
 }
@@ -537,8 +536,9 @@ LRCCS_DEV void stage_row(float2 *dst, const float2 *src, int count, int tid, int
 }
 LRCCS_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 LRCCS_DEV void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-// wait until at most one committed group is still pending (double buffering)
+// wait until at most one (two) committed groups are still pending
 LRCCS_DEV void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+LRCCS_DEV void cp_async_wait_2() { asm volatile("cp.async.wait_group 2;\n" ::: "memory"); }
 
 // ---------------------------------------------------------------- bulk copies (TMA)
 // A bulk copy lands in shared memory and completes a transaction count on an

@@ -21,8 +21,9 @@
 //
 // In init mode the same kernel orthonormalises the given U+ (G1 = U+^H U+)
 // and forms the first right-hand sides U_0^H Z.
-// A block's pixel range stays in shared memory across the phases when it
-// fits; otherwise each phase re-stages it in chunks.
+// A block's pixel range of U and of the gradient stays in shared memory across
+// the phases; its rows of Z stream in behind phase 1 (all of them when they fit,
+// else through two chunk buffers).
 //
 // Z B^H depends only on the B-step's result, so its own kernel k_zb forms it
 // while the adjoint transforms run (a parallel branch of the iteration).
@@ -32,6 +33,8 @@
 // with an iteration limit: a barrier that gives up sets ST_TIMEOUT and the
 // kernel runs to completion with that status raised.
 #include <math.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "internal.h"
@@ -53,7 +56,7 @@ struct GdArgs {
     double *scal;       // SC_* scalars
     unsigned int *bar;  // [0] barrier arrivals, [1] exit count
     unsigned int *status;
-    int n, r, q, zs, chunk, resident, mode;
+    int n, q, per, zs, zc, nbuf, mode;   // per: pixels per block; zc: rows of a Z chunk buffer, nbuf of them
     double eta_c;
     double eta_scale0, eta_decay;   // variable step size: eta_t = eta eta_scale0 eta_decay^k
     long long *ts;             // NULL, or GD_NTS clock64() stamps per block (phase timing)
@@ -142,91 +145,199 @@ static __device__ void stage_rows(float2 *dst, int ds, const float2 *src, int ss
     }
 }
 
-// Rinv = (L^H)^{-1} for the lower-triangular L of warp_chol32 (row-major R x R,
-// invd = 1 / diag), by one warp: lane j forms column j of X = L^{-1} by
-// forward substitution in registers (L read by broadcast), then row j of
-// Rinv = X^H (upper triangular).
+// Row stride (complex values) of U and the gradient in shared memory: rows 16-byte
+// aligned for even R, and eight consecutive rows on distinct banks.
 template <int R>
-static __device__ void warp_rinv(const float2 *L, const float *invd, float2 *Rinv) {
-    const int j = threadIdx.x & 31;
-    float2 x[R];
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-        float2 acc = make_float2(i == j ? 1.f : 0.f, 0.f);
-#pragma unroll
-        for (int m = 0; m < i; ++m) acc = csub(acc, cmul(L[i * R + m], x[m]));
-        x[i] = cscale(acc, invd[i]);   // zero for i < j
-    }
-    if (j < R) {
-#pragma unroll
-        for (int i = 0; i < R; ++i) Rinv[j * R + i] = i >= j ? cconj(x[i]) : make_float2(0.f, 0.f);
-    }
-    __syncwarp();
-}
-
-// 2 x 2 tile of a cross-Gram: acc[2 i + j] += sum_ii conj(X[ii][x_i]) Y[ii][y_j].
-struct Tile {
-    const float2 *X, *Y;
-    int xs, ys, x0, x1, y0, y1;
+struct GdPlan {
+    static constexpr int RS = R % 4 == 0 ? R + 2 : R;
+    static constexpr int TR = (R + 1) / 2, TH = TR * (TR + 1) / 2, NP = R * (R + 1) / 2;
+    // 2 x 2 tiles: [grad^H grad (upper) | U^H grad (all) | U^H U (upper)], init: [U+^H U+ (upper)]
+    static constexpr int T_ITER = 2 * TH + TR * TR, L_ITER = 2 * NP + R * R;
 };
-static __device__ void tile_accumulate(const Tile &g, float2 (&acc)[4], int s, int S, int cn) {
-#pragma unroll 4
-    for (int ii = s; ii < cn; ii += S) {
-        const float2 p0 = g.X[ii * g.xs + g.x0], p1 = g.X[ii * g.xs + g.x1];
-        const float2 q0 = g.Y[ii * g.ys + g.y0], q1 = g.Y[ii * g.ys + g.y1];
-        cfmac(acc[0], p0, q0);
-        cfmac(acc[1], p0, q1);
-        cfmac(acc[2], p1, q0);
-        cfmac(acc[3], p1, q1);
+// pixel slices per tile: the largest power of two <= 32 with tiles x slices <= NTG
+__host__ __device__ constexpr int gd_slices(int tiles) {
+    int s = 1;
+    while (2 * s <= 32 && 2 * s * tiles <= NTG) s *= 2;
+    return s;
+}
+
+// columns 2A, 2A + 1 of a row (the last one twice past R)
+template <int R>
+LRCCS_DEV void gd_pair(const float2 *row, int A, float2 &p0, float2 &p1) {
+    if constexpr (R % 2 == 0) {
+        const float4 v = *reinterpret_cast<const float4 *>(row + 2 * A);
+        p0 = make_float2(v.x, v.y);
+        p1 = make_float2(v.z, v.w);
+    } else {
+        p0 = row[2 * A];
+        p1 = row[min(2 * A + 1, R - 1)];
     }
 }
 
-// Combine the slices of up to two tile items per thread (item w = t + u NTG,
-// tile w mod T, slice w / T) and write entry m of tile w2 to
-// part[blockIdx.x * ld + out(w2, m)] (skipped when out < 0).  One round when
-// the scratch scr (cap complex values) holds all four entries of every item,
-// else one round per entry through s_red2 (2 NTG values).
-template <class OUT>
-static __device__ void tiles_write(const float2 (&acc)[2][4], int T, int S, float2 *scr, int cap, float2 *s_red2,
-                                   float2 *part, int ld, OUT out) {
-    const int W = S * T;
-    __syncthreads();
-    if (cap >= 4 * W) {
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int w = threadIdx.x + u * NTG;
-            if (w < W) {
-#pragma unroll
-                for (int m = 0; m < 4; ++m) scr[m * W + w] = acc[u][m];
-            }
+// The block's partial sums of the cross-Gram tiles: thread (tile, slice) adds
+// pixels slice, slice + SL, ..., the slices of a tile (neighbouring lanes) add by
+// a fixed shuffle tree, and lane m writes entry m to part.
+template <int R, bool ITER>
+static __device__ void gd_grams(const float2 *s_u, const float2 *s_a, int rows, float2 *part) {
+    using PL = GdPlan<R>;
+    constexpr int T = ITER ? PL::T_ITER : PL::TH, SL = gd_slices(T), RS = PL::RS;
+    const int tile = threadIdx.x / SL, sl = threadIdx.x % SL;
+    int kind = 2, A = 0, Bt = 0;
+    if (tile < T) {
+        if (!ITER || tile < PL::TH) {
+            kind = ITER ? 0 : 2;
+            pair_of(tile, PL::TR, A, Bt);
+        } else if (tile < PL::TH + PL::TR * PL::TR) {
+            kind = 1;
+            A = (tile - PL::TH) / PL::TR;
+            Bt = (tile - PL::TH) - A * PL::TR;
+        } else {
+            pair_of(tile - PL::TH - PL::TR * PL::TR, PL::TR, A, Bt);
         }
-        __syncthreads();
-        for (int it = threadIdx.x; it < 4 * T; it += NTG) {
-            const int m = it / T, w2 = it - m * T;
-            const int o = out(w2, m);
-            if (o >= 0) {
-                float2 sum = make_float2(0.f, 0.f);
-                for (int ss = 0; ss < S; ++ss) sum = cadd(sum, scr[m * W + ss * T + w2]);
-                part[(size_t)blockIdx.x * ld + o] = sum;
-            }
+    }
+    const float2 *X = kind == 0 ? s_a : s_u, *Y = kind == 2 ? s_u : s_a;
+    float2 acc[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) acc[m] = make_float2(0.f, 0.f);
+    if (tile < T) {
+#pragma unroll 4
+        for (int i = sl; i < rows; i += SL) {
+            float2 p0, p1, q0, q1;
+            gd_pair<R>(X + i * RS, A, p0, p1);
+            gd_pair<R>(Y + i * RS, Bt, q0, q1);
+            cfmac(acc[0], p0, q0);
+            cfmac(acc[1], p0, q1);
+            cfmac(acc[2], p1, q0);
+            cfmac(acc[3], p1, q1);
         }
-        return;
     }
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        __syncthreads();
+    for (int o = SL / 2; o > 0; o >>= 1)
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int w = threadIdx.x + u * NTG;
-            if (w < W) s_red2[w] = acc[u][m];
+        for (int m = 0; m < 4; ++m) acc[m] = cadd(acc[m], shfl_xor2(acc[m], o));
+    if (tile < T) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int x = 2 * A + (m >> 1), y = 2 * Bt + (m & 1);
+            if (sl != m % SL || x >= R || y >= R) continue;
+            if (kind == 1) part[PL::NP + x * R + y] = acc[m];
+            else if (x <= y) part[(kind == 2 && ITER ? PL::NP + R * R : 0) + pair_index(x, y, R)] = acc[m];
+        }
+    }
+}
+
+// R1^{-1} = (L^{-1})^H of the Hermitian positive definite G1 = L L^H in sG (R
+// rows of [G1 | I], 2 R wide): one entry per thread, one barrier per pivot; row
+// c of the right half ends as the unit-diagonal factor's inverse, scaled by
+// 1 / sqrt(pivot c).  False (the same in every thread) when a pivot is not
+// positive.  With the totals' load: one warp with the rows in registers 4.2 us
+// (R = 10) and 9.2 us (R = 12), most of it instruction fetch of the unrolled
+// triangles; this form 2.7 and 3.1 us.
+template <int R>
+static __device__ bool gd_factor(float2 *sG, float2 *sR) {
+    const int e = threadIdx.x, i = e / (2 * R), j = e - i * 2 * R;
+    bool ok = true;
+    for (int c = 0; c < R; ++c) {
+        const float d = sG[c * 2 * R + c].x;
+        ok = ok && d > 0.f;
+        if (i > c && i < R && (j < R ? j > c : j - R <= c)) {
+            const float2 f = cscale(sG[i * 2 * R + c], 1.f / d);
+            sG[e] = csub(sG[e], cmul(f, sG[c * 2 * R + j]));
         }
         __syncthreads();
-        for (int w2 = threadIdx.x; w2 < T; w2 += NTG) {
-            const int o = out(w2, m);
-            if (o >= 0) {
+    }
+    if (e < R * R) {
+        const int a = e / R, b = e - a * R;   // Rinv[a][b] = conj(Linv[b][a])
+        sR[e] = b >= a ? cscale(cconj(sG[b * 2 * R + R + a]), rsqrtf(sG[b * 2 * R + b].x)) : make_float2(0.f, 0.f);
+        if (!ok) sR[e] = make_float2(a == b ? 1.f : 0.f, 0.f);
+    }
+    __syncthreads();
+    return ok;
+}
+
+// Stage Z rows [c0, c0 + zc) of the block's pixels into buffer `buf` (one
+// committed group, empty past the last row).
+static __device__ void gd_stage_z(const GdArgs &a, float2 *s_z, int i0, int rows, int chunk) {
+    const int c0 = chunk * a.zc, cn = min(a.zc, rows - c0);
+    if (cn > 0)
+        stage_rows(s_z + (size_t)(chunk % a.nbuf) * a.zc * a.zs, a.zs, a.Z + (size_t)(i0 + c0) * a.q, a.q, cn, a.q);
+    cp_async_commit();
+}
+
+// Partial sums of h = U_{t+1}^H Z over the block's pixels into hrow[k R + l]:
+// thread (frame pair, LC columns, pixel slice) reads its two Z values by 16
+// bytes and U's row by broadcast; the slices add in order.  Few frames leave
+// many slices, so the columns are split then (LC = 2 instead of R).
+template <int R, int LC>
+static __device__ __noinline__ void gd_h(const GdArgs &a, const float2 *s_a, float2 *s_z, float2 *scr, int cap, int i0, int rows,
+                            float2 *hrow) {
+    constexpr int RS = GdPlan<R>::RS, NC = R / LC;
+    const int t = threadIdx.x, q = a.q, tq = (q + 1) >> 1, items = tq * NC, Sh = NTG / items;
+    const int hs = t / items, item = t - hs * items, cgp = item / tq, kp = item - cgp * tq;
+    const bool act = hs < Sh;
+    float2 pv[2 * LC];
+#pragma unroll
+    for (int v = 0; v < 2 * LC; ++v) pv[v] = make_float2(0.f, 0.f);
+    const int nch = (rows + a.zc - 1) / a.zc;
+    for (int ch = 0; ch < nch; ++ch) {
+        // groups committed so far: nbuf ahead of this chunk
+        if (a.nbuf == 1) cp_async_wait();
+        else cp_async_wait_1();
+        __syncthreads();
+        if (act) {
+            const int c0 = ch * a.zc, cn = min(a.zc, rows - c0);
+            const float2 *z = s_z + (size_t)(ch % a.nbuf) * a.zc * a.zs + 2 * kp, *u = s_a + c0 * RS + cgp * LC;
+#pragma unroll(LC <= 12 ? 2 : 1)
+            for (int ii = hs; ii < cn; ii += Sh) {
+                const float4 zz = *(const float4 *)(z + ii * a.zs);   // Z[k], Z[k+1] (pad column when k+1 = q)
+                const float2 z0 = make_float2(zz.x, zz.y), z1 = make_float2(zz.z, zz.w);
+                if constexpr (LC % 2 == 0 && R % 2 == 0) {
+                    const float4 *u4 = (const float4 *)(u + ii * RS);
+#pragma unroll
+                    for (int l2 = 0; l2 < LC / 2; ++l2) {
+                        const float4 uu = u4[l2];
+                        const float2 ua = make_float2(uu.x, uu.y), ub = make_float2(uu.z, uu.w);
+                        cfmac(pv[2 * l2], ua, z0);
+                        cfmac(pv[LC + 2 * l2], ua, z1);
+                        cfmac(pv[2 * l2 + 1], ub, z0);
+                        cfmac(pv[LC + 2 * l2 + 1], ub, z1);
+                    }
+                } else {
+#pragma unroll
+                    for (int l = 0; l < LC; ++l) {
+                        const float2 uu = u[ii * RS + l];
+                        cfmac(pv[l], uu, z0);
+                        cfmac(pv[LC + l], uu, z1);
+                    }
+                }
+            }
+        }
+        if (ch + a.nbuf < nch) {
+            __syncthreads();   // the chunk's buffer is free
+            gd_stage_z(a, s_z, i0, rows, ch + a.nbuf);
+        } else if (a.nbuf > 1) {
+            cp_async_commit();
+        }
+    }
+    // slices of V values per thread at a time, through the whole dynamic shared memory
+    const int V = max(2, min(2 * LC, cap / NTG));
+    for (int v0 = 0; v0 < 2 * LC; v0 += V) {
+        __syncthreads();
+        if (act) {
+#pragma unroll
+            for (int v = 0; v < 2 * LC; ++v)
+                if (v >= v0 && v < v0 + V) scr[(v - v0) * NTG + t] = pv[v];
+        }
+        __syncthreads();
+        const int vn = min(V, 2 * LC - v0);
+        for (int w = t; w < vn * items; w += NTG) {
+            const int dv = w / items, it = w - dv * items, v = v0 + dv;
+            const int k = 2 * (it % tq) + v / LC, l = (it / tq) * LC + v % LC;
+            if (k < q) {
                 float2 sum = make_float2(0.f, 0.f);
-                for (int ss = 0; ss < S; ++ss) sum = cadd(sum, s_red2[ss * T + w2]);
-                part[(size_t)blockIdx.x * ld + o] = sum;
+#pragma unroll 8
+                for (int ss = 0; ss < Sh; ++ss) sum = cadd(sum, scr[dv * NTG + ss * items + it]);
+                hrow[k * R + l] = sum;
             }
         }
     }
@@ -234,30 +345,33 @@ static __device__ void tiles_write(const float2 (&acc)[2][4], int T, int S, floa
 
 // ---------------------------------------------------------------- the kernel
 
+// Latency bounds it: two grid barriers, short phases between them.  Time from
+// the first block's entry to the last one's exit (graph replay), inputs staged
+// three wide, tile slices added one by one, a one-warp factorisation and Z
+// re-staged when a block's rows did not fit -> this form: 64 x 64, q = 32, r = 4: 15.6 ->
+// 13.3 us; 128 x 128, q = 8, r = 6: 21.4 -> 13.5 us; 192 x 192, q = 48, r = 10: 24.6 -> 21.3 us;
+// 256 x 256, q = 64, r = 12: 55.0 -> 42.4 us.
 template <int R>
 __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
     GD_GT(9);
+    using PL = GdPlan<R>;
+    constexpr int RS = PL::RS, np = PL::NP, rr = R * R;
     extern __shared__ __align__(16) float2 smem[];
-    constexpr int r = R;
-    const int q = a.q, zs = a.zs, chunk = a.chunk;
-    float2 *s_u = smem;                 // chunk * r : U_t (iteration) or U+ (init)
-    float2 *s_a = s_u + chunk * r;      // chunk * r : Gk, grad, then U_{t+1}
-    float2 *s_w = s_a + chunk * r;      // chunk * r : Z B^H, then U - eta grad
-    float2 *s_z = s_w + chunk * r;      // chunk * zs: Z (for h = U_{t+1}^H Z)
-    __shared__ float2 sL[R * R];
+    const int q = a.q;
+    float2 *s_u = smem;                            // per * RS : U_t (iteration) or U+ (init)
+    float2 *s_a = s_u + (size_t)a.per * RS;        // per * RS : grad, then U_{t+1}
+    float2 *s_z = s_a + (size_t)a.per * RS;        // nbuf * zc * zs: Z (for h = U_{t+1}^H Z)
+    __shared__ float2 sG[R * 2 * R];
     __shared__ float2 sR[R * R];
-    __shared__ float sinv[R];
-    __shared__ float2 s_tot[2 * (R * (R + 1) / 2) + R * R];
-    __shared__ float2 s_red2[2 * NTG];
+    __shared__ float2 s_tot[PL::L_ITER];
     __shared__ float s_c[RMAXC], s_s[RMAXC];
     __shared__ float2 s_e[RMAXC];
     __shared__ int s_cnt, s_flag;
     __shared__ float s_eta;
     const int t = threadIdx.x, G = gridDim.x;
-    const int np = r * (r + 1) / 2, rr = r * r, tr = (r + 1) >> 1;
-    const int per = (a.n + G - 1) / G;
-    const int i0 = min(a.n, (int)blockIdx.x * per), i1 = min(a.n, i0 + per);
+    const int i0 = min(a.n, (int)blockIdx.x * a.per), i1 = min(a.n, i0 + a.per), rows = i1 - i0;
     const bool iter = a.mode == 1;
+    const int len1 = iter ? PL::L_ITER : np;
     // eta as it stands at launch; block 0 updates the device copy only after
     // every block has passed the first barrier (so after every block read it)
     const double eta_in = a.scal[SC_ETA];
@@ -265,90 +379,41 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
     const double tcnt = eta_set ? a.scal[SC_TCNT] : 0.0;   // iterations since eta was set
 
     // ------------------------------------------------ phase 1: gradient and Gram partial sums
-    // tiles: [grad^H grad (upper tiles) | U^H grad (all) | U^H U (upper tiles)], init: [U+^H U+]
-    const int th = tr * (tr + 1) / 2;
-    const int T1 = iter ? 2 * th + tr * tr : th;
-    const int len1 = iter ? 2 * np + rr : np;
-    const int S1 = max(1, NTG / T1);
-    auto tile1 = [&](int w, int &kind, int &A, int &Bt) {
-        if (!iter) {
-            kind = 2;
-            pair_of(w, tr, A, Bt);
-        } else if (w < th) {
-            kind = 0;
-            pair_of(w, tr, A, Bt);
-        } else if (w < th + tr * tr) {
-            kind = 1;
-            A = (w - th) / tr;
-            Bt = (w - th) - A * tr;
-        } else {
-            kind = 2;
-            pair_of(w - th - tr * tr, tr, A, Bt);
-        }
-    };
-    Tile g1[2];
-    int sl1[2];
-    float2 acc[2][4];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const int w = t + u * NTG;
-        sl1[u] = w < S1 * T1 ? w / T1 : S1;   // S1 marks an idle item
-        int kind = 0, A = 0, Bt = 0;
-        if (w < S1 * T1) tile1(w % T1, kind, A, Bt);
-        g1[u].X = kind == 0 ? s_a : s_u;
-        g1[u].Y = kind == 2 ? s_u : s_a;
-        g1[u].xs = g1[u].ys = r;
-        g1[u].x0 = 2 * A;
-        g1[u].x1 = min(2 * A + 1, r - 1);
-        g1[u].y0 = 2 * Bt;
-        g1[u].y1 = min(2 * Bt + 1, r - 1);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) acc[u][m] = make_float2(0.f, 0.f);
-    }
     GD_TS(0);
-    for (int c0 = i0; c0 < i1; c0 += chunk) {
-        const int cn = min(chunk, i1 - c0);
-        __syncthreads();
-        if (iter) {
-            stage_rows(s_a, r, a.Gk + (size_t)c0 * r, r, cn, r);
-            stage_rows(s_u, r, a.U + (size_t)c0 * r, r, cn, r);
-            stage_rows(s_w, r, a.ZB + (size_t)c0 * r, r, cn, r);
-        } else {
-            stage_rows(s_u, r, a.Up + (size_t)c0 * r, r, cn, r);
-        }
-        cp_async_commit();
-        if (a.resident) {   // Z for phase 2 streams in behind phase 1
-            stage_rows(s_z, zs, a.Z + (size_t)c0 * q, q, cn, q);
-            cp_async_commit();
-            cp_async_wait_1();
-        } else {
-            cp_async_wait();
-        }
-        __syncthreads();
-        if (c0 == i0) GD_TS(1);
-        if (iter) {   // grad = Gk - Z B^H
-            for (int e = t; e < cn * r; e += NTG) {
-                const float2 g = csub(s_a[e], s_w[e]);
-                s_a[e] = g;
-                a.Gr[(size_t)c0 * r + e] = g;
+    stage_rows(s_u, RS, (iter ? a.U : a.Up) + (size_t)i0 * R, R, rows, R);
+    cp_async_commit();
+    for (int b = 0; b < a.nbuf; ++b) gd_stage_z(a, s_z, i0, rows, b);   // streams in behind phase 1
+    if (iter) {   // grad = Gk - Z B^H
+        const float2 *gk = a.Gk + (size_t)i0 * R, *zb = a.ZB + (size_t)i0 * R;
+        float2 *gr = a.Gr + (size_t)i0 * R;
+        if constexpr (R % 2 == 0) {
+            constexpr int H = R / 2;
+#pragma unroll 4
+            for (int e = t; e < rows * H; e += NTG) {
+                const float4 x = __ldg((const float4 *)gk + e), y = __ldg((const float4 *)zb + e);
+                const float4 g = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
+                ((float4 *)gr)[e] = g;
+                const int ii = e / H;
+                *(float4 *)(s_a + ii * RS + 2 * (e - ii * H)) = g;
             }
-            __syncthreads();
+        } else {
+#pragma unroll 4
+            for (int e = t; e < rows * R; e += NTG) {
+                const float2 g = csub(__ldg(gk + e), __ldg(zb + e));
+                gr[e] = g;
+                const int ii = e / R;
+                s_a[ii * RS + (e - ii * R)] = g;
+            }
         }
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-            if (sl1[u] < S1) tile_accumulate(g1[u], acc[u], sl1[u], S1, cn);
     }
-    GD_TS(2);
+    if (a.nbuf == 1) cp_async_wait_1();
+    else cp_async_wait_2();
+    __syncthreads();
+    GD_TS(1);
     // partial row: [grad^H grad pairs (np) | U^H grad (rr) | U^H U pairs (np)], init: [U+^H U+ pairs]
-    tiles_write(acc, T1, S1, s_w, chunk * r, s_red2, a.part, len1, [&](int w, int m) {
-        int kind, A, Bt;
-        tile1(w, kind, A, Bt);
-        const int x = 2 * A + (m >> 1), y = 2 * Bt + (m & 1);
-        if (x >= r || y >= r) return -1;
-        if (kind == 1) return np + x * r + y;
-        if (x > y) return -1;
-        return (kind == 2 && iter ? np + rr : 0) + pair_index(x, y, r);
-    });
+    if (iter) gd_grams<R, true>(s_u, s_a, rows, a.part + (size_t)blockIdx.x * len1);
+    else gd_grams<R, false>(s_u, s_a, rows, a.part + (size_t)blockIdx.x * len1);
+    GD_TS(2);
     GD_TS(3);
     grid_sync(a.bar, 1, a.status, a.spin_limit, a.bar_skew, ST_TIMEOUT);
     GD_TS(4);
@@ -370,15 +435,15 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
             // ||grad||_2^2 = lambda_max(grad^H grad) (Alg. 2, t = 1), FP32 Jacobi
             for (int p = t; p < np; p += NTG) {
                 int x, y;
-                pair_of(p, r, x, y);
-                sR[x * r + y] = A1[p];
-                sR[y * r + x] = cconj(A1[p]);
+                pair_of(p, R, x, y);
+                sR[x * R + y] = A1[p];
+                sR[y * R + x] = cconj(A1[p]);
             }
             __syncthreads();
-            block_jacobi(sR, r, r, nullptr, 0, s_c, s_s, s_e, &s_cnt, 30);
+            block_jacobi(sR, R, R, nullptr, 0, s_c, s_s, s_e, &s_cnt, 30);
             if (t == 0) {
                 float lmax = 0.f;
-                for (int x = 0; x < r; ++x) lmax = fmaxf(lmax, sR[x * r + x].x);
+                for (int x = 0; x < R; ++x) lmax = fmaxf(lmax, sR[x * R + x].x);
                 const double gn = sqrt((double)lmax);
                 const double eta = gn > 0.0 ? a.eta_c / gn : 0.0;
                 s_eta = (float)eta;
@@ -398,133 +463,66 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
         }
         __syncthreads();
         const float eta = s_eta, eta2 = s_eta * s_eta;
-        for (int e = t; e < rr; e += NTG) {
-            const int x = e / r, y = e - x * r;
-            const int p = x <= y ? pair_index(x, y, r) : pair_index(y, x, r);
+        if (t < rr) {
+            const int x = t / R, y = t - x * R;
+            const int p = x <= y ? pair_index(x, y, R) : pair_index(y, x, R);
             const float sg = x <= y ? 1.f : -1.f;   // lower half: conjugate of the stored pair
-            const float x2r = A2[x * r + y].x + A2[y * r + x].x;
-            const float x2i = A2[x * r + y].y - A2[y * r + x].y;
-            sL[e] = make_float2(A3[p].x - eta * x2r + eta2 * A1[p].x, sg * A3[p].y - eta * x2i + eta2 * sg * A1[p].y);
+            const float x2r = A2[x * R + y].x + A2[y * R + x].x;
+            const float x2i = A2[x * R + y].y - A2[y * R + x].y;
+            sG[x * 2 * R + y] =
+                make_float2(A3[p].x - eta * x2r + eta2 * A1[p].x, sg * A3[p].y - eta * x2i + eta2 * sg * A1[p].y);
+            sG[x * 2 * R + R + y] = make_float2(x == y ? 1.f : 0.f, 0.f);
         }
-    } else {
-        for (int e = t; e < rr; e += NTG) {
-            const int x = e / r, y = e - x * r;
-            const int p = x <= y ? pair_index(x, y, r) : pair_index(y, x, r);
-            sL[e] = x <= y ? s_tot[p] : cconj(s_tot[p]);
-        }
+    } else if (t < rr) {
+        const int x = t / R, y = t - x * R;
+        const int p = x <= y ? pair_index(x, y, R) : pair_index(y, x, R);
+        sG[x * 2 * R + y] = x <= y ? s_tot[p] : cconj(s_tot[p]);
+        sG[x * 2 * R + R + y] = make_float2(x == y ? 1.f : 0.f, 0.f);
     }
     __syncthreads();
-    // G1 = L L^H and R1^{-1} = (L^H)^{-1} by the first warp in registers (the
-    // other warps wait at the barrier below)
-    if (t < 32) {
-        if (!warp_chol32<R>(sL, R, sinv)) {
-            if (t == 0 && blockIdx.x == 0) atomicOr(a.status, (unsigned)ST_NOT_SPD_QR);
-            for (int e = t; e < rr; e += 32) sL[e] = make_float2(e / r == e % r ? 1.f : 0.f, 0.f);
-            if (t < r) sinv[t] = 1.f;
-            __syncwarp();
-        }
-        warp_rinv<R>(sL, sinv, sR);
-    }
-    __syncthreads();
+    if (!gd_factor<R>(sG, sR) && t == 0 && blockIdx.x == 0) atomicOr(a.status, (unsigned)ST_NOT_SPD_QR);
     GD_TS(7);
     const float etaf = iter ? s_eta : 0.f;
 
     // ------------------------------------------------ phase 2: U_{t+1} = (U - eta grad) R1^{-1}
-    // and the partial sums of h = U_{t+1}^H Z over the block's pixels, thread
-    // (frame pair kp, slice hs) holding all R columns for frames 2 kp, 2 kp + 1
-    const int tq = (q + 1) >> 1;
-    const int Sh = max(1, NTG / tq), Hth = tq * Sh;
-    const bool hthr = t < Hth;
-    const int hk = 2 * (t % tq), hs = t / tq;
-    float2 pv[2 * R];
+    // a thread per pixel row, in place over the gradient: column l needs the
+    // columns up to l only, so they are formed from the last one down
+    for (int i = t; i < rows; i += NTG) {
+        asm volatile("" ::: "memory");   // one turn as a rule: keep R1^{-1} in shared memory
+        float2 w[R];
 #pragma unroll
-    for (int v = 0; v < 2 * R; ++v) pv[v] = make_float2(0.f, 0.f);
-    for (int c0 = i0; c0 < i1; c0 += chunk) {
-        const int cn = min(chunk, i1 - c0);
-        if (!a.resident) {
-            __syncthreads();
-            if (iter) {
-                stage_rows(s_u, r, a.U + (size_t)c0 * r, r, cn, r);
-                stage_rows(s_a, r, a.Gr + (size_t)c0 * r, r, cn, r);
-            } else {
-                stage_rows(s_u, r, a.Up + (size_t)c0 * r, r, cn, r);
-            }
-            stage_rows(s_z, zs, a.Z + (size_t)c0 * q, q, cn, q);
-            cp_async_commit();
+        for (int m = 0; m < R; ++m) {
+            w[m] = s_u[i * RS + m];
+            if (iter) w[m] = csub(w[m], cscale(s_a[i * RS + m], etaf));
         }
-        cp_async_wait();
-        __syncthreads();
-        for (int e = t; e < cn * r; e += NTG) s_w[e] = iter ? csub(s_u[e], cscale(s_a[e], etaf)) : s_u[e];
-        __syncthreads();
-        for (int e = t; e < cn * r; e += NTG) {
-            const int ii = e / r, l = e - ii * r;
+#pragma unroll
+        for (int l = R - 1; l >= 0; --l) {
             float2 v = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int m = 0; m < R; ++m)
-                if (m <= l) cfma(v, s_w[ii * r + m], sR[m * r + l]);
-            s_a[e] = v;
-            a.U[(size_t)c0 * r + e] = v;
-            if (iter) a.Uprev[(size_t)c0 * r + e] = s_u[e];
+            for (int m = 0; m <= l; ++m) cfma(v, w[m], sR[m * R + l]);
+            w[l] = v;
         }
-        __syncthreads();
-        if (hthr) {
-#pragma unroll(R <= 12 ? 2 : 1)
-            for (int ii = hs; ii < cn; ii += Sh) {
-                const float4 z = *(const float4 *)(s_z + ii * zs + hk);   // Z[k], Z[k+1] (pad column when k+1 = q)
-                const float2 z0 = make_float2(z.x, z.y), z1 = make_float2(z.z, z.w);
-                if constexpr ((R & 1) == 0) {   // U_{t+1} row in 16-byte pairs (r even: rows 16-byte aligned)
-                    const float4 *u4 = (const float4 *)(s_a + ii * r);
 #pragma unroll
-                    for (int l2 = 0; l2 < R / 2; ++l2) {
-                        const float4 uu = u4[l2];
-                        const float2 ua = make_float2(uu.x, uu.y), ub = make_float2(uu.z, uu.w);
-                        cfmac(pv[2 * l2], ua, z0);
-                        cfmac(pv[R + 2 * l2], ua, z1);
-                        cfmac(pv[2 * l2 + 1], ub, z0);
-                        cfmac(pv[R + 2 * l2 + 1], ub, z1);
-                    }
-                } else {
-#pragma unroll
-                    for (int l = 0; l < R; ++l) {
-                        const float2 u = s_a[ii * r + l];
-                        cfmac(pv[l], u, z0);
-                        cfmac(pv[R + l], u, z1);
-                    }
-                }
-            }
-        }
+        for (int m = 0; m < R; ++m) s_a[i * RS + m] = w[m];
     }
-    // the block's row of h partial sums, hpart[b][k r + l], slices added in
-    // order, V values per thread per round (s_w and s_z are free now)
+    __syncthreads();
+    for (int e = t; e < rows * R; e += NTG) {
+        const int ii = e / R, l = e - ii * R;
+        a.U[(size_t)i0 * R + e] = s_a[ii * RS + l];
+        if (iter) a.Uprev[(size_t)i0 * R + e] = s_u[ii * RS + l];
+    }
+    // the block's row of h partial sums, hpart[b][k R + l]
     {
-        const int cap2 = chunk * (r + zs);
-        float2 *scr = cap2 >= 2 * NTG ? s_w : s_red2;
-        const int V = max(2, min(2 * R, ((cap2 >= 2 * NTG ? cap2 : 2 * NTG) / NTG) & ~1));
-        float2 *hrow = a.hpart + (size_t)blockIdx.x * q * r;
-        for (int v0 = 0; v0 < 2 * R; v0 += V) {
-            __syncthreads();
-            if (hthr) {
-#pragma unroll
-                for (int v = 0; v < 2 * R; ++v)
-                    if (v >= v0 && v < v0 + V) scr[(v - v0) * NTG + t] = pv[v];
-            }
-            __syncthreads();
-            const int vn = min(V, 2 * R - v0);
-            for (int w = t; w < vn * tq; w += NTG) {
-                const int dv = w / tq, kp = w - dv * tq, v = v0 + dv;
-                const int k = 2 * kp + v / R, l = v % R;
-                if (k < q) {
-                    float2 sum = make_float2(0.f, 0.f);
-                    for (int ss = 0; ss < Sh; ++ss) sum = cadd(sum, scr[dv * NTG + ss * tq + kp]);
-                    hrow[k * r + l] = sum;
-                }
-            }
-        }
+        float2 *hrow = a.hpart + (size_t)blockIdx.x * q * R;
+        const int cap = max(2 * NTG, 2 * a.per * RS + a.nbuf * a.zc * a.zs);   // as launched
+        constexpr int LS = R % 2 == 0 ? 2 : 1;
+        if (NTG / ((q + 1) >> 1) > 64) gd_h<R, LS>(a, s_a, s_z, smem, cap, i0, rows, hrow);
+        else gd_h<R, R>(a, s_a, s_z, smem, cap, i0, rows, hrow);
     }
     GD_TS(8);
     // the last block out: SD(U_t, U_{t+1})^2 = r - ||U_t^H U_{t+1}||_F^2 with
     // U_t^H U_{t+1} = (U_t^H U_t - eta U_t^H grad) R1^{-1} from the totals (no
-    // second reduction; thread x r + y forms entry (x, y)), and the barrier
+    // second reduction; thread x R + y forms entry (x, y)), and the barrier
     // counters back to zero (every block is past its last barrier)
     __syncthreads();
     if (t == 0) {
@@ -540,13 +538,13 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
     double sq = 0.0;
     if (iter && t < rr) {
         const float2 *A2 = s_tot + np, *A3 = s_tot + np + rr;
-        const int x = t / r, y = t - x * r;
+        const int x = t / R, y = t - x * R;
         float2 mv = make_float2(0.f, 0.f);
 #pragma unroll
         for (int m = 0; m < R; ++m) {
             if (m <= y) {
-                const float2 uu = x <= m ? A3[pair_index(x, m, r)] : cconj(A3[pair_index(m, x, r)]);
-                cfma(mv, csub(uu, cscale(A2[x * r + m], etaf)), sR[m * r + y]);
+                const float2 uu = x <= m ? A3[pair_index(x, m, R)] : cconj(A3[pair_index(m, x, R)]);
+                cfma(mv, csub(uu, cscale(A2[x * R + m], etaf)), sR[m * R + y]);
             }
         }
         sq = (double)mv.x * mv.x + (double)mv.y * mv.y;
@@ -561,7 +559,7 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
         sum = warp_sum_d(sum);
         if (t == 0) {
             if (iter) {
-                const double sd2 = (double)r - sum;
+                const double sd2 = (double)R - sum;
                 a.scal[SC_SD] = sqrt(sd2 > 0.0 ? sd2 : 0.0);
             }
             a.bar[0] = 0u;
@@ -643,13 +641,13 @@ cudaError_t launch_gdqr(lrccs_ctx *c, int mode) {
     const int r = c->r, q = c->q, G = c->gd_grid;
     if (r < 1 || r > RMAXC) return cudaErrorInvalidValue;
     const int zs = z_stride(q);
-    const int per = (c->n + G - 1) / G;
-    const size_t bpp = (size_t)(3 * r + zs) * sizeof(float2);
+    const int per = (c->n + G - 1) / G, rs = r % 4 == 0 ? r + 2 : r;
+    const size_t fixed = (size_t)2 * per * rs * sizeof(float2);
     const size_t avail = (size_t)(c->dev_smem_optin - g_gd_static_smem[r - 1]);
-    int chunk = (int)(avail / bpp) & ~1;
-    chunk = min(chunk, 512);
-    chunk = min(chunk, (per + 1) & ~1);
-    if (chunk < 2) return cudaErrorInvalidConfiguration;
+    if (fixed + 4 * zs * sizeof(float2) > avail) return cudaErrorInvalidConfiguration;
+    // Z in one piece, or through two buffers of as many rows as fit
+    const int rows = (int)((avail - fixed) / (zs * sizeof(float2)));
+    const int nbuf = rows >= per ? 1 : 2, zc = nbuf == 1 ? per : rows / 2;
     GdArgs a;
     a.Gk = c->d_Up;
     a.ZB = c->d_ZB;
@@ -665,11 +663,11 @@ cudaError_t launch_gdqr(lrccs_ctx *c, int mode) {
     a.bar = c->d_counters + CNT_BAR;
     a.status = c->d_status;
     a.n = c->n;
-    a.r = r;
     a.q = q;
+    a.per = per;
     a.zs = zs;
-    a.chunk = chunk;
-    a.resident = chunk >= per ? 1 : 0;
+    a.zc = zc;
+    a.nbuf = nbuf;
     a.mode = mode;
     a.eta_c = c->prm.eta_c;
     a.eta_scale0 = c->prm.eta_scale0 > 0.0 ? c->prm.eta_scale0 : 1.0;
@@ -683,7 +681,8 @@ cudaError_t launch_gdqr(lrccs_ctx *c, int mode) {
         c->test_timeout = 0;
     }
     void *args[] = {&a};
-    const size_t smem = (size_t)chunk * bpp;
+    // the h slices go through all of it, two values per thread at least
+    const size_t smem = std::max(fixed + (size_t)nbuf * zc * zs * sizeof(float2), (size_t)2 * NTG * sizeof(float2));
     prof_begin(c, KID_GDQR);
     cudaError_t e = cudaLaunchCooperativeKernel((const void *)kGd[r - 1], dim3(G), dim3(NTG), args, smem, c->stream);
     prof_end(c, KID_GDQR);
