@@ -458,19 +458,23 @@ LRCCS_DEV void block_sum(int nent, int nitem, double *dst, F fetch) {
             }
             continue;
         }
+        // the slices add by a fixed tree (a thread per entry adding them one by
+        // one waits for shared memory S times)
         if (act) s_acc[t] = make_float4(re.hi, re.lo, im.hi, im.lo);
-        __syncthreads();
-        if (t < nent) {
-            fsum2 R = {0.f, 0.f}, I = {0.f, 0.f};
-            for (int ss = 0; ss < S; ++ss) {
-                const float4 a = s_acc[ss * nent + t];
-                fsum_add(R, a.x);
-                R.lo += a.y;
-                fsum_add(I, a.z);
-                I.lo += a.w;
+        int h = 1;
+        while (2 * h < S) h <<= 1;
+        for (; h > 0; h >>= 1) {
+            __syncthreads();
+            if (act && e < nent && s < h && s + h < S) {
+                const float4 b = s_acc[t + h * nent];
+                re = fsum_pair(re, fsum2{b.x, b.y});
+                im = fsum_pair(im, fsum2{b.z, b.w});
+                s_acc[t] = make_float4(re.hi, re.lo, im.hi, im.lo);
             }
-            dst[2 * t] = (double)R.hi + (double)R.lo;
-            dst[2 * t + 1] = (double)I.hi + (double)I.lo;
+        }
+        if (act && s == 0 && e < nent) {
+            dst[2 * e] = (double)re.hi + (double)re.lo;
+            dst[2 * e + 1] = (double)im.hi + (double)im.lo;
         }
     }
     __syncthreads();

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(NT) k_solve(const float2 *__restrict__ Prow, c
 // and solves.  Gather latency bounds it, so nch = gen_chunks(q) makes about
 // eight blocks per multiprocessor whatever q is, between 8 and 64 chunks; with
 // 8 chunks for every q: 31 us (64 frames of 256 x 256, r = 12) and 31 us now, 49 us
-// (8 frames of 224 x 224, r = 13: 64 blocks) -> 18 us, k_solve_gen 7 -> 12 us.
+// (8 frames of 224 x 224, r = 13: 64 blocks) -> 11 us, k_solve_gen 7 -> 12 us.
 static int gen_chunks(int q) { return std::max(8, std::min(64, (8 * 152 + q - 1) / q)); }
 template <int R>
 __global__ void __launch_bounds__(NT) k_frame_gram_gen(const float2 *__restrict__ Pu, const int32_t *__restrict__ fpk,
@@ -413,6 +413,7 @@ struct BstepArgs {
     unsigned int *bar;            // [0] barrier arrivals, [1] exit count
     unsigned int *status;
     int ny, nx, nc, q, P, n;      // P: partial rows of h
+    int area;                     // complex values of the row buffer (and Z staging area)
     unsigned int spin_limit;      // polls before a grid barrier gives up
     long long *ts;                // NULL, or BS_NTS global-timer stamps (ns) per block b < ts_blocks
     int ts_blocks;
@@ -440,7 +441,7 @@ __global__ void __launch_bounds__(BS_NT, 1) k_bstep(const __grid_constant__ Bste
     extern __shared__ __align__(128) float2 bs_smem[];
     // 128-byte aligned start (bulk-copy destination); the launch adds 128 bytes of slack
     float2 *row = (float2 *)(((uintptr_t)bs_smem + 127) & ~(uintptr_t)127);   // nc nx R: T_j[ky] of every coil
-    float2 *sB = row + (size_t)a.nc * a.nx * R;             // q R
+    float2 *sB = row + a.area;                              // q R
     __shared__ __align__(8) uint64_t s_mbar[BS_MAXC];
     __shared__ float s_part[(BS_NT / 32) * 64];
     __shared__ double sP[2 * np];
@@ -609,7 +610,7 @@ __global__ void __launch_bounds__(BS_NT, 1) k_bstep(const __grid_constant__ Bste
     {
         const int per = (a.n + G - 1) / G, i0 = blockIdx.x * per, i1 = min(a.n, i0 + per);
         const int qs = bs_zstride(q);                // staged row stride
-        const int cap = (nc * nx * R) / qs;          // pixels per chunk
+        const int cap = a.area / qs;                 // pixels per chunk
         float2 *zs = row;
         for (int c0 = i0; c0 < i1; c0 += cap) {
             const int c1 = min(i1, c0 + cap), np_ = c1 - c0, cnt = np_ * q;
@@ -694,8 +695,16 @@ __global__ void __launch_bounds__(BS_NT, 1) k_bstep(const __grid_constant__ Bste
 typedef void (*bstep_kernel_t)(const BstepArgs);
 static const bstep_kernel_t kBstep[RMAXC] = RANK_TABLE(k_bstep);
 
+// The row buffer also stages Z for Z B^H.  A short row (few coils) would cut the
+// block's pixels into many small chunks, each with its own copy latency (64 x 64,
+// C = 1, r = 4: ten chunks of 7 pixels, 15.3 of 27.8 us; now 1.1 of 12.7), so the area holds 128
+// pixels of Z at least, up to 72 KB (two blocks a multiprocessor).
+static int bstep_area(int nc, int nx, int q, int r) {
+    const int z = std::min(128, (int)(73728 / (bs_zstride(q) * sizeof(float2)))) * bs_zstride(q);
+    return std::max(nc * nx * r, (z + 1) & ~1);
+}
 static size_t bstep_smem(int nc, int nx, int q, int r) {
-    return ((size_t)nc * nx * r + (size_t)q * r) * sizeof(float2) + 128;
+    return ((size_t)bstep_area(nc, nx, q, r) + (size_t)q * r) * sizeof(float2) + 128;
 }
 
 cudaError_t configure_kernels_solve(int max_smem) {
@@ -714,7 +723,6 @@ cudaError_t configure_kernels_solve(int max_smem) {
 // sampled row does not fit a block's shared memory, or too many coils).
 int bstep_capacity(int nc, int nx, int q, int r, int smem_optin, int nsm) {
     if (r < 1 || r > RMAXC || nc < 1 || nc > BS_MAXC || q < 1 || q > 128 || ((size_t)nx * r) % 2 != 0) return 0;
-    if ((size_t)nc * nx * r < (size_t)bs_zstride(q)) return 0;   // Z B^H stages whole Z rows in the row buffer
     const size_t smem = bstep_smem(nc, nx, q, r);
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kBstep[r - 1]) != cudaSuccess) {
@@ -762,6 +770,7 @@ cudaError_t launch_bstep_fused(lrccs_ctx *c) {
     a.nx = c->nx;
     a.nc = c->nc;
     a.q = c->q;
+    a.area = bstep_area(c->nc, c->nx, c->q, r);
     a.P = c->gd_grid;
     a.spin_limit = 1u << 24;
     // phase stamps after k_gdqr's in the phase-timing buffer (lrccs_gdqr_phases on)
