@@ -124,101 +124,139 @@ LRCCS_DEV bool last_block_arrive(unsigned int *counter) {
 // such indices only mixes columns p and q of V: when every wanted eigenvalue
 // is above tail_tol, the wanted eigenvectors converge without them);
 // the sweeps stop when a whole sweep skips every rotation.
-__device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ldv, float *s_c, float *s_s, float2 *s_e,
-                             int *s_cnt, int max_sweeps, float abs_tol = 0.f, float rel_tol = 1e-7f,
-                             float tail_tol = 0.f) {
-    const int n2 = n + (n & 1);
-    const int npair = n2 / 2;
-    int sh = 0;                             // column index stride 2^sh >= n (no division per task)
-    while ((1 << sh) < n) ++sh;
-    const int mmask = (1 << sh) - 1;
-    int psh = 0;                            // pair index stride 2^psh >= npair
-    while ((1 << psh) < npair) ++psh;
-    const int pmask = (1 << psh) - 1;
-    __shared__ short s_pp[64], s_qq[64];   // the pairs of the current round
+//
+// A round is two phases with a barrier each: the 2 x 2 blocks of A on and above
+// the diagonal (the rest is their mirror image), then the first warp forms the
+// next round's rotations while the others update V with this round's.
+struct JacobiRot {
+    float c[64], s[64];
+    float2 e[64];
+    short p[64], q[64];
+};
+
+// The rotations of round rnd (one warp); returns whether any is not skipped.
+LRCCS_DEV bool jacobi_rotations(const float2 *A, int n, int lda, int rnd, JacobiRot &r, float abs_tol, float rel_tol,
+                                float tail_tol) {
+    const int n2 = n + (n & 1), npair = n2 / 2;
+    bool any = false;
+    for (int i = threadIdx.x & 31; i < npair; i += 32) {
+        int p, qq;
+        if (i == 0) { p = rnd; qq = n2 - 1; }
+        else { p = (rnd + i) % (n2 - 1); qq = (rnd - i + n2 - 1) % (n2 - 1); }
+        float c = 1.f, s = 0.f;
+        float2 e = make_float2(1.f, 0.f);
+        if (p < n && qq < n) {
+            const float2 apq = A[p * lda + qq];
+            const float b2 = apq.x * apq.x + apq.y * apq.y;
+            const float al = A[p * lda + p].x, ga = A[qq * lda + qq].x;
+            if (b2 > 1e-36f && b2 > abs_tol * abs_tol && b2 > rel_tol * rel_tol * fabsf(al) * fabsf(ga) &&
+                (fabsf(al) >= tail_tol || fabsf(ga) >= tail_tol)) {
+                // the rotation only has to be orthogonal: c = 1 / sqrt(1 + t^2),
+                // s = t c hold to rounding whatever the accuracy of t (c rounded
+                // to nearest: rsqrtf's bias took 1e-5 off V's column norms over
+                // 47 x 5 rotations, and off the singular values)
+                const float ib = rsqrtf(b2);
+                e = make_float2(apq.x * ib, apq.y * ib);
+                const float tau = (ga - al) * 0.5f * ib;
+                const float t = copysignf(1.f, tau) * __frcp_rn(fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f)));
+                c = __frsqrt_rn(fmaf(t, t, 1.f));
+                s = t * c;
+                any = true;
+            }
+        }
+        r.c[i] = c;
+        r.s[i] = s;
+        r.e[i] = e;
+        r.p[i] = (short)p;
+        r.q[i] = (short)qq;
+    }
+    return __any_sync(0xffffffffu, any);
+}
+
+__device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ldv, JacobiRot (&rot)[2], int (&cnt)[2],
+                                    int max_sweeps, float abs_tol = 0.f, float rel_tol = 1e-7f, float tail_tol = 0.f) {
+    const int n2 = n + (n & 1), npair = n2 / 2, nblk = npair * (npair + 1) / 2;
+    const int warp = threadIdx.x >> 5;
+    const unsigned inv_n = ((1u << 20) + n - 1) / n;   // tv / n for tv < 64 n
+    __syncthreads();
+    if (warp == 0) {
+        const bool any = jacobi_rotations(A, n, lda, 0, rot[0], abs_tol, rel_tol, tail_tol);
+        if (threadIdx.x == 0) {
+            cnt[0] = any;
+            cnt[1] = 0;
+        }
+    }
+    __syncthreads();
+    int b = 0;
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        if (threadIdx.x == 0) *s_cnt = 0;
-        __syncthreads();
-        for (int rnd = 0; rnd < n2 - 1; ++rnd) {
-            for (int i = threadIdx.x; i < npair; i += blockDim.x) {
-                int p, qq;
-                if (i == 0) { p = rnd; qq = n2 - 1; }
-                else { p = (rnd + i) % (n2 - 1); qq = (rnd - i + n2 - 1) % (n2 - 1); }
-                s_pp[i] = (short)p;
-                s_qq[i] = (short)qq;
-                float c = 1.f, s = 0.f;
-                float2 e = make_float2(1.f, 0.f);
-                if (p < n && qq < n) {
-                    const float2 apq = A[p * lda + qq];
-                    const float b2 = apq.x * apq.x + apq.y * apq.y;
-                    const float al = A[p * lda + p].x, ga = A[qq * lda + qq].x;
-                    if (b2 > 1e-36f && b2 > abs_tol * abs_tol && b2 > rel_tol * rel_tol * fabsf(al) * fabsf(ga) &&
-                        (fabsf(al) >= tail_tol || fabsf(ga) >= tail_tol)) {
-                        // the rotation only has to be orthogonal: c = 1 / sqrt(1 + t^2),
-                        // s = t c hold to rounding whatever the accuracy of t
-                        const float ib = rsqrtf(b2);
-                        e = make_float2(apq.x * ib, apq.y * ib);
-                        const float tau = (ga - al) * 0.5f * ib;
-                        const float t = copysignf(1.f, tau) * __frcp_rn(fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f)));
-                        c = rsqrtf(fmaf(t, t, 1.f));
-                        s = t * c;
-                        *s_cnt = 1;
-                    }
+        for (int rnd = 0; rnd < n2 - 1; ++rnd, b ^= 1) {
+            const JacobiRot &r = rot[b];
+            // A <- G^H A G on the block (rows of pair i, columns of pair i2 >= i):
+            // the row rotation first, then the column rotation
+            for (int task = threadIdx.x; task < nblk; task += blockDim.x) {
+                // task -> (i, i2): row i of the triangle starts at i npair - i (i - 1) / 2
+                int i = (int)(((float)(2 * npair + 1) -
+                               sqrtf((float)((2 * npair + 1) * (2 * npair + 1) - 8 * task))) * 0.5f);
+                while (i > 0 && i * npair - i * (i - 1) / 2 > task) --i;
+                while ((i + 1) * npair - (i + 1) * i / 2 <= task) ++i;
+                const int i2 = i + task - (i * npair - i * (i - 1) / 2);
+                const float si = r.s[i], si2 = r.s[i2];
+                if (si == 0.f && si2 == 0.f) continue;
+                const int p = r.p[i], qq = r.q[i], p2 = r.p[i2], q2 = r.q[i2];
+                const bool r0 = p < n, r1 = qq < n, c0 = p2 < n, c1 = q2 < n;
+                const float2 z = make_float2(0.f, 0.f);
+                float2 a00 = r0 && c0 ? A[p * lda + p2] : z, a01 = r0 && c1 ? A[p * lda + q2] : z;
+                float2 a10 = r1 && c0 ? A[qq * lda + p2] : z, a11 = r1 && c1 ? A[qq * lda + q2] : z;
+                if (si != 0.f) {   // rows p, q of columns p2, q2
+                    const float c = r.c[i];
+                    const float2 e = r.e[i];
+                    float2 eaq = cmul(e, a10);
+                    float2 ap = a00;
+                    a00 = make_float2(c * ap.x - si * eaq.x, c * ap.y - si * eaq.y);
+                    a10 = make_float2(si * ap.x + c * eaq.x, si * ap.y + c * eaq.y);
+                    eaq = cmul(e, a11);
+                    ap = a01;
+                    a01 = make_float2(c * ap.x - si * eaq.x, c * ap.y - si * eaq.y);
+                    a11 = make_float2(si * ap.x + c * eaq.x, si * ap.y + c * eaq.y);
                 }
-                s_c[i] = c;
-                s_s[i] = s;
-                s_e[i] = e;
+                if (si2 != 0.f) {   // columns p2, q2 of rows p, q
+                    const float c = r.c[i2];
+                    const float2 eh = cconj(r.e[i2]);
+                    float2 e2 = cmul(eh, a01);
+                    float2 ap = a00;
+                    a00 = make_float2(c * ap.x - si2 * e2.x, c * ap.y - si2 * e2.y);
+                    a01 = make_float2(si2 * ap.x + c * e2.x, si2 * ap.y + c * e2.y);
+                    e2 = cmul(eh, a11);
+                    ap = a10;
+                    a10 = make_float2(c * ap.x - si2 * e2.x, c * ap.y - si2 * e2.y);
+                    a11 = make_float2(si2 * ap.x + c * e2.x, si2 * ap.y + c * e2.y);
+                }
+                if (r0 && c0) A[p * lda + p2] = a00;
+                if (r0 && c1) A[p * lda + q2] = a01;
+                if (r1 && c0) A[qq * lda + p2] = a10;
+                if (r1 && c1) A[qq * lda + q2] = a11;
+                if (i2 != i) {   // the mirror block
+                    if (r0 && c0) A[p2 * lda + p] = cconj(a00);
+                    if (r0 && c1) A[q2 * lda + p] = cconj(a01);
+                    if (r1 && c0) A[p2 * lda + qq] = cconj(a10);
+                    if (r1 && c1) A[q2 * lda + qq] = cconj(a11);
+                }
             }
             __syncthreads();
-            // A <- G^H A G on the 2 x 2 blocks (rows of pair i, columns of
-            // pair i2: disjoint, so one pass; the row rotation first, then
-            // the column rotation, as two separate passes would), and V <- V G
-            const int nab = npair << psh;
-            for (int task = threadIdx.x; task < nab + (V ? (npair << sh) : 0); task += blockDim.x) {
-                if (task < nab) {
-                    const int i = task >> psh, i2 = task & pmask;
-                    if (i2 >= npair) continue;
-                    const float si = s_s[i], si2 = s_s[i2];
-                    if (si == 0.f && si2 == 0.f) continue;
-                    const int p = s_pp[i], qq = s_qq[i], p2 = s_pp[i2], q2 = s_qq[i2];
-                    const bool r0 = p < n, r1 = qq < n, c0 = p2 < n, c1 = q2 < n;
-                    const float2 z = make_float2(0.f, 0.f);
-                    float2 a00 = r0 && c0 ? A[p * lda + p2] : z, a01 = r0 && c1 ? A[p * lda + q2] : z;
-                    float2 a10 = r1 && c0 ? A[qq * lda + p2] : z, a11 = r1 && c1 ? A[qq * lda + q2] : z;
-                    if (si != 0.f) {   // rows p, q of columns p2, q2
-                        const float c = s_c[i];
-                        const float2 e = s_e[i];
-                        float2 eaq = cmul(e, a10);
-                        float2 ap = a00;
-                        a00 = make_float2(c * ap.x - si * eaq.x, c * ap.y - si * eaq.y);
-                        a10 = make_float2(si * ap.x + c * eaq.x, si * ap.y + c * eaq.y);
-                        eaq = cmul(e, a11);
-                        ap = a01;
-                        a01 = make_float2(c * ap.x - si * eaq.x, c * ap.y - si * eaq.y);
-                        a11 = make_float2(si * ap.x + c * eaq.x, si * ap.y + c * eaq.y);
-                    }
-                    if (si2 != 0.f) {   // columns p2, q2 of rows p, q
-                        const float c = s_c[i2];
-                        const float2 eh = cconj(s_e[i2]);
-                        float2 e2 = cmul(eh, a01);
-                        float2 ap = a00;
-                        a00 = make_float2(c * ap.x - si2 * e2.x, c * ap.y - si2 * e2.y);
-                        a01 = make_float2(si2 * ap.x + c * e2.x, si2 * ap.y + c * e2.y);
-                        e2 = cmul(eh, a11);
-                        ap = a10;
-                        a10 = make_float2(c * ap.x - si2 * e2.x, c * ap.y - si2 * e2.y);
-                        a11 = make_float2(si2 * ap.x + c * e2.x, si2 * ap.y + c * e2.y);
-                    }
-                    if (r0 && c0) A[p * lda + p2] = a00;
-                    if (r0 && c1) A[p * lda + q2] = a01;
-                    if (r1 && c0) A[qq * lda + p2] = a10;
-                    if (r1 && c1) A[qq * lda + q2] = a11;
-                } else {
-                    const int tv = task - nab, i = tv >> sh, m = tv & mmask;
-                    if (m >= n || s_s[i] == 0.f) continue;
-                    const int p = s_pp[i], qq = s_qq[i];
-                    const float c = s_c[i], s = s_s[i];
-                    const float2 eh = cconj(s_e[i]);
+            if (warp == 0) {
+                const bool last = rnd == n2 - 2;
+                if (rnd == 0 && threadIdx.x == 0) cnt[(sweep + 1) & 1] = 0;   // read by every thread before this round
+                const bool any =
+                    jacobi_rotations(A, n, lda, last ? 0 : rnd + 1, rot[b ^ 1], abs_tol, rel_tol, tail_tol);
+                if (any && threadIdx.x == 0) cnt[(last ? sweep + 1 : sweep) & 1] = 1;
+            } else if (V) {
+                for (int tv = threadIdx.x - 32; tv < npair * n; tv += blockDim.x - 32) {   // V <- V G
+                    const int i = (int)((tv * inv_n) >> 20), m = tv - i * n;
+                    const float s = r.s[i];
+                    if (s == 0.f) continue;
+                    const int p = r.p[i], qq = r.q[i];
+                    const float c = r.c[i];
+                    const float2 eh = cconj(r.e[i]);
                     const float2 vp = V[m * ldv + p], vq = V[m * ldv + qq];
                     const float2 e2 = cmul(eh, vq);
                     V[m * ldv + p] = make_float2(c * vp.x - s * e2.x, c * vp.y - s * e2.y);
@@ -227,12 +265,10 @@ __device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ld
             }
             __syncthreads();
         }
-        if (*s_cnt == 0) break;
-        __syncthreads();
+        if (cnt[sweep & 1] == 0) break;   // this sweep skipped every rotation
     }
     __syncthreads();
 }
-
 
 // Allow a kernel the device's opt-in shared memory per block, minus its static
 // shared memory (the launch still requests only what it needs).

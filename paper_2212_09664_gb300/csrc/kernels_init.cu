@@ -636,9 +636,8 @@ __global__ void k_eig(const double *__restrict__ gram, int q, int n, int nc, int
     // A (and the rotation matrix when it fits) in shared memory with an odd row
     // pitch, so that the column updates of the rotations hit distinct banks
     extern __shared__ float2 sA[];
-    __shared__ float s_c[64], s_s[64];
-    __shared__ float2 s_e[64];
-    __shared__ int s_cnt;
+    __shared__ JacobiRot s_rot[2];
+    __shared__ int s_cnt[2];
     __shared__ double s_fro[32];
     __shared__ double s_scale;
     __shared__ float s_lam[128];
@@ -669,7 +668,7 @@ __global__ void k_eig(const double *__restrict__ gram, int q, int n, int nc, int
         // a rotation is skipped once |a_pq| <= 1e-5 sqrt(a_pp a_qq) or <= 1e-6
         // ||A||_F, at most 5 sweeps: this pass only has to leave B = V0^H A V0
         // diagonally dominant; the refine pass converges quadratically from there
-        block_jacobi(sA, q, ld, Vw, ldv, s_c, s_s, s_e, &s_cnt, 5, (float)(1e-6 * sqrt(fro)), 1e-5f);
+        block_jacobi(sA, q, ld, Vw, ldv, s_rot, s_cnt, 5, (float)(1e-6 * sqrt(fro)), 1e-5f);
         if (v_in_smem)
             for (int e = threadIdx.x; e < q * q; e += blockDim.x) V[e] = Vw[(e / q) * ldv + e % q];
         return;
@@ -695,7 +694,7 @@ __global__ void k_eig(const double *__restrict__ gram, int q, int n, int nc, int
         }
         __syncthreads();
     }
-    block_jacobi(sA, q, ld, Vw, ldv, s_c, s_s, s_e, &s_cnt, 6, 0.f, 1e-6f, s_tail);
+    block_jacobi(sA, q, ld, Vw, ldv, s_rot, s_cnt, 6, 0.f, 1e-6f, s_tail);
     // eigenvalues (diagonal of the rotated B, scaled back), then V <- V0 Q,
     // formed in the shared A region (A is no longer needed)
     for (int i = threadIdx.x; i < q; i += blockDim.x) s_lam[i] = sA[i * ld + i].x;
