@@ -565,6 +565,26 @@ LRCCS_DEV void cp_async8(void *dst, const void *src) {
 LRCCS_DEV void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
+// The same copies, or zeros (and no read) when !on.
+LRCCS_DEV void cp_async8_or_zero(void *dst, const void *src, bool on) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 8 : 0)
+                 : "memory");
+}
+LRCCS_DEV void cp_async16_or_zero(void *dst, const void *src, bool on) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 16 : 0)
+                 : "memory");
+}
+// base + k strides of `bytes` bytes (one multiply-add with a constant k)
+template <class V>
+LRCCS_DEV V *step_by(V *base, unsigned bytes, unsigned k) {
+    return (V *)((uintptr_t)base + (unsigned long long)bytes * k);
+}
+// A global store under a predicate: no branch around it.
+LRCCS_DEV void st_global_if(float2 *p, float2 v, uint32_t on) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %3, 0;\n@p st.global.v2.f32 [%0], {%1, %2};\n}\n" ::"l"(p), "f"(v.x),
+                 "f"(v.y), "r"(on)
+                 : "memory");
+}
 // Stage `count` complex64 values from global `src` into shared `dst`, 16 bytes
 // per copy when both are 16-byte aligned and count is even, else 8 bytes.
 LRCCS_DEV void stage_row(float2 *dst, const float2 *src, int count, int tid, int nthr) {

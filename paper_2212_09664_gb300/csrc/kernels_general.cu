@@ -286,8 +286,8 @@ __global__ void __launch_bounds__(256, 3) k_fwd_rows(const float2 *__restrict__ 
 }
 
 // The row's points scattered into a zero row, transformed back along x, the
-// full row written to T_j[ky] for the column pass.  Measured as above: 87 -> 53 us;
-// 65 -> 37 us.
+// full row written to T_j[ky] for the column pass.  Measured as above: 87 -> 48 us;
+// 65 -> 36 us.
 template <int P>
 __global__ void __launch_bounds__(256, 3) k_adj_rows(const float2 *__restrict__ FU, float2 *__restrict__ T,
                                                      const RowArgs a) {
@@ -303,13 +303,16 @@ __global__ void __launch_bounds__(256, 3) k_adj_rows(const float2 *__restrict__ 
     float2 *mine = smem + slot * tile;
     row_positions(s_up, a, ky, NX);
     const uint32_t bits = first ? row_bits(s_up, a, ky, g, l, R2, R1, 16) : 0u;
-    auto stage = [&](int j, int s) {
-        if (j < a.nc) {
+    const unsigned pt = (unsigned)(r * sizeof(float2)), piece = (unsigned)(R1 * r * sizeof(float2));
+    auto stage = [&](int j, int s) {   // zeros at the points that do not exist
+        if (first && j < a.nc) {
             float2 *dst = mine + s * a.CB * tile + i;
             const float2 *src = FU + ((size_t)j * a.nu + u0) * r + l;
 #pragma unroll
-            for (int m = 0; m < R1; ++m)
-                if (bits >> m & 1) cp_async8(dst + m * a.S, src + s_up[g + R2 * m] * r);
+            for (int m = 0; m < R1; ++m) {
+                const uint32_t on = bits & (1u << m);
+                cp_async8_or_zero(dst + m * a.S, step_by(src, pt, on ? (unsigned)s_up[g + R2 * m] : 0u), on);
+            }
         }
         cp_async_commit();
     };
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__(256, 3) k_adj_rows(const float2 *__restrict__ 
         if (first && j < a.nc) {
             float2 v[R1];
 #pragma unroll
-            for (int m = 0; m < R1; ++m) v[m] = (bits >> m & 1) ? ex[m * a.S + i] : make_float2(0.f, 0.f);
+            for (int m = 0; m < R1; ++m) v[m] = ex[m * a.S + i];
             fft::dft_first<R1, R2, true>(v, g, a.tw, [&](int k1, float2 w) { ex[k1 * a.S + i] = w; });
         }
         __syncthreads();
@@ -335,7 +338,7 @@ __global__ void __launch_bounds__(256, 3) k_adj_rows(const float2 *__restrict__ 
             fft::Dft<R2, true>::run(v);
             float2 *dst = T + ((size_t)j * a.ny + ky) * rowlen + i;
 #pragma unroll
-            for (int k2 = 0; k2 < R2; ++k2) dst[k2 * R1 * r] = v[k2];
+            for (int k2 = 0; k2 < R2; ++k2) *step_by(dst, piece, k2) = v[k2];
         }
     }
 }

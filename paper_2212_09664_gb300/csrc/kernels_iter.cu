@@ -75,12 +75,6 @@ int npairs_of(int r) { return r * (r + 1) / 2; }
 // of the adjoint ([e][16..31]); column l uses entry e0 + l estep.
 #define COLW 16
 
-// base + off bytes: a uniform base and a 32-bit per-thread offset address without 64-bit arithmetic
-template <class V>
-LRCCS_DEV V *at(V *base, unsigned off) {
-    return (V *)((uintptr_t)base + off);
-}
-
 template <int P>
 struct ColPlan {
     static constexpr int NY = 32 * P, R1 = fft::Plan<NY>::R1, R2 = fft::Plan<NY>::R2;
@@ -94,17 +88,39 @@ __host__ __device__ inline int col_nxt(int r) { return (COLW - 1 + r - 1) / r + 
 // the tile's nxt x values (the nxl of them inside the image), transposed to
 // dst[xi (CNT + 2) + m] (the pad keeps the 16-byte reads of different xi on
 // different banks); inv = ceil(2^16 / nxt).
+// Up to three x values (r >= 8) every lane's copies are worked out once.
 template <int CNT>
-LRCCS_DEV void stage_map(float2 *dst, const float2 *src, int rowstep, int nxt, int nxl, unsigned inv, int lane) {
-    for (unsigned e = lane; e < (unsigned)(CNT * nxt); e += COLW) {
-        const unsigned m = (e * inv) >> 16, xi = e - m * nxt;
-        if (xi < (unsigned)nxl) cp_async8(dst + xi * (CNT + 2) + m, src + m * rowstep + xi);
+struct MapStage {
+    static constexpr int NI = (3 * CNT + COLW - 1) / COLW;
+    uint32_t at[NI];   // byte offsets: source << 12 | destination, or ~0
+    LRCCS_DEV void init(int rowstep, int nxt, int nxl, unsigned inv, int lane) {
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            const unsigned e = lane + COLW * i, m = (e * inv) >> 16, xi = e - m * nxt;
+            at[i] = ((m * rowstep + xi) << 15) | ((xi * (CNT + 2) + m) << 3);   // rows span less than 2^17 pixels
+            if (e >= (unsigned)(CNT * nxt) || xi >= (unsigned)nxl) at[i] = ~0u;
+        }
     }
-}
+    LRCCS_DEV void run(float2 *d, const float2 *s, int rowstep, int nxt, int nxl, unsigned inv, int lane) const {
+        if (nxt <= 3) {
+#pragma unroll
+            for (int i = 0; i < NI; ++i)
+                if (at[i] != ~0u) cp_async8((char *)d + (at[i] & 4095u), (const char *)s + (at[i] >> 12));
+            return;
+        }
+        for (unsigned e = lane; e < (unsigned)(CNT * nxt); e += COLW) {
+            const unsigned m = (e * inv) >> 16, xi = e - m * nxt;
+            if (xi < (unsigned)nxl) cp_async8(d + xi * (CNT + 2) + m, s + m * rowstep + xi);
+        }
+    }
+};
 
 // Measured (kernel time, L2 warm), TMA-staged tiles of whole columns -> this form:
-// 192 x 192, C = 12, r = 10: 17.9 -> 15.3 us; 256 x 256, C = 20, r = 12: 58 -> 44 us;
-// 256 x 256, C = 32, r = 14: 136 -> 72 us
+// 192 x 192, C = 12, r = 10: 17.9 -> 13.0 us; 256 x 256, C = 20, r = 12: 58 -> 41 us;
+// 256 x 256, C = 32, r = 14: 136 -> 69 us.  Issue bounds it, so addresses step by
+// constant multiples of one row, stores are predicated rather than branched
+// round, and a tile's map copies are worked out once, not per coil (all but
+// the arithmetic was half of the instructions: 15.3, 44 and 72 us before).
 template <int P>
 __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_fwd_cols(
     const float2 *__restrict__ U, const float2 *__restrict__ smaps, const uint32_t *__restrict__ rowtab, int e0,
@@ -122,15 +138,20 @@ __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_fwd_co
     float2 *map = smem + 2 * NY * COLW + g * mstage;
     const float2 *d = smaps + (size_t)g * nx + x0;
     const int nxl = min(nxt, nx - x0);   // x values of this tile inside the image
+    MapStage<R1> ms;
+    ms.init(R2 * nx, nxt, nxl, inv, lane);
     float2 u[R1];
-    const unsigned off = (unsigned)(g * rs + c) * sizeof(float2);
     int j = blockIdx.y;
+    d += (size_t)j * NY * nx;
     if (first) {
-        stage_map<R1>(map, d + (size_t)j * NY * nx, R2 * nx, nxt, nxl, inv, lane);
+        ms.run(map, d, R2 * nx, nxt, nxl, inv, lane);
         cp_async_commit();
 #pragma unroll
-        for (int m = 0; m < R1; ++m) u[m] = __ldg(at(U + (size_t)(m * R2) * rs, off));
+        for (int m = 0; m < R1; ++m) u[m] = __ldg(U + (size_t)(g + m * R2) * rs + c);
     }
+    float2 *dst = T + ((size_t)j * NY + g) * rs + c;
+    const size_t dstep = (size_t)CG * NY * rs;
+    const unsigned rowbytes = (unsigned)(R1 * rs * sizeof(float2));
     float2 *ex = smem;
     for (int s = 0; j < nc; j += CG, s ^= 1) {
         if (first) {
@@ -147,8 +168,9 @@ __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_fwd_co
             fft::dft_first<R1, R2, false>(v, g, g_tw, [&](int k1, float2 w) { ex[(k1 * R2 + g) * COLW + lane] = w; });
         }
         __syncthreads();
+        d += (size_t)CG * NY * nx;
         if (first && j + CG < nc) {
-            stage_map<R1>(map + (s ^ 1) * NG * mstage, d + (size_t)(j + CG) * NY * nx, R2 * nx, nxt, nxl, inv, lane);
+            ms.run(map + (s ^ 1) * NG * mstage, d, R2 * nx, nxt, nxl, inv, lane);
             cp_async_commit();
         }
         if (rows != 0) {
@@ -156,11 +178,10 @@ __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_fwd_co
 #pragma unroll
             for (int j2 = 0; j2 < R2; ++j2) v[j2] = ex[(g * R2 + j2) * COLW + lane];
             fft::Dft<R2, false>::run(v);
-            float2 *dst = T + (size_t)j * NY * rs;
 #pragma unroll
-            for (int k2 = 0; k2 < R2; ++k2)
-                if (rows >> k2 & 1) *at(dst + (size_t)(R1 * k2) * rs, off) = v[k2];
+            for (int k2 = 0; k2 < R2; ++k2) st_global_if(step_by(dst, rowbytes, k2), v[k2], rows & (1u << k2));
         }
+        dst += dstep;
         ex = ex == smem ? smem + NY * COLW : smem;
     }
 }
@@ -318,10 +339,12 @@ __global__ void __launch_bounds__(256) k_row_w(float2 *__restrict__ T, const flo
 // half-warp stages its own rows of T (and of the coil map) by cp.async while
 // the previous coil's second half runs, and transforms them in place: the
 // first half's output k1 replaces row g + R2 k1.  Rows that the tables leave
-// out are zero and not read.
+// out are staged as zeros and not read.
 // Measured (kernel time, L2 warm), one image column per block staged by 8-byte
-// cp.async -> this form: 192 x 192, C = 12, r = 10: 28.9 -> 17.4 us; 256 x 256,
-// C = 20, r = 12: 121 -> 65 us; 256 x 256, C = 32, r = 14: 291 -> 114 us
+// cp.async -> this form: 192 x 192, C = 12, r = 10: 28.9 -> 16.9 us; 256 x 256,
+// C = 20, r = 12: 121 -> 55 us; 256 x 256, C = 32, r = 14: 291 -> 93 us (zeros
+// staged instead of rows masked at the read, steps as in k_fwd_cols: from
+// 17.4, 65 and 114 us).
 // Where k_adj_cols writes: element (pixel i, column l < cols) at p[i stride + l],
 // times scale[l] when scale is not NULL.
 struct AdjOut {
@@ -343,10 +366,7 @@ __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_adj_co
     const int x = (int)((unsigned)c / (unsigned)r), l = c - x * r;
     const bool first = R2 == NG || g < R2, second = R1 == NG || g < R1;
     const uint32_t rows = first ? __ldg(rowtab + (e0 + l * estep) * 32 + 16 + g) : 0u;
-    // rows either column of the lane pair needs: the pair's 16-byte pieces
-    const uint32_t prow = (rows | __shfl_xor_sync(0xffffffffu, rows, 1)) >> (lane & 1);
     const size_t plane = (size_t)NY * rs;
-    const unsigned off = (unsigned)((g + R2 * (lane & 1)) * rs + c0 + (lane & ~1)) * sizeof(float2);
     const int mstage = nxt * (R2 + 2);
     float2 *map = smem + 2 * NY * COLW + g * mstage;
     const float2 *d = smaps + (size_t)g * nx + x0;
@@ -354,18 +374,34 @@ __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_adj_co
     float2 acc[R2];
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) acc[k2] = make_float2(0.f, 0.f);
-    auto stage = [&](int j, int s) {
+    // the next coil's rows (zeros where the tables leave them out) and map; one
+    // table for every column: 16-byte pieces of the pair's rows, else its own 8 bytes
+    const unsigned rowbytes = (unsigned)(R2 * rs * sizeof(float2));
+    const float2 *src = T + grp * plane +
+                        (estep == 0 ? (size_t)(g + R2 * (lane & 1)) * rs + c0 + (lane & ~1) : (size_t)g * rs + c);
+    MapStage<R2> ms;
+    ms.init(R1 * nx, nxt, nxl, inv, lane);
+    d += (size_t)grp * NY * nx;
+    auto stage = [&](int s) {
         if (first) {
-            float2 *dst = smem + s * NY * COLW + (g + R2 * (lane & 1)) * COLW + (lane & ~1);
-            const float2 *sj = T + j * plane;
+            if (estep == 0) {
+                float2 *dst = smem + s * NY * COLW + (g + R2 * (lane & 1)) * COLW + (lane & ~1);
 #pragma unroll
-            for (int m = 0; m < R1; m += 2)
-                if (prow >> m & 1) cp_async16(dst + m * R2 * COLW, at(sj + (size_t)(m * R2) * rs, off));
+                for (int m = 0; m < R1; m += 2)
+                    cp_async16_or_zero(dst + m * R2 * COLW, step_by(src, rowbytes, m), rows & (1u << m << (lane & 1)));
+            } else {
+                float2 *dst = smem + s * NY * COLW + g * COLW + lane;
+#pragma unroll
+                for (int m = 0; m < R1; ++m)
+                    cp_async8_or_zero(dst + m * R2 * COLW, step_by(src, rowbytes, m), rows & (1u << m));
+            }
         }
-        if (second) stage_map<R2>(map + s * NG * mstage, d + (size_t)j * NY * nx, R1 * nx, nxt, nxl, inv, lane);
+        if (second) ms.run(map + s * NG * mstage, d, R1 * nx, nxt, nxl, inv, lane);
         cp_async_commit();
+        src += CG * plane;
+        d += (size_t)CG * NY * nx;
     };
-    if (grp < nc) stage(grp, 0);
+    if (grp < nc) stage(0);
     int s = 0;
     for (int j = grp; j < nc; j += CG, s ^= 1) {
         float2 *sm = smem + s * NY * COLW + lane;
@@ -374,11 +410,11 @@ __global__ void __launch_bounds__(ColPlan<P>::NT, 768 / ColPlan<P>::NT) k_adj_co
         if (first) {
             float2 v[R1];
 #pragma unroll
-            for (int m = 0; m < R1; ++m) v[m] = (rows >> m & 1) ? sm[(g + R2 * m) * COLW] : make_float2(0.f, 0.f);
+            for (int m = 0; m < R1; ++m) v[m] = sm[(g + R2 * m) * COLW];
             fft::dft_first<R1, R2, true>(v, g, g_tw, [&](int k1, float2 w) { sm[(g + R2 * k1) * COLW] = w; });
         }
         __syncthreads();
-        if (j + CG < nc) stage(j + CG, s ^ 1);
+        if (j + CG < nc) stage(s ^ 1);
         if (second) {
             float2 v[R2];
 #pragma unroll
