@@ -142,7 +142,10 @@ LRCCS_DEV bool jacobi_rotations(const float2 *A, int n, int lda, int rnd, Jacobi
     for (int i = threadIdx.x & 31; i < npair; i += 32) {
         int p, qq;
         if (i == 0) { p = rnd; qq = n2 - 1; }
-        else { p = (rnd + i) % (n2 - 1); qq = (rnd - i + n2 - 1) % (n2 - 1); }
+        else {   // (rnd + i) and (rnd - i) mod (n2 - 1)
+            p = rnd + i < n2 - 1 ? rnd + i : rnd + i - (n2 - 1);
+            qq = rnd >= i ? rnd - i : rnd - i + (n2 - 1);
+        }
         float c = 1.f, s = 0.f;
         float2 e = make_float2(1.f, 0.f);
         if (p < n && qq < n) {
@@ -152,13 +155,15 @@ LRCCS_DEV bool jacobi_rotations(const float2 *A, int n, int lda, int rnd, Jacobi
             if (b2 > 1e-36f && b2 > abs_tol * abs_tol && b2 > rel_tol * rel_tol * fabsf(al) * fabsf(ga) &&
                 (fabsf(al) >= tail_tol || fabsf(ga) >= tail_tol)) {
                 // the rotation only has to be orthogonal: c = 1 / sqrt(1 + t^2),
-                // s = t c hold to rounding whatever the accuracy of t (c rounded
-                // to nearest: rsqrtf's bias took 1e-5 off V's column norms over
-                // 47 x 5 rotations, and off the singular values)
+                // s = t c hold to rounding whatever the accuracy of t, so t takes
+                // the short forms (tau^2 held finite); c is rounded to nearest:
+                // rsqrtf's bias took 1e-5 off V's column norms over 47 x 5
+                // rotations, and off the singular values
                 const float ib = rsqrtf(b2);
                 e = make_float2(apq.x * ib, apq.y * ib);
                 const float tau = (ga - al) * 0.5f * ib;
-                const float t = copysignf(1.f, tau) * __frcp_rn(fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f)));
+                const float h2 = fminf(fmaf(tau, tau, 1.f), 1e38f);
+                const float t = __fdividef(copysignf(1.f, tau), fabsf(tau) + h2 * rsqrtf(h2));
                 c = __frsqrt_rn(fmaf(t, t, 1.f));
                 s = t * c;
                 any = true;
@@ -178,6 +183,17 @@ __device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ld
     const int n2 = n + (n & 1), npair = n2 / 2, nblk = npair * (npair + 1) / 2;
     const int warp = threadIdx.x >> 5;
     const unsigned inv_n = ((1u << 20) + n - 1) / n;   // tv / n for tv < 64 n
+    // this thread's blocks (i, i2), the same in every round: block `task` of the
+    // triangle whose row i starts at i npair - i (i - 1) / 2 (n <= 128: at most
+    // 2080 blocks; the launch has at least a third as many threads)
+    int blk[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int task = threadIdx.x + k * blockDim.x;
+        int i = 0, first = 0;
+        while (task < nblk && first + npair - i <= task) first += npair - i++;
+        blk[k] = task < nblk ? i << 8 | (i + task - first) : -1;
+    }
     __syncthreads();
     if (warp == 0) {
         const bool any = jacobi_rotations(A, n, lda, 0, rot[0], abs_tol, rel_tol, tail_tol);
@@ -193,13 +209,10 @@ __device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ld
             const JacobiRot &r = rot[b];
             // A <- G^H A G on the block (rows of pair i, columns of pair i2 >= i):
             // the row rotation first, then the column rotation
-            for (int task = threadIdx.x; task < nblk; task += blockDim.x) {
-                // task -> (i, i2): row i of the triangle starts at i npair - i (i - 1) / 2
-                int i = (int)(((float)(2 * npair + 1) -
-                               sqrtf((float)((2 * npair + 1) * (2 * npair + 1) - 8 * task))) * 0.5f);
-                while (i > 0 && i * npair - i * (i - 1) / 2 > task) --i;
-                while ((i + 1) * npair - (i + 1) * i / 2 <= task) ++i;
-                const int i2 = i + task - (i * npair - i * (i - 1) / 2);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (blk[k] < 0) break;
+                const int i = blk[k] >> 8, i2 = blk[k] & 255;
                 const float si = r.s[i], si2 = r.s[i2];
                 if (si == 0.f && si2 == 0.f) continue;
                 const int p = r.p[i], qq = r.q[i], p2 = r.p[i2], q2 = r.q[i2];

@@ -644,11 +644,12 @@ __global__ void k_eig(const double *__restrict__ gram, int q, int n, int nc, int
     const int ld = q | 1;
     float2 *Vw = v_in_smem ? sA + q * ld : (refine ? Q : V);
     const int ldv = v_in_smem ? ld : q;
-    if (threadIdx.x == 0) {   // the refine pass works on B / max diag(B)
+    if (threadIdx.x < 32) {   // the refine pass works on B / max diag(B)
         double mx = 0.0;
         if (refine)
-            for (int i = 0; i < q; ++i) mx = fmax(mx, gram[2 * (i * q + i)]);
-        s_scale = mx > 0.0 ? mx : 1.0;
+            for (int i = threadIdx.x; i < q; i += 32) mx = fmax(mx, gram[2 * (i * q + i)]);
+        for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (threadIdx.x == 0) s_scale = mx > 0.0 ? mx : 1.0;
     }
     __syncthreads();
     const double isc = refine ? 1.0 / s_scale : 1.0;
@@ -803,8 +804,10 @@ cudaError_t launch_gram_x0(lrccs_ctx *c) {
     const int v_in_smem = (size_t)2 * q * ld * sizeof(float2) + 4096 <= (size_t)c->dev_smem_optin;
     const size_t smem2 = (size_t)(v_in_smem ? 2 : 1) * q * ld * sizeof(float2);
     double *T = c->d_gram + 2 * (size_t)q * q, *Bm = T + 2 * (size_t)q * q;
+    // a thread per element of a round's V update, beside the rotations' warp
+    const int nthr = std::min(1024, 32 + ((q + 1) / 2 * q + 31) / 32 * 32);
     prof_begin(c, KID_EIG);
-    k_eig<<<1, 1024, smem2, c->stream>>>(gram, q, c->n, c->nc, c->dims.rank, c->rmax, c->prm.energy_pct, c->d_V,
+    k_eig<<<1, nthr, smem2, c->stream>>>(gram, q, c->n, c->nc, c->dims.rank, c->rmax, c->prm.energy_pct, c->d_V,
                                         c->d_Q, c->d_meta + MT_COUNT, c->d_sigma, c->d_meta, c->d_status, v_in_smem,
                                         0);
     prof_end(c, KID_EIG);
@@ -815,7 +818,7 @@ cudaError_t launch_gram_x0(lrccs_ctx *c) {
     k_refine_vhb<<<q, 128, 0, c->stream>>>(c->d_V, T, q, Bm);
     prof_end(c, KID_EIG);
     prof_begin(c, KID_EIG);
-    k_eig<<<1, 1024, smem2, c->stream>>>(Bm, q, c->n, c->nc, c->dims.rank, c->rmax, c->prm.energy_pct, c->d_V,
+    k_eig<<<1, nthr, smem2, c->stream>>>(Bm, q, c->n, c->nc, c->dims.rank, c->rmax, c->prm.energy_pct, c->d_V,
                                         c->d_Q, c->d_meta + MT_COUNT, c->d_sigma, c->d_meta, c->d_status, v_in_smem,
                                         1);
     prof_end(c, KID_EIG);
