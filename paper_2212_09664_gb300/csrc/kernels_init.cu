@@ -225,10 +225,8 @@ __global__ void __launch_bounds__(ST_NT) k_structure(
     }
 }
 
-__global__ void k_fill_idx(const int32_t *__restrict__ framerows, const int32_t *__restrict__ meta,
-                           int nx, int32_t *idx) {
+__global__ void k_fill_idx(const int32_t *__restrict__ framerows, int nx, int32_t *idx) {
     const int g = blockIdx.x;
-    if (g >= meta[MT_NLINES]) return;
     const int ky = framerows[g];
     for (int kx = threadIdx.x; kx < nx; kx += blockDim.x) idx[(size_t)g * nx + kx] = ky * nx + kx;
 }
@@ -253,7 +251,7 @@ cudaError_t launch_compact(lrccs_ctx *c, const uint8_t *d_mask, const int64_t *d
 // Sample indices of masks that are unions of full lines (meta[MT_GENERAL] = 0).
 cudaError_t launch_fill_lines(lrccs_ctx *c) {
     prof_begin(c, KID_FILL_IDX);
-    k_fill_idx<<<c->q * c->ny, 128, 0, c->stream>>>(c->d_framerows, c->d_meta, c->nx, c->d_idx);
+    k_fill_idx<<<c->n_lines, 128, 0, c->stream>>>(c->d_framerows, c->nx, c->d_idx);
     prof_end(c, KID_FILL_IDX);
     return cudaGetLastError();
 }
