@@ -25,18 +25,19 @@
 // issues MMAs.
 //
 // Tiles: M = 128 output rows (64 sampled rows), N = 128 columns, K chunks of
-// 32 (16 y values); one CTA of 256 threads per (N tile, coil) covers every M
-// tile (up to four accumulators of 128 columns in tensor memory), so each B
-// tile is read once.  Thread 0 (producer) streams the chunks' A and B tiles
+// 32 (16 y values); one CTA of 256 threads per (N tile, coil, M tile), a
+// few on a multiprocessor (one accumulator of 128 tensor-memory columns each).
+// Thread 0 (producer) streams the chunks' A and B tiles
 // into two shared-memory stages with bulk asynchronous copies
 // (cp.async.bulk, completing on the stage's "full" mbarrier); thread 32 (MMA
-// issuer) waits for a stage, issues tcgen05.mma (M 128, N 128, K 16) for every
-// M tile and commits to the stage's "empty" mbarrier, which the producer
+// issuer) waits for a stage, issues tcgen05.mma (M 128, N 128, K 16)
+// and commits to the stage's "empty" mbarrier, which the producer
 // waits on before it refills the stage; the last commit arms a "done"
 // mbarrier for the epilogue.  Every wait is bounded.  The epilogue reads the
-// accumulators from tensor memory (tcgen05.ld), pairs real and imaginary rows
+// accumulator from tensor memory (tcgen05.ld), pairs real and imaginary rows
 // through a warp shuffle and writes T_j[ky_s] as complex64.
 #include <math.h>
+#include <algorithm>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -49,7 +50,8 @@
 #define TC_TILE (TC_M * TC_KC)         // elements of one operand tile (128 x 32)
 #define TC_TILE_BYTES (TC_TILE * 2)
 #define TC_THREADS 256
-#define TC_MT_MAX 4                    // M tiles per CTA (2 ny / 128 for ny <= 256)
+#define TC_MT_MAX 4                    // M tiles (2 ny / 128 for ny <= 256)
+#define TC_COLS 128                    // tensor-memory columns of a CTA: one accumulator
 // no-swizzle K-major layout: core matrix (8 rows x 8 elements, 128 bytes)
 // (rg, kb) at (rg * (TC_KC / 8) + kb) * 128 bytes; adjacent core matrices
 // along K are 128 bytes apart, along M/N 512 bytes apart
@@ -242,8 +244,7 @@ LRCCS_DEV void tc_expect(uint32_t mbar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar), "r"(bytes) : "memory");
 }
 
-// Stage layout: [A tiles: array a (0: hi / fp16, 1: lo), M tile m at
-// (a MT + m)] then [B tiles: array a at a].  NA = 2 (BF16X3) or 1 (FP16S).
+// Stage layout: [A tiles: array a (0: hi / fp16, 1: lo) at a] then [B tiles: array a at NA + a].  NA = 2 (BF16X3) or 1 (FP16S).
 template <int MODE>
 __global__ void __launch_bounds__(TC_THREADS) k_fwd_gemm(const uint16_t *__restrict__ A0,
                                                          const uint16_t *__restrict__ A1,
@@ -251,7 +252,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_fwd_gemm(const uint16_t *__restr
                                                          const uint16_t *__restrict__ B1,
                                                          const int32_t *__restrict__ usedrows,
                                                          const float *__restrict__ tmax, float2 *__restrict__ T,
-                                                         int ny, int nx, int r, int n_used, int mt, int tcols,
+                                                         int ny, int nx, int r, int n_used,
                                                          unsigned int *status) {
     constexpr int NA = MODE == 1 ? 2 : 1;
     extern __shared__ __align__(1024) uint8_t tc_smem[];
@@ -259,9 +260,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_fwd_gemm(const uint16_t *__restr
     __shared__ uint32_t tmem_slot;
     __shared__ int s_fail;
     const int t = threadIdx.x;
-    const int nb = blockIdx.x, j = blockIdx.y, NB = gridDim.x, m0 = blockIdx.z * mt;
+    const int nb = blockIdx.x, j = blockIdx.y, NB = gridDim.x, mb = blockIdx.z;
     const int N = nx * r, K2 = 2 * ny, KC = K2 / TC_KC;
-    const uint32_t stage_bytes = (uint32_t)((NA * mt + NA) * TC_TILE_BYTES);
+    const uint32_t stage_bytes = (uint32_t)(2 * NA * TC_TILE_BYTES);
     uint32_t full[2], empty[2], done;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_fwd_gemm(const uint16_t *__restr
     if (t < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          (uint32_t)__cvta_generic_to_shared(&tmem_slot)),
-                     "r"((uint32_t)tcols));
+                     "r"((uint32_t)TC_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -299,11 +300,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_fwd_gemm(const uint16_t *__restr
             const uint32_t sst = sbase + st * stage_bytes;
             for (int a = 0; a < NA; ++a) {
                 const uint16_t *Ag = a == 0 ? A0 : A1;
-                for (int m = 0; m < mt; ++m)
-                    tc_bulk(sst + (a * mt + m) * TC_TILE_BYTES, Ag + ((size_t)(m0 + m) * KC + kc) * TC_TILE, TC_TILE_BYTES,
-                            full[st]);
+                tc_bulk(sst + a * TC_TILE_BYTES, Ag + ((size_t)mb * KC + kc) * TC_TILE, TC_TILE_BYTES, full[st]);
                 const uint16_t *Bg = a == 0 ? B0 : B1;
-                tc_bulk(sst + (NA * mt + a) * TC_TILE_BYTES, Bg + (((size_t)j * NB + nb) * KC + kc) * TC_TILE,
+                tc_bulk(sst + (NA + a) * TC_TILE_BYTES, Bg + (((size_t)j * NB + nb) * KC + kc) * TC_TILE,
                         TC_TILE_BYTES, full[st]);
             }
         }
@@ -320,18 +319,15 @@ __global__ void __launch_bounds__(TC_THREADS) k_fwd_gemm(const uint16_t *__restr
             if (*(volatile int *)&s_fail) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint32_t sst = sbase + st * stage_bytes;
-            const uint32_t b0 = sst + (NA * mt) * TC_TILE_BYTES, b1 = b0 + TC_TILE_BYTES;
-            for (int m = 0; m < mt; ++m) {
-                const uint32_t a0 = sst + m * TC_TILE_BYTES, a1 = sst + (mt + m) * TC_TILE_BYTES;
-                const uint32_t acc_t = tmem + (uint32_t)(m * TC_N);
+            const uint32_t a0 = sst, a1 = sst + TC_TILE_BYTES;
+            const uint32_t b0 = sst + NA * TC_TILE_BYTES, b1 = b0 + TC_TILE_BYTES;
 #pragma unroll
-                for (int ks = 0; ks < TC_KC / 16; ++ks) {
-                    const uint32_t ko = ks * 2 * 128;   // two K core matrices per MMA
-                    tc_mma(acc_t, tc_desc(a0 + ko), tc_desc(b0 + ko), idesc, (kc > 0 || ks > 0) ? 1u : 0u);
-                    if (MODE == 1) {
-                        tc_mma(acc_t, tc_desc(a0 + ko), tc_desc(b1 + ko), idesc, 1u);
-                        tc_mma(acc_t, tc_desc(a1 + ko), tc_desc(b0 + ko), idesc, 1u);
-                    }
+            for (int ks = 0; ks < TC_KC / 16; ++ks) {
+                const uint32_t ko = ks * 2 * 128;   // two K core matrices per MMA
+                tc_mma(tmem, tc_desc(a0 + ko), tc_desc(b0 + ko), idesc, (kc > 0 || ks > 0) ? 1u : 0u);
+                if (MODE == 1) {
+                    tc_mma(tmem, tc_desc(a0 + ko), tc_desc(b1 + ko), idesc, 1u);
+                    tc_mma(tmem, tc_desc(a1 + ko), tc_desc(b0 + ko), idesc, 1u);
                 }
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -353,37 +349,35 @@ __global__ void __launch_bounds__(TC_THREADS) k_fwd_gemm(const uint16_t *__restr
     if (ok) {
         const float binv = MODE == 2 ? 1.f / tile_scale(tmax[nb], tmax[-1]) : 1.f;
         // epilogue: warp w reads rows 32 (w % 4) .. + 31 (TMEM lanes), columns
-        // 64 (w / 4) .. + 63 of each M tile's accumulator; the even lane of a
+        // 64 (w / 4) .. + 63 of the accumulator; the even lane of a
         // pair holds the real part of output row s, the odd lane its imaginary part
         const int w = t >> 5, lane = t & 31;
         const int row = 32 * (w & 3) + lane, cb = 64 * (w >> 2);
         const bool odd = lane & 1;
         const int n0 = nb * TC_N;
-        for (int m = 0; m < mt; ++m) {
-            const int s = ((m0 + m) * TC_M + row) >> 1;
-            const int ky = s < n_used ? usedrows[s] : -1;
-            float2 *Trow = T + ((size_t)j * ny + (ky < 0 ? 0 : ky)) * N;
+        const int s = (mb * TC_M + row) >> 1;
+        const int ky = s < n_used ? usedrows[s] : -1;
+        float2 *Trow = T + ((size_t)j * ny + (ky < 0 ? 0 : ky)) * N;
 #pragma unroll
-            for (int c0 = 0; c0 < 64; c0 += 16) {
-                uint32_t v[16];
-                const uint32_t ta = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(m * TC_N + cb + c0);
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
-                    "%12, %13, %14, %15}, [%16];\n"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                      "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-                      "=r"(v[14]), "=r"(v[15])
-                    : "r"(ta));
-                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        for (int c0 = 0; c0 < 64; c0 += 16) {
+            uint32_t v[16];
+            const uint32_t ta = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(cb + c0);
+            asm volatile(
+                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+                "%12, %13, %14, %15}, [%16];\n"
+                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+                  "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+                  "=r"(v[14]), "=r"(v[15])
+                : "r"(ta));
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float mine = __uint_as_float(v[i]) * binv;
-                    const float other = __shfl_xor_sync(0xffffffffu, mine, 1);
-                    // even lanes write the first 8 columns of the 16, odd lanes the last 8
-                    const int col = n0 + cb + c0 + i;
-                    if (ky >= 0 && col < N && ((i < 8) != odd))
-                        Trow[col] = odd ? make_float2(other, mine) : make_float2(mine, other);
-                }
+            for (int i = 0; i < 16; ++i) {
+                const float mine = __uint_as_float(v[i]) * binv;
+                const float other = __shfl_xor_sync(0xffffffffu, mine, 1);
+                // even lanes write the first 8 columns of the 16, odd lanes the last 8
+                const int col = n0 + cb + c0 + i;
+                if (ky >= 0 && col < N && ((i < 8) != odd))
+                    Trow[col] = odd ? make_float2(other, mine) : make_float2(mine, other);
             }
         }
     } else if (t == 0) {
@@ -391,7 +385,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_fwd_gemm(const uint16_t *__restr
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"((uint32_t)tcols));
+    if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"((uint32_t)TC_COLS));
 }
 
 // ---------------------------------------------------------------- launchers
@@ -417,12 +411,9 @@ cudaError_t launch_dft_a(lrccs_ctx *c) {
     return cudaGetLastError();
 }
 
-static size_t gemm_smem(int mode, int mt, int tcols) {
-    const int na = mode == 1 ? 2 : 1;
-    size_t sm = (size_t)2 * (na * mt + na) * TC_TILE_BYTES;
-    // keep the CTAs of one SM within its 512 tensor-memory columns
-    const size_t floor_ = (size_t)(tcols >= 512 ? 120 : tcols >= 256 ? 80 : 56) * 1024;
-    return sm > floor_ ? sm : floor_;
+// two stages, and no more CTAs on a multiprocessor than its 512 tensor-memory columns hold
+static size_t gemm_smem(int mode) {
+    return std::max((size_t)4 * (mode == 1 ? 2 : 1) * TC_TILE_BYTES, (size_t)56 * 1024);
 }
 
 cudaError_t launch_fwd_gemm(lrccs_ctx *c) {
@@ -434,8 +425,6 @@ cudaError_t launch_fwd_gemm(lrccs_ctx *c) {
     // another; one M tile per CTA puts three on it, which overlap, for B tiles read
     // `mall` times from L2.  192 x 192, C = 12, r = 10 (180 or 540 CTAs), BF16X3:
     // 55 -> 43 us.
-    const int mt = 1;
-    const int tcols = mt <= 1 ? 128 : (mt == 2 ? 256 : 512);
     cudaError_t e;
     if (c->dims.precision == LRCCS_PREC_FP16S_GEMM) {   // per-tile max |U| (d_tcscale[0] holds max |d|)
         prof_begin(c, KID_TC_SCALE);
@@ -454,16 +443,16 @@ cudaError_t launch_fwd_gemm(lrccs_ctx *c) {
                                                                           c->d_tcB0, c->d_tcB1, c->ny, c->nx, c->r);
     prof_end(c, KID_TC_B);
     prof_begin(c, KID_TC_GEMM);
-    const size_t smem = gemm_smem(bf ? 1 : 2, mt, tcols);
+    const size_t smem = gemm_smem(bf ? 1 : 2);
     if (bf)
         k_fwd_gemm<1><<<dim3(NB, c->nc, mall), TC_THREADS, smem, c->stream>>>(c->d_tcA0, c->d_tcA1, c->d_tcB0, c->d_tcB1,
                                                                         c->d_usedrows, c->d_tcscale + 1, c->d_T,
-                                                                        c->ny, c->nx, c->r, c->n_used, mt, tcols,
+                                                                        c->ny, c->nx, c->r, c->n_used,
                                                                         c->d_status);
     else
         k_fwd_gemm<2><<<dim3(NB, c->nc, mall), TC_THREADS, smem, c->stream>>>(c->d_tcA0, c->d_tcA1, c->d_tcB0, c->d_tcB1,
                                                                         c->d_usedrows, c->d_tcscale + 1, c->d_T,
-                                                                        c->ny, c->nx, c->r, c->n_used, mt, tcols,
+                                                                        c->ny, c->nx, c->r, c->n_used,
                                                                         c->d_status);
     prof_end(c, KID_TC_GEMM);
     e = cudaGetLastError();
