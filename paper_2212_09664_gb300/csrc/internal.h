@@ -253,6 +253,7 @@ cudaError_t launch_gram_x0(lrccs_ctx *c);
 cudaError_t launch_u0(lrccs_ctx *c);
 cudaError_t launch_gdqr(lrccs_ctx *c, int mode);      // F: GD step + Cholesky QR (mode 0: init U+)
 cudaError_t launch_zb(lrccs_ctx *c);                  // d_ZB <- Z B^H
+void launch_zb_of(lrccs_ctx *c, const float2 *Z, const float2 *B, float2 *dst);
 cudaError_t launch_solve(lrccs_ctx *c);                // C kernel
 bool bstep_fused_ok(const lrccs_ctx *c);               // k_bstep applies (line masks, rows resident)
 cudaError_t launch_bstep_fused(lrccs_ctx *c);          // B + C + D in one cooperative launch

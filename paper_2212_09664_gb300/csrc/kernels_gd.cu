@@ -693,13 +693,15 @@ typedef void (*zb_kernel_t)(const float2 *, const float2 *, int, int, float2 *);
 static const zb_kernel_t kZb[RMAXC] = RANK_TABLE(k_zb);
 
 static size_t zb_smem(int q, int r) { return ((size_t)ZB_PIX * (q | 1) + (size_t)q * r) * sizeof(float2); }
+// dst (n x r) <- Z B^H of an n x q Z and a q x r B (b_k contiguous)
+void launch_zb_of(lrccs_ctx *c, const float2 *Z, const float2 *B, float2 *dst) {
+    kZb[c->r - 1]<<<(c->n + ZB_PIX - 1) / ZB_PIX, 256, zb_smem(c->q, c->r), c->stream>>>(Z, B, c->n, c->q, dst);
+}
 // d_ZB <- Z B^H (the data term of the next gradient), from the current B.
 cudaError_t launch_zb(lrccs_ctx *c) {
-    const int r = c->r;
-    if (r < 1 || r > RMAXC) return cudaErrorInvalidValue;
+    if (c->r < 1 || c->r > RMAXC) return cudaErrorInvalidValue;
     prof_begin(c, KID_ZB);
-    kZb[r - 1]<<<(c->n + ZB_PIX - 1) / ZB_PIX, 256, zb_smem(c->q, r), c->stream>>>(c->d_Z, c->d_B, c->n, c->q,
-                                                                                   c->d_ZB);
+    launch_zb_of(c, c->d_Z, c->d_B, c->d_ZB);
     prof_end(c, KID_ZB);
     return cudaGetLastError();
 }

@@ -521,47 +521,85 @@ cudaError_t launch_init_adjoint(lrccs_ctx *c, const float2 *d_y, bool trunc) {
 
 // ---------------------------------------------------------------- Gram of X0 and its eigensolver
 
+// X0^H X0: thread (4 x 4 tile of frame pairs on or above the diagonal, pixel
+// slice) adds its 16 products per pixel from four 16-byte reads; the slices of a
+// tile add in order at the end.  Two 8-byte reads per product bounded one pair
+// per item: 36864 x 48: 60 -> 25 us, 65536 x 64: 152 -> 63 us.
 #define GRAM_CHUNK 32
 #define GRAM_THREADS 512
-#define MAXPP 17   // pairs per thread: q(q+1)/2 <= 512 * 17 for q <= 128
 
-template <int NS>   // pair slots per thread: q(q+1)/2 <= GRAM_THREADS NS
-__global__ void __launch_bounds__(GRAM_THREADS) k_gram_x0(const float2 *__restrict__ X0, int n, int q,
-                                                           float2 *part) {
-    extern __shared__ float2 s_x[];  // GRAM_CHUNK * q, then the pair table
-    short2 *s_pair = (short2 *)(s_x + GRAM_CHUNK * q);
-    const int np = q * (q + 1) / 2;
-    for (int p = threadIdx.x; p < np; p += blockDim.x) {
-        int a, b;
-        pair_of(p, q, a, b);
-        s_pair[p] = make_short2((short)a, (short)b);
-    }
+__host__ __device__ inline int gram_tiles(int q) { const int t = (q + 3) / 4; return t * (t + 1) / 2; }
+__host__ __device__ inline int gram_slices(int q) {   // pixel slices per tile
+    const int t = gram_tiles(q), s = GRAM_THREADS / t;
+    return t >= GRAM_THREADS ? 1 : (s < GRAM_CHUNK ? s : GRAM_CHUNK);
+}
+
+template <int NS>   // tiles per thread: gram_tiles(q) <= GRAM_THREADS NS
+__global__ void __launch_bounds__(GRAM_THREADS) k_gram_x0(const float2 *__restrict__ X0, int n, int q, float2 *part) {
+    extern __shared__ __align__(16) float2 s_x[];   // GRAM_CHUNK x qp (columns past q zero), then the slices' sums
+    const int nt = (q + 3) / 4, qp = 4 * nt + 2, T = gram_tiles(q), S = gram_slices(q);
     const int per = (n + gridDim.x - 1) / gridDim.x;
     const int i0 = blockIdx.x * per, i1 = min(n, i0 + per);
-    float2 acc[NS];
+    const int sl = threadIdx.x / T;
+    float2 acc[NS][16];
+    int ta[NS], tb[NS];
 #pragma unroll
-    for (int u = 0; u < NS; ++u) acc[u] = make_float2(0.f, 0.f);
+    for (int u = 0; u < NS; ++u) {
+        const int w = NS == 1 ? threadIdx.x - sl * T : threadIdx.x + u * GRAM_THREADS;
+        int A = 0, B = 0;
+        const bool live = NS == 1 ? sl < S : w < T;
+        if (live) pair_of(w, nt, A, B);
+        ta[u] = live ? 4 * A : -1;
+        tb[u] = 4 * B;
+#pragma unroll
+        for (int m = 0; m < 16; ++m) acc[u][m] = make_float2(0.f, 0.f);
+    }
+    const int s0 = NS == 1 ? sl : 0, step = NS == 1 ? S : 1;
     for (int c0 = i0; c0 < i1; c0 += GRAM_CHUNK) {
         const int cn = min(GRAM_CHUNK, i1 - c0);
         __syncthreads();
-        for (int e = threadIdx.x; e < cn * q; e += blockDim.x) s_x[e] = X0[(size_t)c0 * q + e];
+        for (int e = threadIdx.x; e < cn * qp; e += GRAM_THREADS) {
+            const int ii = e / qp, k = e - ii * qp;
+            s_x[e] = k < q ? __ldg(X0 + (size_t)(c0 + ii) * q + k) : make_float2(0.f, 0.f);
+        }
         __syncthreads();
-        for (int ii = 0; ii < cn; ++ii) {   // all of this thread's pairs per pixel (independent chains)
-            const float2 *xr = s_x + ii * q;
 #pragma unroll
-            for (int u = 0; u < NS; ++u) {
-                const int p = threadIdx.x + GRAM_THREADS * u;
-                if (p < np) {
-                    const short2 ab = s_pair[p];
-                    cfmac(acc[u], xr[ab.x], xr[ab.y]);
-                }
+        for (int u = 0; u < NS; ++u) {
+            if (ta[u] < 0) continue;
+            for (int ii = s0; ii < cn; ii += step) {
+                const float4 *x4 = reinterpret_cast<const float4 *>(s_x + ii * qp + ta[u]);
+                const float4 *y4 = reinterpret_cast<const float4 *>(s_x + ii * qp + tb[u]);
+                const float4 xa = x4[0], xb = x4[1], ya = y4[0], yb = y4[1];
+                const float2 x[4] = {make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xb.x, xb.y),
+                                     make_float2(xb.z, xb.w)};
+                const float2 y[4] = {make_float2(ya.x, ya.y), make_float2(ya.z, ya.w), make_float2(yb.x, yb.y),
+                                     make_float2(yb.z, yb.w)};
+#pragma unroll
+                for (int m = 0; m < 16; ++m) cfmac(acc[u][m], x[m >> 2], y[m & 3]);
             }
         }
     }
+    // the slices' sums, a row of the tiles at a time, then pair (a, b), a <= b, to part
+    float2 *out = part + (size_t)blockIdx.x * (q * (q + 1) / 2);
 #pragma unroll
-    for (int u = 0; u < NS; ++u) {
-        const int p = threadIdx.x + GRAM_THREADS * u;
-        if (p < np) part[(size_t)blockIdx.x * np + p] = acc[u];
+    for (int h = 0; h < 4; ++h) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < NS; ++u)
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (ta[u] >= 0) s_x[x * NS * GRAM_THREADS + u * GRAM_THREADS + threadIdx.x] = acc[u][4 * h + x];
+        __syncthreads();
+        for (int e = threadIdx.x; e < 4 * T; e += GRAM_THREADS) {
+            const int x = e / T, w = e - x * T;
+            int A, B;
+            pair_of(w, nt, A, B);
+            const int a = 4 * A + h, b = 4 * B + x;
+            if (a > b || b >= q) continue;
+            float2 sum = make_float2(0.f, 0.f);
+            for (int ss = 0; ss < S; ++ss) sum = cadd(sum, s_x[x * NS * GRAM_THREADS + ss * T + w]);
+            out[pair_index(a, b, q)] = sum;
+        }
     }
 }
 
@@ -783,17 +821,12 @@ cudaError_t launch_gram_x0(lrccs_ctx *c) {
     int blocks = (c->n + 127) / 128;
     if (blocks > 152) blocks = 152;
     if ((size_t)blocks * np > c->gpart_cap) blocks = (int)(c->gpart_cap / np);
-    const size_t smem = (size_t)GRAM_CHUNK * q * sizeof(float2) + (size_t)np * sizeof(short2);
+    const int ns = gram_tiles(q) <= GRAM_THREADS ? 1 : 2;
+    const size_t smem = std::max(GRAM_CHUNK * (4 * ((q + 3) / 4) + 2), 4 * ns * GRAM_THREADS) * sizeof(float2);
     double *gram = c->d_gram;
     prof_begin(c, KID_GRAM_X0);
-    const int ns = (np + GRAM_THREADS - 1) / GRAM_THREADS;
-    if (ns <= 1) k_gram_x0<1><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
-    else if (ns <= 2) k_gram_x0<2><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
-    else if (ns <= 3) k_gram_x0<3><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
-    else if (ns <= 5) k_gram_x0<5><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
-    else if (ns <= 8) k_gram_x0<8><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
-    else if (ns <= 12) k_gram_x0<12><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
-    else k_gram_x0<MAXPP><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
+    if (ns == 1) k_gram_x0<1><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
+    else k_gram_x0<2><<<blocks, GRAM_THREADS, smem, c->stream>>>(c->d_X0, c->n, q, c->d_gpart);
     k_gram_sum<<<(np + 63) / 64, 256, 0, c->stream>>>(c->d_gpart, blocks, q, gram);
     prof_end(c, KID_GRAM_X0);
     cudaError_t e = cudaGetLastError();
@@ -825,31 +858,22 @@ cudaError_t launch_gram_x0(lrccs_ctx *c) {
 
 // ---------------------------------------------------------------- U_0
 // U_0 = X0 V_r Sigma_r^{-1}: the top-r left singular vectors of X0 (Alg. 2),
-// written to the U+ buffer and then orthonormalised by CholeskyQR2.
-
-__global__ void k_u0(const float2 *__restrict__ X0, const float2 *__restrict__ V, const int32_t *__restrict__ order,
-                     const double *__restrict__ sigma, int n, int q, int r, float2 *Up) {
-    extern __shared__ float2 s_v[];  // q * r, scaled by 1/sigma
+// written to the U+ buffer and then orthonormalised by Cholesky QR.  The
+// product is k_zb's X0 conj(Q) with Q = conj(V_r Sigma_r^{-1}) (q x r), formed
+// here; a thread per entry with both factors re-read took 21 us (36864 x 48, r = 10)
+// and 49 us (65536 x 64, r = 12), k_zb 13 and 26 us, both launches.
+__global__ void k_u0(const float2 *__restrict__ V, const int32_t *__restrict__ order, const double *__restrict__ sigma,
+                     int q, int r, float2 *__restrict__ Q) {
     for (int e = threadIdx.x; e < q * r; e += blockDim.x) {
-        const int k = e / r, l = e % r;
-        const float is = (float)(1.0 / sigma[l]);
-        s_v[e] = cscale(V[k * q + order[l]], is);
-    }
-    __syncthreads();
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * r; e += gridDim.x * blockDim.x) {
-        const int i = e / r, l = e % r;
-        float2 acc = make_float2(0.f, 0.f);
-        const float2 *xr = X0 + (size_t)i * q;
-        for (int k = 0; k < q; ++k) cfma(acc, xr[k], s_v[k * r + l]);
-        Up[e] = acc;
+        const int k = e / r, l = e - k * r;
+        Q[e] = cconj(cscale(V[k * q + order[l]], (float)(1.0 / sigma[l])));
     }
 }
 
 cudaError_t launch_u0(lrccs_ctx *c) {
-    const size_t smem = (size_t)c->q * c->r * sizeof(float2);
     prof_begin(c, KID_U0);
-    k_u0<<<304, 256, smem, c->stream>>>(c->d_X0, c->d_V, c->d_meta + MT_COUNT, c->d_sigma, c->n, c->q, c->r,
-                                        c->d_Up);
+    k_u0<<<1, 256, 0, c->stream>>>(c->d_V, c->d_meta + MT_COUNT, c->d_sigma, c->q, c->r, c->d_B);
+    launch_zb_of(c, c->d_X0, c->d_B, c->d_Up);
     prof_end(c, KID_U0);
     return cudaGetLastError();
 }
@@ -861,10 +885,8 @@ cudaError_t launch_u0(lrccs_ctx *c) {
 cudaError_t configure_kernels_init(int max_smem) {
     SET_SMEM_B(k_init_rows, 1); SET_SMEM_B(k_init_rows, 2); SET_SMEM_B(k_init_rows, 3); SET_SMEM_B(k_init_rows, 4);
     SET_SMEM_B(k_init_rows, 5); SET_SMEM_B(k_init_rows, 6); SET_SMEM_B(k_init_rows, 7); SET_SMEM_B(k_init_rows, 8);
-    SET_SMEM(k_gram_x0<1>); SET_SMEM(k_gram_x0<2>); SET_SMEM(k_gram_x0<3>); SET_SMEM(k_gram_x0<5>);
-    SET_SMEM(k_gram_x0<8>); SET_SMEM(k_gram_x0<12>); SET_SMEM(k_gram_x0<MAXPP>);
+    SET_SMEM(k_gram_x0<1>); SET_SMEM(k_gram_x0<2>);
     SET_SMEM(k_eig);
     SET_SMEM(k_structure);
-    SET_SMEM(k_u0);
     return cudaGetLastError();
 }
