@@ -125,118 +125,151 @@ LRCCS_DEV bool last_block_arrive(unsigned int *counter) {
 // is above tail_tol, the wanted eigenvectors converge without them);
 // the sweeps stop when a whole sweep skips every rotation.
 //
-// A round is two phases with a barrier each: the 2 x 2 blocks of A on and above
-// the diagonal (the rest is their mirror image), then the first warp forms the
-// next round's rotations while the others update V with this round's.
+// One barrier a round: latency bounds a round, so the thread that rotates the
+// 2 x 2 block holding a pivot of the next round forms that rotation from it at
+// once (the pivot's two diagonal entries follow from the last round's and this
+// round's t |a_pq|).  Only the blocks on and above the diagonal are rotated, the
+// rest is their mirror image; other warps update V meanwhile.
+// One matrix, first pass, whole-matrix rotations in two phases -> half blocks,
+// rotations by one warp beside the V update -> this form: q = 32: 162 -> 145 ->
+// 116 us, q = 48: 405 -> 269 -> 247, q = 64: 601 -> 429 -> 388,
+// q = 96: 2040 -> 1173 -> 1006.
 struct JacobiRot {
-    float c[64], s[64];
-    float2 e[64];
-    short p[64], q[64];
+    float4 g[64];      // c, s, e
+    float tb[64];      // t |a_pq|: a_pp falls by it, a_qq grows
+    uint32_t pq[64];   // p | q << 16
+};
+struct JacobiWork {
+    JacobiRot rot[2];
+    float diag[2][128];   // the diagonal after an even / odd round
+    int cnt[2];           // a sweep rotated something (by the sweep's parity)
 };
 
-// The rotations of round rnd (one warp); returns whether any is not skipped.
-LRCCS_DEV bool jacobi_rotations(const float2 *A, int n, int lda, int rnd, JacobiRot &r, float abs_tol, float rel_tol,
-                                float tail_tol) {
-    const int n2 = n + (n & 1), npair = n2 / 2;
-    bool any = false;
-    for (int i = threadIdx.x & 31; i < npair; i += 32) {
-        int p, qq;
-        if (i == 0) { p = rnd; qq = n2 - 1; }
-        else {   // (rnd + i) and (rnd - i) mod (n2 - 1)
-            p = rnd + i < n2 - 1 ? rnd + i : rnd + i - (n2 - 1);
-            qq = rnd >= i ? rnd - i : rnd - i + (n2 - 1);
-        }
-        float c = 1.f, s = 0.f;
-        float2 e = make_float2(1.f, 0.f);
-        if (p < n && qq < n) {
-            const float2 apq = A[p * lda + qq];
-            const float b2 = apq.x * apq.x + apq.y * apq.y;
-            const float al = A[p * lda + p].x, ga = A[qq * lda + qq].x;
-            if (b2 > 1e-36f && b2 > abs_tol * abs_tol && b2 > rel_tol * rel_tol * fabsf(al) * fabsf(ga) &&
-                (fabsf(al) >= tail_tol || fabsf(ga) >= tail_tol)) {
-                // the rotation only has to be orthogonal: c = 1 / sqrt(1 + t^2),
-                // s = t c hold to rounding whatever the accuracy of t, so t takes
-                // the short forms (tau^2 held finite); c is rounded to nearest:
-                // rsqrtf's bias took 1e-5 off V's column norms over 47 x 5
-                // rotations, and off the singular values
-                const float ib = rsqrtf(b2);
-                e = make_float2(apq.x * ib, apq.y * ib);
-                const float tau = (ga - al) * 0.5f * ib;
-                const float h2 = fminf(fmaf(tau, tau, 1.f), 1e38f);
-                const float t = __fdividef(copysignf(1.f, tau), fabsf(tau) + h2 * rsqrtf(h2));
-                c = __frsqrt_rn(fmaf(t, t, 1.f));
-                s = t * c;
-                any = true;
-            }
-        }
-        r.c[i] = c;
-        r.s[i] = s;
-        r.e[i] = e;
-        r.p[i] = (short)p;
-        r.q[i] = (short)qq;
+// Rotation i of a round, of indices p and q; returns whether it is not skipped.
+LRCCS_DEV bool jacobi_rotation(JacobiRot &r, int i, int p, int q, float2 apq, float al, float ga, float abs_tol,
+                               float rel_tol, float tail_tol) {
+    const float b2 = apq.x * apq.x + apq.y * apq.y;
+    float c = 1.f, s = 0.f, tb = 0.f;
+    float2 e = make_float2(1.f, 0.f);
+    const bool live = b2 > 1e-36f && b2 > abs_tol * abs_tol &&
+                      b2 > rel_tol * rel_tol * fabsf(al) * fabsf(ga) && (fabsf(al) >= tail_tol || fabsf(ga) >= tail_tol);
+    if (live) {
+        // the rotation only has to be orthogonal: c = 1 / sqrt(1 + t^2), s = t c
+        // hold to rounding whatever the accuracy of t, so t takes the short forms
+        // (tau^2 held finite); c is rounded to nearest: rsqrtf's bias took 1e-5
+        // off V's column norms over 47 x 5 rotations, and off the singular values
+        const float ib = rsqrtf(b2);
+        e = make_float2(apq.x * ib, apq.y * ib);
+        const float tau = (ga - al) * 0.5f * ib;
+        const float h2 = fminf(fmaf(tau, tau, 1.f), 1e38f);
+        const float t = __fdividef(copysignf(1.f, tau), fabsf(tau) + h2 * rsqrtf(h2));
+        c = __frsqrt_rn(fmaf(t, t, 1.f));
+        s = t * c;
+        tb = t * (b2 * ib);
     }
-    return __any_sync(0xffffffffu, any);
+    r.g[i] = make_float4(c, s, e.x, e.y);
+    r.tb[i] = tb;
+    r.pq[i] = p | q << 16;
+    return live;
 }
 
-__device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ldv, JacobiRot (&rot)[2], int (&cnt)[2],
-                                    int max_sweeps, float abs_tol = 0.f, float rel_tol = 1e-7f, float tail_tol = 0.f) {
-    const int n2 = n + (n & 1), npair = n2 / 2, nblk = npair * (npair + 1) / 2;
-    const int warp = threadIdx.x >> 5;
-    const unsigned inv_n = ((1u << 20) + n - 1) / n;   // tv / n for tv < 64 n
-    // this thread's blocks (i, i2), the same in every round: block `task` of the
-    // triangle whose row i starts at i npair - i (i - 1) / 2 (n <= 128: at most
-    // 2080 blocks; the launch has at least a third as many threads)
-    int blk[3];
+// Threads that hold blocks of A beside others that update V: one block each up
+// to 17 warps (n = 64), then several; 1024 threads leave 15 warps for V.
+__host__ __device__ inline int jacobi_block_threads(int n) {
+    const int np = n > 5 ? (n + 1) / 2 : 3, t = (np * (np + 1) / 2 + 31) / 32 * 32;
+    return t < 544 ? t : 544;
+}
+
+// PAD: A holds jacobi_rows(n) rows and columns, zero past n.
+__host__ __device__ inline int jacobi_rows(int n) { return n > 5 ? n + (n & 1) : 6; }
+
+template <bool PAD>
+__device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ldv, JacobiWork &w, int max_sweeps,
+                                    float abs_tol = 0.f, float rel_tol = 1e-7f, float tail_tol = 0.f) {
+    // at least three pairs (indices past n are never rotated): a block then holds at most one pivot
+    const int n2 = jacobi_rows(n), npair = n2 / 2, nblk = npair * (npair + 1) / 2, N = n2 - 1;
+    // This thread's blocks (i, i2), the same in every round: at most 2080 of them
+    // (n <= 128), four a thread; the other warps update V.  Round rnd pairs
+    // (rnd + i, rnd - i) mod N for i >= 1 and (rnd, N), so pivot x of the next round
+    // lies in the rows of pair x - 1 and the columns of pair x + 1 (or at the ends
+    // (0, 1) and (npair - 2, npair - 1)).  The pivots' blocks go to the first threads,
+    // for few warps to run the rotations' code; the rest follow by rows.
+    const int na = V ? jacobi_block_threads(n) : (int)blockDim.x;
+    int blk[4];   // i << 8 | i2, -1: none
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const int task = threadIdx.x + k * blockDim.x;
-        int i = 0, first = 0;
-        while (task < nblk && first + npair - i <= task) first += npair - i++;
-        blk[k] = task < nblk ? i << 8 | (i + task - first) : -1;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        const bool any = jacobi_rotations(A, n, lda, 0, rot[0], abs_tol, rel_tol, tail_tol);
-        if (threadIdx.x == 0) {
-            cnt[0] = any;
-            cnt[1] = 0;
+    for (int k = 0; k < 4; ++k) {
+        const int task = threadIdx.x < na ? threadIdx.x + k * na : nblk;
+        int i, i2;
+        if (task < npair) {
+            i = task == 0 ? 0 : task == npair - 1 ? npair - 2 : task - 1;
+            i2 = task == 0 ? 1 : task == npair - 1 ? npair - 1 : task + 1;
+        } else {
+            int left = task - npair;
+            for (i = 0; i < npair; ++i) {
+                const bool e1 = i == 0 || i == npair - 2, e2 = i + 2 < npair;   // pivots at i + 1, i + 2
+                const int cnt = npair - i - e1 - e2;
+                if (left < cnt) {
+                    i2 = i + left;
+                    if (e1 && i2 >= i + 1) ++i2;
+                    if (e2 && i2 >= i + 2) ++i2;
+                    break;
+                }
+                left -= cnt;
+            }
         }
+        blk[k] = task < nblk ? i << 8 | i2 : -1;
+    }
+    const bool pivot = threadIdx.x < npair;   // blk[0] holds pivot threadIdx.x of the next round: its
+    const bool prow = threadIdx.x != 1, pcol = threadIdx.x == npair - 1;   // second row, second column
+    __syncthreads();
+    if (threadIdx.x < 2) w.cnt[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < n2; i += blockDim.x) w.diag[1][i] = i < n ? A[i * lda + i].x : 0.f;
+    __syncthreads();
+    for (int i = threadIdx.x; i < npair; i += blockDim.x) {
+        const int p = i, q = i == 0 ? N : N - i;   // round 0
+        const bool in = p < n && q < n;
+        if (jacobi_rotation(w.rot[0], i, p, q, in ? A[p * lda + q] : make_float2(0.f, 0.f), w.diag[1][p],
+                            w.diag[1][q], abs_tol, rel_tol, tail_tol))
+            w.cnt[0] = 1;
     }
     __syncthreads();
     int b = 0;
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        for (int rnd = 0; rnd < n2 - 1; ++rnd, b ^= 1) {
-            const JacobiRot &r = rot[b];
+        for (int rnd = 0; rnd < N; ++rnd, b ^= 1) {
+            const JacobiRot &r = w.rot[b];
+            const int nsweep = rnd == N - 1 ? sweep + 1 : sweep;   // the sweep of the next round
+            if (rnd == 1 && threadIdx.x == 0) w.cnt[(sweep + 1) & 1] = 0;   // read by every thread before round 0
             // A <- G^H A G on the block (rows of pair i, columns of pair i2 >= i):
             // the row rotation first, then the column rotation
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
+            for (int k = 0; k < 4; ++k) {
                 if (blk[k] < 0) break;
                 const int i = blk[k] >> 8, i2 = blk[k] & 255;
-                const float si = r.s[i], si2 = r.s[i2];
-                if (si == 0.f && si2 == 0.f) continue;
-                const int p = r.p[i], qq = r.q[i], p2 = r.p[i2], q2 = r.q[i2];
-                const bool r0 = p < n, r1 = qq < n, c0 = p2 < n, c1 = q2 < n;
+                const float4 g = r.g[i], g2 = r.g[i2];
+                const bool turn = g.y != 0.f || g2.y != 0.f;
+                if (!turn && !(k == 0 && pivot) && i != i2) continue;
+                const uint32_t pq = r.pq[i], pq2 = r.pq[i2];
+                const int p = pq & 0xffff, qq = pq >> 16, p2 = pq2 & 0xffff, q2 = pq2 >> 16;
+                const bool r0 = PAD || p < n, r1 = PAD || qq < n, c0 = PAD || p2 < n, c1 = PAD || q2 < n;
                 const float2 z = make_float2(0.f, 0.f);
                 float2 a00 = r0 && c0 ? A[p * lda + p2] : z, a01 = r0 && c1 ? A[p * lda + q2] : z;
                 float2 a10 = r1 && c0 ? A[qq * lda + p2] : z, a11 = r1 && c1 ? A[qq * lda + q2] : z;
-                if (si != 0.f) {   // rows p, q of columns p2, q2
-                    const float c = r.c[i];
-                    const float2 e = r.e[i];
-                    float2 eaq = cmul(e, a10);
-                    float2 ap = a00;
+                if (turn) {
+                    // rows p, q of columns p2, q2 (the identity when skipped)
+                    float c = g.x;
+                    const float si = g.y, si2 = g2.y;
+                    const float2 e = make_float2(g.z, g.w), eh = make_float2(g2.z, -g2.w);
+                    float2 eaq = cmul(e, a10), ap = a00;
                     a00 = make_float2(c * ap.x - si * eaq.x, c * ap.y - si * eaq.y);
                     a10 = make_float2(si * ap.x + c * eaq.x, si * ap.y + c * eaq.y);
                     eaq = cmul(e, a11);
                     ap = a01;
                     a01 = make_float2(c * ap.x - si * eaq.x, c * ap.y - si * eaq.y);
                     a11 = make_float2(si * ap.x + c * eaq.x, si * ap.y + c * eaq.y);
-                }
-                if (si2 != 0.f) {   // columns p2, q2 of rows p, q
-                    const float c = r.c[i2];
-                    const float2 eh = cconj(r.e[i2]);
+                    // columns p2, q2 of rows p, q
+                    c = g2.x;
                     float2 e2 = cmul(eh, a01);
-                    float2 ap = a00;
+                    ap = a00;
                     a00 = make_float2(c * ap.x - si2 * e2.x, c * ap.y - si2 * e2.y);
                     a01 = make_float2(si2 * ap.x + c * e2.x, si2 * ap.y + c * e2.y);
                     e2 = cmul(eh, a11);
@@ -244,6 +277,20 @@ __device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ld
                     a10 = make_float2(c * ap.x - si2 * e2.x, c * ap.y - si2 * e2.y);
                     a11 = make_float2(si2 * ap.x + c * e2.x, si2 * ap.y + c * e2.y);
                 }
+                if (k == 0 && pivot) {   // (p', q') of the next round: column p', row q' of this block
+                    const int pn = pcol ? q2 : p2, qn = prow ? qq : p;
+                    const float *d = w.diag[b ^ 1];
+                    const float al = d[pn] + (pcol ? r.tb[i2] : -r.tb[i2]), ga = d[qn] + (prow ? r.tb[i] : -r.tb[i]);
+                    const float2 aqp = prow ? (pcol ? a11 : a10) : a00;
+                    if (jacobi_rotation(w.rot[b ^ 1], threadIdx.x, pn, qn, cconj(aqp), al, ga, abs_tol, rel_tol,
+                                        tail_tol))
+                        w.cnt[nsweep & 1] = 1;
+                }
+                if (i2 == i) {
+                    w.diag[b][p] = a00.x;
+                    w.diag[b][qq] = a11.x;
+                }
+                if (!turn) continue;
                 if (r0 && c0) A[p * lda + p2] = a00;
                 if (r0 && c1) A[p * lda + q2] = a01;
                 if (r1 && c0) A[qq * lda + p2] = a10;
@@ -255,30 +302,25 @@ __device__ inline void block_jacobi(float2 *A, int n, int lda, float2 *V, int ld
                     if (r1 && c1) A[q2 * lda + qq] = cconj(a11);
                 }
             }
-            __syncthreads();
-            if (warp == 0) {
-                const bool last = rnd == n2 - 2;
-                if (rnd == 0 && threadIdx.x == 0) cnt[(sweep + 1) & 1] = 0;   // read by every thread before this round
-                const bool any =
-                    jacobi_rotations(A, n, lda, last ? 0 : rnd + 1, rot[b ^ 1], abs_tol, rel_tol, tail_tol);
-                if (any && threadIdx.x == 0) cnt[(last ? sweep + 1 : sweep) & 1] = 1;
-            } else if (V) {
-                for (int tv = threadIdx.x - 32; tv < npair * n; tv += blockDim.x - 32) {   // V <- V G
-                    const int i = (int)((tv * inv_n) >> 20), m = tv - i * n;
-                    const float s = r.s[i];
+            if (threadIdx.x >= na) {   // V <- V G: a warp takes columns p, q of pair i, a lane rows lane, lane + 32, ...
+                const int nw = (blockDim.x - na) >> 5, lane = threadIdx.x & 31;
+                for (int i = (threadIdx.x - na) >> 5; i < npair; i += nw) {
+                    const float4 g = r.g[i];
+                    const float c = g.x, s = g.y;
                     if (s == 0.f) continue;
-                    const int p = r.p[i], qq = r.q[i];
-                    const float c = r.c[i];
-                    const float2 eh = cconj(r.e[i]);
-                    const float2 vp = V[m * ldv + p], vq = V[m * ldv + qq];
-                    const float2 e2 = cmul(eh, vq);
-                    V[m * ldv + p] = make_float2(c * vp.x - s * e2.x, c * vp.y - s * e2.y);
-                    V[m * ldv + qq] = make_float2(s * vp.x + c * e2.x, s * vp.y + c * e2.y);
+                    const float2 eh = make_float2(g.z, -g.w);
+                    float2 *vp = V + (r.pq[i] & 0xffff), *vq = V + (r.pq[i] >> 16);
+#pragma unroll 2
+                    for (int m = lane * ldv; m < n * ldv; m += 32 * ldv) {
+                        const float2 a = vp[m], e2 = cmul(eh, vq[m]);
+                        vp[m] = make_float2(c * a.x - s * e2.x, c * a.y - s * e2.y);
+                        vq[m] = make_float2(s * a.x + c * e2.x, s * a.y + c * e2.y);
+                    }
                 }
             }
             __syncthreads();
         }
-        if (cnt[sweep & 1] == 0) break;   // this sweep skipped every rotation
+        if (w.cnt[sweep & 1] == 0) break;   // this sweep skipped every rotation
     }
     __syncthreads();
 }

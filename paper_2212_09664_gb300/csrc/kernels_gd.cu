@@ -364,8 +364,8 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
     __shared__ float2 sG[R * 2 * R];
     __shared__ float2 sR[R * R];
     __shared__ float2 s_tot[PL::L_ITER];
-    __shared__ JacobiRot s_rot[2];
-    __shared__ int s_cnt[2], s_flag;
+    __shared__ JacobiWork s_jac;
+    __shared__ int s_flag;
     __shared__ float s_eta;
     const int t = threadIdx.x, G = gridDim.x;
     const int i0 = min(a.n, (int)blockIdx.x * a.per), i1 = min(a.n, i0 + a.per), rows = i1 - i0;
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
                 sR[y * R + x] = cconj(A1[p]);
             }
             __syncthreads();
-            block_jacobi(sR, R, R, nullptr, 0, s_rot, s_cnt, 30);
+            block_jacobi<false>(sR, R, R, nullptr, 0, s_jac, 30);
             if (t == 0) {
                 float lmax = 0.f;
                 for (int x = 0; x < R; ++x) lmax = fmaxf(lmax, sR[x * R + x].x);

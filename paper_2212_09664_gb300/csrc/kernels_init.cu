@@ -666,19 +666,18 @@ __global__ void __launch_bounds__(256) k_gram_sum(const float2 *__restrict__ par
 // The refine pass also sorts: sigma_j = sqrt(lambda_j) descending, and the
 // rank rule of Alg. 2 when rank_in == 0: the smallest r whose leading sigma^2
 // reach b% of the energy of the first floor(min(n, q, C min m_k)/10) (at least 1).
-__global__ void k_eig(const double *__restrict__ gram, int q, int n, int nc, int rank_in, int rmax,
+__global__ void __launch_bounds__(1024) k_eig(const double *__restrict__ gram, int q, int n, int nc, int rank_in, int rmax,
                       double energy_pct, float2 *V, float2 *Q, int32_t *order, double *sigma, int32_t *meta,
                       unsigned int *status, int v_in_smem, int refine) {
     // A (and the rotation matrix when it fits) in shared memory with an odd row
     // pitch, so that the column updates of the rotations hit distinct banks
     extern __shared__ float2 sA[];
-    __shared__ JacobiRot s_rot[2];
-    __shared__ int s_cnt[2];
+    __shared__ JacobiWork s_jac;
     __shared__ double s_fro[32];
     __shared__ double s_scale;
     __shared__ float s_lam[128];
-    const int ld = q | 1;
-    float2 *Vw = v_in_smem ? sA + q * ld : (refine ? Q : V);
+    const int n2 = jacobi_rows(q), ld = n2 | 1;
+    float2 *Vw = v_in_smem ? sA + n2 * ld : (refine ? Q : V);
     const int ldv = v_in_smem ? ld : q;
     if (threadIdx.x < 32) {   // the refine pass works on B / max diag(B)
         double mx = 0.0;
@@ -690,6 +689,8 @@ __global__ void k_eig(const double *__restrict__ gram, int q, int n, int nc, int
     __syncthreads();
     const double isc = refine ? 1.0 / s_scale : 1.0;
     double fro = 0.0;
+    for (int e = threadIdx.x; e < n2 * ld; e += blockDim.x) sA[e] = make_float2(0.f, 0.f);
+    __syncthreads();
     for (int e = threadIdx.x; e < q * q; e += blockDim.x) {
         const int a = e / q, b = e - a * q;
         sA[a * ld + b] = make_float2((float)(gram[2 * e] * isc), (float)(gram[2 * e + 1] * isc));
@@ -705,7 +706,7 @@ __global__ void k_eig(const double *__restrict__ gram, int q, int n, int nc, int
         // a rotation is skipped once |a_pq| <= 1e-5 sqrt(a_pp a_qq) or <= 1e-6
         // ||A||_F, at most 5 sweeps: this pass only has to leave B = V0^H A V0
         // diagonally dominant; the refine pass converges quadratically from there
-        block_jacobi(sA, q, ld, Vw, ldv, s_rot, s_cnt, 5, (float)(1e-6 * sqrt(fro)), 1e-5f);
+        block_jacobi<true>(sA, q, ld, Vw, ldv, s_jac, 5, (float)(1e-6 * sqrt(fro)), 1e-5f);
         if (v_in_smem)
             for (int e = threadIdx.x; e < q * q; e += blockDim.x) V[e] = Vw[(e / q) * ldv + e % q];
         return;
@@ -731,7 +732,7 @@ __global__ void k_eig(const double *__restrict__ gram, int q, int n, int nc, int
         }
         __syncthreads();
     }
-    block_jacobi(sA, q, ld, Vw, ldv, s_rot, s_cnt, 6, 0.f, 1e-6f, s_tail);
+    block_jacobi<true>(sA, q, ld, Vw, ldv, s_jac, 6, 0.f, 1e-6f, s_tail);
     // eigenvalues (diagonal of the rotated B, scaled back), then V <- V0 Q,
     // formed in the shared A region (A is no longer needed)
     for (int i = threadIdx.x; i < q; i += blockDim.x) s_lam[i] = sA[i * ld + i].x;
@@ -831,12 +832,12 @@ cudaError_t launch_gram_x0(lrccs_ctx *c) {
     prof_end(c, KID_GRAM_X0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int ld = q | 1;
-    const int v_in_smem = (size_t)2 * q * ld * sizeof(float2) + 4096 <= (size_t)c->dev_smem_optin;
-    const size_t smem2 = (size_t)(v_in_smem ? 2 : 1) * q * ld * sizeof(float2);
+    const int n2 = jacobi_rows(q), ld = n2 | 1;
+    const int v_in_smem = (size_t)2 * n2 * ld * sizeof(float2) + sizeof(JacobiWork) + 2048 <= (size_t)c->dev_smem_optin;
+    const size_t smem2 = (size_t)(v_in_smem ? 2 : 1) * n2 * ld * sizeof(float2);
     double *T = c->d_gram + 2 * (size_t)q * q, *Bm = T + 2 * (size_t)q * q;
-    // a thread per element of a round's V update, beside the rotations' warp
-    const int nthr = std::min(1024, 32 + ((q + 1) / 2 * q + 31) / 32 * 32);
+    // one warp a pair for V, as far as 1024 threads go
+    const int nthr = std::min(1024, jacobi_block_threads(q) + 32 * std::max(3, (q + 1) / 2));
     prof_begin(c, KID_EIG);
     k_eig<<<1, nthr, smem2, c->stream>>>(gram, q, c->n, c->nc, c->dims.rank, c->rmax, c->prm.energy_pct, c->d_V,
                                         c->d_Q, c->d_meta + MT_COUNT, c->d_sigma, c->d_meta, c->d_status, v_in_smem,
