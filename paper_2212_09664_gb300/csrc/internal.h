@@ -167,6 +167,8 @@ struct lrccs_ctx {
     float2 *d_hpart;             // gd_grid * q * rmax  per-block partial sums of h = U^H Z (k_gdqr)
     cudaStream_t side;           // parallel branch of the iteration (k_zb beside the adjoint passes)
     cudaEvent_t ev_fork, ev_join;
+    cudaEvent_t ev_counts;       // h_counts has arrived
+    int32_t *h_counts;           // pinned: the data load's meta block, then its status word
 
     // general (2D) masks: the union Omega_u of the frames' samples, kept row by
     // row (points of row ky at u in [uptr[ky], uptr[ky+1]), ascending kx)
