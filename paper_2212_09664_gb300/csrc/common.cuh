@@ -467,6 +467,28 @@ LRCCS_DEV void two_sum(float a, float b, float &s, float &e) {
     const float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
 }
+// FP32 sums of products without error: a product is the exact pair (p,
+// fma(a, b, -p)), and p, its error term and the rounding of every addition go
+// into three levels of two_sum (about 72 bits, more than an FP64 accumulator
+// holds).  A product that leaves the FP32 range, or whose error term would (and
+// NaN), goes to the FP64 sum `wide`.
+struct fsum3 {
+    float a, b, c;
+};
+LRCCS_DEV void fsum3_mul(fsum3 &s, double &wide, float a, float b) {
+    const float p = __fmul_rn(a, b), ap = fabsf(p);
+    if (!(ap <= 1e30f && (ap >= 1e-26f || a == 0.f || b == 0.f))) {
+        wide += (double)a * (double)b;
+        return;
+    }
+    float e, f;
+    two_sum(s.a, p, s.a, e);
+    two_sum(s.b, e, s.b, f);
+    s.c += f;
+    two_sum(s.b, fmaf(a, b, -p), s.b, f);
+    s.c += f;
+}
+LRCCS_DEV double fsum3_total(const fsum3 &s) { return (double)s.a + ((double)s.b + (double)s.c); }
 LRCCS_DEV void fsum_add(fsum2 &acc, float x) {
     float s, e;
     two_sum(acc.hi, x, s, e);

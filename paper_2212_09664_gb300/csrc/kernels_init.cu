@@ -260,34 +260,8 @@ cudaError_t launch_fill_lines(lrccs_ctx *c) {
 // gamma = trunc * sum |y|^2 / (number of measured entries)  (Alg. 2, init).
 // FP64 adds bound an FP64 sum here (two a cycle per multiprocessor: 50 us for
 // 2.7 M entries, 403 us for 34 M), so each thread sums in FP32 without error:
-// a square is the exact pair (p, fma(x, x, -p)), and p, its error term and the
-// rounding of every addition go into three levels of two_sum (about 72 bits,
-// more than an FP64 accumulator holds); threads and blocks add in FP64 in a
-// fixed order: 17 us and 93 us.
-
-struct fsum3 {
-    float a, b, c;
-};
-LRCCS_DEV void fsum3_add(fsum3 &s, float x) {
-    float e, f;
-    two_sum(s.a, x, s.a, e);
-    two_sum(s.b, e, s.b, f);
-    s.c += f;
-}
-// x^2, exactly, where neither the square nor its error term leaves the FP32
-// range (and not NaN); anything else goes to the FP64 sum
-LRCCS_DEV void fsum3_sq(fsum3 &s, double &wide, float x) {
-    const float ax = fabsf(x);
-    if (!(ax <= 1e15f && (ax >= 1e-13f || ax == 0.f))) {
-        wide += (double)x * (double)x;
-        return;
-    }
-    const float p = __fmul_rn(x, x);
-    float f;
-    fsum3_add(s, p);
-    two_sum(s.b, fmaf(x, x, -p), s.b, f);
-    s.c += f;
-}
+// fsum3 (common.cuh); threads and blocks add in FP64 in a fixed order: 17 us and
+// 93 us.
 
 __global__ void __launch_bounds__(256) k_energy(const float2 *__restrict__ y, int64_t count, double trunc, double *part,
                                                 unsigned int *counter, double *scal) {
@@ -302,16 +276,16 @@ __global__ void __launch_bounds__(256) k_energy(const float2 *__restrict__ y, in
         for (int u = 0; u < 4; ++u) v[u] = __ldg(y + i + u * step);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            fsum3_sq(s, wide, v[u].x);
-            fsum3_sq(s, wide, v[u].y);
+            fsum3_mul(s, wide, v[u].x, v[u].x);
+            fsum3_mul(s, wide, v[u].y, v[u].y);
         }
     }
     for (; i < count; i += step) {
         const float2 v = __ldg(y + i);
-        fsum3_sq(s, wide, v.x);
-        fsum3_sq(s, wide, v.y);
+        fsum3_mul(s, wide, v.x, v.x);
+        fsum3_mul(s, wide, v.y, v.y);
     }
-    const double acc = warp_sum_d(wide + ((double)s.a + ((double)s.b + (double)s.c)));
+    const double acc = warp_sum_d(wide + fsum3_total(s));
     if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -70,7 +70,7 @@ int npairs_of(int r) { return r * (r + 1) / 2; }
 // twiddles, and a half-warp stages the coil map's few x of its own rows by
 // cp.async one coil ahead, which needs no further block barrier.
 //
-// Which rows are sampled comes as bit tables (k_row_tables): entry e holds, per
+// Which rows are sampled comes as bit tables (k_structure): entry e holds, per
 // group, the rows of pass 2 of the forward transform ([e][0..15]) and of pass 1
 // of the adjoint ([e][16..31]); column l uses entry e0 + l estep.
 #define COLW 16
