@@ -84,10 +84,11 @@ static void free_all(lrccs_ctx *c) {
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->ev_counts) cudaEventDestroy(c->ev_counts);
+    if (c->ev_copied) cudaEventDestroy(c->ev_copied);
     if (c->side) cudaStreamDestroy(c->side);
     if (c->h_counts) cudaFreeHost(c->h_counts);
     c->side = nullptr;
-    c->ev_fork = c->ev_join = c->ev_counts = nullptr;
+    c->ev_fork = c->ev_join = c->ev_counts = c->ev_copied = nullptr;
     c->h_counts = nullptr;
     void *ptrs[] = {c->d_twy, c->d_twx, c->d_smaps, c->d_rowcnt, c->d_rowidx, c->d_framerows, c->d_lineptr,
                     c->d_rfptr, c->d_rflist, c->d_usedrows, c->d_rowused, c->d_idx, c->d_meta, c->d_status,
@@ -268,6 +269,7 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_counts, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_copied, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->h_counts, (MT_COUNT + 1) * sizeof(int32_t), cudaHostAllocDefault);
     if (e == cudaSuccess) e = launch_twiddles(c->d_twy, ny, c->stream);
     if (e == cudaSuccess) e = launch_twiddles(c->d_twx, c->nx, c->stream);
@@ -393,16 +395,14 @@ static bool grow_work(lrccs_ctx *c, float2 **buf, size_t *cap, size_t need) {
     return true;
 }
 
-// Mask compaction, the sampled-row structure and Z = [A_k^H y_k] for the data
-// of one lrccs_init or tracking call; with_energy also forms gamma and the
-// truncated X0, which only the spectral initialisation uses.  Waits for the compaction's
-// counts (twice for a general 2D mask: once for the row structure, once for
-// the union of the frames' samples): counts and status come together in pinned
-// memory, and the copies of the maps and the mask run while the host wakes (one
-// online frame, 128 x 128, 12 coils: 321 us a call with two waits through
-// pageable memory behind those copies, 302 us so).
-static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_frame_ptr, const uint8_t *d_mask,
-                              const void *d_smaps, bool with_energy) {
+// The work of load_data, queued.  Waits for the compaction's counts (twice for a
+// general 2D mask: once for the row structure, once for the union of the frames'
+// samples): counts and status come together in pinned memory, and the copies of
+// the maps and the mask run while the host wakes (one online frame, 128 x 128,
+// 12 coils: 321 us a call with two waits through pageable memory behind those
+// copies, 302 us so).
+static lrccs_status queue_load(lrccs_ctx *c, const void *d_y, const int64_t *d_frame_ptr, const uint8_t *d_mask,
+                               const void *d_smaps, bool with_energy) {
     CK(cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream));
     CK(cudaMemsetAsync(c->d_counters, 0, CNT_COUNT * sizeof(unsigned), c->stream));
     CK(cudaMemsetAsync(c->d_meta, 0, MT_COUNT * sizeof(int32_t), c->stream));
@@ -414,12 +414,10 @@ static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_fr
     CK(cudaMemcpyAsync(c->d_smaps, d_smaps, (size_t)c->nc * c->n * sizeof(float2), cudaMemcpyDeviceToDevice,
                        c->stream));
     CK(cudaMemcpyAsync(c->d_maskc, d_mask, (size_t)c->q * c->n, cudaMemcpyDeviceToDevice, c->stream));
+    CK(cudaEventRecord(c->ev_copied, c->stream));
     CK(cudaEventSynchronize(c->ev_counts));
     lrccs_status s = status_to_code(c, (unsigned)meta[MT_COUNT]);
-    if (s != LRCCS_OK) {
-        cudaStreamSynchronize(c->stream);   // the copies read the caller's arrays
-        return s;
-    }
+    if (s != LRCCS_OK) return s;
     c->n_used = meta[MT_NUSED];
     c->n_lines = meta[MT_NLINES];
     c->m_max = meta[MT_MMAX];
@@ -428,7 +426,6 @@ static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_fr
     c->n_u = 0;
     if (c->total == 0 || c->n_used == 0) {
         set_err(c, "no sampled k-space");
-        cudaStreamSynchronize(c->stream);
         return LRCCS_E_INVALID;
     }
     if (c->general) {
@@ -447,6 +444,20 @@ static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_fr
     if (with_energy) CK(launch_energy(c, (const float2 *)d_y));
     CK(launch_init_adjoint(c, (const float2 *)d_y, with_energy));
     return LRCCS_OK;
+}
+
+// Mask compaction, the sampled-row structure and Z = [A_k^H y_k] for the data
+// of one lrccs_init or tracking call; with_energy also forms gamma and the
+// truncated X0, which only the spectral initialisation uses.  The caller may
+// change its frame offsets, mask and maps as soon as this returns, whatever it
+// returns: the copies out of them are waited for here, behind the launches that
+// follow them.
+static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_frame_ptr, const uint8_t *d_mask,
+                              const void *d_smaps, bool with_energy) {
+    const lrccs_status s = queue_load(c, d_y, d_frame_ptr, d_mask, d_smaps, with_energy);
+    if (s == LRCCS_OK) CK(cudaEventSynchronize(c->ev_copied));
+    else cudaStreamSynchronize(c->stream);
+    return s;
 }
 
 extern "C" lrccs_status lrccs_init(lrccs_ctx *c, const void *d_y, const int64_t *d_frame_ptr, const uint8_t *d_mask,

@@ -168,6 +168,7 @@ struct lrccs_ctx {
     cudaStream_t side;           // parallel branch of the iteration (k_zb beside the adjoint passes)
     cudaEvent_t ev_fork, ev_join;
     cudaEvent_t ev_counts;       // h_counts has arrived
+    cudaEvent_t ev_copied;       // the data load has read the caller's maps and mask
     int32_t *h_counts;           // pinned: the data load's meta block, then its status word
 
     // general (2D) masks: the union Omega_u of the frames' samples, kept row by
