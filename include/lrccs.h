@@ -206,7 +206,8 @@ lrccs_status lrccs_get_images(lrccs_ctx *ctx, void *d_X);
 
 /* Diagnostics: copy an internal array to caller device memory.
  *   LRCCS_BUF_Z     Z = [A_k^H y_k]            n x q, row-major (i * q + k)
- *   LRCCS_BUF_X0    truncated, scaled X0       n x q, row-major (of the last lrccs_init)
+ *   LRCCS_BUF_X0    truncated, scaled X0       n x q, row-major: of the data loaded last,
+ *                   truncated at the gamma of the last lrccs_init (zeros before any)
  *   LRCCS_BUF_GRAD  last gradient              n x r, row-major
  *   LRCCS_BUF_SIGMA singular values of X0      q float64, descending
  *   LRCCS_BUF_IDX   compacted sample indices   fp[q] int32 (ascending per frame)

@@ -279,6 +279,8 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_scal, 0, SC_COUNT * sizeof(double), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_meta, 0, ((size_t)MT_COUNT + q) * sizeof(int32_t), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_X0, 0, (size_t)n * q * F2, c->stream);
+    c->x0_zero = 1;
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         set_err(nullptr, "lrccs_create: %s", cudaGetErrorString(e));
@@ -441,14 +443,25 @@ static lrccs_status queue_load(lrccs_ctx *c, const void *d_y, const int64_t *d_f
     if (c->dims.precision != LRCCS_PREC_FP32_FFT) CK(launch_dft_a(c));   // DFT rows of the sampled rows
     // the init transforms up to 16 frames at a time where the memory allows it (rmax otherwise)
     grow_work(c, &c->d_T, &c->T_cap, (size_t)c->nc * c->n * std::min(16, c->q));
-    if (with_energy) CK(launch_energy(c, (const float2 *)d_y));
-    CK(launch_init_adjoint(c, (const float2 *)d_y, with_energy));
+    if (with_energy) {
+        CK(launch_energy(c, (const float2 *)d_y));
+        c->has_gamma = 1;
+    }
+    // X0 of the loaded data, truncated at the gamma of the last lrccs_init (0 before
+    // any: everything is dropped and no transform has to run for it)
+    if (c->has_gamma) {
+        c->x0_zero = 0;
+    } else if (!c->x0_zero) {
+        CK(cudaMemsetAsync(c->d_X0, 0, (size_t)c->n * c->q * sizeof(float2), c->stream));
+        c->x0_zero = 1;
+    }
+    CK(launch_init_adjoint(c, (const float2 *)d_y, c->has_gamma != 0));
     return LRCCS_OK;
 }
 
 // Mask compaction, the sampled-row structure and Z = [A_k^H y_k] for the data
-// of one lrccs_init or tracking call; with_energy also forms gamma and the
-// truncated X0, which only the spectral initialisation uses.  The caller may
+// of one lrccs_init or tracking call; with_energy also forms gamma, which only
+// the spectral initialisation's truncation uses.  The caller may
 // change its frame offsets, mask and maps as soon as this returns, whatever it
 // returns: the copies out of them are waited for here, behind the launches that
 // follow them.
@@ -475,6 +488,7 @@ extern "C" lrccs_status lrccs_init(lrccs_ctx *c, const void *d_y, const int64_t 
     c->has_u = 0;
     c->need_h = 0;
     c->t = 0;
+    c->has_gamma = 0;
     CK(cudaMemsetAsync(c->d_scal, 0, SC_COUNT * sizeof(double), c->stream));
     lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, true);
     if (s != LRCCS_OK) return s;

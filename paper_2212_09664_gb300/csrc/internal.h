@@ -96,6 +96,8 @@ struct lrccs_ctx {
     int r;             // rank in use (after init)
     int initialized;   // data and subspace loaded (lrccs_init or a tracking call succeeded)
     int has_u;         // d_U holds a subspace (init, lrccs_set_subspace, lrccs_set_state, tracking)
+    int has_gamma;     // d_scal[SC_GAMMA] is the last lrccs_init's
+    int x0_zero;       // d_X0 holds zeros
     int need_h;        // d_U was set from outside: re-orthonormalise it and form U^H Z before iterating
     int t;             // iterations run since init
     int px, py;        // nx / 32, ny / 32

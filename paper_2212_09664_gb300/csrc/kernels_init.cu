@@ -320,9 +320,8 @@ cudaError_t launch_energy(lrccs_ctx *c, const float2 *d_y) {
 // rest and writes column k0 + l of Z or X0.  Any mask takes this path (full
 // lines only make the scatter the identity).  Z and X0, kernel time: 16 spokes on
 // 256 x 256, q = 64, C = 20: direct sums over each row's samples in one kernel 3.22 ms
-// -> 8 chunks of 108 + 89 us; 8 frames of 224 x 224 (Z alone, which is all that
-// tracking needs): 0.98 ms -> 26 + 50 us; lines of 192 x 192, q = 48, C = 12: 36 + 175 us
-// -> 6 chunks of 15 + 23 us.
+// -> 8 chunks of 108 + 89 us; 8 frames of 224 x 224 (Z alone): 0.98 ms -> 26 + 50 us;
+// lines of 192 x 192, q = 48, C = 12: 36 + 175 us -> 6 chunks of 15 + 23 us.
 //
 // Row pass: block (row ky, coil group); only the nf frames of the chunk that
 // sample ky take part.  Item (frame c, g): its length-R1 DFT takes kx = g + R2 m
@@ -476,7 +475,7 @@ static cudaError_t launch_init_rows(lrccs_ctx *c, const float2 *d_y, int w, int 
     return cudaGetLastError();
 }
 
-// Z, and with trunc also X0 (which only the spectral initialisation reads).
+// Z, and with trunc also X0.
 cudaError_t launch_init_adjoint(lrccs_ctx *c, const float2 *d_y, bool trunc) {
     const int wmax = (int)std::min<size_t>(16, c->T_cap / ((size_t)c->nc * c->n));
     const int nch = (c->q + wmax - 1) / wmax, w = (c->q + nch - 1) / nch;
