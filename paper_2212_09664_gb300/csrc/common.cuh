@@ -475,18 +475,22 @@ LRCCS_DEV void two_sum(float a, float b, float &s, float &e) {
 struct fsum3 {
     float a, b, c;
 };
-LRCCS_DEV void fsum3_mul(fsum3 &s, double &wide, float a, float b) {
-    const float p = __fmul_rn(a, b), ap = fabsf(p);
-    if (!(ap <= 1e30f && (ap >= 1e-26f || a == 0.f || b == 0.f))) {
-        wide += (double)a * (double)b;
-        return;
-    }
+LRCCS_DEV void fsum3_product(fsum3 &s, float a, float b) {   // 0 or 1e-26 <= |a b| <= 1e30
+    const float p = __fmul_rn(a, b);
     float e, f;
     two_sum(s.a, p, s.a, e);
     two_sum(s.b, e, s.b, f);
     s.c += f;
     two_sum(s.b, fmaf(a, b, -p), s.b, f);
     s.c += f;
+}
+LRCCS_DEV void fsum3_mul(fsum3 &s, double &wide, float a, float b) {
+    const float ap = fabsf(__fmul_rn(a, b));
+    if (!(ap <= 1e30f && (ap >= 1e-26f || a == 0.f || b == 0.f))) {
+        wide += (double)a * (double)b;
+        return;
+    }
+    fsum3_product(s, a, b);
 }
 LRCCS_DEV double fsum3_total(const fsum3 &s) { return (double)s.a + ((double)s.b + (double)s.c); }
 LRCCS_DEV void fsum_add(fsum2 &acc, float x) {

@@ -213,9 +213,11 @@ __global__ void __launch_bounds__(256) k_mec_dir(const float2 *__restrict__ S, f
 // thread forms output f (with q even also f + q/2, whose sum differs only in the
 // sign of the odd inputs, so half the products serve both) for TD_P pixels at
 // once: per input frame one twiddle and four broadcast 16-byte reads feed the
-// 8 complex products, which FP32 issue bounds.  H = q/2 or q output pairs by
-// 256 / H pixel groups fill the block.  192 x 192, q = 48, kernel time: 327 + 42
-// (the sums of its blocks) -> 63 us forward, 45 -> 29 us back.
+// 8 complex products.  H = q/2 or q output pairs by 256 / H pixel groups fill
+// the block.  192 x 192, q = 48, kernel time: 327 + 42 (the sums of its blocks) ->
+// 35 us forward, 45 -> 28 us back: about six times what their products take at
+// the FP32 rate; 461 blocks on the 456 places that 77 registers a thread leave, so
+// a second, nearly empty round is about half of either.
 #define TD_P 8                  // pixels per thread
 #define TD_S (TD_P + 2)         // shared stride of a frame's pixels (16-byte aligned, spread over the banks)
 
@@ -292,24 +294,16 @@ LRCCS_DEV void td_fill(float2 *s_g, int q, int w, int n, int pix, GET get) {
 }
 
 // M[:, i] = F_t (E + S0 - V)[i, :] (unitary DFT over the q frames, tw[t] =
-// exp(-2 pi i t / q)), and over the whole grid max |M| (first step only, Mprev
-// NULL) or sum |M - Mprev|^2 and sum |Mprev|^2 into out[3]: FP32 pairs that keep
-// the rounding of every square and addition per thread, FP64 from there, in a
-// fixed order.
-LRCCS_DEV void fsum_sq(fsum2 &s, float x) {
-    const float p = __fmul_rn(x, x);
-    fsum_add(s, p);
-    s.lo += fmaf(x, x, -p);
-}
+// exp(-2 pi i t / q)); with part != NULL (the first step) also max |M| over the
+// whole grid into *top.
 __global__ void __launch_bounds__(256, 3) k_tdft_fwd(const float2 *__restrict__ E, const float2 *__restrict__ S0,
-                                                     const float2 *__restrict__ V, const float2 *__restrict__ Mprev,
-                                                     const float2 *__restrict__ tw, int n, int q, int w,
-                                                     float2 *__restrict__ M, double *part, unsigned int *counter,
-                                                     double *out) {
+                                                     const float2 *__restrict__ V, const float2 *__restrict__ tw, int n,
+                                                     int q, int w, float2 *__restrict__ M, double *part,
+                                                     unsigned int *counter, double *top) {
     extern __shared__ __align__(16) float2 s_g[];
     const TdShape t = td_shape(q);
     float2 *s_tw = s_g + (size_t)t.groups * q * TD_S;
-    __shared__ double s_r[3][8];
+    __shared__ double s_r[8];
     const int i0 = blockIdx.x * t.pix, lane = threadIdx.x & 31;
     const float sc = rsqrtf((float)q);
     for (int i = threadIdx.x; i < q; i += blockDim.x) s_tw[i] = tw[i];
@@ -319,8 +313,7 @@ __global__ void __launch_bounds__(256, 3) k_tdft_fwd(const float2 *__restrict__ 
         return g;
     });
     __syncthreads();
-    double mx = 0.0;
-    fsum2 dd = {0.f, 0.f}, pp = {0.f, 0.f};
+    double mx = 0.0;   // max |M|^2
     const int pg = threadIdx.x / t.H, f0 = threadIdx.x - pg * t.H;
     if (pg < t.groups) {
         float2 lo[TD_P], hi[TD_P];
@@ -331,60 +324,101 @@ __global__ void __launch_bounds__(256, 3) k_tdft_fwd(const float2 *__restrict__ 
             for (int p = 0; p < TD_P; ++p) {
                 const int i = i0 + pg * TD_P + p;
                 if (i >= n) continue;
-                const size_t o = ((size_t)cc * n + i) * w + l;
                 const float2 m = cscale(v[p], sc);
-                M[o] = m;
-                if (Mprev) {
-                    const float2 m0 = Mprev[o];
-                    float d, e;   // the difference and its rounding, exactly
-                    two_sum(m.x, -m0.x, d, e);
-                    fsum_sq(dd, d);
-                    dd.lo += 2.f * d * e;
-                    two_sum(m.y, -m0.y, d, e);
-                    fsum_sq(dd, d);
-                    dd.lo += 2.f * d * e;
-                    fsum_sq(pp, m0.x);
-                    fsum_sq(pp, m0.y);
-                } else {
-                    mx = fmax(mx, (double)m.x * m.x + (double)m.y * m.y);
-                }
+                M[((size_t)cc * n + i) * w + l] = m;
+                if (part) mx = fmax(mx, (double)m.x * m.x + (double)m.y * m.y);
             }
         };
         put(lo, f0);
         if (!(q & 1)) put(hi, f0 + t.H);
     }
-    // block, then grid: [0] max |M|^2, [1] sum |M - Mprev|^2, [2] sum |Mprev|^2
-    double v[3] = {mx, (double)dd.hi + (double)dd.lo, (double)pp.hi + (double)pp.lo};
-    for (int o = 16; o > 0; o >>= 1) v[0] = fmax(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
-    v[1] = warp_sum_d(v[1]);
-    v[2] = warp_sum_d(v[2]);
-    if (lane == 0)
-        for (int c = 0; c < 3; ++c) s_r[c][threadIdx.x >> 5] = v[c];
+    if (!part) return;
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) s_r[threadIdx.x >> 5] = mx;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0, c = 0.0;
-        for (int x = 0; x < 8; ++x) {
-            a = fmax(a, s_r[0][x]);
-            b += s_r[1][x];
-            c += s_r[2][x];
+        for (int x = 1; x < 8; ++x) mx = fmax(mx, s_r[x]);
+        part[blockIdx.x] = mx;
+    }
+    if (!last_block_arrive(counter) || threadIdx.x >= 32) return;
+    mx = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) mx = fmax(mx, __ldcg(part + b));
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) *top = sqrt(mx);
+}
+
+// sum |M - Mprev|^2 and sum |Mprev|^2 over the frames k < q into out[0], out[1]
+// (blocks along the pixels, chunks).  FP32 without error per thread (fsum3; a
+// difference is its rounded value d and that rounding e, exactly), FP64 from
+// there, in a fixed order.  FP64 work bounds every form that does more of it
+// (192 x 192, q = 48: 43 us all in FP64, 52 us with a range test and an FP64 side
+// path at each product), so one test covers an entry's four values and an entry
+// outside the range goes to FP64 as a whole: 21 us.  As a part of k_tdft_fwd, where
+// few warps are in flight, FP32 pairs took 28 us and lost the squares that leave
+// the FP32 range.
+#define TD_CHANGE_BLOCKS 1024   // at most
+LRCCS_DEV void td_diff(fsum3 &s, float d, float e) {   // (d + e)^2, |e| at most half an ulp of d
+    fsum3_product(s, d, d);
+    const float a = 2.f * d, p = __fmul_rn(a, e);
+    float f;
+    two_sum(s.b, p, s.b, f);
+    s.c += f + (fmaf(a, e, -p) + e * e);
+}
+__global__ void __launch_bounds__(256) k_tdft_change(const float2 *__restrict__ M, const float2 *__restrict__ Mprev,
+                                                     int n, int q, int w, double *part, unsigned int *counter,
+                                                     double *out) {
+    __shared__ double s_r[2][8];
+    const unsigned total = (unsigned)n * w;
+    const int cc = blockIdx.y, live = min(w, q - cc * w), lane = threadIdx.x & 31;
+    const float2 *Mc = M + (size_t)cc * total, *Pc = Mprev + (size_t)cc * total;
+    double dw = 0.0, pw = 0.0;
+    fsum3 dd = {0.f, 0.f, 0.f}, pp = {0.f, 0.f, 0.f};
+#pragma unroll 2
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        if (live < w && (int)(i % (unsigned)w) >= live) continue;   // columns past q
+        const float2 m = __ldg(Mc + i), m0 = __ldg(Pc + i);
+        float dx, ex, dy, ey;
+        two_sum(m.x, -m0.x, dx, ex);
+        two_sum(m.y, -m0.y, dy, ey);
+        // the smallest (zeros left out) and the largest magnitude, NaN above all, as bits
+        unsigned lo = ~0u, hi = 0u;
+        auto span = [&](float v) {
+            const unsigned b = __float_as_uint(v) & 0x7fffffffu;
+            lo = min(lo, b - 1u);
+            hi = max(hi, b);
+        };
+        span(dx);
+        span(dy);
+        span(m0.x);
+        span(m0.y);
+        if (lo >= __float_as_uint(1e-13f) && hi <= __float_as_uint(1e15f)) {
+            td_diff(dd, dx, ex);
+            td_diff(dd, dy, ey);
+            fsum3_product(pp, m0.x, m0.x);
+            fsum3_product(pp, m0.y, m0.y);
+        } else {
+            const double x = (double)m.x - (double)m0.x, y = (double)m.y - (double)m0.y;
+            dw += x * x + y * y;
+            pw += (double)m0.x * m0.x + (double)m0.y * m0.y;
         }
-        part[(size_t)blockIdx.x * 3] = a;
-        part[(size_t)blockIdx.x * 3 + 1] = b;
-        part[(size_t)blockIdx.x * 3 + 2] = c;
     }
-    if (!last_block_arrive(counter) || threadIdx.x >= 96) return;
-    const int c = threadIdx.x >> 5;   // a warp per result
+    const double a = warp_sum_d(dw + fsum3_total(dd)), b = warp_sum_d(pw + fsum3_total(pp));
+    if (lane == 0) {
+        s_r[0][threadIdx.x >> 5] = a;
+        s_r[1][threadIdx.x >> 5] = b;
+    }
+    __syncthreads();
+    const int id = blockIdx.y * gridDim.x + blockIdx.x, nb = gridDim.x * gridDim.y;
+    if (threadIdx.x < 2) {
+        double v = 0.0;
+        for (int x = 0; x < 8; ++x) v += s_r[threadIdx.x][x];
+        part[2 * id + threadIdx.x] = v;
+    }
+    if (!last_block_arrive(counter) || threadIdx.x >= 64) return;
+    const int c = threadIdx.x >> 5;   // a warp per sum
     double r = 0.0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) {
-        const double x = __ldcg(part + (size_t)b * 3 + c);
-        r = c == 0 ? fmax(r, x) : r + x;
-    }
-    if (c == 0) {
-        for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
-        r = sqrt(r);
-    } else {
-        r = warp_sum_d(r);
-    }
+    for (int x = lane; x < nb; x += 32) r += __ldcg(part + 2 * x + c);
+    r = warp_sum_d(r);
     if (lane == 0) out[c] = r;
 }
 
@@ -465,14 +499,23 @@ cudaError_t launch_mec_out(lrccs_ctx *c, const float2 *E, const float2 *zbar, fl
     return launch_images_mec(c, KID_MEC_ELEM, zbar, E, c->mec_w, Eout, Xout);
 }
 
+// M, then out[0] = max |M| (Mprev NULL: the first step), or out[1], out[2] = the sums of k_tdft_change
 cudaError_t launch_tdft_fwd(lrccs_ctx *c, const float2 *E, const float2 *S0, const float2 *V, const float2 *Mprev,
                             float2 *M, double *out) {
     const TdShape t = td_shape(c->q);
     double *part = c->d_mscal + 3 * c->q;
+    unsigned int *cnt = c->d_counters + CNT_MEC;
     prof_begin(c, KID_MEC_TDFT);
-    k_tdft_fwd<<<(c->n + t.pix - 1) / t.pix, 256, t.smem, c->stream>>>(E, S0, V, Mprev, c->d_twq, c->n, c->q, c->mec_w, M,
-                                                                      part, c->d_counters + CNT_MEC, out);
+    k_tdft_fwd<<<(c->n + t.pix - 1) / t.pix, 256, t.smem, c->stream>>>(E, S0, V, c->d_twq, c->n, c->q, c->mec_w, M,
+                                                                       Mprev ? nullptr : part, cnt, out);
     prof_end(c, KID_MEC_TDFT);
+    if (Mprev) {
+        dim3 grid = mec_grid(c);
+        grid.x = std::max(1u, std::min(grid.x, (unsigned)TD_CHANGE_BLOCKS / grid.y));
+        prof_begin(c, KID_MEC_TDFT);
+        k_tdft_change<<<grid, 256, 0, c->stream>>>(M, Mprev, c->n, c->q, c->mec_w, part, cnt, out + 1);
+        prof_end(c, KID_MEC_TDFT);
+    }
     return cudaGetLastError();
 }
 
@@ -485,11 +528,12 @@ cudaError_t launch_tdft_inv(lrccs_ctx *c, const float2 *M, float omega, float2 *
 }
 
 // Scratch of the reductions: 3 q FP64 scalars, then the partials of the frame
-// sums (G per column) or of the temporal transform (3 per block).
+// sums (G per column), of the temporal transform (1 per block) or of its change
+// (2 per block).
 size_t mec_scal_count(int n, int q, int w) {
     const int nch = (q + w - 1) / w, pix = td_shape(q).pix;
-    const size_t a = (size_t)MEC_G * nch * w, b = (size_t)3 * ((n + pix - 1) / pix);
-    return (size_t)3 * q + (a > b ? a : b) + 8;
+    const size_t a = (size_t)MEC_G * nch * w, b = (n + pix - 1) / pix;
+    return (size_t)3 * q + std::max({a, b, (size_t)2 * TD_CHANGE_BLOCKS}) + 8;
 }
 
 cudaError_t configure_kernels_mec(int max_smem) {
