@@ -95,7 +95,8 @@ typedef struct lrccs_params {
     int32_t t_max;         /* 70   : iteration cap used by callers that solve to completion */
     int32_t exit_enabled;  /* 1: lrccs_iterate stops at the exit test (one host sync per iteration) */
     double admit_reserve_bytes;  /* 256 MiB: device memory that must stay free after lrccs_create's
-                                    buffers, or the context is not admitted (LRCCS_E_ADMISSION) */
+                                    buffers, or the context is not admitted (LRCCS_E_ADMISSION);
+                                    later calls widen their transform buffers only beside it */
     /* tuning variants from the paper's discussion of its limitations (the
        defaults give Alg. 2 as printed) */
     int32_t exit_patience; /* 1    : with exit_enabled, stop once this many consecutive iterations
@@ -152,9 +153,8 @@ lrccs_status lrccs_create(const lrccs_dims *dims, const lrccs_params *params,
 
 /* Device bytes lrccs_create would allocate for dims (each buffer rounded up to
  * 256 bytes).  Not included: the general-mask and MEC work space and wider
- * transform buffers, allocated by the first call that needs them where the
- * memory allows (see lrccs_init, lrccs_mec1).  Allocates
- * nothing.  Errors: LRCCS_E_INVALID, LRCCS_E_UNSUPPORTED. */
+ * transform buffers, allocated by the first call that needs them (see
+ * lrccs_init, lrccs_mec1).  Allocates nothing.  Errors: LRCCS_E_INVALID, LRCCS_E_UNSUPPORTED. */
 lrccs_status lrccs_context_bytes(const lrccs_dims *dims, size_t *bytes);
 
 /* Spectral initialisation (Alg. 2, initialisation) from the measurements.
@@ -170,7 +170,8 @@ lrccs_status lrccs_context_bytes(const lrccs_dims *dims, size_t *bytes);
  * The first general (2D) mask a context sees allocates that path's buffers
  * (about 2 q n int32 plus C n rank_max complex64).  The first data load widens
  * the transform buffer to min(q, 16) frames (C n min(q, 16) complex64) if that
- * is above rank_max and fits the device memory.
+ * is above rank_max and leaves admit_reserve_bytes of device memory free; the
+ * context gives it back when one of its calls needs the memory.
  * Errors: LRCCS_E_INVALID (frame_ptr inconsistent with the mask, or a fixed
  * rank above q: the top-r singular vectors of the n x q X0 need r <= q),
  * LRCCS_E_RANK_DEFICIENT (sigma_r(X0) = 0), LRCCS_E_NOMEM, LRCCS_E_CUDA. */
@@ -263,9 +264,9 @@ lrccs_status lrccs_mean_step(lrccs_ctx *ctx, const void *d_y, const int64_t *d_f
  * The frames are processed up to 16 at a time through the per-frame normal
  * operators A_k^H A_k (the iteration's transforms with each frame's own
  * sampling between them).  The first call allocates 5 q n complex64 of work
- * space in the context and, where the memory allows, widens its transform
- * buffers to the frames processed at a time.  Both calls synchronise (MEC-2 reads its stopping test
- * after every step).  Errors: LRCCS_E_STATE (no iterate yet), LRCCS_E_INVALID,
+ * space in the context and then, where admit_reserve_bytes stay free, widens its
+ * transform buffers to the frames processed at a time.  Both calls synchronise
+ * (MEC-2 reads its stopping test after every step).  Errors: LRCCS_E_STATE (no iterate yet), LRCCS_E_INVALID,
  * LRCCS_E_NOMEM, LRCCS_E_CUDA. */
 lrccs_status lrccs_mec1(lrccs_ctx *ctx, int32_t iters, const void *d_zbar, void *d_E, void *d_X);
 lrccs_status lrccs_mec2(lrccs_ctx *ctx, int32_t max_iter, double rel_change, double omega_frac,

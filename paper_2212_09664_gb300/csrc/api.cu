@@ -361,32 +361,19 @@ static lrccs_status sync_status(lrccs_ctx *c) {
     return status_to_code(c, st);
 }
 
-// Buffers of the general-mask path (allocated the first time a context sees
-// a mask with partly sampled rows).
-static lrccs_status ensure_general_buffers(lrccs_ctx *c) {
-    if (c->gen_cap_q) return LRCCS_OK;
-    const size_t n = (size_t)c->n, q = (size_t)c->q, ny = (size_t)c->ny;
-    const size_t npm = (size_t)c->rmax * (c->rmax + 1) / 2;
-    const bool ok = dalloc(c, &c->d_ucnt, n) && dalloc(c, &c->d_uloc, n) && dalloc(c, &c->d_floc, n) &&
-                    dalloc(c, &c->d_urow, 2 * ny) && dalloc(c, &c->d_uptr, ny + 1) &&
-                    dalloc(c, &c->d_ufrow, ny + 1) && dalloc(c, &c->d_upos, n) && dalloc(c, &c->d_uidx, n) &&
-                    dalloc(c, &c->d_ufptr, n + 1) && dalloc(c, &c->d_uflist, q * n) && dalloc(c, &c->d_fu, q * n) &&
-                    dalloc(c, &c->d_FU, (size_t)c->nc * n * c->rmax) && dalloc(c, &c->d_Pu, n * npm) &&
-                    dalloc(c, &c->d_fpart, frame_gram_part_count(c->q, c->rmax));
-    if (!ok) return LRCCS_E_NOMEM;
-    c->gen_cap_q = q;
-    c->FU_cap = (size_t)c->nc * n * c->rmax;
-    return LRCCS_OK;
-}
+// The transform work buffers T and FU hold rank_max columns; up to 16 columns
+// (frames) at a time run faster, so calls widen them where the memory allows it.
+static size_t base_work(const lrccs_ctx *c) { return (size_t)c->nc * c->n * c->rmax; }
 
-static void drop_iter_graph(lrccs_ctx *c);
-
-// Grow a transform work buffer to `need` complex values, keeping the old one
-// when the larger does not fit the device memory.
+// Widen a work buffer to `need` complex values, if the new buffer beside the old
+// one leaves the caller's reserve free; else keep the old one.
 static bool grow_work(lrccs_ctx *c, float2 **buf, size_t *cap, size_t need) {
     if (need <= *cap) return true;
+    size_t fr = 0, tot = 0;
+    const double reserve = c->prm.admit_reserve_bytes > 0.0 ? c->prm.admit_reserve_bytes : 0.0;
     float2 *p = nullptr;
-    if (cudaMalloc((void **)&p, need * sizeof(float2)) != cudaSuccess) {
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || (double)(need * sizeof(float2)) + reserve > (double)fr ||
+        cudaMalloc((void **)&p, need * sizeof(float2)) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -395,6 +382,45 @@ static bool grow_work(lrccs_ctx *c, float2 **buf, size_t *cap, size_t need) {
     *buf = p;
     *cap = need;
     return true;
+}
+
+// Give widened work buffers back; false when there was none.
+static bool shrink_work(lrccs_ctx *c) {
+    const struct { float2 **buf; size_t *cap; } w[] = {{&c->d_T, &c->T_cap}, {&c->d_FU, &c->FU_cap}};
+    bool any = false;
+    for (const auto &b : w) {
+        if (*b.cap <= base_work(c)) continue;
+        any = true;
+        drop_iter_graph(c);
+        cudaFree(*b.buf);
+        *b.cap = dalloc(c, b.buf, base_work(c)) ? base_work(c) : 0;
+    }
+    return any;
+}
+
+// A buffer that the call cannot do without, unless it is there: the widened work buffers make room for it.
+template <typename T>
+static bool need_buf(lrccs_ctx *c, T **p, size_t count) {
+    return *p || dalloc(c, p, count) || (shrink_work(c) && dalloc(c, p, count));
+}
+
+// Buffers of the general-mask path (allocated the first time a context sees
+// a mask with partly sampled rows).
+static lrccs_status ensure_general_buffers(lrccs_ctx *c) {
+    if (c->gen_cap_q) return LRCCS_OK;
+    const size_t n = (size_t)c->n, q = (size_t)c->q, ny = (size_t)c->ny;
+    const size_t npm = (size_t)c->rmax * (c->rmax + 1) / 2;
+    const bool ok = need_buf(c, &c->d_ucnt, n) && need_buf(c, &c->d_uloc, n) && need_buf(c, &c->d_floc, n) &&
+                    need_buf(c, &c->d_urow, 2 * ny) && need_buf(c, &c->d_uptr, ny + 1) &&
+                    need_buf(c, &c->d_ufrow, ny + 1) && need_buf(c, &c->d_upos, n) && need_buf(c, &c->d_uidx, n) &&
+                    need_buf(c, &c->d_ufptr, n + 1) && need_buf(c, &c->d_uflist, q * n) &&
+                    need_buf(c, &c->d_fu, q * n) && need_buf(c, &c->d_FU, base_work(c)) &&
+                    need_buf(c, &c->d_Pu, n * npm) &&
+                    need_buf(c, &c->d_fpart, frame_gram_part_count(c->q, c->rmax));
+    if (!ok) return LRCCS_E_NOMEM;
+    c->gen_cap_q = q;
+    c->FU_cap = base_work(c);
+    return LRCCS_OK;
 }
 
 // The work of load_data, queued.  Waits for the compaction's counts (twice for a
@@ -408,6 +434,10 @@ static lrccs_status queue_load(lrccs_ctx *c, const void *d_y, const int64_t *d_f
     CK(cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream));
     CK(cudaMemsetAsync(c->d_counters, 0, CNT_COUNT * sizeof(unsigned), c->stream));
     CK(cudaMemsetAsync(c->d_meta, 0, MT_COUNT * sizeof(int32_t), c->stream));
+    // (null only after a failed narrowing)
+    if (!c->d_T && dalloc(c, &c->d_T, base_work(c))) c->T_cap = base_work(c);
+    if (c->gen_cap_q && !c->d_FU && dalloc(c, &c->d_FU, base_work(c))) c->FU_cap = base_work(c);
+    if (!c->d_T || (c->gen_cap_q && !c->d_FU)) return LRCCS_E_NOMEM;
     CK(launch_compact(c, d_mask, d_frame_ptr));
     const int32_t *meta = c->h_counts;
     CK(cudaMemcpyAsync(c->h_counts, c->d_meta, MT_COUNT * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
@@ -819,31 +849,28 @@ extern "C" lrccs_status lrccs_mean_step(lrccs_ctx *c, const void *d_y, const int
 // costs little more for 16 columns than for 4, so the frames go in the fewest
 // chunks of at most 16 with the least padding: w = ceil(q / ceil(q / 16)), which
 // is also one column instead of rank_max for a single online frame.  Wider than
-// rank_max, the transform buffers grow once; when they cannot, w = rank_max.
+// rank_max, the transform buffers grow once, after the vectors (sized for either
+// width) have their memory; when they cannot, w = rank_max.
 static lrccs_status mec_ensure(lrccs_ctx *c) {
     int nch = (c->q + 15) / 16, w = (c->q + nch - 1) / nch;
-    const size_t need = (size_t)c->nc * c->n * w;
-    if (!grow_work(c, &c->d_T, &c->T_cap, need) || (c->general && !grow_work(c, &c->d_FU, &c->FU_cap, need))) {
-        w = w < c->rmax ? w : c->rmax;
-        nch = (c->q + w - 1) / w;
-    }
-    if (c->general) {   // the loaded masks' point tables
-        if (!c->d_ptab && !dalloc(c, &c->d_ptab, (size_t)c->q * c->ny * 32)) return LRCCS_E_NOMEM;
-        CK(launch_point_tables(c));
-    }
-    if (c->d_mec && c->mec_w == w) return LRCCS_OK;
-    if (c->d_mec) cudaFree(c->d_mec);
-    if (c->d_mscal) cudaFree(c->d_mscal);
-    c->d_mec = nullptr;
-    c->d_mscal = nullptr;
-    if (!dalloc(c, &c->d_mec, (size_t)5 * nch * c->n * w) || !dalloc(c, &c->d_mscal, mec_scal_count(c->n, c->q, w)) ||
-        (!c->d_mout && !dalloc(c, &c->d_mout, 8))) {
-        if (c->d_mec) cudaFree(c->d_mec);
-        if (c->d_mscal) cudaFree(c->d_mscal);
+    const int wn = std::min(w, c->rmax), nn = (c->q + wn - 1) / wn;
+    const size_t cols = std::max(nch * w, nn * wn);
+    const size_t scal = std::max(mec_scal_count(c->n, c->q, w), mec_scal_count(c->n, c->q, wn));
+    if (!need_buf(c, &c->d_mec, 5 * cols * c->n) || !need_buf(c, &c->d_mscal, scal) || !need_buf(c, &c->d_mout, 8) ||
+        (c->general && !need_buf(c, &c->d_ptab, (size_t)c->q * c->ny * 32)) || !c->d_T || (c->general && !c->d_FU)) {
+        cudaFree(c->d_mec);
+        cudaFree(c->d_mscal);
         c->d_mec = nullptr;
         c->d_mscal = nullptr;
+        if (!c->d_T || (c->gen_cap_q && !c->d_FU)) c->initialized = 0;   // the next data load brings them back
         return LRCCS_E_NOMEM;
     }
+    const size_t need = (size_t)c->nc * c->n * w;
+    if (!grow_work(c, &c->d_T, &c->T_cap, need) || (c->general && !grow_work(c, &c->d_FU, &c->FU_cap, need))) {
+        w = wn;
+        nch = nn;
+    }
+    if (c->general) CK(launch_point_tables(c));   // of the loaded masks
     c->mec_w = w;
     c->mec_nch = nch;
     return LRCCS_OK;
