@@ -175,8 +175,10 @@ LRCCS_DEV void gd_pair(const float2 *row, int A, float2 &p0, float2 &p1) {
 }
 
 // The block's partial sums of the cross-Gram tiles: thread (tile, slice) adds
-// pixels slice, slice + SL, ..., the slices of a tile (neighbouring lanes) add by
-// a fixed shuffle tree, and lane m writes entry m to part.
+// pixels slice, slice + SL, ... in two FP32 chains (SL is a power of two: one
+// chain a slice would be almost twice as long as NTG / tiles slices make it),
+// the slices of a tile (neighbouring lanes) add by a fixed shuffle tree, and lane
+// m writes entry m to part.
 template <int R, bool ITER>
 static __device__ void gd_grams(const float2 *s_u, const float2 *s_a, int rows, float2 *part) {
     using PL = GdPlan<R>;
@@ -196,20 +198,28 @@ static __device__ void gd_grams(const float2 *s_u, const float2 *s_a, int rows, 
         }
     }
     const float2 *X = kind == 0 ? s_a : s_u, *Y = kind == 2 ? s_u : s_a;
-    float2 acc[4];
+    float2 acc[4], ac2[4];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) acc[m] = make_float2(0.f, 0.f);
+    for (int m = 0; m < 4; ++m) acc[m] = ac2[m] = make_float2(0.f, 0.f);
     if (tile < T) {
-#pragma unroll 4
-        for (int i = sl; i < rows; i += SL) {
+        auto add = [&](float2 (&c)[4], int i) {
             float2 p0, p1, q0, q1;
             gd_pair<R>(X + i * RS, A, p0, p1);
             gd_pair<R>(Y + i * RS, Bt, q0, q1);
-            cfmac(acc[0], p0, q0);
-            cfmac(acc[1], p0, q1);
-            cfmac(acc[2], p1, q0);
-            cfmac(acc[3], p1, q1);
+            cfmac(c[0], p0, q0);
+            cfmac(c[1], p0, q1);
+            cfmac(c[2], p1, q0);
+            cfmac(c[3], p1, q1);
+        };
+        int i = sl;
+#pragma unroll 2
+        for (; i + SL < rows; i += 2 * SL) {
+            add(acc, i);
+            add(ac2, i + SL);
         }
+        if (i < rows) add(acc, i);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc[m] = cadd(acc[m], ac2[m]);
     }
 #pragma unroll
     for (int o = SL / 2; o > 0; o >>= 1)
