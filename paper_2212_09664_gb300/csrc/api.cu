@@ -565,7 +565,7 @@ static lrccs_status warm_start(lrccs_ctx *c) {
 // Capture n iterations (launch_iteration's kernels and, when kernels are being
 // timed, their event records; nothing else) as one CUDA graph on the
 // context's stream, cached per (n, timed kernels, rank, sampled rows, work
-// buffer).  Returns false when the graph cannot be built here (the legacy
+// buffers).  Returns false when the graph cannot be built here (the legacy
 // default stream cannot be captured); the caller then launches directly.
 static void drop_iter_graph(lrccs_ctx *c) {
     if (!c->iter_exec) return;
@@ -583,8 +583,8 @@ static void drop_iter_graph(lrccs_ctx *c) {
 
 static bool graph_matches(const lrccs_ctx *c, int n_iter) {
     return c->iter_exec && c->iter_n == n_iter && c->iter_mask == c->prof_mask && c->iter_r == c->r &&
-           c->iter_nused == c->n_used && c->iter_T == c->d_T && c->iter_general == c->general &&
-           c->iter_nu == c->n_u;
+           c->iter_nused == c->n_used && c->iter_T == c->d_T && c->iter_FU == c->d_FU &&
+           c->iter_general == c->general && c->iter_nu == c->n_u;
 }
 
 static bool ensure_iter_graph(lrccs_ctx *c, int n_iter) {
@@ -660,6 +660,7 @@ static bool ensure_iter_graph(lrccs_ctx *c, int n_iter) {
     c->iter_r = c->r;
     c->iter_nused = c->n_used;
     c->iter_T = c->d_T;
+    c->iter_FU = c->d_FU;
     c->iter_general = c->general;
     c->iter_nu = c->n_u;
     return true;

@@ -83,7 +83,7 @@ struct lrccs_ctx {
     std::vector<prof_rec> iter_prof;    // timing events recorded by the graph
     int iter_n, iter_r, iter_nused, iter_general, iter_nu;
     unsigned long long iter_mask;
-    const void *iter_T;
+    const void *iter_T, *iter_FU;
     bool iter_graph_failed;             // capture not possible here: launch directly
     bool capturing;                     // inside the library's own capture
     int capture_iter;                   // iteration being captured

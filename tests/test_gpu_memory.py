@@ -72,3 +72,31 @@ def test_optional_memory_is_given_back(kind):
     fill.clear()
     torch.cuda.empty_cache()
     assert rel(got[0], wide[0]) < 1e-6 and rel(got[2], wide[2]) < 3e-6
+
+
+@pytest.mark.parametrize("kind", ["lines", "radial"])
+def test_iterations_and_batches_go_on_after_a_buffer_has_grown(kind):
+    """Captured iterations hold the work buffers' addresses; model-error correction grows them in between."""
+    c = Case(96, 64, 17, 3, 2, kind, 11)
+    res = []
+    for grow in (False, True):
+        solo, stream = torch.cuda.Stream(), torch.cuda.Stream()
+        a = lrccs.Solver(c.ny, c.nx, c.q, c.nc, 2, stream=solo)
+        b = lrccs.Solver(c.ny, c.nx, c.q, c.nc, 2, stream=stream)
+        batch = lrccs.lrccs_batch_create([b.ctx], stream)
+        torch.cuda.synchronize()
+        for s, step in ((a, a.iterate), (b, lambda n: lrccs.lrccs_batch_iterate(batch, n))):
+            with torch.cuda.stream(s.stream):
+                s.init(*c.inp)
+                step(4)
+                s.sync()
+                if grow:
+                    s.mec1(1)
+                step(4)
+                s.sync()
+                res.append(s.subspace())
+        torch.cuda.synchronize()
+        lrccs.lrccs_batch_destroy(batch)
+        a.close()
+        b.close()
+    assert all(torch.equal(res[0], u) for u in res[1:])
