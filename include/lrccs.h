@@ -530,6 +530,15 @@ lrccs_status lrccs_bstep_phases(lrccs_ctx *ctx, double *out);
  * Errors: LRCCS_E_INVALID (null ctx). */
 lrccs_status lrccs_test_wait_timeout(lrccs_ctx *ctx, int32_t enable);
 
+/* Test support (the paper has no counterpart): the context's GD/QR kernel runs
+ * with `blocks` blocks from now on, as it does on a device or a partition of one
+ * with that many multiprocessors; the next iteration then starts from the
+ * current subspace as after lrccs_set_subspace.
+ * Errors: LRCCS_E_INVALID (null ctx, blocks outside 1 .. the device's
+ * multiprocessors, or a count that needs more buffers than the context has),
+ * LRCCS_E_STATE (phase timing is on). */
+lrccs_status lrccs_test_few_blocks(lrccs_ctx *ctx, int32_t blocks);
+
 /* Wait for the context's stream and return any device-side failure. */
 lrccs_status lrccs_synchronize(lrccs_ctx *ctx);
 

@@ -167,6 +167,12 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     if (gd > nsm) gd = nsm;
     if (gd < 1) gd = 1;
     c->gd_grid = gd;
+    int optin = 0, coop = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    c->dev_smem_optin = optin;
+    gd = gdqr_parts(c->n, d.q, rmax, gd, optin);
+    c->gd_parts = c->gd_cap = gd;
     const size_t gd_len = std::max((size_t)2 * npm + rmax * rmax, (size_t)rmax * rmax + (size_t)q * rmax);
     size_t gcap = (size_t)gd * gd_len;
     if ((size_t)nblk * rmax * rmax > gcap) gcap = (size_t)nblk * rmax * rmax;
@@ -247,10 +253,6 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
         delete c;
         return LRCCS_E_NOMEM;
     }
-    int optin = 0, coop = 0;
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    c->dev_smem_optin = optin;
     cudaError_t e = configure_kernels_init(optin);
     if (e == cudaSuccess) e = configure_kernels_iter(optin);
     if (e == cudaSuccess) e = configure_kernels_gd(optin);
@@ -1497,7 +1499,7 @@ static lrccs_status save_state(lrccs_ctx *c, solver_state &s, size_t tot_len) {
     s.B.resize((size_t)c->q * c->r);
     s.scal.resize(SC_COUNT);
     s.tot.resize(tot_len);
-    s.hpart.resize((size_t)c->gd_grid * c->q * c->r);
+    s.hpart.resize((size_t)c->gd_parts * c->q * c->r);
     CK(cudaStreamSynchronize(c->stream));
     CK(cudaMemcpy(s.hpart.data(), c->d_hpart, s.hpart.size() * sizeof(float2), cudaMemcpyDeviceToHost));
     CK(cudaMemcpy(s.U.data(), c->d_U, nu * sizeof(float2), cudaMemcpyDeviceToHost));
@@ -1841,6 +1843,26 @@ extern "C" lrccs_status lrccs_bstep_phases(lrccs_ctx *c, double *out) {
 extern "C" lrccs_status lrccs_test_wait_timeout(lrccs_ctx *c, int32_t enable) {
     if (!c) return LRCCS_E_INVALID;
     c->test_timeout = enable ? 1 : 0;
+    return LRCCS_OK;
+}
+
+extern "C" lrccs_status lrccs_test_few_blocks(lrccs_ctx *c, int32_t blocks) {
+    if (!c) return LRCCS_E_INVALID;
+    const int g = std::min(blocks, c->n / 32);
+    const int parts = blocks > 0 ? gdqr_parts(c->n, c->q, c->rmax, g, c->dev_smem_optin) : 0;
+    if (c->d_gdts) {
+        set_err(c, "lrccs_test_few_blocks: phase timing is on (its buffer is laid out by blocks)");
+        return LRCCS_E_STATE;
+    }
+    if (blocks < 1 || blocks > c->nsm || parts > c->gd_cap) {
+        set_err(c, "lrccs_test_few_blocks: blocks outside [1, %d], or more parts than the buffers hold", c->nsm);
+        return LRCCS_E_INVALID;
+    }
+    CK(cudaStreamSynchronize(c->stream));
+    drop_iter_graph(c);
+    c->gd_grid = g;
+    c->gd_parts = parts;
+    if (c->has_u) c->need_h = 1;   // the right-hand sides' partial sums are laid out by parts
     return LRCCS_OK;
 }
 

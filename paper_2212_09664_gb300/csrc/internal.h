@@ -103,6 +103,8 @@ struct lrccs_ctx {
     int px, py;        // nx / 32, ny / 32
     int nblk;          // blocks of the pixel-parallel init kernels
     int gd_grid;       // blocks of the cooperative GD/QR kernel (all resident)
+    int gd_parts;      // parts of the pixels it works on, one or more a block: partial rows of h = U^H Z
+    int gd_cap;        // parts the buffers hold
     int nsm;           // multiprocessors of the device
     int smem_sm;       // shared memory per multiprocessor (bytes)
     int bs_cap[17];    // resident k_bstep<r> blocks for this shape, r = 1..16 (0: rows do not fit)
@@ -166,7 +168,7 @@ struct lrccs_ctx {
     float2 *d_Q;                 // q * q rotations of the eigensolver's refine pass
     double2 *d_tot;              // k_gdqr totals: [grad^H grad | U^H grad | U^H U] (iteration), [U+^H U+] (init)
     float2 *d_ZB;                // n * rmax  Z B^H (k_zb)
-    float2 *d_hpart;             // gd_grid * q * rmax  per-block partial sums of h = U^H Z (k_gdqr)
+    float2 *d_hpart;             // gd_cap * q * rmax  per-part partial sums of h = U^H Z (k_gdqr)
     cudaStream_t side;           // parallel branch of the iteration (k_zb beside the adjoint passes)
     cudaEvent_t ev_fork, ev_join;
     cudaEvent_t ev_counts;       // h_counts has arrived
@@ -256,6 +258,7 @@ cudaError_t launch_energy(lrccs_ctx *c, const float2 *d_y);
 cudaError_t launch_init_adjoint(lrccs_ctx *c, const float2 *d_y, bool trunc);   // Z (and X0)
 cudaError_t launch_gram_x0(lrccs_ctx *c);
 cudaError_t launch_u0(lrccs_ctx *c);
+int gdqr_parts(int n, int q, int rmax, int blocks, int smem_optin);
 cudaError_t launch_gdqr(lrccs_ctx *c, int mode);      // F: GD step + Cholesky QR (mode 0: init U+)
 cudaError_t launch_zb(lrccs_ctx *c);                  // d_ZB <- Z B^H
 void launch_zb_of(lrccs_ctx *c, const float2 *Z, const float2 *B, float2 *dst);

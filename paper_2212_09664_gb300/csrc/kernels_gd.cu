@@ -21,8 +21,9 @@
 //
 // In init mode the same kernel orthonormalises the given U+ (G1 = U+^H U+)
 // and forms the first right-hand sides U_0^H Z.
-// A block's pixel range of U and of the gradient stays in shared memory across
-// the phases; its rows of Z stream in behind phase 1 (all of them when they fit,
+// A block has one part of the pixels (several where a device has few
+// multiprocessors: gdqr_parts) and its rows of U and of the gradient stay in shared
+// memory across the phases; its rows of Z stream in behind phase 1 (all of them when they fit,
 // else through two chunk buffers).
 //
 // Z B^H depends only on the B-step's result, so its own kernel k_zb forms it
@@ -46,17 +47,17 @@ struct GdArgs {
     const float2 *Gk;   // n x r   sum_j conj(d_j) F^H K_j (iteration mode)
     const float2 *ZB;   // n x r   Z B^H (iteration mode)
     const float2 *Z;    // n x q   A_k^H y_k, row-major (i q + k)
-    float2 *hpart;      // G x q r partial sums of h = U_{t+1}^H Z (row b: block b)
+    float2 *hpart;      // parts x q r partial sums of h = U_{t+1}^H Z (row b: part b)
     float2 *U;          // n x r   U_t in, U_{t+1} out
     float2 *Uprev;      // n x r   receives U_t (iteration mode)
     const float2 *Up;   // n x r   U+ (init mode)
     float2 *Gr;         // n x r   receives the gradient (iteration mode)
-    float2 *part;       // G x len partial sums
+    float2 *part;       // parts x len partial sums
     double2 *tot;       // len totals (FP64)
     double *scal;       // SC_* scalars
     unsigned int *bar;  // [0] barrier arrivals, [1] exit count
     unsigned int *status;
-    int n, q, per, zs, zc, nbuf, mode;   // per: pixels per block; zc: rows of a Z chunk buffer, nbuf of them
+    int n, q, parts, per, zs, zc, nbuf, mode;   // per: pixels per part; zc: rows of a Z chunk buffer, nbuf of them
     double eta_c;
     double eta_scale0, eta_decay;   // variable step size: eta_t = eta eta_scale0 eta_decay^k
     long long *ts;             // NULL, or GD_NTS clock64() stamps per block (phase timing)
@@ -85,18 +86,18 @@ struct GdArgs {
 
 // grid_sync (common.cuh) is the grid-wide barrier of this cooperative kernel.
 
-// Block b reduces entries e = b, b + G, b + 2G, ... (< len) of the G partial
+// Block b reduces entries e = b, b + G, b + 2G, ... (< len) of the P partial
 // rows part[g len + e], four entries at a time (128 threads each), into FP64
 // totals: per thread in g order, then a fixed shuffle tree, then the warps in
 // order.
-static __device__ void grid_reduce(const float2 *part, int len, double2 *tot) {
+static __device__ void grid_reduce(const float2 *part, int P, int len, double2 *tot) {
     __shared__ float4 s_w[NTG / 32];   // per warp: (re.hi, re.lo, im.hi, im.lo)
     const int G = gridDim.x, l128 = threadIdx.x & 127, slot = threadIdx.x >> 7;
     for (int j0 = 0; (int)blockIdx.x + G * j0 < len; j0 += NTG / 128) {
         const int e = blockIdx.x + G * (j0 + slot);
         fsum2 re = {0.f, 0.f}, im = {0.f, 0.f};
         if (e < len)
-            for (int g = l128; g < G; g += 128) {
+            for (int g = l128; g < P; g += 128) {
                 const float2 v = __ldcg(part + (size_t)g * len + e);
                 fsum_add(re, v.x);
                 fsum_add(im, v.y);
@@ -361,7 +362,9 @@ static __device__ __noinline__ void gd_h(const GdArgs &a, const float2 *s_a, flo
 // re-staged when a block's rows did not fit -> this form: 64 x 64, q = 32, r = 4: 15.6 ->
 // 13.3 us; 128 x 128, q = 8, r = 6: 21.4 -> 13.5 us; 192 x 192, q = 48, r = 10: 24.6 -> 21.3 us;
 // 256 x 256, q = 64, r = 12: 55.0 -> 42.4 us.
-template <int R>
+// MANY: several parts a block, staged in turn by each phase (a form of its own: the
+// loops alone cost the usual one up to 3 us).
+template <int R, bool MANY>
 __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
     GD_GT(9);
     using PL = GdPlan<R>;
@@ -378,7 +381,15 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
     __shared__ int s_flag;
     __shared__ float s_eta;
     const int t = threadIdx.x, G = gridDim.x;
-    const int i0 = min(a.n, (int)blockIdx.x * a.per), i1 = min(a.n, i0 + a.per), rows = i1 - i0;
+    int part = blockIdx.x, i0 = min(a.n, part * a.per), rows = min(a.n, i0 + a.per) - i0;
+    auto next = [&](int p) {   // part p, when there is one
+        if (!MANY || p >= a.parts) return false;
+        part = p;
+        i0 = min(a.n, p * a.per);
+        rows = min(a.n, i0 + a.per) - i0;
+        __syncthreads();   // the last part's rows are read
+        return true;
+    };
     const bool iter = a.mode == 1;
     const int len1 = iter ? PL::L_ITER : np;
     // eta as it stands at launch; block 0 updates the device copy only after
@@ -389,44 +400,46 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
 
     // ------------------------------------------------ phase 1: gradient and Gram partial sums
     GD_TS(0);
-    stage_rows(s_u, RS, (iter ? a.U : a.Up) + (size_t)i0 * R, R, rows, R);
-    cp_async_commit();
-    for (int b = 0; b < a.nbuf; ++b) gd_stage_z(a, s_z, i0, rows, b);   // streams in behind phase 1
-    if (iter) {   // grad = Gk - Z B^H
-        const float2 *gk = a.Gk + (size_t)i0 * R, *zb = a.ZB + (size_t)i0 * R;
-        float2 *gr = a.Gr + (size_t)i0 * R;
-        if constexpr (R % 2 == 0) {
-            constexpr int H = R / 2;
+    do {
+        stage_rows(s_u, RS, (iter ? a.U : a.Up) + (size_t)i0 * R, R, rows, R);
+        cp_async_commit();
+        for (int b = 0; b < a.nbuf; ++b) gd_stage_z(a, s_z, i0, MANY ? 0 : rows, b);   // streams in behind phase 1
+        if (iter) {   // grad = Gk - Z B^H
+            const float2 *gk = a.Gk + (size_t)i0 * R, *zb = a.ZB + (size_t)i0 * R;
+            float2 *gr = a.Gr + (size_t)i0 * R;
+            if constexpr (R % 2 == 0) {
+                constexpr int H = R / 2;
 #pragma unroll 4
-            for (int e = t; e < rows * H; e += NTG) {
-                const float4 x = __ldg((const float4 *)gk + e), y = __ldg((const float4 *)zb + e);
-                const float4 g = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
-                ((float4 *)gr)[e] = g;
-                const int ii = e / H;
-                *(float4 *)(s_a + ii * RS + 2 * (e - ii * H)) = g;
-            }
-        } else {
+                for (int e = t; e < rows * H; e += NTG) {
+                    const float4 x = __ldg((const float4 *)gk + e), y = __ldg((const float4 *)zb + e);
+                    const float4 g = make_float4(x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w);
+                    ((float4 *)gr)[e] = g;
+                    const int ii = e / H;
+                    *(float4 *)(s_a + ii * RS + 2 * (e - ii * H)) = g;
+                }
+            } else {
 #pragma unroll 4
-            for (int e = t; e < rows * R; e += NTG) {
-                const float2 g = csub(__ldg(gk + e), __ldg(zb + e));
-                gr[e] = g;
-                const int ii = e / R;
-                s_a[ii * RS + (e - ii * R)] = g;
+                for (int e = t; e < rows * R; e += NTG) {
+                    const float2 g = csub(__ldg(gk + e), __ldg(zb + e));
+                    gr[e] = g;
+                    const int ii = e / R;
+                    s_a[ii * RS + (e - ii * R)] = g;
+                }
             }
         }
-    }
-    if (a.nbuf == 1) cp_async_wait_1();
-    else cp_async_wait_2();
-    __syncthreads();
-    GD_TS(1);
-    // partial row: [grad^H grad pairs (np) | U^H grad (rr) | U^H U pairs (np)], init: [U+^H U+ pairs]
-    if (iter) gd_grams<R, true>(s_u, s_a, rows, a.part + (size_t)blockIdx.x * len1);
-    else gd_grams<R, false>(s_u, s_a, rows, a.part + (size_t)blockIdx.x * len1);
+        if (a.nbuf == 1) cp_async_wait_1();
+        else cp_async_wait_2();
+        __syncthreads();
+        GD_TS(1);
+        // partial row: [grad^H grad pairs (np) | U^H grad (rr) | U^H U pairs (np)], init: [U+^H U+ pairs]
+        if (iter) gd_grams<R, true>(s_u, s_a, rows, a.part + (size_t)part * len1);
+        else gd_grams<R, false>(s_u, s_a, rows, a.part + (size_t)part * len1);
+    } while (next(part + G));
     GD_TS(2);
     GD_TS(3);
     grid_sync(a.bar, 1, a.status, a.spin_limit, a.bar_skew, ST_TIMEOUT);
     GD_TS(4);
-    grid_reduce(a.part, len1, a.tot);
+    grid_reduce(a.part, a.parts, len1, a.tot);
     GD_TS(5);
     grid_sync(a.bar, 2, a.status, a.spin_limit, a.bar_skew, ST_TIMEOUT);
     GD_TS(6);
@@ -496,38 +509,48 @@ __global__ void __launch_bounds__(NTG, 1) k_gdqr(GdArgs a) {
     // ------------------------------------------------ phase 2: U_{t+1} = (U - eta grad) R1^{-1}
     // a thread per pixel row, in place over the gradient: column l needs the
     // columns up to l only, so they are formed from the last one down
-    for (int i = t; i < rows; i += NTG) {
-        asm volatile("" ::: "memory");   // one turn as a rule: keep R1^{-1} in shared memory
-        float2 w[R];
-#pragma unroll
-        for (int m = 0; m < R; ++m) {
-            w[m] = s_u[i * RS + m];
-            if (iter) w[m] = csub(w[m], cscale(s_a[i * RS + m], etaf));
+    next(blockIdx.x);
+    do {
+        if (MANY) {
+            stage_rows(s_u, RS, (iter ? a.U : a.Up) + (size_t)i0 * R, R, rows, R);
+            if (iter) stage_rows(s_a, RS, a.Gr + (size_t)i0 * R, R, rows, R);
+            cp_async_commit();
+            for (int b = 0; b < a.nbuf; ++b) gd_stage_z(a, s_z, i0, rows, b);
+            if (a.nbuf == 1) cp_async_wait_1();
+            else cp_async_wait_2();
+            __syncthreads();
         }
+        for (int i = t; i < rows; i += NTG) {
+            asm volatile("" ::: "memory");   // one turn as a rule: keep R1^{-1} in shared memory
+            float2 w[R];
 #pragma unroll
-        for (int l = R - 1; l >= 0; --l) {
-            float2 v = make_float2(0.f, 0.f);
+            for (int m = 0; m < R; ++m) {
+                w[m] = s_u[i * RS + m];
+                if (iter) w[m] = csub(w[m], cscale(s_a[i * RS + m], etaf));
+            }
 #pragma unroll
-            for (int m = 0; m <= l; ++m) cfma(v, w[m], sR[m * R + l]);
-            w[l] = v;
+            for (int l = R - 1; l >= 0; --l) {
+                float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int m = 0; m <= l; ++m) cfma(v, w[m], sR[m * R + l]);
+                w[l] = v;
+            }
+#pragma unroll
+            for (int m = 0; m < R; ++m) s_a[i * RS + m] = w[m];
         }
-#pragma unroll
-        for (int m = 0; m < R; ++m) s_a[i * RS + m] = w[m];
-    }
-    __syncthreads();
-    for (int e = t; e < rows * R; e += NTG) {
-        const int ii = e / R, l = e - ii * R;
-        a.U[(size_t)i0 * R + e] = s_a[ii * RS + l];
-        if (iter) a.Uprev[(size_t)i0 * R + e] = s_u[ii * RS + l];
-    }
-    // the block's row of h partial sums, hpart[b][k R + l]
-    {
-        float2 *hrow = a.hpart + (size_t)blockIdx.x * q * R;
+        __syncthreads();
+        for (int e = t; e < rows * R; e += NTG) {
+            const int ii = e / R, l = e - ii * R;
+            a.U[(size_t)i0 * R + e] = s_a[ii * RS + l];
+            if (iter) a.Uprev[(size_t)i0 * R + e] = s_u[ii * RS + l];
+        }
+        // the part's row of h partial sums, hpart[part][k R + l]
+        float2 *hrow = a.hpart + (size_t)part * q * R;
         const int cap = max(2 * NTG, 2 * a.per * RS + a.nbuf * a.zc * a.zs);   // as launched
         constexpr int LS = R % 2 == 0 ? 2 : 1;
         if (NTG / ((q + 1) >> 1) > 64) gd_h<R, LS>(a, s_a, s_z, smem, cap, i0, rows, hrow);
         else gd_h<R, R>(a, s_a, s_z, smem, cap, i0, rows, hrow);
-    }
+    } while (next(part + G));
     GD_TS(8);
     // the last block out: SD(U_t, U_{t+1})^2 = r - ||U_t^H U_{t+1}||_F^2 with
     // U_t^H U_{t+1} = (U_t^H U_t - eta U_t^H grad) R1^{-1} from the totals (no
@@ -624,19 +647,22 @@ __global__ void __launch_bounds__(256) k_zb(const float2 *__restrict__ Z, const 
 // ---------------------------------------------------------------- launcher
 
 typedef void (*gd_kernel_t)(GdArgs);
-static const gd_kernel_t kGd[RMAXC] = {k_gdqr<1>,  k_gdqr<2>,  k_gdqr<3>,  k_gdqr<4>,  k_gdqr<5>,  k_gdqr<6>,
-                                       k_gdqr<7>,  k_gdqr<8>,  k_gdqr<9>,  k_gdqr<10>, k_gdqr<11>, k_gdqr<12>,
-                                       k_gdqr<13>, k_gdqr<14>, k_gdqr<15>, k_gdqr<16>};
-static int g_gd_static_smem[RMAXC];
+#define GD_TABLE(M) {k_gdqr<1, M>,  k_gdqr<2, M>,  k_gdqr<3, M>,  k_gdqr<4, M>,  k_gdqr<5, M>,  k_gdqr<6, M>, \
+                     k_gdqr<7, M>,  k_gdqr<8, M>,  k_gdqr<9, M>,  k_gdqr<10, M>, k_gdqr<11, M>, k_gdqr<12, M>, \
+                     k_gdqr<13, M>, k_gdqr<14, M>, k_gdqr<15, M>, k_gdqr<16, M>}
+static const gd_kernel_t kGd[2][RMAXC] = {GD_TABLE(false), GD_TABLE(true)};
+static int g_gd_static_smem[2 * RMAXC];
+#define GD_STATIC_MAX 16384   // no rank's static shared memory is above this (14880 bytes at 16)
 
 cudaError_t configure_kernels_gd(int max_smem) {
-    for (int i = 0; i < RMAXC; ++i) {
+    for (int i = 0; i < 2 * RMAXC; ++i) {
+        const gd_kernel_t k = kGd[i / RMAXC][i % RMAXC];
         cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, kGd[i]);
+        cudaError_t e = cudaFuncGetAttributes(&fa, k);
         if (e != cudaSuccess) return e;
+        if (fa.sharedSizeBytes > GD_STATIC_MAX) return cudaErrorInvalidConfiguration;
         g_gd_static_smem[i] = (int)fa.sharedSizeBytes;
-        e = cudaFuncSetAttribute(kGd[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 max_smem - (int)fa.sharedSizeBytes);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - (int)fa.sharedSizeBytes);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -646,13 +672,36 @@ cudaError_t configure_kernels_gd(int max_smem) {
 // that 16-byte loads of consecutive pixels' rows hit distinct banks.
 static int z_stride(int q) { return ((q + 1) | 3) - 1; }
 
+// Shared memory of k_gdqr for a part's rows of U and of the gradient.
+static size_t gd_fixed(int n, int r, int parts) {
+    const int per = (n + parts - 1) / parts, rs = r % 4 == 0 ? r + 2 : r;
+    return (size_t)2 * per * rs * sizeof(float2);
+}
+
+// Parts the n pixels are cut into for `blocks` blocks: as many, unless their rows
+// of U and the gradient (rank up to rmax) and four rows of Z leave a block's
+// shared memory, which few multiprocessors cause (65536 pixels at rank 16: fewer
+// than 89 of them, a partition of the device): then two or more a block.
+int gdqr_parts(int n, int q, int rmax, int blocks, int smem_optin) {
+    for (int m = 1;; ++m) {
+        bool fits = smem_optin <= 0;   // no device to ask: sizes only
+        int r = 1;
+        while (!fits && r <= rmax &&
+               gd_fixed(n, r, m * blocks) + 4 * z_stride(q) * sizeof(float2) + GD_STATIC_MAX <= (size_t)smem_optin)
+            ++r;
+        fits = fits || r > rmax;
+        if (fits || m * blocks >= n) return m * blocks;
+    }
+}
+
 cudaError_t launch_gdqr(lrccs_ctx *c, int mode) {
     const int r = c->r, q = c->q, G = c->gd_grid;
     if (r < 1 || r > RMAXC) return cudaErrorInvalidValue;
     const int zs = z_stride(q);
-    const int per = (c->n + G - 1) / G, rs = r % 4 == 0 ? r + 2 : r;
-    const size_t fixed = (size_t)2 * per * rs * sizeof(float2);
-    const size_t avail = (size_t)(c->dev_smem_optin - g_gd_static_smem[r - 1]);
+    const int per = (c->n + c->gd_parts - 1) / c->gd_parts;
+    const size_t fixed = gd_fixed(c->n, r, c->gd_parts);
+    const bool many = c->gd_parts > G;
+    const size_t avail = (size_t)(c->dev_smem_optin - g_gd_static_smem[many * RMAXC + r - 1]);
     if (fixed + 4 * zs * sizeof(float2) > avail) return cudaErrorInvalidConfiguration;
     // Z in one piece, or through two buffers of as many rows as fit
     const int rows = (int)((avail - fixed) / (zs * sizeof(float2)));
@@ -673,6 +722,7 @@ cudaError_t launch_gdqr(lrccs_ctx *c, int mode) {
     a.status = c->d_status;
     a.n = c->n;
     a.q = q;
+    a.parts = c->gd_parts;
     a.per = per;
     a.zs = zs;
     a.zc = zc;
@@ -693,7 +743,7 @@ cudaError_t launch_gdqr(lrccs_ctx *c, int mode) {
     // the h slices go through all of it, two values per thread at least
     const size_t smem = std::max(fixed + (size_t)nbuf * zc * zs * sizeof(float2), (size_t)2 * NTG * sizeof(float2));
     prof_begin(c, KID_GDQR);
-    cudaError_t e = cudaLaunchCooperativeKernel((const void *)kGd[r - 1], dim3(G), dim3(NTG), args, smem, c->stream);
+    cudaError_t e = cudaLaunchCooperativeKernel((const void *)kGd[many][r - 1], dim3(G), dim3(NTG), args, smem, c->stream);
     prof_end(c, KID_GDQR);
     return e;
 }

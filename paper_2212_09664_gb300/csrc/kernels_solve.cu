@@ -200,19 +200,19 @@ size_t frame_gram_part_count(int q, int rmax) { return (size_t)q * gen_chunks(q)
 
 cudaError_t launch_solve(lrccs_ctx *c) {
     if (c->r < 1 || c->r > RMAXC) return cudaErrorInvalidValue;
-    if (c->gd_grid > HMAX * (NT / c->r)) return cudaErrorInvalidConfiguration;   // frame_h_load's reach
+    if (c->gd_parts > HMAX * (NT / c->r)) return cudaErrorInvalidConfiguration;   // frame_h_load's reach
     if (c->general) {
         prof_begin(c, KID_SOLVE_GEN);
         kFrameGramGen[c->r - 1]<<<dim3(c->q, gen_chunks(c->q)), NT, 0, c->stream>>>(c->d_Pu, c->d_fpk, c->d_fu, c->d_fpart);
         prof_end(c, KID_SOLVE_GEN);
         prof_begin(c, KID_SOLVE_GEN);
-        kSolveGen[c->r - 1]<<<c->q, NT, 0, c->stream>>>(c->d_fpart, c->d_hpart, c->gd_grid, c->q,
+        kSolveGen[c->r - 1]<<<c->q, NT, 0, c->stream>>>(c->d_fpart, c->d_hpart, c->gd_parts, c->q,
                                                         gen_chunks(c->q), c->d_fpk, c->d_B, c->d_status);
         prof_end(c, KID_SOLVE_GEN);
         return cudaGetLastError();
     }
     prof_begin(c, KID_SOLVE);
-    kSolve[c->r - 1]<<<c->q, NT, 0, c->stream>>>(c->d_P, c->d_hpart, c->gd_grid, c->q, c->d_lineptr,
+    kSolve[c->r - 1]<<<c->q, NT, 0, c->stream>>>(c->d_P, c->d_hpart, c->gd_parts, c->q, c->d_lineptr,
                                                  c->d_framerows, c->d_B, c->d_status);
     prof_end(c, KID_SOLVE);
     return cudaGetLastError();
@@ -769,7 +769,7 @@ int bstep_capacity(int nc, int nx, int q, int r, int smem_optin, int nsm) {
 // resident block (and the plan does not ask for the separate kernels).
 bool bstep_fused_ok(const lrccs_ctx *c) {
     if (c->plan.bstep_form != 0 || c->general || c->r < 1 || c->r > RMAXC) return false;
-    if (c->gd_grid > HMAX * (NT / c->r)) return false;   // frame_h_load's reach
+    if (c->gd_parts > HMAX * (NT / c->r)) return false;   // frame_h_load's reach
     return c->n_used >= 1 && c->n_used <= c->bs_cap[c->r];
 }
 
@@ -798,7 +798,7 @@ cudaError_t launch_bstep_fused(lrccs_ctx *c) {
     a.nc = c->nc;
     a.q = c->q;
     a.area = bstep_area(c->nc, c->nx, c->q, r);
-    a.P = c->gd_grid;
+    a.P = c->gd_parts;
     a.spin_limit = 1u << 24;
     // phase stamps after k_gdqr's in the phase-timing buffer (lrccs_gdqr_phases on)
     a.ts = c->d_gdts ? c->d_gdts + (size_t)c->gd_grid * 11 : nullptr;

@@ -78,6 +78,7 @@ _sig = {
     "lrccs_get_state": (_st, [_vp, _vp, C.POINTER(C.c_size_t)]),
     "lrccs_set_state": (_st, [_vp, C.c_char_p, C.c_size_t]),
     "lrccs_test_wait_timeout": (_st, [_vp, C.c_int32]),
+    "lrccs_test_few_blocks": (_st, [_vp, C.c_int32]),
     "lrccs_gdqr_phases": (_st, [_vp, C.c_int32, C.POINTER(C.c_double)]),
     "lrccs_bstep_phases": (_st, [_vp, C.POINTER(C.c_double)]),
     "lrccs_forward_transform": (_st, [_vp, _vp, C.c_size_t]),
@@ -338,6 +339,10 @@ def lrccs_bstep_phases(ctx):
 
 def lrccs_test_wait_timeout(ctx, enable: bool = True):
     _check(ctx, _lib.lrccs_test_wait_timeout(ctx, 1 if enable else 0))
+
+
+def lrccs_test_few_blocks(ctx, blocks: int):
+    _check(ctx, _lib.lrccs_test_few_blocks(ctx, int(blocks)))
 
 
 def lrccs_mec1(ctx, iters: int = 3, zbar=None, E=None, X=None):
