@@ -90,12 +90,12 @@ static void free_all(lrccs_ctx *c) {
     c->side = nullptr;
     c->ev_fork = c->ev_join = c->ev_counts = c->ev_copied = nullptr;
     c->h_counts = nullptr;
-    void *ptrs[] = {c->d_twy, c->d_twx, c->d_smaps, c->d_rowcnt, c->d_rowidx, c->d_framerows, c->d_lineptr,
-                    c->d_rfptr, c->d_rflist, c->d_usedrows, c->d_rowused, c->d_idx, c->d_meta, c->d_status,
+    void *ptrs[] = {c->d_twx, c->d_smaps, c->d_rowcnt, c->d_framerows, c->d_lineptr,
+                    c->d_rfptr, c->d_rflist, c->d_usedrows, c->d_idx, c->d_meta, c->d_status,
                     c->d_counters, c->d_scal, c->d_Z, c->d_X0, c->d_T, c->d_U, c->d_Uprev, c->d_Up, c->d_G,
-                    c->d_B, c->d_P, c->d_gpart, c->d_sigma, c->d_gram, c->d_V, c->d_tot, c->d_framek,
+                    c->d_B, c->d_P, c->d_gpart, c->d_sigma, c->d_gram, c->d_V, c->d_tot,
                     c->d_mks, c->d_fpk, c->d_rowoff, c->d_ucnt, c->d_uloc, c->d_floc, c->d_urow, c->d_uptr,
-                    c->d_ufrow, c->d_upos, c->d_uidx, c->d_ufptr, c->d_uflist, c->d_fu, c->d_FU, c->d_Pu,
+                    c->d_ufrow, c->d_upos, c->d_ufptr, c->d_uflist, c->d_fu, c->d_FU, c->d_Pu,
                     c->d_maskc, c->d_mec, c->d_mscal, c->d_mout, c->d_twq, c->d_Q, c->d_gdts, c->d_fpart,
                     c->d_tcA0, c->d_tcA1, c->d_tcscale, c->d_ZB, c->d_hpart,
                     c->d_tcB0, c->d_tcB1, c->d_twsy, c->d_twsx, c->d_rowtab, c->d_ptab, c->d_xs};
@@ -185,12 +185,13 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     // against the free device memory before anything is allocated
     const size_t F2 = sizeof(float2), I4 = sizeof(int32_t), D8 = sizeof(double);
     const struct { void **p; size_t bytes; } plan[] = {
-        {(void **)&c->d_twy, ny * F2}, {(void **)&c->d_twx, c->nx * F2},
-        {(void **)&c->d_twsy, ny * F2}, {(void **)&c->d_twsx, c->nx * F2}, {(void **)&c->d_rowtab, ((size_t)q + 17) * 32 * I4}, {(void **)&c->d_xs, (size_t)q * 4}, {(void **)&c->d_smaps, (size_t)nc * n * F2},
-        {(void **)&c->d_rowcnt, (size_t)q * ny * I4}, {(void **)&c->d_rowidx, (size_t)q * ny * I4},
+        {(void **)&c->d_twx, c->nx * F2}, {(void **)&c->d_twsy, ny * F2}, {(void **)&c->d_twsx, c->nx * F2},
+        {(void **)&c->d_rowtab, ((size_t)q + 17) * 32 * I4}, {(void **)&c->d_xs, (size_t)q * 4},
+        {(void **)&c->d_smaps, (size_t)nc * n * F2},
+        {(void **)&c->d_rowcnt, (size_t)q * ny * I4},
         {(void **)&c->d_framerows, (size_t)q * ny * I4}, {(void **)&c->d_lineptr, ((size_t)q + 1) * I4},
         {(void **)&c->d_rfptr, ((size_t)ny + 1) * I4}, {(void **)&c->d_rflist, (size_t)q * ny * I4},
-        {(void **)&c->d_usedrows, (size_t)ny * I4}, {(void **)&c->d_rowused, (size_t)ny},
+        {(void **)&c->d_usedrows, (size_t)ny * I4},
         {(void **)&c->d_idx, (size_t)q * n * I4}, {(void **)&c->d_meta, ((size_t)MT_COUNT + q) * I4},
         {(void **)&c->d_status, sizeof(unsigned)}, {(void **)&c->d_counters, CNT_COUNT * sizeof(unsigned)},
         {(void **)&c->d_scal, SC_COUNT * D8}, {(void **)&c->d_Z, (size_t)n * q * F2},
@@ -202,7 +203,7 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
         {(void **)&c->d_ZB, (size_t)n * rmax * F2}, {(void **)&c->d_hpart, (size_t)gd * q * rmax * F2},
         {(void **)&c->d_sigma, (size_t)q * D8}, {(void **)&c->d_gram, (size_t)6 * q * q * D8},
         {(void **)&c->d_V, (size_t)q * q * F2}, {(void **)&c->d_Q, (size_t)q * q * F2},
-        {(void **)&c->d_framek, (size_t)q * ny * I4}, {(void **)&c->d_mks, (size_t)q * I4},
+        {(void **)&c->d_mks, (size_t)q * I4},
         {(void **)&c->d_fpk, ((size_t)q + 1) * I4}, {(void **)&c->d_rowoff, (size_t)q * ny * I4},
         {(void **)&c->d_maskc, (size_t)q * n}, {(void **)&c->d_twq, (size_t)q * F2},
         {(void **)&c->d_tcA0, d.precision != LRCCS_PREC_FP32_FFT ? tc_a_elems(ny) * 2 : 0},
@@ -273,7 +274,6 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_counts, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_copied, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->h_counts, (MT_COUNT + 1) * sizeof(int32_t), cudaHostAllocDefault);
-    if (e == cudaSuccess) e = launch_twiddles(c->d_twy, ny, c->stream);
     if (e == cudaSuccess) e = launch_twiddles(c->d_twx, c->nx, c->stream);
     if (e == cudaSuccess) e = launch_twiddles(c->d_twq, q, c->stream);
     if (e == cudaSuccess) e = launch_col_twiddles(c);
@@ -414,7 +414,7 @@ static lrccs_status ensure_general_buffers(lrccs_ctx *c) {
     const size_t npm = (size_t)c->rmax * (c->rmax + 1) / 2;
     const bool ok = need_buf(c, &c->d_ucnt, n) && need_buf(c, &c->d_uloc, n) && need_buf(c, &c->d_floc, n) &&
                     need_buf(c, &c->d_urow, 2 * ny) && need_buf(c, &c->d_uptr, ny + 1) &&
-                    need_buf(c, &c->d_ufrow, ny + 1) && need_buf(c, &c->d_upos, n) && need_buf(c, &c->d_uidx, n) &&
+                    need_buf(c, &c->d_ufrow, ny + 1) && need_buf(c, &c->d_upos, n) &&
                     need_buf(c, &c->d_ufptr, n + 1) && need_buf(c, &c->d_uflist, q * n) &&
                     need_buf(c, &c->d_fu, q * n) && need_buf(c, &c->d_FU, base_work(c)) &&
                     need_buf(c, &c->d_Pu, n * npm) &&
@@ -1371,10 +1371,9 @@ extern "C" lrccs_status lrccs_get_buffer(lrccs_ctx *c, lrccs_buffer which, void 
 // ---------------------------------------------------------------- profiling
 
 const char *const kKernelNames[KID_COUNT] = {
-    "k_rowcount", "k_structure", "k_fill_idx", "k_energy", "k_init_rows", "k_init_cols", "k_gram_x0",
+    "k_rowcount", "k_structure", "k_fill_idx", "k_energy", "k_init_rows", "k_gram_x0",
     "k_eig", "k_u0", "k_gdqr", "k_fwd_cols", "k_row_gram", "k_solve", "k_row_w", "k_adj_cols",
-    "k_images", "k_cg_init", "k_cg_step", "k_mean_resid", "k_union", "k_fill_general", "k_init_gen",
-    "k_fwd_rows", "k_sample_gram", "k_solve_gen", "k_sample_w", "k_adj_rows", "k_mean_resid_gen", "k_mec_mask",
+    "k_images", "k_cg_init", "k_cg_step", "k_mean_resid", "k_union", "k_fill_general", "k_fwd_rows", "k_sample_gram", "k_solve_gen", "k_sample_w", "k_adj_rows", "k_mean_resid_gen", "k_mec_mask",
     "k_mec_elem", "k_mec_tdft", "k_dft_a", "k_fwd_gemm", "k_tile_max", "k_b_operand", "k_zb", "k_bstep"};
 
 static cudaEvent_t get_event(lrccs_ctx *c) {

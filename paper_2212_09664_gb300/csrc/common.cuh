@@ -46,15 +46,6 @@ LRCCS_DEV float2 shfl_xor2(float2 v, int m) {
     return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
 }
 
-struct dcomplex { double x, y; };
-LRCCS_DEV dcomplex dc(double x, double y) { dcomplex r; r.x = x; r.y = y; return r; }
-LRCCS_DEV dcomplex dmul(dcomplex a, dcomplex b) { return dc(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-LRCCS_DEV dcomplex dmulc(dcomplex a, dcomplex b) { return dc(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }
-LRCCS_DEV dcomplex dadd(dcomplex a, dcomplex b) { return dc(a.x + b.x, a.y + b.y); }
-LRCCS_DEV dcomplex dsub(dcomplex a, dcomplex b) { return dc(a.x - b.x, a.y - b.y); }
-
-LRCCS_DEV int brev5(int v) { return (int)(__brev((unsigned)v) >> 27); }
-
 // Upper-triangle pair enumeration of an r x r Hermitian matrix: p -> (a, b), a <= b.
 LRCCS_DEV void pair_of(int p, int r, int &a, int &b) {
     int aa = 0;
@@ -67,7 +58,6 @@ LRCCS_DEV int pair_index(int a, int b, int r) {  // a <= b
     return a * r - (a * (a - 1)) / 2 + (b - a);
 }
 
-// Load the twiddle table of length N into shared memory.
 // |v|^2 in FP64 without contraction: the truncation decision |y|^2 <= gamma of
 // the spectral initialisation is taken on exactly the squares an FP64
 // reference forms.
@@ -87,6 +77,7 @@ LRCCS_DEV bool trunc_drop(float2 v, double gam, float glo, float ghi) {
     return abs2_rn(v) > gam;
 }
 
+// Load the twiddle table of length N into shared memory.
 LRCCS_DEV void load_twiddles(float2 *s_tw, const float2 *g_tw, int N) {
     for (int t = threadIdx.x; t < N; t += blockDim.x) s_tw[t] = g_tw[t];
 }
@@ -335,126 +326,10 @@ static inline cudaError_t allow_smem(K kernel, int optin) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
 }
 
-// ---------------------------------------------------------------- warp-level FP64 small linear algebra
-// For the r x r (r <= 32) Hermitian systems of the B-step and of CholeskyQR2.
-// Matrices are FP64 (re, im) pairs, row-major, in shared memory; one full warp
-// calls each routine.  GB300's FP64 pipe is narrow, so the work is spread over
-// the lanes instead of running on one thread.
-
 LRCCS_DEV double warp_sum_d(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;  // identical in every lane (each level adds the same two numbers)
-}
-
-// In place A = L L^H: the lower triangle of A receives L (real positive
-// diagonal).  Returns false (in every lane) if A is not positive definite.
-LRCCS_DEV bool warp_cholesky(double *A, int r) {
-    const int lane = threadIdx.x & 31;
-    for (int c = 0; c < r; ++c) {
-        double part = 0.0;
-        if (lane < c) {
-            const double ar = A[(c * r + lane) * 2], ai = A[(c * r + lane) * 2 + 1];
-            part = ar * ar + ai * ai;
-        }
-        part = warp_sum_d(part);
-        double d = A[(c * r + c) * 2] - part;
-        if (!(d > 0.0)) return false;
-        d = sqrt(d);
-        __syncwarp();
-        if (lane > c && lane < r) {
-            double vr = A[(lane * r + c) * 2], vi = A[(lane * r + c) * 2 + 1];
-            for (int m = 0; m < c; ++m) {  // v -= L[lane][m] conj(L[c][m])
-                const double ar = A[(lane * r + m) * 2], ai = A[(lane * r + m) * 2 + 1];
-                const double br = A[(c * r + m) * 2], bi = A[(c * r + m) * 2 + 1];
-                vr -= ar * br + ai * bi;
-                vi -= ai * br - ar * bi;
-            }
-            A[(lane * r + c) * 2] = vr / d;
-            A[(lane * r + c) * 2 + 1] = vi / d;
-        }
-        __syncwarp();
-        if (lane == 0) {
-            A[(c * r + c) * 2] = d;
-            A[(c * r + c) * 2 + 1] = 0.0;
-        }
-        __syncwarp();
-    }
-    return true;
-}
-
-// Rinv = (L^H)^{-1} (upper triangular) from the lower factor L in A.
-// Li: r * r * 2 doubles of shared scratch.  Lane j computes column j of L^{-1}.
-LRCCS_DEV void warp_rinv(const double *A, int r, double *Li, double *Rinv) {
-    const int lane = threadIdx.x & 31;
-    if (lane < r) {
-        const int j = lane;
-        for (int i = 0; i < j; ++i) {
-            Li[(i * r + j) * 2] = 0.0;
-            Li[(i * r + j) * 2 + 1] = 0.0;
-        }
-        Li[(j * r + j) * 2] = 1.0 / A[(j * r + j) * 2];
-        Li[(j * r + j) * 2 + 1] = 0.0;
-        for (int i = j + 1; i < r; ++i) {
-            double vr = 0.0, vi = 0.0;
-            for (int m = j; m < i; ++m) {
-                const double ar = A[(i * r + m) * 2], ai = A[(i * r + m) * 2 + 1];
-                const double br = Li[(m * r + j) * 2], bi = Li[(m * r + j) * 2 + 1];
-                vr += ar * br - ai * bi;
-                vi += ar * bi + ai * br;
-            }
-            const double d = A[(i * r + i) * 2];
-            Li[(i * r + j) * 2] = -vr / d;
-            Li[(i * r + j) * 2 + 1] = -vi / d;
-        }
-    }
-    __syncwarp();
-    for (int e = lane; e < r * r; e += 32) {
-        const int a = e / r, b = e - a * r;
-        Rinv[e * 2] = Li[(b * r + a) * 2];
-        Rinv[e * 2 + 1] = -Li[(b * r + a) * 2 + 1];
-    }
-    __syncwarp();
-}
-
-// Solve L L^H x = h (L lower in A); h and x are r (re, im) pairs in shared memory.
-LRCCS_DEV void warp_chol_solve(const double *A, int r, const double *h, double *x) {
-    const int lane = threadIdx.x & 31;
-    for (int c = 0; c < r; ++c) {  // L z = h
-        double pr = 0.0, pi = 0.0;
-        if (lane < c) {
-            const double ar = A[(c * r + lane) * 2], ai = A[(c * r + lane) * 2 + 1];
-            const double zr = x[2 * lane], zi = x[2 * lane + 1];
-            pr = ar * zr - ai * zi;
-            pi = ar * zi + ai * zr;
-        }
-        pr = warp_sum_d(pr);
-        pi = warp_sum_d(pi);
-        const double d = A[(c * r + c) * 2];
-        if (lane == 0) {
-            x[2 * c] = (h[2 * c] - pr) / d;
-            x[2 * c + 1] = (h[2 * c + 1] - pi) / d;
-        }
-        __syncwarp();
-    }
-    for (int c = r - 1; c >= 0; --c) {  // L^H x = z
-        double pr = 0.0, pi = 0.0;
-        if (lane > c && lane < r) {  // conj(L[lane][c]) x[lane]
-            const double ar = A[(lane * r + c) * 2], ai = -A[(lane * r + c) * 2 + 1];
-            const double zr = x[2 * lane], zi = x[2 * lane + 1];
-            pr = ar * zr - ai * zi;
-            pi = ar * zi + ai * zr;
-        }
-        pr = warp_sum_d(pr);
-        pi = warp_sum_d(pi);
-        const double d = A[(c * r + c) * 2];
-        __syncwarp();
-        if (lane == 0) {
-            x[2 * c] = (x[2 * c] - pr) / d;
-            x[2 * c + 1] = (x[2 * c + 1] - pi) / d;
-        }
-        __syncwarp();
-    }
 }
 
 // Compensated FP32 summation (Knuth's two-sum): a (hi, lo) pair carries ~48
@@ -521,21 +396,6 @@ LRCCS_DEV fsum2 fsum_pair(fsum2 a, fsum2 b) {
     r.lo = (a.lo + b.lo) + e;
     return r;
 }
-// Warp-wide sum of (hi, lo) pairs; identical result in every lane.
-LRCCS_DEV double warp_fsum(fsum2 v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float oh = __shfl_xor_sync(0xffffffffu, v.hi, o), ol = __shfl_xor_sync(0xffffffffu, v.lo, o);
-        float s, e;
-        // order the pair so that both lanes of a butterfly compute the same sum
-        const bool first = (threadIdx.x & o) == 0;
-        two_sum(first ? v.hi : oh, first ? oh : v.hi, s, e);
-        v.lo = (first ? v.lo + ol : ol + v.lo) + e;
-        v.hi = s;
-    }
-    return (double)v.hi + (double)v.lo;
-}
-
 // Block-wide compensated sums dst[e] = sum_{m < nitem} fetch(e, m) for
 // e < nent, written as FP64 (re, im) pairs.  Thread (entry e, slice s) sums
 // items s, s + S, s + 2S, ... in that order with RB loads in flight, and the S
@@ -595,12 +455,6 @@ LRCCS_DEV void block_sum(int nent, int nitem, double *dst, F fetch) {
         }
     }
     __syncthreads();
-}
-
-// Sum nblk rows of float2 partials (row length len, row b at part + b * len)
-// into dst (FP64 re, im pairs).
-LRCCS_DEV void block_reduce_rows(const float2 *part, int nblk, int len, double *dst) {
-    block_sum(len, nblk, dst, [=](int e, int b) { return __ldcg(part + (size_t)b * len + e); });
 }
 
 // ---------------------------------------------------------------- grid barrier of a cooperative launch
@@ -700,170 +554,4 @@ LRCCS_DEV bool mbar_wait(uint64_t *bar, unsigned parity, unsigned limit) {
             : "memory");
     }
     return done != 0;
-}
-
-// ---------------------------------------------------------------- FP32 r x r factorisation
-
-// In place A = L L^H for a Hermitian r x r A (FP32, row-major, r <= RMAX) by
-// one warp, lane i holding row i in registers: the lower triangle of A
-// receives L, invd[i] = 1 / L[i][i].  Returns false (every lane) if a pivot
-// is not positive.
-template <int RMAX>
-LRCCS_DEV bool warp_chol32(float2 *A, int r, float *invd) {
-    const int i = threadIdx.x & 31;
-    float2 row[RMAX];
-#pragma unroll
-    for (int j = 0; j < RMAX; ++j) row[j] = (i < r && j <= i) ? A[i * r + j] : make_float2(0.f, 0.f);
-    float myinv = 1.f;
-    bool ok = true;
-#pragma unroll
-    for (int c = 0; c < RMAX; ++c) {
-        if (c < r && ok) {   // uniform across the warp
-            const float d = __shfl_sync(0xffffffffu, row[c].x, c);
-            ok = d > 0.f;
-            const float is = ok ? rsqrtf(d) : 0.f;
-            float2 lic = make_float2(0.f, 0.f);
-            if (i == c) {
-                lic = make_float2(d * is, 0.f);
-                myinv = is;
-            } else if (i > c && i < r) {
-                lic = cscale(row[c], is);
-            }
-            if (i >= c) row[c] = lic;
-#pragma unroll
-            for (int j = c + 1; j < RMAX; ++j) {
-                if (j < r) {
-                    const float ljx = __shfl_sync(0xffffffffu, lic.x, j), ljy = __shfl_sync(0xffffffffu, lic.y, j);
-                    if (i >= j && i < r) {   // A[i][j] -= L[i][c] conj(L[j][c])
-                        row[j].x -= lic.x * ljx + lic.y * ljy;
-                        row[j].y -= lic.y * ljx - lic.x * ljy;
-                    }
-                }
-            }
-        }
-    }
-    __syncwarp();
-    if (ok && i < r) {
-#pragma unroll
-        for (int j = 0; j < RMAX; ++j)
-            if (j < r) A[i * r + j] = j <= i ? row[j] : make_float2(0.f, 0.f);
-        invd[i] = myinv;
-    }
-    __syncwarp();
-    return ok;
-}
-
-// Solve L L^H x = h (L from warp_chol32, lower triangle of the row-major r x r
-// FP32 matrix, invd = 1 / diag) by one warp; lane i holds h_i on entry and
-// returns x_i (lanes >= r return 0).  Right-looking substitutions.
-LRCCS_DEV float2 warp_chol_solve32(const float2 *L, const float *invd, int r, float2 h) {
-    const int i = threadIdx.x & 31;
-    for (int c = 0; c < r; ++c) {            // L z = h
-        const float2 hc = make_float2(__shfl_sync(0xffffffffu, h.x, c), __shfl_sync(0xffffffffu, h.y, c));
-        const float2 z = cscale(hc, invd[c]);
-        if (i == c) h = z;
-        else if (i > c && i < r) h = csub(h, cmul(L[i * r + c], z));
-    }
-    for (int c = r - 1; c >= 0; --c) {       // L^H x = z
-        const float2 hc = make_float2(__shfl_sync(0xffffffffu, h.x, c), __shfl_sync(0xffffffffu, h.y, c));
-        const float2 x = cscale(hc, invd[c]);
-        if (i == c) h = x;
-        else if (i < c) h = csub(h, cmulc(L[c * r + i], x));
-    }
-    return i < r ? h : make_float2(0.f, 0.f);
-}
-
-// ---------------------------------------------------------------- latency-lean FP64 r x r kernels
-// On this GPU a dependent FP64 FMA costs ~64 cycles and an FP64 square root or
-// division several hundred, so the r x r factorizations below avoid both: a
-// reciprocal square root / reciprocal is seeded in FP32 and refined by one
-// Newton step in FP64 (relative error ~1e-14), and every step spreads its
-// updates over the lanes of a warp (right-looking forms).
-
-LRCCS_DEV double d_rsqrt(double x) {   // 1/sqrt(x), x > 0
-    double y = (double)rsqrtf((float)x);
-    const double t = x * y * y;
-    return y * fma(-0.5, t, 1.5);
-}
-LRCCS_DEV double d_rcp(double x) {     // 1/x, x != 0
-    const double r = (double)__frcp_rn((float)x);
-    return fma(r, fma(-x, r, 1.0), r);
-}
-
-// In place A = L L^H (A Hermitian, FP64 (re, im) pairs, row-major, r <= 32):
-// the lower triangle of A receives L and invd[c] = 1 / L[c][c].  One warp;
-// lane i owns row i of the trailing matrix.  Returns false if A is not
-// positive definite (same value in every lane).
-LRCCS_DEV bool warp_cholesky_rl(double *A, int r, double *invd) {
-    const int lane = threadIdx.x & 31;
-    for (int c = 0; c < r; ++c) {
-        const double d = A[(c * r + c) * 2];
-        if (!(d > 0.0)) return false;
-        const double is = d_rsqrt(d);
-        // column c below the diagonal: L[i][c] = A[i][c] / sqrt(d)
-        double lr = 0.0, li = 0.0;
-        if (lane > c && lane < r) {
-            lr = A[(lane * r + c) * 2] * is;
-            li = A[(lane * r + c) * 2 + 1] * is;
-        }
-        __syncwarp();
-        if (lane == c) {
-            A[(c * r + c) * 2] = d * is;
-            A[(c * r + c) * 2 + 1] = 0.0;
-            invd[c] = is;
-        }
-        if (lane > c && lane < r) {
-            A[(lane * r + c) * 2] = lr;
-            A[(lane * r + c) * 2 + 1] = li;
-        }
-        __syncwarp();
-        // trailing update A[i][j] -= L[i][c] conj(L[j][c]) for c < j <= i, the
-        // (r-c-1)(r-c)/2 entries spread over the lanes
-        const int rt = r - c - 1;
-        for (int e = lane; e < rt * (rt + 1) / 2; e += 32) {
-            int a, b;
-            pair_of(e, rt, a, b);
-            const int j = c + 1 + a, i = c + 1 + b;
-            const double ar = A[(i * r + c) * 2], ai = A[(i * r + c) * 2 + 1];
-            const double br = A[(j * r + c) * 2], bi = A[(j * r + c) * 2 + 1];
-            A[(i * r + j) * 2] -= ar * br + ai * bi;
-            A[(i * r + j) * 2 + 1] -= ai * br - ar * bi;
-        }
-        __syncwarp();
-    }
-    return true;
-}
-
-// Solve L L^H x = h with the factor of warp_cholesky_rl; h and x are r (re, im)
-// pairs in shared memory (h is consumed).  Right-looking substitutions.
-LRCCS_DEV void warp_chol_solve_rl(const double *L, const double *invd, int r, double *h, double *x) {
-    const int lane = threadIdx.x & 31;
-    for (int c = 0; c < r; ++c) {            // L z = h  (z in h)
-        const double zr = h[2 * c] * invd[c], zi = h[2 * c + 1] * invd[c];
-        __syncwarp();
-        if (lane == c) {
-            h[2 * c] = zr;
-            h[2 * c + 1] = zi;
-        }
-        if (lane > c && lane < r) {          // h[i] -= L[i][c] z
-            const double ar = L[(lane * r + c) * 2], ai = L[(lane * r + c) * 2 + 1];
-            h[2 * lane] -= ar * zr - ai * zi;
-            h[2 * lane + 1] -= ar * zi + ai * zr;
-        }
-        __syncwarp();
-    }
-    for (int c = r - 1; c >= 0; --c) {       // L^H x = z
-        const double xr = h[2 * c] * invd[c], xi = h[2 * c + 1] * invd[c];
-        __syncwarp();
-        if (lane == c) {
-            x[2 * c] = xr;
-            x[2 * c + 1] = xi;
-        }
-        if (lane < c) {                      // z[i] -= conj(L[c][i]) x_c
-            const double ar = L[(c * r + lane) * 2], ai = -L[(c * r + lane) * 2 + 1];
-            h[2 * lane] -= ar * xr - ai * xi;
-            h[2 * lane + 1] -= ar * xi + ai * xr;
-        }
-        __syncwarp();
-    }
 }

@@ -41,11 +41,11 @@ enum { CNT_ENERGY = 0, CNT_GRAMX0, CNT_BAR, CNT_BAR_EXIT, CNT_BS_BAR, CNT_BS_EXI
 
 // Kernel ids (launch counting and optional CUDA-event timing).
 enum {
-    KID_ROWCOUNT = 0, KID_STRUCTURE, KID_FILL_IDX, KID_ENERGY, KID_INIT_ROWS, KID_INIT_COLS, KID_GRAM_X0,
+    KID_ROWCOUNT = 0, KID_STRUCTURE, KID_FILL_IDX, KID_ENERGY, KID_INIT_ROWS, KID_GRAM_X0,
     KID_EIG, KID_U0, KID_GDQR, KID_FWD_COLS, KID_ROW_GRAM, KID_SOLVE, KID_ROW_W, KID_ADJ_COLS,
     KID_IMAGES, KID_CG_INIT, KID_CG_STEP, KID_MEAN_RESID,
     // general (2D) masks
-    KID_UNION, KID_FILL_GEN, KID_INIT_GEN, KID_FWD_ROWS, KID_SAMPLE_GRAM, KID_SOLVE_GEN, KID_SAMPLE_W,
+    KID_UNION, KID_FILL_GEN, KID_FWD_ROWS, KID_SAMPLE_GRAM, KID_SOLVE_GEN, KID_SAMPLE_W,
     KID_ADJ_ROWS, KID_MEAN_RESID_GEN,
     // model-error correction (Alg. 3) and online tracking (Alg. 5)
     KID_MEC_MASK, KID_MEC_ELEM, KID_MEC_TDFT,
@@ -126,15 +126,13 @@ struct lrccs_ctx {
     std::string err;
 
     // geometry / sampling
-    float2 *d_twy, *d_twx;       // twiddles w_N^t, N = ny / nx
+    float2 *d_twx;               // twiddles w_nx^t
     float2 *d_twsy, *d_twsx;     // ny, nx: twiddles of the column and row passes with their scale, [j2][k1]
     uint16_t *d_ptab;            // q * ny * 32 sampled-point tables of the row passes (general masks, MEC)
     uint32_t *d_rowtab;          // (q + 17) * 32 sampled-row tables of the column passes (k_structure)
     float2 *d_smaps;             // nc * n
     int32_t *d_rowcnt;           // q * ny  samples of frame k in row ky
-    int32_t *d_rowidx;           // q * ny  line index of row ky in frame k, or -1
     int32_t *d_framerows;        // q * ny  row ky of line i of frame k, at lineptr[k] + i
-    int32_t *d_framek;           // q * ny  frame k of frame row lineptr[k] + i
     int32_t *d_mks;              // q       m_k, samples per coil of frame k
     int32_t *d_fpk;              // q + 1   frame sample offsets (the running sum of m_k)
     int32_t *d_rowoff;           // q * ny  first sample of (frame k, row ky) in the frame-ordered sample list
@@ -142,7 +140,6 @@ struct lrccs_ctx {
     int32_t *d_rfptr;            // ny + 1  frames sampling row ky: rflist[rfptr[ky] .. rfptr[ky+1])
     int32_t *d_rflist;           // q * ny
     int32_t *d_usedrows;         // ny      rows sampled by some frame
-    uint8_t *d_rowused;          // ny
     int32_t *d_idx;              // sample indices (capacity q * n)
     int32_t *d_meta;             // MT_COUNT ints, then the eigenvalue order (q ints)
     unsigned int *d_status;      // status word (ST_* bits)
@@ -184,7 +181,6 @@ struct lrccs_ctx {
     int32_t *d_uptr;             // ny + 1
     int32_t *d_ufrow;            // ny + 1
     int32_t *d_upos;             // n       union index of point i, or -1
-    int32_t *d_uidx;             // n_u     k-space index of union point u
     int32_t *d_ufptr;            // n_u + 1 frames sampling u: uflist[ufptr[u] .. ufptr[u+1])
     int32_t *d_uflist;           // sum m_k
     int32_t *d_fu;               // sum m_k union index of every frame sample (frame-ordered)
@@ -275,7 +271,6 @@ cudaError_t launch_fwd_only(lrccs_ctx *c);            // T <- F_y(d_j o U) on th
 cudaError_t launch_cg_init(lrccs_ctx *c, double *cg);
 cudaError_t launch_cg_step(lrccs_ctx *c, double *cg);
 cudaError_t launch_mean_resid(lrccs_ctx *c, const float2 *d_y, float2 *d_ytil, int nl_max);
-int npairs_of(int r);
 
 // Bits of the device status word ctx->d_status.
 enum {

@@ -126,13 +126,13 @@ __global__ void k_union_scan(const int32_t *__restrict__ urow, int ny, int32_t *
     }
 }
 
-// Per union point u (k-space index i): upos[i] = u, uidx[u] = i, and its frames
+// Per union point u (k-space index i): upos[i] = u, and its frames
 // in ascending order at uflist[ufptr[u] ..] (a deterministic order, so that
 // W_u is summed the same way on every run).
 __global__ void k_union_fill(const uint8_t *__restrict__ mask, const int32_t *__restrict__ uloc,
                              const int32_t *__restrict__ floc, const int32_t *__restrict__ uptr,
                              const int32_t *__restrict__ ufrow, int q, int nx, int n, int32_t *__restrict__ upos,
-                             int32_t *__restrict__ uidx, int32_t *__restrict__ ufptr, int32_t *__restrict__ uflist) {
+                             int32_t *__restrict__ ufptr, int32_t *__restrict__ uflist) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int l = uloc[i];
         if (l < 0) {
@@ -142,7 +142,6 @@ __global__ void k_union_fill(const uint8_t *__restrict__ mask, const int32_t *__
         const int ky = i / nx;
         const int u = uptr[ky] + l;
         upos[i] = u;
-        uidx[u] = i;
         const int f0 = ufrow[ky] + floc[i];
         ufptr[u] = f0;
         int cnt = 0;
@@ -188,7 +187,7 @@ cudaError_t launch_compact_general(lrccs_ctx *c, const uint8_t *d_mask) {
     prof_end(c, KID_UNION);
     prof_begin(c, KID_UNION);
     k_union_fill<<<blocks, 256, 0, c->stream>>>(d_mask, c->d_uloc, c->d_floc, c->d_uptr, c->d_ufrow, q, nx, n,
-                                                c->d_upos, c->d_uidx, c->d_ufptr, c->d_uflist);
+                                                c->d_upos, c->d_ufptr, c->d_uflist);
     prof_end(c, KID_UNION);
     prof_begin(c, KID_FILL_GEN);
     k_fill_general<<<(q * ny * 32 + 255) / 256, 256, 0, c->stream>>>(d_mask, c->d_rowcnt, c->d_rowoff, c->d_upos,

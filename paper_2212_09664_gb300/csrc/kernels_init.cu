@@ -56,8 +56,8 @@ __global__ void k_rowcount(const uint8_t *__restrict__ mask, int rows, int nx, i
 
 // Per-frame and per-row structure of the masks from the per-(frame, row)
 // sample counts.  Rows of a frame with at least one sample are the frame's
-// "frame rows" (its lines, for 1D Cartesian masks): lineptr / framerows /
-// framek / rowidx.  Also the frames' sample counts m_k and offsets fpk (checked
+// "frame rows" (its lines, for 1D Cartesian masks): lineptr /
+// framerows.  Also the frames' sample counts m_k and offsets fpk (checked
 // against the caller's frame_ptr), each (frame, row)'s first sample rowoff, the
 // rows sampled by some frame, meta[MT_GENERAL] = 1 when some row is only
 // partly sampled (a general 2D mask), and the column passes' row tables
@@ -83,9 +83,8 @@ LRCCS_DEV int warp_excl_sum(int v, int lane, int &total) {   // exclusive prefix
 }
 __global__ void __launch_bounds__(ST_NT) k_structure(
     const int32_t *__restrict__ rowcnt, const int64_t *__restrict__ fp_user, int q, int ny, int nx, int R1, int R2,
-    int32_t *rowidx, int32_t *framerows, int32_t *framek, int32_t *lineptr, int32_t *rfptr, int32_t *rflist,
-    int32_t *usedrows, uint8_t *rowused, int32_t *mks, int32_t *fpk, int32_t *rowoff, uint32_t *rowtab, float *xs, int32_t *meta,
-    unsigned int *status, double *scal) {
+    int32_t *framerows, int32_t *lineptr, int32_t *rfptr, int32_t *rflist, int32_t *usedrows, int32_t *mks,
+    int32_t *fpk, int32_t *rowoff, uint32_t *rowtab, float *xs, int32_t *meta, unsigned int *status, double *scal) {
     extern __shared__ int16_t s_cnt[];   // q x ny (a count is at most nx <= 256)
     __shared__ int s_lines[129], s_fp[129], s_rf[257], s_nu[257];
     __shared__ int s_partial, s_min, s_max, s_total;
@@ -125,10 +124,7 @@ __global__ void __launch_bounds__(ST_NT) k_structure(
         for (int k = lane; k < q; k += 32) c += s_cnt[k * ny + ky] > 0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (lane == 0) {
-            s_rf[ky] = c;
-            rowused[ky] = (uint8_t)(c > 0);
-        }
+        if (lane == 0) s_rf[ky] = c;
     }
     __syncthreads();
     if (warp == 0) {                              // prefixes over the frames (q <= 128)
@@ -186,17 +182,12 @@ __global__ void __launch_bounds__(ST_NT) k_structure(
     }
     for (int k = warp; k < q; k += nw) {          // frame k's rows, in order
         int i = s_lines[k], off = s_fp[k];
-        const int base = i;
         for (int y0 = 0; y0 < ny; y0 += 32) {
             const int ky = y0 + lane, e = k * ny + ky, c = s_cnt[e];
             int tl, tm;
             const int el = warp_excl_sum(c > 0, lane, tl), em = warp_excl_sum(c, lane, tm);
             rowoff[e] = off + em;
-            rowidx[e] = c > 0 ? i + el - base : -1;
-            if (c > 0) {
-                framerows[i + el] = ky;
-                framek[i + el] = k;
-            }
+            if (c > 0) framerows[i + el] = ky;
             i += tl;
             off += tm;
         }
@@ -240,9 +231,9 @@ cudaError_t launch_compact(lrccs_ctx *c, const uint8_t *d_mask, const int64_t *d
     DISPATCH_P(c->py, {
         using PL = fft::Plan<32 * P_>;
         k_structure<<<1, ST_NT, (size_t)c->q * c->ny * sizeof(int16_t), c->stream>>>(
-            c->d_rowcnt, d_fp_user, c->q, c->ny, c->nx, PL::R1, PL::R2, c->d_rowidx, c->d_framerows, c->d_framek,
-            c->d_lineptr, c->d_rfptr, c->d_rflist, c->d_usedrows, c->d_rowused, c->d_mks, c->d_fpk, c->d_rowoff,
-            c->d_rowtab, c->d_xs, c->d_meta, c->d_status, c->d_scal);
+            c->d_rowcnt, d_fp_user, c->q, c->ny, c->nx, PL::R1, PL::R2, c->d_framerows, c->d_lineptr, c->d_rfptr,
+            c->d_rflist, c->d_usedrows, c->d_mks, c->d_fpk, c->d_rowoff, c->d_rowtab, c->d_xs, c->d_meta, c->d_status,
+            c->d_scal);
     });
     prof_end(c, KID_STRUCTURE);
     return cudaGetLastError();

@@ -52,8 +52,6 @@ namespace cg = cooperative_groups;
 
 #define RMAXC 16   // compile-time bound on the rank
 
-int npairs_of(int r) { return r * (r + 1) / 2; }
-
 // ---------------------------------------------------------------- A: forward, along y
 //
 // The transforms along y act on the flat columns c = x r + l (rows of nx r
