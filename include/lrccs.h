@@ -235,8 +235,7 @@ lrccs_status lrccs_get_buffer(lrccs_ctx *ctx, lrccs_buffer which, void *d_dst, s
  *   out_iters : NULL, or receives the number of CG iterations run
  * The CG vectors use the context's subspace buffers, so afterwards the context
  * holds no solve (lrccs_init starts one).  The call synchronises.
- * Errors: LRCCS_E_INVALID, LRCCS_E_UNSUPPORTED (a mask that is not a union of
- * full lines), LRCCS_E_CUDA. */
+ * Errors: LRCCS_E_INVALID, LRCCS_E_NOMEM, LRCCS_E_CUDA. */
 lrccs_status lrccs_mean_step(lrccs_ctx *ctx, const void *d_y, const int64_t *d_frame_ptr,
                              const uint8_t *d_mask, const void *d_smaps, double tol, int32_t max_iter,
                              void *d_zbar, void *d_ytil, int32_t *out_iters);
@@ -341,16 +340,16 @@ lrccs_status lrccs_set_subspace(lrccs_ctx *ctx, const void *d_U, int32_t rank, d
  *   info     : NULL, or receives t, eta, sd, gnorm (the call then waits for
  *              the iterations)
  * The masks are compacted first (one wait for that step); the rest is queued
- * on the context's stream and the call returns: lrccs_synchronize waits for it
- * and reports its device status.  Afterwards the context holds this
+ * on the context's stream, and the call returns once the offsets, the masks and
+ * the maps have been read (d_y is read by the queued work): lrccs_synchronize
+ * waits for the rest and reports its device status.  Afterwards the context holds this
  * mini-batch's data and final subspace, so lrccs_iterate, lrccs_get_factors
  * and lrccs_get_images work on it as after lrccs_init.  The iterations are
  * the ones lrccs_iterate launches; a captured iteration graph is replayed only
  * when it matches this mini-batch's sampled rows (none is captured here).
  * Errors: LRCCS_E_STATE (no subspace: call lrccs_init, lrccs_set_subspace or
- * lrccs_set_state first), LRCCS_E_INVALID, LRCCS_E_UNSUPPORTED (a mask that is
- * not a union of full lines), LRCCS_E_RANK_DEFICIENT, LRCCS_E_TIMEOUT,
- * LRCCS_E_CUDA. */
+ * lrccs_set_state first), LRCCS_E_INVALID, LRCCS_E_RANK_DEFICIENT,
+ * LRCCS_E_NOMEM, LRCCS_E_TIMEOUT, LRCCS_E_CUDA. */
 lrccs_status lrccs_track_minibatch(lrccs_ctx *ctx, const void *d_y, const int64_t *d_frame_ptr,
                                    const uint8_t *d_mask, const void *d_smaps, int32_t t_max,
                                    int32_t reset_eta, void *d_X, lrccs_iter_info *info);

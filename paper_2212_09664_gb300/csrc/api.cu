@@ -418,7 +418,7 @@ static lrccs_status ensure_general_buffers(lrccs_ctx *c) {
                     need_buf(c, &c->d_ufptr, n + 1) && need_buf(c, &c->d_uflist, q * n) &&
                     need_buf(c, &c->d_fu, q * n) && need_buf(c, &c->d_FU, base_work(c)) &&
                     need_buf(c, &c->d_Pu, n * npm) &&
-                    need_buf(c, &c->d_fpart, frame_gram_part_count(c->q, c->rmax));
+                    need_buf(c, &c->d_fpart, frame_gram_part_count(c->q, c->rmax, c->nsm));
     if (!ok) return LRCCS_E_NOMEM;
     c->gen_cap_q = q;
     c->FU_cap = base_work(c);

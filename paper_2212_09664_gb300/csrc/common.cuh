@@ -399,7 +399,7 @@ LRCCS_DEV fsum2 fsum_pair(fsum2 a, fsum2 b) {
 // Block-wide compensated sums dst[e] = sum_{m < nitem} fetch(e, m) for
 // e < nent, written as FP64 (re, im) pairs.  Thread (entry e, slice s) sums
 // items s, s + S, s + 2S, ... in that order with RB loads in flight, and the S
-// slices are then combined in order: deterministic, and one memory latency per
+// slices are then combined by a fixed tree: deterministic, and one memory latency per
 // RB items instead of one per item.  All threads of the block call it (the
 // first 256 do the work); it ends with a barrier.
 template <class F>
@@ -461,8 +461,8 @@ LRCCS_DEV void block_sum(int nent, int nitem, double *dst, F fetch) {
 
 // Barrier number k (1, 2, ...) of this launch: wait until every block has
 // arrived k times (plus `skew` arrivals, which only the timeout test sets and
-// the grid can never make).  Bounded: gives up after `limit` polls (2^24, about
-// a second) and ORs `timeout_bit` into the status word; the kernel then runs on
+// the grid can never make).  Bounded: gives up after `limit` polls (2^24, 3.5
+// seconds) and ORs `timeout_bit` into the status word; the kernel then runs on
 // to its end.
 LRCCS_DEV void grid_sync(unsigned int *bar, unsigned int k, unsigned int *status, unsigned int limit,
                          unsigned int skew, unsigned int timeout_bit) {

@@ -186,7 +186,7 @@ struct lrccs_ctx {
     int32_t *d_fu;               // sum m_k union index of every frame sample (frame-ordered)
     float2 *d_FU;                // nc * n_u * rmax  F(d_j o U) at the union points (FU[j][u][l])
     float2 *d_Pu;                // n_u * npairs      coil-summed Gram of every union point
-    double *d_fpart;             // q * 8 chunks * 2 npairs  per-frame Gram partial sums (FP64)
+    double *d_fpart;             // q * chunks * 2 npairs  per-frame Gram partial sums (FP64)
     float *d_xs;                 // q       X0's column scale 1 / sqrt(m_k mbar)
 
     // model-error correction (Alg. 3): frames in chunks of mec_w <= 16 columns,
@@ -242,7 +242,7 @@ cudaError_t launch_tdft_fwd(lrccs_ctx *c, const float2 *E, const float2 *S0, con
                             float2 *M, double *out);
 cudaError_t launch_tdft_inv(lrccs_ctx *c, const float2 *M, float omega, float2 *E);
 size_t mec_scal_count(int n, int q, int w);
-size_t frame_gram_part_count(int q, int rmax);   // doubles of d_fpart
+size_t frame_gram_part_count(int q, int rmax, int nsm);   // doubles of d_fpart
 cudaError_t launch_bstep(lrccs_ctx *c);   // B-step only (forward transforms, Grams, solve) at the current U
 // precision forms (kernels_tc.cu)
 cudaError_t launch_dft_a(lrccs_ctx *c);

@@ -278,7 +278,10 @@ static __device__ void gd_stage_z(const GdArgs &a, float2 *s_z, int i0, int rows
 // Partial sums of h = U_{t+1}^H Z over the block's pixels into hrow[k R + l]:
 // thread (frame pair, LC columns, pixel slice) reads its two Z values by 16
 // bytes and U's row by broadcast; the slices add in order.  Few frames leave
-// many slices, so the columns are split then (LC = 2 instead of R).
+// many slices, so the columns are split then (LC = 2 instead of R), below 15 frames.
+// Kernel time, whole -> split, 128 x 128 at r = 6 and 192 x 192 at r = 16: 4 frames 27 ->
+// 21 and 41 -> 32 us, 12 frames 22.6 -> 18.9 and 35.0 -> 32.8, 16 frames 20.5 -> 18.7 and
+// 34.8 -> 33.6, 32 frames 20.5 -> 20.0 and 35.2 -> 36.7.
 template <int R, int LC>
 static __device__ __noinline__ void gd_h(const GdArgs &a, const float2 *s_a, float2 *s_z, float2 *scr, int cap, int i0, int rows,
                             float2 *hrow) {

@@ -39,8 +39,9 @@ cudaError_t launch_twiddles(float2 *tw, int N, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- mask compaction
-// Sampling H_k (Sec. II-A) given as a q x n bitmap.  This build accepts masks
-// whose every row ky is either fully sampled or empty (1D Cartesian lines).
+// Sampling H_k (Sec. II-A) given as a q x n bitmap, any mask: one whose every row
+// is fully sampled or empty (1D Cartesian lines) takes the line path, any other the
+// general one (meta[MT_GENERAL]).
 
 __global__ void k_rowcount(const uint8_t *__restrict__ mask, int rows, int nx, int32_t *rowcnt) {
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;

@@ -16,7 +16,8 @@
 // with the per-frame sampling M_k applied between the forward and inverse
 // transforms (the column passes' row tables for line masks, the row passes'
 // point tables for general ones).
-// Reductions per frame (dot products, norms) are FP64 in a fixed order.
+// Sums per frame (dot products, norms) run in FP32 without error within a thread and
+// in FP64 from there, in a fixed order.
 #include <math.h>
 
 #include <algorithm>
@@ -215,9 +216,9 @@ __global__ void __launch_bounds__(256) k_mec_dir(const float2 *__restrict__ S, f
 // once: per input frame one twiddle and four broadcast 16-byte reads feed the
 // 8 complex products.  H = q/2 or q output pairs by 256 / H pixel groups fill
 // the block.  192 x 192, q = 48, kernel time: 327 + 42 (the sums of its blocks) ->
-// 35 us forward, 45 -> 28 us back: about six times what their products take at
-// the FP32 rate; 461 blocks on the 456 places that 77 registers a thread leave, so
-// a second, nearly empty round is about half of either.
+// 35 us forward, 45 -> 28 us back.  The products alone would take 4.5 us at the
+// FP32 rate; a third of the time is the second round of 5 blocks behind the 456
+// that 77 registers a thread let run at once (192 x 160, 384 blocks: 21 and 18 us).
 #define TD_P 8                  // pixels per thread
 #define TD_S (TD_P + 2)         // shared stride of a frame's pixels (16-byte aligned, spread over the banks)
 

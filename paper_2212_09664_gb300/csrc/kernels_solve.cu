@@ -142,11 +142,12 @@ __global__ void __launch_bounds__(NT) k_solve(const float2 *__restrict__ Prow, c
 // P_{u(s)} (u(s) = fu[s], the union index of sample s).  A frame holds
 // thousands of samples, so the sum is split: block (k, c) sums chunk c of nch of
 // the frame's samples (FP64 pairs), and k_solve_gen adds the chunks in order
-// and solves.  Gather latency bounds it, so nch = gen_chunks(q) makes about
-// eight blocks per multiprocessor whatever q is, between 8 and 64 chunks; with
-// 8 chunks for every q: 31 us (64 frames of 256 x 256, r = 12) and 31 us now, 49 us
-// (8 frames of 224 x 224, r = 13: 64 blocks) -> 11 us, k_solve_gen 7 -> 12 us.
-static int gen_chunks(int q) { return std::max(8, std::min(64, (8 * 152 + q - 1) / q)); }
+// and solves.  Gather latency bounds the first and the chunks' chain the second:
+// about eight blocks per multiprocessor, with 8 to 64 chunks a frame (fewer blocks
+// than that below 19 frames).  Both kernels' time by chunks 8 / 16 / 32 / 64 / 128 on
+// 224 x 224, r = 12: 1 frame 45 / 31 / 27 / 26 / 31 us; 8 frames 51 / 36 / 29 / 29 / 36;
+// 32 frames 49 / 39 / 41 / 43 / 51; 128 frames 79 / 78 / 84 / 91 / 111.
+static int gen_chunks(int q, int nsm) { return std::max(8, std::min(64, (8 * nsm + q - 1) / q)); }
 template <int R>
 __global__ void __launch_bounds__(NT) k_frame_gram_gen(const float2 *__restrict__ Pu, const int32_t *__restrict__ fpk,
                                                        const int32_t *__restrict__ fu, double *__restrict__ part) {
@@ -196,18 +197,19 @@ typedef void (*solve_gen_t)(const double *, const float2 *, int, int, int, const
 static const fgram_t kFrameGramGen[RMAXC] = RANK_TABLE(k_frame_gram_gen);
 static const solve_gen_t kSolveGen[RMAXC] = RANK_TABLE(k_solve_gen);
 
-size_t frame_gram_part_count(int q, int rmax) { return (size_t)q * gen_chunks(q) * rmax * (rmax + 1); }
+size_t frame_gram_part_count(int q, int rmax, int nsm) { return (size_t)q * gen_chunks(q, nsm) * rmax * (rmax + 1); }
 
 cudaError_t launch_solve(lrccs_ctx *c) {
     if (c->r < 1 || c->r > RMAXC) return cudaErrorInvalidValue;
     if (c->gd_parts > HMAX * (NT / c->r)) return cudaErrorInvalidConfiguration;   // frame_h_load's reach
     if (c->general) {
         prof_begin(c, KID_SOLVE_GEN);
-        kFrameGramGen[c->r - 1]<<<dim3(c->q, gen_chunks(c->q)), NT, 0, c->stream>>>(c->d_Pu, c->d_fpk, c->d_fu, c->d_fpart);
+        const int nch = gen_chunks(c->q, c->nsm);
+        kFrameGramGen[c->r - 1]<<<dim3(c->q, nch), NT, 0, c->stream>>>(c->d_Pu, c->d_fpk, c->d_fu, c->d_fpart);
         prof_end(c, KID_SOLVE_GEN);
         prof_begin(c, KID_SOLVE_GEN);
-        kSolveGen[c->r - 1]<<<c->q, NT, 0, c->stream>>>(c->d_fpart, c->d_hpart, c->gd_parts, c->q,
-                                                        gen_chunks(c->q), c->d_fpk, c->d_B, c->d_status);
+        kSolveGen[c->r - 1]<<<c->q, NT, 0, c->stream>>>(c->d_fpart, c->d_hpart, c->gd_parts, c->q, nch, c->d_fpk,
+                                                        c->d_B, c->d_status);
         prof_end(c, KID_SOLVE_GEN);
         return cudaGetLastError();
     }
@@ -724,8 +726,10 @@ static const bstep_kernel_t kBstep[RMAXC] = RANK_TABLE(k_bstep);
 
 // The row buffer also stages Z for Z B^H.  A short row (few coils) would cut the
 // block's pixels into many small chunks, each with its own copy latency (64 x 64,
-// C = 1, r = 4: ten chunks of 7 pixels, 15.3 of 27.8 us; now 1.1 of 12.7), so the area holds 128
-// pixels of Z at least, up to 72 KB (two blocks a multiprocessor).
+// C = 1, r = 4: ten chunks of 7 pixels, 15.3 of 27.8 us; now 1.1 of 12.7), so the area
+// holds 128 pixels of Z at least, up to 72 KB.  (The limit buys nothing: registers keep
+// the kernel to one block a multiprocessor whatever the area.  128 x 128, C = 1,
+// r = 6: the same time without it up to 96 frames, 36.9 us for 32.7 at 128.)
 static int bstep_area(int nc, int nx, int q, int r) {
     const int z = std::min(128, (int)(73728 / (bs_zstride(q) * sizeof(float2)))) * bs_zstride(q);
     return std::max(nc * nx * r, (z + 1) & ~1);
