@@ -13,7 +13,7 @@ LRCCS_DEV float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y *
 // conj(a) * b
 LRCCS_DEV float2 cmulc(float2 a, float2 b) { return make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }
 // one packed instruction for both parts (the same two roundings): the transform
-// kernels are bound by instruction issue
+// kernels issue an instruction in up to half of their cycles
 LRCCS_DEV float2 cadd(float2 a, float2 b) {
     float2 d;
     asm("{\n.reg .b64 a, b, d;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nadd.rn.f32x2 d, a, b;\n"
