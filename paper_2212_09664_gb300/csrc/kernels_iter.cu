@@ -63,9 +63,9 @@ namespace cg = cooperative_groups;
 // (lane, group g) runs the length-R1 DFT of rows g + R2 m, the groups exchange
 // through shared memory once per coil (one block barrier: two exchange tiles),
 // and thread (lane, g) finishes with the length-R2 DFT of rows g + R1 k2.  The
-// tiles sit in L2; instructions issue in 49% of the forward and 37% of the adjoint
-// pass's cycles, the waits are for loads first (192 x 192, C = 12, r = 10, caches
-// cold, 18 warps a multiprocessor).  Both cost, so every shared address is a
+// tiles sit in L2; instructions issue in just under half of the forward and over a
+// third of the adjoint pass's cycles, the waits are for loads first (192 x 192,
+// C = 12, r = 10, caches cold, 18 warps a multiprocessor).  Both cost, so every shared address is a
 // constant offset from a per-thread base, the scale rides in the twiddles, and a
 // half-warp stages the coil map's few x of its own rows by cp.async one coil
 // ahead, which needs no further block barrier.
