@@ -432,7 +432,7 @@ static lrccs_status ensure_general_buffers(lrccs_ctx *c) {
 // 12 coils: 321 us a call with two waits through pageable memory behind those
 // copies, 302 us so).
 static lrccs_status queue_load(lrccs_ctx *c, const void *d_y, const int64_t *d_frame_ptr, const uint8_t *d_mask,
-                               const void *d_smaps, bool with_energy) {
+                               const void *d_smaps, bool with_energy, bool record) {
     CK(cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream));
     CK(cudaMemsetAsync(c->d_counters, 0, CNT_COUNT * sizeof(unsigned), c->stream));
     CK(cudaMemsetAsync(c->d_meta, 0, MT_COUNT * sizeof(int32_t), c->stream));
@@ -448,7 +448,7 @@ static lrccs_status queue_load(lrccs_ctx *c, const void *d_y, const int64_t *d_f
     CK(cudaMemcpyAsync(c->d_smaps, d_smaps, (size_t)c->nc * c->n * sizeof(float2), cudaMemcpyDeviceToDevice,
                        c->stream));
     CK(cudaMemcpyAsync(c->d_maskc, d_mask, (size_t)c->q * c->n, cudaMemcpyDeviceToDevice, c->stream));
-    CK(cudaEventRecord(c->ev_copied, c->stream));
+    if (record) CK(cudaEventRecord(c->ev_copied, c->stream));
     CK(cudaEventSynchronize(c->ev_counts));
     lrccs_status s = status_to_code(c, (unsigned)meta[MT_COUNT]);
     if (s != LRCCS_OK) return s;
@@ -493,17 +493,28 @@ static lrccs_status queue_load(lrccs_ctx *c, const void *d_y, const int64_t *d_f
 
 // Mask compaction, the sampled-row structure and Z = [A_k^H y_k] for the data
 // of one lrccs_init or tracking call; with_energy also forms gamma, which only
-// the spectral initialisation's truncation uses.  The caller may
-// change its frame offsets, mask and maps as soon as this returns, whatever it
-// returns: the copies out of them are waited for here, behind the launches that
-// follow them.
+// the spectral initialisation's truncation uses; record marks the point where
+// the caller's arrays have been copied.
 static lrccs_status load_data(lrccs_ctx *c, const void *d_y, const int64_t *d_frame_ptr, const uint8_t *d_mask,
-                              const void *d_smaps, bool with_energy) {
-    const lrccs_status s = queue_load(c, d_y, d_frame_ptr, d_mask, d_smaps, with_energy);
-    if (s == LRCCS_OK) CK(cudaEventSynchronize(c->ev_copied));
-    else cudaStreamSynchronize(c->stream);
+                              const void *d_smaps, bool with_energy, bool record) {
+    const lrccs_status s = queue_load(c, d_y, d_frame_ptr, d_mask, d_smaps, with_energy, record);
+    if (s != LRCCS_OK) cudaStreamSynchronize(c->stream);
     return s;
 }
+
+// The caller may change its frame offsets, mask and maps as soon as a call that
+// loads them returns, whatever it returns.  Each such call holds one of these,
+// which waits behind everything the call has queued: for the copies alone in the
+// call that returns before its work is done, else for the stream, which a call
+// that succeeds has waited for anyway.
+struct copies_guard {
+    lrccs_ctx *c;
+    bool recorded;
+    ~copies_guard() {
+        if (recorded) cudaEventSynchronize(c->ev_copied);
+        else cudaStreamSynchronize(c->stream);
+    }
+};
 
 extern "C" lrccs_status lrccs_init(lrccs_ctx *c, const void *d_y, const int64_t *d_frame_ptr, const uint8_t *d_mask,
                                    const void *d_smaps, int32_t *out_rank) {
@@ -522,7 +533,8 @@ extern "C" lrccs_status lrccs_init(lrccs_ctx *c, const void *d_y, const int64_t 
     c->t = 0;
     c->has_gamma = 0;
     CK(cudaMemsetAsync(c->d_scal, 0, SC_COUNT * sizeof(double), c->stream));
-    lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, true);
+    const copies_guard guard{c, false};
+    lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, true, false);
     if (s != LRCCS_OK) return s;
     CK(launch_gram_x0(c));
     if (c->dims.rank > 0 && c->dims.rank <= c->rmax) {
@@ -772,7 +784,8 @@ extern "C" lrccs_status lrccs_track_minibatch(lrccs_ctx *c, const void *d_y, con
         CK(cudaMemsetAsync(c->d_scal + SC_ETASET, 0, sizeof(double), c->stream));
         CK(cudaMemsetAsync(c->d_scal + SC_TCNT, 0, sizeof(double), c->stream));
     }
-    lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, false);
+    const copies_guard guard{c, true};
+    lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, false, true);
     if (s != LRCCS_OK) return s;
     s = warm_start(c);
     if (s != LRCCS_OK) return s;
@@ -837,7 +850,8 @@ extern "C" lrccs_status lrccs_mean_step(lrccs_ctx *c, const void *d_y, const int
     c->has_u = 0;
     c->need_h = 0;
     c->t = 0;
-    lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, false);
+    const copies_guard guard{c, false};
+    lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, false, false);
     if (s != LRCCS_OK) return s;
     const int r_save = c->r;
     c->r = 1;
@@ -988,7 +1002,8 @@ extern "C" lrccs_status lrccs_online_frames(lrccs_ctx *c, const void *d_y, const
         return LRCCS_E_STATE;
     }
     c->initialized = 0;
-    lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, false);
+    const copies_guard guard{c, false};
+    lrccs_status s = load_data(c, d_y, d_frame_ptr, d_mask, d_smaps, false, false);
     if (s != LRCCS_OK) return s;
     s = mec_ensure(c);
     if (s != LRCCS_OK) return s;
