@@ -32,6 +32,7 @@ void set_err(lrccs_ctx *c, const char *fmt, ...) {
 cudaError_t configure_kernels_init(int max_smem);
 cudaError_t configure_kernels_iter(int max_smem);
 cudaError_t configure_kernels_gd(int max_smem);
+cudaError_t configure_kernels_gd_many(int max_smem);
 cudaError_t configure_kernels_general(int max_smem);
 cudaError_t configure_kernels_tc(int max_smem);
 cudaError_t configure_kernels_zh(int max_smem);
@@ -257,6 +258,7 @@ static lrccs_status create_impl(const lrccs_dims *dims, const lrccs_params *para
     cudaError_t e = configure_kernels_init(optin);
     if (e == cudaSuccess) e = configure_kernels_iter(optin);
     if (e == cudaSuccess) e = configure_kernels_gd(optin);
+    if (e == cudaSuccess && c->gd_parts > c->gd_grid) e = configure_kernels_gd_many(optin);
     if (e == cudaSuccess) e = configure_kernels_general(optin);
     if (e == cudaSuccess) e = configure_kernels_tc(optin);
     if (e == cudaSuccess) e = configure_kernels_zh(optin);
@@ -1872,6 +1874,7 @@ extern "C" lrccs_status lrccs_test_few_blocks(lrccs_ctx *c, int32_t blocks) {
         set_err(c, "lrccs_test_few_blocks: blocks outside [1, %d], or more parts than the buffers hold", c->nsm);
         return LRCCS_E_INVALID;
     }
+    if (parts > g) CK(configure_kernels_gd_many(c->dev_smem_optin));
     CK(cudaStreamSynchronize(c->stream));
     drop_iter_graph(c);
     c->gd_grid = g;

@@ -654,22 +654,27 @@ typedef void (*gd_kernel_t)(GdArgs);
                      k_gdqr<7, M>,  k_gdqr<8, M>,  k_gdqr<9, M>,  k_gdqr<10, M>, k_gdqr<11, M>, k_gdqr<12, M>, \
                      k_gdqr<13, M>, k_gdqr<14, M>, k_gdqr<15, M>, k_gdqr<16, M>}
 static const gd_kernel_t kGd[2][RMAXC] = {GD_TABLE(false), GD_TABLE(true)};
-static int g_gd_static_smem[2 * RMAXC];
+static int g_gd_static_smem[2][RMAXC];
 #define GD_STATIC_MAX 16384   // no rank's static shared memory is above this (14880 bytes at 16)
 
-cudaError_t configure_kernels_gd(int max_smem) {
-    for (int i = 0; i < 2 * RMAXC; ++i) {
-        const gd_kernel_t k = kGd[i / RMAXC][i % RMAXC];
+static cudaError_t configure_gd(int max_smem, bool many) {
+    for (int i = 0; i < RMAXC; ++i) {
         cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, k);
+        cudaError_t e = cudaFuncGetAttributes(&fa, kGd[many][i]);
         if (e != cudaSuccess) return e;
         if (fa.sharedSizeBytes > GD_STATIC_MAX) return cudaErrorInvalidConfiguration;
-        g_gd_static_smem[i] = (int)fa.sharedSizeBytes;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - (int)fa.sharedSizeBytes);
+        g_gd_static_smem[many][i] = (int)fa.sharedSizeBytes;
+        e = cudaFuncSetAttribute(kGd[many][i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 max_smem - (int)fa.sharedSizeBytes);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
+cudaError_t configure_kernels_gd(int max_smem) { return configure_gd(max_smem, false); }
+// The form for several parts a block, loaded by the contexts that use it only: with
+// its 16 kernels beside the usual ones the others' code lies elsewhere, and an
+// iteration at 192 x 192, r = 10 took 2 us more.
+cudaError_t configure_kernels_gd_many(int max_smem) { return configure_gd(max_smem, true); }
 
 // Z row stride in shared memory: q rounded up to 2 mod 4 complex values, so
 // that 16-byte loads of consecutive pixels' rows hit distinct banks.
@@ -704,7 +709,7 @@ cudaError_t launch_gdqr(lrccs_ctx *c, int mode) {
     const int per = (c->n + c->gd_parts - 1) / c->gd_parts;
     const size_t fixed = gd_fixed(c->n, r, c->gd_parts);
     const bool many = c->gd_parts > G;
-    const size_t avail = (size_t)(c->dev_smem_optin - g_gd_static_smem[many * RMAXC + r - 1]);
+    const size_t avail = (size_t)(c->dev_smem_optin - g_gd_static_smem[many][r - 1]);
     if (fixed + 4 * zs * sizeof(float2) > avail) return cudaErrorInvalidConfiguration;
     // Z in one piece, or through two buffers of as many rows as fit
     const int rows = (int)((avail - fixed) / (zs * sizeof(float2)));
