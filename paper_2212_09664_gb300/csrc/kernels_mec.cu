@@ -349,14 +349,14 @@ __global__ void __launch_bounds__(256, 3) k_tdft_fwd(const float2 *__restrict__ 
 }
 
 // sum |M - Mprev|^2 and sum |Mprev|^2 over the frames k < q into out[0], out[1]
-// (blocks along the pixels, chunks).  FP32 without error per thread (fsum3; a
+// (blocks along the pixels, chunks).  FP32 without error within a warp (fsum3; a
 // difference is its rounded value d and that rounding e, exactly), FP64 from
 // there, in a fixed order.  FP64 work bounds every form that does more of it
 // (192 x 192, q = 48: 43 us all in FP64, 52 us with a range test and an FP64 side
 // path at each product), so one test covers an entry's four values and an entry
-// outside the range goes to FP64 as a whole: 21 us.  As a part of k_tdft_fwd, where
-// few warps are in flight, FP32 pairs took 28 us and lost the squares that leave
-// the FP32 range.
+// outside the range goes to FP64 as a whole: 21 us, and the warps add in FP32 too:
+// 19 us.  As a part of k_tdft_fwd, where few warps are in flight, FP32 pairs took
+// 28 us and lost the squares that leave the FP32 range.
 #define TD_CHANGE_BLOCKS 1024   // at most
 LRCCS_DEV void td_diff(fsum3 &s, float d, float e) {   // (d + e)^2, |e| at most half an ulp of d
     fsum3_product(s, d, d);
@@ -365,10 +365,24 @@ LRCCS_DEV void td_diff(fsum3 &s, float d, float e) {   // (d + e)^2, |e| at most
     two_sum(s.b, p, s.b, f);
     s.c += f + (fmaf(a, e, -p) + e * e);
 }
+LRCCS_DEV fsum3 td_warp_sum(fsum3 s) {   // the same in every lane
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float a = __shfl_xor_sync(0xffffffffu, s.a, o), b = __shfl_xor_sync(0xffffffffu, s.b, o);
+        const float c = __shfl_xor_sync(0xffffffffu, s.c, o);
+        float e, f, g;
+        two_sum(s.a, a, s.a, e);
+        two_sum(s.b, b, s.b, f);
+        two_sum(s.b, e, s.b, g);
+        s.c = (s.c + c) + (f + g);
+    }
+    return s;
+}
 __global__ void __launch_bounds__(256) k_tdft_change(const float2 *__restrict__ M, const float2 *__restrict__ Mprev,
                                                      int n, int q, int w, double *part, unsigned int *counter,
                                                      double *out) {
-    __shared__ double s_r[2][8];
+    __shared__ fsum3 s_f[2][8];
+    __shared__ double s_w[2][8];
     const unsigned total = (unsigned)n * w;
     const int cc = blockIdx.y, live = min(w, q - cc * w), lane = threadIdx.x & 31;
     const float2 *Mc = M + (size_t)cc * total, *Pc = Mprev + (size_t)cc * total;
@@ -403,17 +417,24 @@ __global__ void __launch_bounds__(256) k_tdft_change(const float2 *__restrict__ 
             pw += (double)m0.x * m0.x + (double)m0.y * m0.y;
         }
     }
-    const double a = warp_sum_d(dw + fsum3_total(dd)), b = warp_sum_d(pw + fsum3_total(pp));
+    dd = td_warp_sum(dd);
+    pp = td_warp_sum(pp);
+    if (__any_sync(0xffffffffu, dw != 0.0 || pw != 0.0)) {
+        dw = warp_sum_d(dw);
+        pw = warp_sum_d(pw);
+    }
     if (lane == 0) {
-        s_r[0][threadIdx.x >> 5] = a;
-        s_r[1][threadIdx.x >> 5] = b;
+        s_f[0][threadIdx.x >> 5] = dd;
+        s_f[1][threadIdx.x >> 5] = pp;
+        s_w[0][threadIdx.x >> 5] = dw;
+        s_w[1][threadIdx.x >> 5] = pw;
     }
     __syncthreads();
     const int id = blockIdx.y * gridDim.x + blockIdx.x, nb = gridDim.x * gridDim.y;
-    if (threadIdx.x < 2) {
-        double v = 0.0;
-        for (int x = 0; x < 8; ++x) v += s_r[threadIdx.x][x];
-        part[2 * id + threadIdx.x] = v;
+    if (threadIdx.x < 32) {   // lane (sum, warp)
+        double v = lane < 16 ? s_w[lane >> 3][lane & 7] + fsum3_total(s_f[lane >> 3][lane & 7]) : 0.0;
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0 || lane == 8) part[2 * id + (lane >> 3)] = v;
     }
     if (!last_block_arrive(counter) || threadIdx.x >= 64) return;
     const int c = threadIdx.x >> 5;   // a warp per sum
